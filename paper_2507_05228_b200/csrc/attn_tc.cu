@@ -55,12 +55,8 @@ namespace tc {
 constexpr int kThreads = 384;
 constexpr int kM = 128;                  // MMA rows per sub-tile
 constexpr int kNMax = 128;               // keys per KV tile (upper bound)
-constexpr int kD = 128;                  // head_dim
-constexpr int kTileBytes = kM * kD * 2;  // 32 KiB, laid out [2 halves][128 rows][128 bytes]
-constexpr int kHalfBytes = kTileBytes / 2;
-constexpr int kKStages = 2;  // (a third stage bought nothing)
-constexpr int kVStages = 2;
-constexpr uint32_t kTmemCols = 512;       // S0 | S1 | O0 | O1, 128 columns each; P_s aliases the start of S_s
+constexpr int kHalfBytes = kM * 128;     // one 64-column half of a 128-row tile: 128 rows of 128 bytes
+constexpr uint32_t kTmemCols = 512;
 constexpr float kRescaleThreshold = 8.f;  // log2 units
 // setmaxnreg only redistributes the registers the CTA was launched with (168 per thread x 384 threads = 64512), and
 // all four warps of an allocation group execute the same instruction: 8 warps x 32 x 216 + 4 warps x 32 x 72 = 64512.
@@ -71,32 +67,51 @@ static_assert(8 * 32 * kRegsSoftmax + 4 * 32 * kRegsOther <= 168 * kThreads, "se
 constexpr int kChunk = 32;                // keys per chunk of the KV stream
 constexpr int kChunkBytes = kChunk * 128; // one 64-column half of a chunk in a tile
 constexpr int kMaxShards = 256;           // KV shards per CTA whose bookkeeping fits in shared memory
-constexpr int kStageRowBytes = 272;       // output rows staged for the bulk copies: 256 bytes + 16 of padding
+constexpr int kMaxStages = 4;
 
-// shared memory map (offsets from a 1024-byte aligned base)
-constexpr int kOffQ = 0;
-constexpr int kOffK = kOffQ + 2 * kTileBytes;
-constexpr int kOffV = kOffK + kKStages * kTileBytes;
-constexpr int kOffBar = kOffV + kVStages * kTileBytes;
-static_assert(2 * kM * kStageRowBytes <= kOffV, "the output staging area must fit in the Q and K tiles");
-constexpr int kNumBars = 24;
-constexpr int kOffMisc = kOffBar + kNumBars * 8;   // tmem slot, abort flag, 12 progress words
-constexpr int kOffShard = kOffMisc + 64;           // int32 [5][kMaxShards], see ShardTab
-constexpr int kSmemBytes = kOffShard + 5 * kMaxShards * 4 + 1024;  // + alignment slack
-static_assert(kSmemBytes <= 232448, "exceeds the 227 KiB a CTA may use");
+// What depends on the head_dim D.
+//   D = 128: TMEM = S0 | S1 | O0 | O1, 128 columns each; the probabilities P_s overwrite the start of S_s, so the next
+//            logits of a sub-tile wait for the product that reads its P.
+//   D = 64:  TMEM = three logit buffers of 128 columns | O0 | O1 of 64.  The sub-tiles take turns on the three buffers
+//            (sub-tile s, tile i: buffer (2 i + s) mod 3), so the next logits of a sub-tile are computed while it is still
+//            in the softmax of the current tile.  P is kept to twice the precision there: a bf16 part and the bf16
+//            rest, which together fill the 128 columns of the buffer they overwrite.
+template <int D>
+struct Cfg {
+  static constexpr int kHalves = D / 64;
+  static constexpr int kTileBytes = kHalves * kHalfBytes;  // [halves][128 rows][128 bytes]
+  static constexpr int kKStages = D == 64 ? 4 : 2;         // (D = 128: a third stage bought nothing)
+  static constexpr int kVStages = D == 64 ? 3 : 2;
+  static constexpr bool kRing = D == 64;                   // three logit buffers, P in two parts
+  static constexpr uint32_t kOCol = kRing ? 384u : 256u;   // first accumulator column
+  static constexpr int kRowBytes = D * 2;
+  static constexpr int kStageRowBytes = kRowBytes + 16;    // output rows staged for the bulk copies, padded by 16 bytes
+  // shared memory map (offsets from a 1024-byte aligned base)
+  static constexpr int kOffQ = 0;
+  static constexpr int kOffK = kOffQ + 2 * kTileBytes;
+  static constexpr int kOffV = kOffK + kKStages * kTileBytes;
+  static constexpr int kOffBar = kOffV + kVStages * kTileBytes;
+  static_assert(2 * kM * kStageRowBytes <= kOffV, "the output staging area must fit in the Q and K tiles");
+  static constexpr int kNumBars = 28;
+  static constexpr int kOffMisc = kOffBar + kNumBars * 8;   // tmem slot, abort flag, 12 progress words
+  static constexpr int kOffShard = kOffMisc + 64;           // int32 [5][kMaxShards], see ShardTab
+  static constexpr int kSmemBytes = kOffShard + 5 * kMaxShards * 4 + 1024;  // + alignment slack
+  static_assert(kSmemBytes <= 232448, "exceeds the 227 KiB a CTA may use");
+};
 
 enum Bar {
-  Q_FULL = 0,                     // [2]
-  K_FULL = 2,                     // [kKStages]
-  K_EMPTY = K_FULL + kKStages,    // [kKStages]
-  V_FULL = K_EMPTY + kKStages,    // [kVStages]
-  V_EMPTY = V_FULL + kVStages,    // [kVStages]
-  S_FULL = V_EMPTY + kVStages,    // [2]
-  P_FULL = S_FULL + 2,            // [2]
-  O_FULL = P_FULL + 2,            // [1]
-  O_RDY = O_FULL + 1              // [2]  kWalk: the accumulator of a sub-tile holds a finished shard
+  Q_FULL = 0,                       // [2]
+  K_FULL = 2,                       // [kKStages]
+  K_EMPTY = K_FULL + kMaxStages,    // [kKStages]
+  V_FULL = K_EMPTY + kMaxStages,    // [kVStages]
+  V_EMPTY = V_FULL + kMaxStages,    // [kVStages]
+  S_FULL = V_EMPTY + kMaxStages,    // [2]; kRing: [2][2], see s_full
+  P_FULL = S_FULL + 4,              // [2]
+  O_FULL = P_FULL + 2,              // [1]
+  O_RDY = O_FULL + 1                // [2]  kWalk: the accumulator of a sub-tile holds a finished shard;
+                                    //      kRing: the product of a sub-tile's latest tile is in its accumulator
 };
-static_assert(O_RDY + 2 <= kNumBars, "barrier table too small");
+static_assert(O_RDY + 2 <= Cfg<128>::kNumBars, "barrier table too small");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -358,19 +373,29 @@ struct TmaArgs {
 // one after another): the shards are walked as in the fused mode, but a tile never mixes two shards, and at a shard
 // boundary the softmax threads write that shard's (u, m, l) out and start over.  The query tile, the TMEM allocation,
 // the barriers and the K/V pipelines are set up once per query tile instead of once per (query tile, KV shard).
-template <bool kRope, bool kWalk>
+template <int D, bool kRope, bool kWalk>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_constant__ AttnParams p, int lg,
                                                               int tile_major,
                                                               const __grid_constant__ TmaArgs tma) {
+  using C = Cfg<D>;
+  constexpr int kD = D, kTileBytes = C::kTileBytes, kKStages = C::kKStages, kVStages = C::kVStages;
+  constexpr int kOffQ = C::kOffQ, kOffK = C::kOffK, kOffV = C::kOffV, kOffMisc = C::kOffMisc;
+  constexpr int kStageRowBytes = C::kStageRowBytes;
+  constexpr bool kRing = C::kRing;
+  static_assert(!kRope || D == 128, "the rotary step is fused for head_dim 128 only");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
-  const uint32_t bar0 = smem_base + kOffBar;
+  const uint32_t bar0 = smem_base + C::kOffBar;
   auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+  // Logits of sub-tile s, tile i.  With kRing they may be two tiles ahead of a softmax thread, which a phase parity cannot
+  // tell from "not there yet": even and odd tiles have a barrier each (tile i + 2 is issued after the thread's P(i)).
+  auto s_full = [&](int s, int i) { return bar(S_FULL + (kRing ? 2 * (i & 1) : 0) + s); };
+  auto s_parity = [&](int i) { return (uint32_t)((kRing ? i >> 1 : i) & 1); };
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kOffMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 4);
   volatile int* progress = reinterpret_cast<volatile int*>(smem + kOffMisc + 8);  // [12]
-  ShardTab* tab = reinterpret_cast<ShardTab*>(smem + kOffShard);
+  ShardTab* tab = reinterpret_cast<ShardTab*>(smem + C::kOffShard);
   volatile int* stream_info = reinterpret_cast<volatile int*>(smem + kOffMisc + 56);  // [0] active shards, [1] chunks
 
   // lg = log2(Gp): Gp heads stacked per tile, R = 128 / Gp slots per sub-tile, 2 R slots per CTA
@@ -419,8 +444,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   // caller's tensor, 16 bytes per thread and row, half a warp per 256-byte row.  The loads are issued here, before the
   // set-up below, and land in shared memory (128-byte-swizzled [2][128][128 B] layout) after it.  Rows past the end
   // of the sub-tile repeat its last row (their results are discarded).
-  uint4 qv[16];
-  const int q_chunk = tid & 15;
+  constexpr int kRowChunks = kD / 8;            // 16-byte pieces of a row
+  constexpr int kRowsPerPass = 128 / kRowChunks;  // rows the 128 threads of a sub-tile load at a time
+  uint4 qv[kRowChunks];
+  const int q_chunk = tid & (kRowChunks - 1);
+  const int q_row = (tid & 127) / kRowChunks;
   const float4* rope_row[kRope ? 8 : 1];  // this thread's slice of the table row of each of its query rows
   float4 cs[kRope ? 4 : 1][4];            // (cos, sin) of four rows: 8 pairs each
   if (warp < 8 && (warp >> 2) < n_sub) {
@@ -449,8 +477,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     } else {
       const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(p.q) + (int64_t)b * p.qs.batch + q_chunk * 8;
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int r = (tid >> 4 & 7) + 8 * j;
+      for (int j = 0; j < kRowChunks; ++j) {
+        const int r = q_row + kRowsPerPass * j;
         const int tok =
             (int)CASCADE_CHECKED((int64_t)__ldg(q_idx + sub_row0 + min(r >> lg, sub_nrows - 1)), pl.n_q, pl.status, 108);
         qv[j] = __ldg(reinterpret_cast<const uint4*>(qb + (int64_t)tok * p.qs.token +
@@ -507,6 +535,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(bar(S_FULL + s), 1);
+      mbar_init(bar(S_FULL + 2 + s), 1);
       mbar_init(bar(P_FULL + s), 128);
     }
     mbar_init(bar(O_FULL), 1);
@@ -548,8 +577,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       const int32_t* vis_row = vis + (size_t)slot * P;
       const int32_t* vis_first = tab->first[s];  // shortest prefix of the sub-tile, per active shard
       const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-      const uint32_t s_addr = lane_base + (uint32_t)(s * 128);
-      const uint32_t o_addr = lane_base + 256u + (uint32_t)(s * 128);
+      uint32_t s_addr = lane_base + (uint32_t)(s * 128);  // kRing: the buffer of the current tile
+      const uint32_t o_addr = lane_base + C::kOCol + (uint32_t)(s * kD);
       const float c = p.scale * 1.4426950408889634f;  // logits are kept in log2 units: x = s * scale * log2(e)
       const uint64_t c2 = pack2(c, c);
       float m_run = -INFINITY;   // reference max the accumulators are scaled by (may lag by < 2^8)
@@ -587,8 +616,8 @@ if constexpr (kRope) {
         } else {
           uint8_t* q_tile = smem + kOffQ + s * kTileBytes + (q_chunk >> 3) * kHalfBytes;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int r = (tid >> 4 & 7) + 8 * j;
+          for (int j = 0; j < kRowChunks; ++j) {
+            const int r = q_row + kRowsPerPass * j;
             *reinterpret_cast<uint4*>(q_tile + r * 128 + (((q_chunk & 7) ^ (r & 7)) << 4)) = qv[j];
           }
         }
@@ -622,7 +651,7 @@ if constexpr (kRope) {
         // 64 columns per round trip, then 32-byte stores: a row's 16-byte pieces would half-fill 32 sectors per store
         // instruction
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
+        for (int half = 0; half < C::kHalves; ++half) {
         uint32_t o[64];
         CASCADE_TMEM_LD32(o_addr + (uint32_t)(half * 64), o, 0);
         CASCADE_TMEM_LD32(o_addr + (uint32_t)(half * 64 + 32), o, 32);
@@ -684,7 +713,7 @@ if constexpr (kRope) {
           // product of this shard (which overwrites the accumulator) waits for this thread's arrival on P_FULL(i).
           if (opens) {
             if (i > 0) {
-              wait_bar(wc, bar(O_RDY + s), (uint32_t)(n_flushed & 1), 2, i);
+              wait_bar(wc, bar(O_RDY + s), (uint32_t)((kRing ? i - 1 : n_flushed) & 1), 2, i);
               tc_fence_after();
               flush_shard(kk_open);
               ++n_flushed;
@@ -692,8 +721,9 @@ if constexpr (kRope) {
             kk_open = kk_tile;
           }
         }
-        wait_bar(wc, bar(S_FULL + s), (uint32_t)(i & 1), 1, i);
+        wait_bar(wc, s_full(s, i), s_parity(i), 1, i);
         tc_fence_after();
+        if constexpr (kRing) s_addr = lane_base + (uint32_t)((2 * i + s) % 3) * 128u;
         uint32_t sr[128];
         CASCADE_TMEM_LD32(s_addr, sr, 0);
         if (nch > 1) CASCADE_TMEM_LD32(s_addr + 32, sr, 32);
@@ -733,7 +763,7 @@ if constexpr (kRope) {
         const uint64_t neg_m2 = pack2(neg_m, neg_m);
         uint64_t psum2 = pack2(0.f, 0.f);
         auto exp_chunk = [&](int ch) {
-          uint32_t pk[16];
+          uint32_t pk[16], pr[kRing ? 16 : 1];
 #pragma unroll
           for (int j = 0; j < 32; j += 2) {
             float x0, x1;
@@ -741,10 +771,18 @@ if constexpr (kRope) {
                     x1);
             const float p0 = ex2(x0), p1 = ex2(x1);
             psum2 = fadd2(psum2, pack2(p0, p1));
-            pk[j >> 1] = pack_bf16x2(p0, p1);
+            if constexpr (kRing) {
+              // the upper 16 bits, and what they leave out rounded to bf16: together within 2^-17 of the fp32 weight
+              pk[j >> 1] = __byte_perm(__float_as_uint(p0), __float_as_uint(p1), 0x7632);
+              pr[j >> 1] = pack_bf16x2(p0 - __uint_as_float(__float_as_uint(p0) & 0xffff0000u),
+                                       p1 - __uint_as_float(__float_as_uint(p1) & 0xffff0000u));
+            } else {
+              pk[j >> 1] = pack_bf16x2(p0, p1);
+            }
           }
           // P as the A operand of the PV product: lane = row, column kk holds keys 2 kk and 2 kk + 1
           CASCADE_TMEM_ST16(s_addr + (uint32_t)(16 * ch), pk);
+          if constexpr (kRing) CASCADE_TMEM_ST16(s_addr + 64u + (uint32_t)(16 * ch), pr);
         };
         if (nch == 4) {
           // The full tile is one straight-line block, so that the scheduler can run the MUFU instructions of one chunk
@@ -766,16 +804,25 @@ if constexpr (kRope) {
         // dominates a row its rounding error (up to 2^-9 relative) would go straight into O / l: 0.009 at |v| = 4.5.
         // The sum therefore takes the tile's largest weight as the tensor core sees it (same fma and ex2 as in the
         // loop above, so the same bits); the other weights' errors are small against l or average out.
-        const float p_top = ex2(fmaf(smax, c, neg_m));
-        const float p_top_seen = __uint_as_float(pack_bf16x2(0.f, p_top) & 0xffff0000u);
-        l_run = l_run * alpha + ((psum0 + psum1) + (p_top_seen - p_top));
+        // (Not with kRing, whose weights keep 16 bits of mantissa.)
+        float top_err = 0.f;
+        if constexpr (!kRing) {
+          const float p_top = ex2(fmaf(smax, c, neg_m));
+          top_err = __uint_as_float(pack_bf16x2(0.f, p_top) & 0xffff0000u) - p_top;
+        }
+        l_run = l_run * alpha + ((psum0 + psum1) + top_err);
         // S_FULL(i) was committed after PV(i-1), so the output accumulator is quiescent until this thread's
-        // arrival on P_FULL(i) below
+        // arrival on P_FULL(i) below.  With kRing the logits run ahead of the products, and O_RDY says when PV(i-1) is in
+        // (it cannot complete twice without this thread's arrival, so waiting only when needed keeps the parity exact).
         if (!opens && __any_sync(0xffffffffu, changed)) {
+          if constexpr (kRing) {
+            wait_bar(wc, bar(O_RDY + s), (uint32_t)((i - 1) & 1), 2, i);
+            tc_fence_after();
+          }
           // rescale this warp's 32 rows of the output accumulator
           const float f = changed ? alpha : 1.f;
 #pragma unroll
-          for (int cc = 0; cc < 4; ++cc) {
+          for (int cc = 0; cc < kD / 32; ++cc) {
             uint32_t o[32];
             CASCADE_TMEM_LD32(o_addr + (uint32_t)(cc * 32), o, 0);
             tmem_wait_ld();
@@ -825,11 +872,11 @@ if constexpr (kRope) {
         }
       }
       // Every product of the CTA has completed, so the Q / K tiles in shared memory are free: the thread stages its
-      // 256-byte output row there (rows 272 bytes apart, which spreads a warp's 16-byte stores over all banks) and hands
+      // output row there (rows 16 bytes further apart than they are long, which spreads a warp's 16-byte stores over all banks) and hands
       // it to the copy engine as one bulk copy, instead of writing 32-byte pieces of 32 different rows per instruction.
       uint8_t* stage = smem + kOffQ + (s * kM + m) * kStageRowBytes;
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
+      for (int cc = 0; cc < kD / 32; ++cc) {
         uint32_t o[32];
         if (n_tiles > 0) {
           CASCADE_TMEM_LD32(o_addr + (uint32_t)(cc * 32), o, 0);
@@ -850,7 +897,8 @@ if constexpr (kRope) {
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // this thread's writes -> the copy engine's reads
       if (row_ok) {
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], 256;" ::"l"(dst), "r"(smem_u32(stage))
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(stage)),
+                     "n"(C::kRowBytes)
                      : "memory");
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the row has left shared memory
@@ -870,7 +918,7 @@ if constexpr (kRope) {
             p.l_part[st2] = 0.f;
             uint4* row = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.o_part) + st2 * kD);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) row[j] = make_uint4(0u, 0u, 0u, 0u);
+            for (int j = 0; j < kRowChunks; ++j) row[j] = make_uint4(0u, 0u, 0u, 0u);
           }
         }
       }
@@ -890,6 +938,9 @@ if constexpr (kRope) {
       const uint32_t k_lo0 = desc_lo(smem_base + kOffK, 16);
       const uint32_t v_lo0 = desc_lo(smem_base + kOffV, kHalfBytes);  // the two 64-column halves of d
       if (n_tiles > 0) {
+        auto s_col = [&](int s, int i) {  // logit buffer of sub-tile s, tile i
+          return tmem + (uint32_t)((kRing ? (2 * i + s) % 3 : s) * 128);
+        };
         auto issue_qk = [&](int s, int i, int n) {  // S_s = Q_s K(i)^T, n keys wide
           const uint32_t q_lo = q_lo0 + (uint32_t)(s * (kTileBytes >> 4));
           const uint32_t k_lo = k_lo0 + (uint32_t)((i % kKStages) * (kTileBytes >> 4));
@@ -899,9 +950,9 @@ if constexpr (kRope) {
             for (int ks = 0; ks < kD / 16; ++ks) {
               // 16 elements of head_dim = 32 bytes along the 128-byte row; elements 64.. live in the second half
               const uint32_t off = (uint32_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4);
-              mma_ss(tmem + (uint32_t)(s * 128), q_lo + off, k_lo + off, hi_kmajor, idesc_qk, ks > 0);
+              mma_ss(s_col(s, i), q_lo + off, k_lo + off, hi_kmajor, idesc_qk, ks > 0);
             }
-            mma_commit(bar(S_FULL + s));
+            mma_commit(s_full(s, i));
           }
         };
         // O_s (+)= P_s V(i) over n keys; a tile that opens a shard (kWalk) or the stream starts the accumulator afresh
@@ -913,8 +964,16 @@ if constexpr (kRope) {
             for (int ks = 0; ks < kNMax / 16; ++ks) {
               // A = P from TMEM: 16 keys = 8 columns; B = V (MN-major): 16 keys = 16 rows of 128 bytes
               if (ks < ksteps)
-                mma_ts(tmem + 256u + (uint32_t)(s * 128), tmem + (uint32_t)(s * 128 + ks * 8),
+                mma_ts(tmem + C::kOCol + (uint32_t)(s * kD), s_col(s, i) + (uint32_t)(ks * 8),
                        v_lo + (uint32_t)(ks * (2048 >> 4)), hi_v, idesc_pv, !opens || ks > 0);
+            }
+            if constexpr (kRing) {  // the rest of P
+#pragma unroll
+              for (int ks = 0; ks < kNMax / 16; ++ks)
+                if (ks < ksteps)
+                  mma_ts(tmem + C::kOCol + (uint32_t)(s * kD), s_col(s, i) + (uint32_t)(64 + ks * 8),
+                         v_lo + (uint32_t)(ks * (2048 >> 4)), hi_v, idesc_pv, true);
+              mma_commit(bar(O_RDY + s));
             }
           }
         };
@@ -928,6 +987,48 @@ if constexpr (kRope) {
           issue_qk(s, 0, n_cur);
         }
         if (leader) mma_commit(bar(K_EMPTY));
+        if constexpr (kRing) {
+          // Order: QK_0(0) QK_1(0) QK_0(1), then per tile i: PV_0(i) QK_1(i+1) PV_1(i) QK_0(i+2).  QK_1(i+1) takes the
+          // buffer PV_0(i) has read, QK_0(i+2) the one of PV_1(i); MMAs execute in issue order, so neither needs a
+          // barrier.  K(j) is released after QK_1(j), the later of its two readers.
+          const int last_sub = n_sub - 1;
+          auto wait_k = [&](int i) {
+            wait_bar(wc, bar(K_FULL + i % kKStages), (uint32_t)((i / kKStages) & 1), 7, i);
+            tc_fence_after();
+          };
+          bool opens_2 = false;
+          int n_2 = 0;
+          if (n_tiles > 1) {
+            n_next = kChunk * seq.next(opens_next);
+            wait_k(1);
+            issue_qk(0, 1, n_next);
+            if (last_sub == 0 && leader) mma_commit(bar(K_EMPTY + 1 % kKStages));
+          }
+          for (int i = 0; i < n_tiles; ++i) {
+            n_2 = i + 2 < n_tiles ? kChunk * seq.next(opens_2) : 0;
+            wait_bar(wc, bar(V_FULL + i % kVStages), (uint32_t)((i / kVStages) & 1), 4, i);
+            for (int s = 0; s < n_sub; ++s) {
+              note(8 * i + 2 + s);
+              wait_bar(wc, bar(P_FULL + s), (uint32_t)(i & 1), 5, i);
+              tc_fence_after();
+              issue_pv(s, i, n_cur, opens_cur);
+              if (s == last_sub && leader) mma_commit(bar(V_EMPTY + i % kVStages));
+              if (s == 0 && n_sub == 2 && i + 1 < n_tiles) {
+                issue_qk(1, i + 1, n_next);
+                if (leader) mma_commit(bar(K_EMPTY + (i + 1) % kKStages));
+              }
+              if (s == last_sub && i + 2 < n_tiles) {
+                wait_k(i + 2);
+                issue_qk(0, i + 2, n_2);
+                if (last_sub == 0 && leader) mma_commit(bar(K_EMPTY + (i + 2) % kKStages));
+              }
+            }
+            n_cur = n_next;
+            opens_cur = opens_next;
+            n_next = n_2;
+            opens_next = opens_2;
+          }
+        } else
         for (int i = 0; i < n_tiles; ++i) {
           const bool has_next = i + 1 < n_tiles;
           if (i > 0) {
@@ -985,14 +1086,14 @@ if constexpr (kRope) {
           note(8 * i + 1);
           wait_bar(wc, bar(empty0 + st), (uint32_t)(((i / n_stages) & 1) ^ 1), is_k ? 9 : 10, i);
           const uint32_t dst = tiles_s + (uint32_t)(st * kTileBytes), fb = bar(full0 + st);
-          if (leader) mbar_expect_tx(fb, (uint32_t)(nch * 2 * kChunkBytes));
+          if (leader) mbar_expect_tx(fb, (uint32_t)(nch * C::kHalves * kChunkBytes));
           for (int ch = 0; ch < nch; ++ch) {
             // A chunk is 32 consecutive rows of the shard-major copy.  Rows past the shard's visible prefix belong
             // to later keys or, past the end of the matrix, are zero-filled: they are masked either way.
             const int slot = tab->slot0[cur.j] + cur.c * kChunk;
             if (leader) {
               tma_tile3(dst + (uint32_t)(ch * kChunkBytes), map, 0, slot, z, fb);
-              tma_tile3(dst + (uint32_t)(kHalfBytes + ch * kChunkBytes), map, 64, slot, z, fb);
+              if (C::kHalves == 2) tma_tile3(dst + (uint32_t)(kHalfBytes + ch * kChunkBytes), map, 64, slot, z, fb);
             }
             cur.advance(tab, n_act);
           }
@@ -1031,11 +1132,11 @@ EncodeTiledFn encode_tiled_fn() {
 }
 
 // Shard-major K or V copy as a 3-D tensor [batch * kv_heads][n_kv][head_dim]; box = one chunk (32 rows) x 64 columns.
-bool encode_sorted(CUtensorMap* map, const void* base, int64_t n_kv, int64_t n_mats) {
+bool encode_sorted(CUtensorMap* map, const void* base, int d, int64_t n_kv, int64_t n_mats) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return false;
-  const cuuint64_t dims[3] = {(cuuint64_t)tc::kD, (cuuint64_t)n_kv, (cuuint64_t)n_mats};
-  const cuuint64_t strides[2] = {(cuuint64_t)tc::kD * 2, (cuuint64_t)n_kv * tc::kD * 2};
+  const cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)n_kv, (cuuint64_t)n_mats};
+  const cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)n_kv * d * 2};
   const cuuint32_t box[3] = {64, (cuuint32_t)tc::kChunk, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
@@ -1061,13 +1162,16 @@ int sm_count() {
 cudaError_t launch_attn_tc(const AttnParams& p, const void* k_sorted, const void* v_sorted, cudaStream_t stream) {
   // the unfused route walks all KV shards of a query tile in one CTA (CASCADE_PARTIALS_WALK=0: a CTA per pair)
   const bool walk = !p.fused && CASCADE_PARTIALS_WALK && p.plan.n_kv_shards > 1;
-  auto kernel = p.rope ? tc::attn_tc_kernel<true, false>
-                       : (walk ? tc::attn_tc_kernel<false, true> : tc::attn_tc_kernel<false, false>);
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes);
+  auto kernel = p.d == 64 ? (walk ? tc::attn_tc_kernel<64, false, true> : tc::attn_tc_kernel<64, false, false>)
+                : p.rope  ? tc::attn_tc_kernel<128, true, false>
+                          : (walk ? tc::attn_tc_kernel<128, false, true> : tc::attn_tc_kernel<128, false, false>);
+  const int smem_bytes = p.d == 64 ? tc::Cfg<64>::kSmemBytes : tc::Cfg<128>::kSmemBytes;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
   tc::TmaArgs tma;
   const int64_t n_mats = (int64_t)p.batch * p.Hkv;
-  if (!encode_sorted(&tma.k, k_sorted, p.plan.n_kv, n_mats) || !encode_sorted(&tma.v, v_sorted, p.plan.n_kv, n_mats)) {
+  if (!encode_sorted(&tma.k, k_sorted, p.d, p.plan.n_kv, n_mats) ||
+      !encode_sorted(&tma.v, v_sorted, p.d, p.plan.n_kv, n_mats)) {
     set_error("tensor-core attention: could not build the TMA descriptors of the shard-major K/V copies");
     return cudaErrorInvalidValue;
   }
@@ -1084,7 +1188,7 @@ cudaError_t launch_attn_tc(const AttnParams& p, const void* k_sorted, const void
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)n_ctas);
   cfg.blockDim = dim3(tc::kThreads);
-  cfg.dynamicSmemBytes = tc::kSmemBytes;
+  cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -600,12 +600,12 @@ static bool use_decode(const cascade_plan_t* plan, cascade_dtype_t dtype, int H,
 }
 static bool use_tc(const cascade_plan_t* plan, cascade_dtype_t dtype, int d) {
   // the tensor-core kernel keeps per-shard bookkeeping in shared memory: at most 256 KV shards
-  return dtype == CASCADE_BF16 && d == 128 && plan->dev.n_q > 1 && plan->dev.n_kv_shards <= 256;
+  return dtype == CASCADE_BF16 && (d == 64 || d == 128) && plan->dev.n_q > 1 && plan->dev.n_kv_shards <= 256;
 }
 
-// Shard-major K and V copies for the tensor-core path: two regions of batch * kv_heads * n_kv rows of 256 bytes.
-static size_t sorted_kv_bytes(const cascade_plan_t* plan, int batch, int Hkv) {
-  return align_up((size_t)batch * Hkv * plan->dev.n_kv * 128 * 2, 256);
+// Shard-major K and V copies for the tensor-core path: two regions of batch * kv_heads * n_kv rows of 2 d bytes.
+static size_t sorted_kv_bytes(const cascade_plan_t* plan, int batch, int Hkv, int d) {
+  return align_up((size_t)batch * Hkv * plan->dev.n_kv * d * 2, 256);
 }
 
 static size_t decode_ws_bytes(const cascade_plan_t* plan, cascade_dtype_t dtype, int batch, int H, int d) {
@@ -616,7 +616,7 @@ static size_t decode_ws_bytes(const cascade_plan_t* plan, cascade_dtype_t dtype,
 // Tensor-core route: shard gather of K and V into the workspace, then the attention kernel (two launches).
 static cascade_status_t run_tc(const AttnParams& p, const char* fn, const cascade_plan_t* plan, void* workspace,
                                size_t workspace_bytes, cudaStream_t st, cudaError_t* launch_error) {
-  const size_t each = sorted_kv_bytes(plan, p.batch, p.Hkv);
+  const size_t each = sorted_kv_bytes(plan, p.batch, p.Hkv, p.d);
   if (!workspace || workspace_bytes < 2 * each || ((uintptr_t)workspace & 255)) {
     set_error("%s: workspace of %zu bytes (256-byte aligned) required for the shard-major K/V copies, got %zu", fn,
               2 * each, workspace_bytes);
@@ -659,7 +659,7 @@ static HostCallLayout host_call_layout(const cascade_plan_t* plan, cascade_dtype
   // gs KV heads and their query heads per inner call
   const bool decode = use_decode(plan, dtype, G * gs, gs, d);
   L.inner_bytes = decode ? decode_ws_bytes(plan, dtype, batch, G * gs, d)
-                         : (use_tc(plan, dtype, d) ? 2 * sorted_kv_bytes(plan, batch, gs) : 0);
+                         : (use_tc(plan, dtype, d) ? 2 * sorted_kv_bytes(plan, batch, gs, d) : 0);
   L.total = L.inner + align_up(L.inner_bytes, 256);
   return L;
 }
@@ -689,7 +689,7 @@ cascade_status_t cascade_workspace_bytes(const cascade_plan_t* plan, int32_t whi
     return CASCADE_ERR_INVALID_ARG;
   }
   const bool decode = use_decode(plan, dtype, n_heads, n_kv_heads, head_dim);
-  const size_t tc_bytes = !decode && use_tc(plan, dtype, head_dim) ? 2 * sorted_kv_bytes(plan, batch, n_kv_heads) : 0;
+  const size_t tc_bytes = !decode && use_tc(plan, dtype, head_dim) ? 2 * sorted_kv_bytes(plan, batch, n_kv_heads, head_dim) : 0;
   if (which_call == CASCADE_CALL_PARTIALS) {
     *out_bytes = tc_bytes;
   } else if (which_call == CASCADE_CALL_SHARDED) {
@@ -738,7 +738,7 @@ cascade_status_t cascade_attn_partials(const cascade_plan_t* plan, cascade_dtype
   cudaError_t e;
   if (use_decode(plan, dtype, n_heads, n_kv_heads, head_dim)) {
     e = launch_decode(p, st);
-  } else if (use_tc(plan, dtype, head_dim)) {
+  } else if (use_tc(plan, dtype, head_dim) && !(head_dim == 64 && !workspace)) {
     cascade_status_t ws = run_tc(p, "cascade_attn_partials", plan, workspace, workspace_bytes, st, &e);
     if (ws != CASCADE_OK) return ws;
   } else {
@@ -898,7 +898,7 @@ static cascade_status_t attn_sharded_impl(const char* fn, const cascade_plan_t* 
                 "(cascade_shard_plan_resident) does not have", fn);
       return CASCADE_ERR_UNSUPPORTED;
     }
-    if (use_decode(plan, dtype, n_heads, n_kv_heads, head_dim) || !use_tc(plan, dtype, head_dim)) {
+    if (head_dim != 128 || use_decode(plan, dtype, n_heads, n_kv_heads, head_dim) || !use_tc(plan, dtype, head_dim)) {
       set_error("%s: the rotary step is fused on the tensor-core route only (bf16, head_dim 128, more than one query "
                 "row, at most %d KV shards)", fn, 256);
       return CASCADE_ERR_UNSUPPORTED;
@@ -944,7 +944,8 @@ static cascade_status_t attn_sharded_impl(const char* fn, const cascade_plan_t* 
   p.os = {o_strides.batch, o_strides.token, o_strides.head};
   p.lse_out = lse_out;
   cudaError_t e;
-  if (use_tc(plan, dtype, head_dim)) {
+  // (heads of 64 columns without a workspace take the ALU kernel, which needs none)
+  if (use_tc(plan, dtype, head_dim) && !(head_dim == 64 && !workspace)) {
     cascade_status_t ws = run_tc(p, fn, plan, workspace, workspace_bytes, st, &e);
     if (ws != CASCADE_OK) return ws;
   } else {

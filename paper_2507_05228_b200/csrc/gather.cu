@@ -26,8 +26,11 @@ __device__ __forceinline__ bool slot_is_visible(const PlanDev& pl, int map, int 
   return slot - __ldg(pl.kv_off + (size_t)map * (P + 1) + kk) < longest;
 }
 
+template <int D>
 __global__ void __launch_bounds__(256) gather_kv_kernel(AttnParams p, __nv_bfloat16* k_out, __nv_bfloat16* v_out) {
-  constexpr int D = 128;
+  constexpr int kLanes = D / 8;              // 16 bytes per thread
+  constexpr int kRows = 256 / kLanes;        // rows per pass
+  constexpr int kPasses = kGatherRowsPerCta / kRows;
   // The attention kernel that follows may be launched as a programmatic dependent: its CTAs may start their set-up
   // (query loads, shard tables, TMEM) now; they wait for this grid to finish before they touch the copies.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -35,15 +38,15 @@ __global__ void __launch_bounds__(256) gather_kv_kernel(AttnParams p, __nv_bfloa
   const int g = blockIdx.y, b = blockIdx.z;
   const int map = pl.n_maps == 1 ? 0 : b;
   const int32_t* kv_idx = pl.kv_idx + (size_t)map * pl.n_kv;
-  const int chunk = threadIdx.x & 15, r0 = threadIdx.x >> 4;  // 16 rows per pass, 16 bytes per thread
+  const int chunk = threadIdx.x % kLanes, r0 = threadIdx.x / kLanes;
   const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(p.k) + (int64_t)b * p.ks.batch + (int64_t)g * p.ks.head;
   const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(p.v) + (int64_t)b * p.vs.batch + (int64_t)g * p.vs.head;
   const int64_t out_base = ((int64_t)b * p.Hkv + g) * pl.n_kv;
   const int slot0 = blockIdx.x * kGatherRowsPerCta;
-  uint4 kr[kGatherRowsPerCta / 16], vr[kGatherRowsPerCta / 16];
+  uint4 kr[kPasses], vr[kPasses];
 #pragma unroll
-  for (int i = 0; i < kGatherRowsPerCta / 16; ++i) {
-    const int slot = slot0 + 16 * i + r0;
+  for (int i = 0; i < kPasses; ++i) {
+    const int slot = slot0 + kRows * i + r0;
     kr[i] = vr[i] = make_uint4(0u, 0u, 0u, 0u);
     if (slot < pl.n_kv && slot_is_visible(pl, map, slot)) {
       const int64_t tok = CASCADE_CHECKED((int64_t)__ldg(kv_idx + slot), pl.n_kv, pl.status, 101);
@@ -52,8 +55,8 @@ __global__ void __launch_bounds__(256) gather_kv_kernel(AttnParams p, __nv_bfloa
     }
   }
 #pragma unroll
-  for (int i = 0; i < kGatherRowsPerCta / 16; ++i) {
-    const int slot = slot0 + 16 * i + r0;
+  for (int i = 0; i < kPasses; ++i) {
+    const int slot = slot0 + kRows * i + r0;
     if (slot < pl.n_kv) {
       *reinterpret_cast<uint4*>(k_out + (out_base + slot) * D + chunk * 8) = kr[i];
       *reinterpret_cast<uint4*>(v_out + (out_base + slot) * D + chunk * 8) = vr[i];
@@ -131,8 +134,8 @@ cudaError_t launch_gather_kv(const AttnParams& p, void* k_out, void* v_out, cuda
     gather_kv_rope_kernel<<<grid, 256, 0, stream>>>(p, static_cast<__nv_bfloat16*>(k_out),
                                                     static_cast<__nv_bfloat16*>(v_out));
   } else {
-    gather_kv_kernel<<<grid, 256, 0, stream>>>(p, static_cast<__nv_bfloat16*>(k_out),
-                                               static_cast<__nv_bfloat16*>(v_out));
+    auto kernel = p.d == 64 ? gather_kv_kernel<64> : gather_kv_kernel<128>;
+    kernel<<<grid, 256, 0, stream>>>(p, static_cast<__nv_bfloat16*>(k_out), static_cast<__nv_bfloat16*>(v_out));
   }
   count_launch();
   return cudaGetLastError();
