@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cmath>
 #include <atomic>
+#include <mutex>
 #include <new>
 
 #include "cascade_internal.cuh"
@@ -58,6 +59,17 @@ static cascade_status_t cuda_fail(cudaError_t e, const char* what) {
   return CASCADE_ERR_CUDA;
 }
 
+// Number of keys of all shards that a query at position `pos` sees.
+static int64_t visible_keys(const cascade_plan& pl, int map, int64_t pos) {
+  const int n_kv = pl.dev.n_kv;
+  if (!pl.dev.causal) return n_kv;
+  if (!pl.kv_pos.empty()) {
+    const int32_t* kp = pl.kv_pos.data() + (size_t)map * n_kv;
+    return std::upper_bound(kp, kp + n_kv, pos) - kp;
+  }
+  return std::min<int64_t>(std::max<int64_t>(pos + 1, 0), n_kv);
+}
+
 // Query tiles of `rows_per_tile` slots that stay inside one shard, heaviest first.
 static void build_qtiles(const cascade_plan& pl, int map, int rows_per_tile, std::vector<int4>& out) {
   struct Tile {
@@ -65,15 +77,14 @@ static void build_qtiles(const cascade_plan& pl, int map, int rows_per_tile, std
     int64_t work;
   };
   std::vector<Tile> tiles;
-  const int nq = pl.dev.n_q, P = pl.dev.n_kv_shards, J = pl.dev.n_q_shards;
+  const int J = pl.dev.n_q_shards;
   const int32_t* off = pl.q_off.data() + (size_t)map * (J + 1);
-  const int32_t* vis = pl.vis.data() + (size_t)map * nq * P;
+  const int32_t* qi = pl.q_idx.data() + (size_t)map * pl.dev.n_q;
   for (int j = 0; j < J; ++j) {
     for (int r0 = off[j]; r0 < off[j + 1]; r0 += rows_per_tile) {
       const int n = std::min(rows_per_tile, off[j + 1] - r0);
-      int64_t work = 0;
-      for (int k = 0; k < P; ++k) work += vis[(size_t)(r0 + n - 1) * P + k];
-      tiles.push_back({make_int4(r0, n, j, 0), work});
+      // the shards partition the keys, so the last row's prefixes add up to the keys at or before its position
+      tiles.push_back({make_int4(r0, n, j, 0), visible_keys(pl, map, (int64_t)qi[r0 + n - 1] + pl.dev.q_pos_offset)});
     }
   }
   std::stable_sort(tiles.begin(), tiles.end(), [](const Tile& a, const Tile& b) { return a.work > b.work; });
@@ -110,6 +121,13 @@ static void fill_vis(const cascade_plan& pl, int mp, int q_pos_offset, int32_t* 
   }
 }
 
+// Whether vis and pair_class of a device plan are computed on the host.  A decode step (one query row, a few KV shards) is
+// a handful of binary searches and a 64-byte upload: 3 us on the host against 12 us for a dependent-load kernel.  Anything
+// larger goes to the device, except with kv_pos, which the device arrays do not hold.
+static bool vis_from_host(const cascade_plan& pl) {
+  return !pl.kv_pos.empty() || (int64_t)pl.dev.n_maps * pl.dev.n_q * pl.dev.n_kv_shards <= 256;
+}
+
 // EMPTY / PARTIAL / FULL per (query shard, KV shard) from the prefix lengths of the shard's first and last row
 // (rows ascend in position, so the first row has the shortest prefix and the last the longest).
 static void fill_pair_class(const cascade_plan& pl, int mp, const int32_t* vis, uint8_t* pc) {
@@ -128,11 +146,16 @@ static void fill_pair_class(const cascade_plan& pl, int mp, const int32_t* vis, 
     }
 }
 
-// Host copies of vis and pair_class for the plan's current q_pos_offset.
+// Host copies of vis and pair_class for the plan's current q_pos_offset.  A device plan may never need them, so they are
+// made by the first call that reads them (several threads may read one plan).  May throw std::bad_alloc.
+static std::mutex g_host_vis_mutex;
 static void refresh_host_vis(const cascade_plan& pl, bool force) {
+  std::lock_guard<std::mutex> lock(g_host_vis_mutex);
   if (!force && !pl.host_vis_stale) return;
   cascade_plan& w = const_cast<cascade_plan&>(pl);
   const PlanDev& d = pl.dev;
+  w.vis.resize((size_t)d.n_maps * d.n_q * d.n_kv_shards);
+  w.pair_class.resize((size_t)d.n_maps * d.n_q_shards * d.n_kv_shards);
   for (int mp = 0; mp < d.n_maps; ++mp) {
     int32_t* vis = w.vis.data() + (size_t)mp * d.n_q * d.n_kv_shards;
     fill_vis(pl, mp, d.q_pos_offset, vis);
@@ -175,7 +198,7 @@ cascade_status_t cascade_kernel_timing_end(double* total_ms, int64_t* n_launches
 
 static cascade_status_t plan_host(int32_t n_maps, int32_t n_q, int32_t n_kv, const int32_t* q_shard_of,
                                   const int32_t* kv_shard_of, const int32_t* kv_pos, int32_t n_q_shards,
-                                  int32_t n_kv_shards, int32_t q_pos_offset, int32_t causal,
+                                  int32_t n_kv_shards, int32_t q_pos_offset, int32_t causal, bool vis_on_device,
                                   cascade_plan_t** out_plan) {
   if (!out_plan || !q_shard_of || !kv_shard_of) {
     set_error("cascade_shard_plan: null pointer");
@@ -229,8 +252,6 @@ static cascade_status_t plan_host(int32_t n_maps, int32_t n_q, int32_t n_kv, con
     pl->kv_idx.assign((size_t)n_maps * n_kv, 0);
     pl->kv_inv.assign((size_t)n_maps * n_kv, 0);
     pl->kv_slot_shard.assign((size_t)n_maps * n_kv, 0);
-    pl->vis.assign((size_t)n_maps * n_q * P, 0);
-    pl->pair_class.assign((size_t)n_maps * J * P, 0);
     if (kv_pos) pl->kv_pos.assign(kv_pos, kv_pos + (size_t)n_maps * n_kv);
     int max_len = 0;
     // counting sort of token ids by shard id: ascending ids inside every shard
@@ -257,11 +278,10 @@ static cascade_status_t plan_host(int32_t n_maps, int32_t n_q, int32_t n_kv, con
         max_len = std::max(max_len, (int)(ko[k + 1] - ko[k]));
         std::fill(slot_shard + ko[k], slot_shard + ko[k + 1], k);
       }
-      int32_t* vis = pl->vis.data() + (size_t)mp * n_q * P;
-      fill_vis(*pl, mp, q_pos_offset, vis);
-      fill_pair_class(*pl, mp, vis, pl->pair_class.data() + (size_t)mp * J * P);
     }
     pl->dev.max_kv_shard_len = max_len;
+    pl->host_vis_stale = true;
+    if (!vis_on_device || vis_from_host(*pl)) refresh_host_vis(*pl, true);
     // tile lists, padded to the same length for every map
     for (int ts = 0; ts < kNumTileSizes; ++ts) {
       std::vector<std::vector<int4>> lists(n_maps);
@@ -288,7 +308,7 @@ cascade_status_t cascade_shard_plan_host(int32_t n_maps, int32_t n_q, int32_t n_
                                          const int32_t* kv_shard_of, int32_t n_q_shards, int32_t n_kv_shards,
                                          int32_t q_pos_offset, int32_t causal, cascade_plan_t** out_plan) {
   return plan_host(n_maps, n_q, n_kv, q_shard_of, kv_shard_of, nullptr, n_q_shards, n_kv_shards, q_pos_offset, causal,
-                   out_plan);
+                   false, out_plan);
 }
 
 cascade_status_t cascade_shard_plan_resident_host(int32_t n_maps, int32_t n_q, int32_t n_kv, const int32_t* q_shard_of,
@@ -300,7 +320,55 @@ cascade_status_t cascade_shard_plan_resident_host(int32_t n_maps, int32_t n_q, i
     return CASCADE_ERR_INVALID_ARG;
   }
   return plan_host(n_maps, n_q, n_kv, q_shard_of, kv_shard_of, kv_pos, n_q_shards, n_kv_shards, q_pos_offset, causal,
-                   out_plan);
+                   false, out_plan);
+}
+
+// Device memory of plans comes from one CUDA memory pool per device, so that a server that builds a plan per request does
+// not pay for cudaMalloc and cudaFree each time (400 us to over 1 ms per pair once other allocations are around; 2 to 3 us
+// from the pool).  The pool keeps at most kPlanPoolBytes of freed memory; what is beyond goes back to the device at
+// the next synchronisation.  The driver makes it safe for several threads and streams.  Without pool support: cudaMalloc.
+constexpr uint64_t kPlanPoolBytes = 32u << 20;
+static cudaMemPool_t plan_pool(int dev) {
+  static std::mutex mutex;
+  static cudaMemPool_t pools[64] = {};
+  static bool tried[64] = {};
+  if (dev < 0 || dev >= 64) return nullptr;
+  std::lock_guard<std::mutex> lock(mutex);
+  if (!tried[dev]) {
+    tried[dev] = true;
+    cudaMemPoolProps props;
+    memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kPlanPoolBytes;
+    if (cudaMemPoolCreate(&pool, &props) == cudaSuccess &&
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+      pools[dev] = pool;
+    else
+      cudaGetLastError();
+  }
+  return pools[dev];
+}
+
+static cudaError_t plan_blob_alloc(size_t bytes, cudaStream_t st, cascade_plan* pl) {
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  cudaMemPool_t pool = plan_pool(dev);
+  pl->dev_blob_pooled = pool != nullptr;
+  e = pool ? cudaMallocFromPoolAsync(&pl->dev_blob, bytes, pool, st) : cudaMalloc(&pl->dev_blob, bytes);
+  pl->device = dev;
+  if (e == cudaSuccess) pl->dev_blob_bytes = bytes;
+  else pl->dev_blob = nullptr;
+  return e;
+}
+
+// The caller has synchronised the device (or nothing but the failed upload ever used the memory).
+static void plan_blob_free(cascade_plan* pl) {
+  if (pl->dev_blob_pooled) cudaFreeAsync(pl->dev_blob, nullptr);
+  else cudaFree(pl->dev_blob);
 }
 
 static cascade_status_t plan_device(int32_t n_maps, int32_t n_q, int32_t n_kv, const int32_t* q_shard_of,
@@ -309,11 +377,15 @@ static cascade_status_t plan_device(int32_t n_maps, int32_t n_q, int32_t n_kv, c
                                     cascade_plan_t** out_plan) {
   cascade_plan* pl = nullptr;
   cascade_status_t hs = plan_host(n_maps, n_q, n_kv, q_shard_of, kv_shard_of, kv_pos, n_q_shards, n_kv_shards,
-                                  q_pos_offset, causal, &pl);
+                                  q_pos_offset, causal, true, &pl);
   if (hs != CASCADE_OK) return hs;
   *out_plan = nullptr;
 
-  // one device blob, every array 256-byte aligned
+  // One device blob, every array 256-byte aligned: the status word, the arrays that are uploaded, and at the end vis and
+  // pair_class, which kernels fill in from the uploaded lists unless the host has them already.  The uploaded part is put
+  // together in host memory and goes up in one copy (one copy per array cost 5 us each).
+  const bool host_vis = vis_from_host(*pl);
+  const size_t vis_bytes = (size_t)n_maps * n_q * n_kv_shards * 4, class_bytes = (size_t)n_maps * n_q_shards * n_kv_shards;
   struct Seg {
     const void* src;
     size_t bytes;
@@ -323,35 +395,37 @@ static cascade_status_t plan_device(int32_t n_maps, int32_t n_q, int32_t n_kv, c
       {pl->q_off.data(), pl->q_off.size() * 4, 0},       {pl->q_idx.data(), pl->q_idx.size() * 4, 0},
       {pl->q_inv.data(), pl->q_inv.size() * 4, 0},       {pl->kv_off.data(), pl->kv_off.size() * 4, 0},
       {pl->kv_idx.data(), pl->kv_idx.size() * 4, 0},     {pl->kv_inv.data(), pl->kv_inv.size() * 4, 0},
-      {pl->vis.data(), pl->vis.size() * 4, 0},           {pl->pair_class.data(), pl->pair_class.size(), 0},
       {pl->qtiles[0].data(), pl->qtiles[0].size() * 16, 0}, {pl->qtiles[1].data(), pl->qtiles[1].size() * 16, 0},
       {pl->qtiles[2].data(), pl->qtiles[2].size() * 16, 0}, {pl->qtiles[3].data(), pl->qtiles[3].size() * 16, 0},
       {pl->kv_slot_shard.data(), pl->kv_slot_shard.size() * 4, 0},
+      {host_vis ? pl->vis.data() : nullptr, vis_bytes, 0}, {host_vis ? pl->pair_class.data() : nullptr, class_bytes, 0},
   };
   static_assert(kNumTileSizes == 4, "one upload segment per tile list");
-  size_t total = 256;  // status word first
+  size_t total = 256, upload = 256;  // status word first
   for (auto& s : segs) {
     s.off = total;
     total += align_up(s.bytes, 256);
+    if (s.src) upload = total;
   }
-  cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = cudaMalloc(&pl->dev_blob, total);
-  if (e != cudaSuccess) {
+  std::vector<char> staging;
+  try {
+    staging.assign(upload, 0);
+  } catch (const std::bad_alloc&) {
     delete pl;
-    set_error("cascade_shard_plan: cudaMalloc(%zu): %s", total, cudaGetErrorString(e));
+    set_error("cascade_shard_plan: host allocation failed");
     return CASCADE_ERR_ALLOC;
   }
-  pl->dev_blob_bytes = total;
-  char* base = (char*)pl->dev_blob;
-  e = cudaMemsetAsync(base, 0, 256, st);
   for (auto& s : segs)
-    if (e == cudaSuccess && s.bytes) e = cudaMemcpyAsync(base + s.off, s.src, s.bytes, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (s.src && s.bytes) memcpy(staging.data() + s.off, s.src, s.bytes);
+  cudaStream_t st = (cudaStream_t)stream;
+  cudaError_t e = plan_blob_alloc(total, st, pl);
   if (e != cudaSuccess) {
-    cudaFree(pl->dev_blob);
     delete pl;
-    return cuda_fail(e, "cascade_shard_plan: upload");
+    set_error("cascade_shard_plan: device allocation of %zu bytes: %s", total, cudaGetErrorString(e));
+    return CASCADE_ERR_ALLOC;
   }
+  char* base = (char*)pl->dev_blob;
+  e = cudaMemcpyAsync(base, staging.data(), upload, cudaMemcpyHostToDevice, st);
   pl->dev.status = (int32_t*)base;
   pl->dev.q_off = (const int32_t*)(base + segs[0].off);
   pl->dev.q_idx = (const int32_t*)(base + segs[1].off);
@@ -359,10 +433,17 @@ static cascade_status_t plan_device(int32_t n_maps, int32_t n_q, int32_t n_kv, c
   pl->dev.kv_off = (const int32_t*)(base + segs[3].off);
   pl->dev.kv_idx = (const int32_t*)(base + segs[4].off);
   pl->dev.kv_inv = (const int32_t*)(base + segs[5].off);
-  pl->dev.vis = (const int32_t*)(base + segs[6].off);
-  pl->dev.pair_class = (const uint8_t*)(base + segs[7].off);
-  for (int ts = 0; ts < kNumTileSizes; ++ts) pl->dev.qtiles[ts] = (const int4*)(base + segs[8 + ts].off);
-  pl->dev.kv_slot_shard = (const int32_t*)(base + segs[12].off);
+  for (int ts = 0; ts < kNumTileSizes; ++ts) pl->dev.qtiles[ts] = (const int4*)(base + segs[6 + ts].off);
+  pl->dev.kv_slot_shard = (const int32_t*)(base + segs[10].off);
+  pl->dev.vis = (const int32_t*)(base + segs[11].off);
+  pl->dev.pair_class = (const uint8_t*)(base + segs[12].off);
+  if (e == cudaSuccess && !host_vis) e = launch_plan_advance(pl->dev, q_pos_offset, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) {
+    plan_blob_free(pl);
+    delete pl;
+    return cuda_fail(e, "cascade_shard_plan: upload");
+  }
   *out_plan = pl;
   return CASCADE_OK;
 }
@@ -393,11 +474,25 @@ cascade_status_t cascade_plan_destroy(cascade_plan_t* plan) {
     delete plan;
     return CASCADE_OK;
   }
-  cudaError_t e = cudaDeviceSynchronize();
-  cudaFree(plan->dev_blob);
+  int current = plan->device;
+  cudaError_t e = cudaGetDevice(&current);
+  if (e == cudaSuccess && current != plan->device) e = cudaSetDevice(plan->device);
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  plan_blob_free(plan);
+  if (current != plan->device) cudaSetDevice(current);
   delete plan;
   if (e != cudaSuccess) return cuda_fail(e, "cascade_plan_destroy: device synchronize");
   return CASCADE_OK;
+}
+
+static bool host_vis_ready(const cascade_plan& pl) {
+  try {
+    refresh_host_vis(pl, false);
+  } catch (const std::bad_alloc&) {
+    set_error("cascade plan: host allocation failed");
+    return false;
+  }
+  return true;
 }
 
 cascade_status_t cascade_plan_get(const cascade_plan_t* plan, int32_t field, const void** host_ptr,
@@ -417,11 +512,13 @@ cascade_status_t cascade_plan_get(const cascade_plan_t* plan, int32_t field, con
     case CASCADE_PLAN_KV_IDX: h = plan->kv_idx.data(); d = plan->dev.kv_idx; n = plan->kv_idx.size(); break;
     case CASCADE_PLAN_KV_INV: h = plan->kv_inv.data(); d = plan->dev.kv_inv; n = plan->kv_inv.size(); break;
     case CASCADE_PLAN_VIS:
-      refresh_host_vis(*plan, false);
-      h = plan->vis.data(); d = plan->dev.vis; n = plan->vis.size(); break;
+      if (host_ptr && !host_vis_ready(*plan)) return CASCADE_ERR_ALLOC;
+      h = plan->vis.data(); d = plan->dev.vis;
+      n = (int64_t)plan->dev.n_maps * plan->dev.n_q * plan->dev.n_kv_shards; break;
     case CASCADE_PLAN_PAIR_CLASS:
-      refresh_host_vis(*plan, false);
-      h = plan->pair_class.data(); d = plan->dev.pair_class; n = plan->pair_class.size(); break;
+      if (host_ptr && !host_vis_ready(*plan)) return CASCADE_ERR_ALLOC;
+      h = plan->pair_class.data(); d = plan->dev.pair_class;
+      n = (int64_t)plan->dev.n_maps * plan->dev.n_q_shards * plan->dev.n_kv_shards; break;
     default:
       set_error("cascade_plan_get: unknown field %d", field);
       return CASCADE_ERR_INVALID_ARG;
@@ -438,7 +535,7 @@ cascade_status_t cascade_plan_dense_mask(const cascade_plan_t* plan, int32_t map
     set_error("cascade_plan_dense_mask: null pointer");
     return CASCADE_ERR_INVALID_ARG;
   }
-  refresh_host_vis(*plan, false);
+  if (!host_vis_ready(*plan)) return CASCADE_ERR_ALLOC;
   const PlanDev& d = plan->dev;
   if (map < 0 || map >= d.n_maps || j < 0 || j >= d.n_q_shards || k < 0 || k >= d.n_kv_shards) {
     set_error("cascade_plan_dense_mask: index out of range");
@@ -465,11 +562,8 @@ cascade_status_t cascade_plan_advance(cascade_plan_t* plan, int32_t q_pos_offset
     return CASCADE_ERR_INVALID_ARG;
   }
   const PlanDev& d = plan->dev;
-  // A decode step (one query row, a few KV shards) is a handful of binary searches and a 64-byte upload: 3 us on the
-  // host against 12 us for a dependent-load kernel.  Anything larger goes to the device.
-  const int64_t n_vis = (int64_t)d.n_maps * d.n_q * d.n_kv_shards;
-  if (plan->dev_blob && plan->kv_pos.empty() && n_vis > 256) {
-    // Two small kernels rewrite vis and pair_class in stream order from the plan's own index arrays; nothing is
+  if (plan->dev_blob && !vis_from_host(*plan)) {
+    // A small kernel rewrites vis and pair_class in stream order from the plan's own index arrays; nothing is
     // computed on the host and nothing is uploaded.  The host copies follow when they are next read.
     plan->dev.q_pos_offset = q_pos_offset;
     plan->host_vis_stale = true;

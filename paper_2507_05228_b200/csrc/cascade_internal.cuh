@@ -111,8 +111,10 @@ struct cascade_plan {
   std::vector<int4> qtiles[cascade::kNumTileSizes];
   void* dev_blob = nullptr;
   size_t dev_blob_bytes = 0;
-  // cascade_plan_advance moves the device arrays with a kernel; the host copies of vis and pair_class are then brought
-  // up to date only when something reads them (cascade_plan_get, cascade_plan_dense_mask)
+  int device = 0;                // the device that holds dev_blob
+  bool dev_blob_pooled = false;  // dev_blob came from the device's plan pool
+  // The device arrays vis and pair_class are made by a kernel (cascade_shard_plan, cascade_plan_advance); their host
+  // copies are brought up to date only when something reads them (cascade_plan_get, cascade_plan_dense_mask)
   mutable bool host_vis_stale = false;
 };
 

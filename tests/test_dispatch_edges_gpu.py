@@ -1,0 +1,66 @@
+"""Sizes at which a kernel or a dispatch rule changes what it does: edges of tiles, remainders, the smallest and the largest
+of a range.  Reference and tolerances are those of the parity tests."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2507_05228_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gu():
+    import gpu_util
+    return gpu_util
+
+
+@pytest.mark.parametrize("n,H,Hkv,shards,causal", [
+    (2, 4, 4, 1, True),        # one tile of one chunk
+    (129, 8, 1, 3, True),      # eight stacked heads, a last tile of one row
+    (1153, 16, 4, 2, True),    # ten 128-key tiles: every logit buffer and stage is used several times over
+    (700, 12, 12, 5, False),   # no stacking, one sub-tile per CTA, bidirectional
+    (1500, 6, 2, 40, True),    # three heads per KV head: no stacking although heads are shared; many short shards
+])
+def test_head_dim_64_on_the_tensor_cores(gu, n, H, Hkv, shards, causal):
+    gu.full_parity(wl.make_workload(f"d64_{n}", 2, n, n, H, Hkv, 64, "bf16", "random", "random", shards, shards, seed=n,
+                                    causal=causal))
+
+
+def test_head_dim_64_without_a_workspace_takes_the_alu_kernel(gu):
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload("d64_nows", 1, 200, 200, 8, 2, 64, "bf16", "random", "random", 3, 3, seed=7)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    o = torch.empty_like(q)
+    S = cb._strides
+    rc = cb.lib().cascade_attn_sharded(plan.handle, cb.BF16, w.B, w.H, w.Hkv, w.d, w.scale, q.data_ptr(), S(q), k.data_ptr(),
+                                       S(k), v.data_ptr(), S(v), o.data_ptr(), S(o), None, None, 0,
+                                       torch.cuda.current_stream().cuda_stream)
+    assert rc == 0
+    o_ref, _ = oracle.attention_unsharded(w.q, w.k, w.v, w.scale)
+    gu.check_output(o, None, o_ref, None, w.tol, "no workspace")
+    plan.destroy()
+
+
+@pytest.mark.parametrize("n_q,n_kv,P,causal", [(128, 128, 2, True), (129, 200, 2, True), (300, 900, 7, False), (40, 64, 64, True)])
+def test_new_plans_have_the_same_arrays_on_the_device(gu, n_q, n_kv, P, causal):
+    """vis and pair_class come from the host up to 256 entries and from a kernel above; two plans alive at a time, and a
+    third in memory that a destroyed one gave back."""
+    from paper_2507_05228_b200 import binding as cb
+    rng = np.random.default_rng(n_kv)
+    plans = []
+    for _ in range(3):
+        q_of, kv_of = rng.integers(0, 3, n_q).astype(np.int32), rng.integers(0, P, n_kv).astype(np.int32)
+        plan = cb.cascade_shard_plan(q_of, kv_of, 3, P, n_kv - n_q, causal)
+        ref = oracle.shard_plan(q_of, kv_of, 3, P, q_pos_offset=n_kv - n_q, causal=causal)
+        for f in ("q_off", "q_idx", "q_inv", "kv_off", "kv_idx", "kv_inv", "vis", "pair_class"):
+            assert np.array_equal(gu.read_plan_device_array(plan, f)[0], getattr(ref, f)), f
+            assert np.array_equal(plan.get(f)[0], getattr(ref, f)), f
+        assert plan.device_status() == 0
+        plans.append(plan)
+        if len(plans) == 2:
+            plans.pop(0).destroy()
+    for plan in plans:
+        plan.destroy()
