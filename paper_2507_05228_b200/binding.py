@@ -1,4 +1,5 @@
-"""ctypes binding of libcascade_b200.so: argument marshalling only -- every step runs in the CUDA library.
+"""Binding of libcascade_b200.so: argument marshalling only -- every step runs in the CUDA library.  The calls made once per
+plan or request go through ctypes; those made per layer or per token go through _fastcall.so (csrc/fastcall.cpp).
 
 Function names match the C ABI (include/cascade.h).  torch supplies device memory and the current stream.
 The library must have been built (``python -m paper_2507_05228_b200.build``); loading fails loudly otherwise:
@@ -48,11 +49,19 @@ class Strides(ctypes.Structure):
 
 
 _lib = None
+_fast = None  # the _fastcall module, once the library is loaded
+
+
+def _native():
+    """The native marshalling of the per-layer calls, bound to the loaded library."""
+    if _fast is None:
+        lib()
+    return _fast
 
 
 def lib() -> ctypes.CDLL:
     """The loaded shared library.  Raises if it has not been built."""
-    global _lib
+    global _lib, _fast
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise ImportError(
@@ -98,7 +107,9 @@ def lib() -> ctypes.CDLL:
         for name in EXPORTS:
             if name not in ("cascade_version", "cascade_last_error", "cascade_launch_count"):
                 getattr(L, name).restype = i32
-        _lib = L
+        from . import _fastcall  # built with the library; like it, there is no fallback
+        _fastcall.load(LIB_PATH, CascadeError)
+        _fast, _lib = _fastcall, L
     return _lib
 
 
@@ -187,7 +198,7 @@ class Plan:
     def advance(self, q_pos_offset: int):
         """Move the query block to position ``q_pos_offset`` (token-sharded KV caching): the causal prefixes are
         recomputed, on the device in the order of the current stream.  A host-only plan needs no stream."""
-        _check(lib().cascade_plan_advance(self.handle, int(q_pos_offset), _stream() if torch.cuda.is_available() else None))
+        _native().plan_advance(self.handle, int(q_pos_offset))
 
     def destroy(self):
         if self.handle:
@@ -262,47 +273,18 @@ def cascade_workspace_bytes(plan: Plan, which_call: int, dtype_code: int, batch:
     return out.value
 
 
-def _ws(nbytes: int, device, workspace: Optional[torch.Tensor]):
-    if nbytes == 0:
-        return None, 0, 0
-    if workspace is None:
-        workspace = torch.empty(nbytes, dtype=torch.uint8, device=device)
-    return workspace, workspace.data_ptr(), workspace.numel() * workspace.element_size()
-
-
 def cascade_attn_partials(plan: Plan, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, scale: float, out=None,
                           workspace=None):
     """Returns (o_part [B, n_kv_shards, n_q, H, d] in q.dtype, m_part, l_part [B, n_kv_shards, n_q, H] fp32);
     rows in shard-major order."""
-    B, n_q, H, d = q.shape
-    Hkv = k.shape[2]
-    code = _dtype_code(q)
-    if out is None:
-        P = plan.n_kv_shards
-        out = (torch.empty((B, P, n_q, H, d), dtype=q.dtype, device=q.device),
-               torch.empty((B, P, n_q, H), dtype=torch.float32, device=q.device),
-               torch.empty((B, P, n_q, H), dtype=torch.float32, device=q.device))
-    o_part, m_part, l_part = out
-    nbytes = cascade_workspace_bytes(plan, CALL_PARTIALS, code, B, H, Hkv, d)
-    ws, ws_ptr, ws_bytes = _ws(nbytes, q.device, workspace)
-    _check(lib().cascade_attn_partials(plan.handle, code, B, H, Hkv, d, scale, q.data_ptr(), _strides(q),
-                                       k.data_ptr(), _strides(k), v.data_ptr(), _strides(v), o_part.data_ptr(),
-                                       m_part.data_ptr(), l_part.data_ptr(), ws_ptr, ws_bytes, _stream()))
-    return o_part, m_part, l_part
+    return _native().attn_partials(plan.handle, plan.n_kv_shards, q, k, v, scale, out, workspace)
 
 
 def cascade_merge(o_part: torch.Tensor, m_part: torch.Tensor, l_part: torch.Tensor, row_scatter_ptr: int = 0,
                   row_scatter_batch_stride: int = 0, out=None, want_lse: bool = True):
     """o_part [B, P, n_rows, H, d]; row_scatter_ptr: device pointer of an int32 [n_rows] map (a plan's q_idx) or 0.
     Returns (o [B, n_rows, H, d], lse [B, n_rows, H] or None)."""
-    B, P, n_rows, H, d = o_part.shape
-    code = _dtype_code(o_part)
-    o = out if out is not None else torch.empty((B, n_rows, H, d), dtype=o_part.dtype, device=o_part.device)
-    lse = torch.empty((B, n_rows, H), dtype=torch.float32, device=o_part.device) if want_lse else None
-    _check(lib().cascade_merge(code, B, P, n_rows, H, d, o_part.data_ptr(), m_part.data_ptr(), l_part.data_ptr(),
-                               row_scatter_ptr or None, row_scatter_batch_stride, o.data_ptr(), _strides(o),
-                               lse.data_ptr() if lse is not None else None, _stream()))
-    return o, lse
+    return _native().merge(o_part, m_part, l_part, row_scatter_ptr or None, row_scatter_batch_stride, out, want_lse)
 
 
 def cascade_merge_peers(sources, row_gather: Optional[torch.Tensor], n_rows: int, out=None, want_lse: bool = True):
@@ -329,18 +311,7 @@ def cascade_merge_peers(sources, row_gather: Optional[torch.Tensor], n_rows: int
 def cascade_attn_sharded(plan: Plan, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, scale: float, out=None,
                          want_lse: bool = True, workspace=None):
     """Fused attention-pass + post-pass.  Returns (o [B, n_q, H, d] in token order, lse or None)."""
-    B, n_q, H, d = q.shape
-    Hkv = k.shape[2]
-    code = _dtype_code(q)
-    o = out if out is not None else torch.empty((B, n_q, H, d), dtype=q.dtype, device=q.device)
-    lse = torch.empty((B, n_q, H), dtype=torch.float32, device=q.device) if want_lse else None
-    nbytes = cascade_workspace_bytes(plan, CALL_SHARDED, code, B, H, Hkv, d)
-    ws, ws_ptr, ws_bytes = _ws(nbytes, q.device, workspace)
-    _check(lib().cascade_attn_sharded(plan.handle, code, B, H, Hkv, d, scale, q.data_ptr(), _strides(q),
-                                      k.data_ptr(), _strides(k), v.data_ptr(), _strides(v), o.data_ptr(),
-                                      _strides(o), lse.data_ptr() if lse is not None else None, ws_ptr, ws_bytes,
-                                      _stream()))
-    return o, lse
+    return _native().attn_sharded(plan.handle, q, k, v, scale, None, out, want_lse, workspace)
 
 
 def cascade_rope_table(n_positions: int, head_dim: int, base: float, device="cuda") -> torch.Tensor:
@@ -353,19 +324,7 @@ def cascade_rope_table(n_positions: int, head_dim: int, base: float, device="cud
 def cascade_attn_sharded_rope(plan: Plan, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, scale: float,
                               rope_table: torch.Tensor, out=None, want_lse: bool = True, workspace=None):
     """cascade_attn_sharded on unrotated q, k with the rotary step fused into the staging of their rows."""
-    B, n_q, H, d = q.shape
-    Hkv = k.shape[2]
-    code = _dtype_code(q)
-    assert rope_table.dtype == torch.float32 and rope_table.is_contiguous() and rope_table.shape[1:] == (d // 2, 2)
-    o = out if out is not None else torch.empty((B, n_q, H, d), dtype=q.dtype, device=q.device)
-    lse = torch.empty((B, n_q, H), dtype=torch.float32, device=q.device) if want_lse else None
-    nbytes = cascade_workspace_bytes(plan, CALL_SHARDED, code, B, H, Hkv, d)
-    ws, ws_ptr, ws_bytes = _ws(nbytes, q.device, workspace)
-    _check(lib().cascade_attn_sharded_rope(plan.handle, code, B, H, Hkv, d, scale, q.data_ptr(), _strides(q),
-                                           k.data_ptr(), _strides(k), v.data_ptr(), _strides(v),
-                                           rope_table.data_ptr(), rope_table.shape[0], o.data_ptr(), _strides(o),
-                                           lse.data_ptr() if lse is not None else None, ws_ptr, ws_bytes, _stream()))
-    return o, lse
+    return _native().attn_sharded(plan.handle, q, k, v, scale, rope_table, out, want_lse, workspace)
 
 
 CALL_SHARDED_HOST = 2
@@ -385,19 +344,8 @@ def cascade_decode_step_rope(plan: Plan, q_new: torch.Tensor, k_new: torch.Tenso
                              rope_table: torch.Tensor, out=None, want_lse: bool = True, workspace=None):
     """One decode step over a token-sharded cache: advances the plan to `position`, appends the new token's rotated k
     row and its v row to the caches, rotates q and runs decode + merge.  Returns (o [B, 1, H, 128], lse or None)."""
-    B, _, H, d = q_new.shape
-    Hkv = k_new.shape[2]
-    o = out if out is not None else torch.empty_like(q_new)
-    lse = torch.empty((B, 1, H), dtype=torch.float32, device=q_new.device) if want_lse else None
-    nbytes = cascade_workspace_bytes(plan, CALL_DECODE_STEP_ROPE, BF16, B, H, Hkv, d)
-    ws, ws_ptr, ws_bytes = _ws(nbytes, q_new.device, workspace)
-    _check(lib().cascade_decode_step_rope(plan.handle, B, H, Hkv, scale, q_new.data_ptr(), _strides(q_new),
-                                          k_new.data_ptr(), _strides(k_new), v_new.data_ptr(), _strides(v_new),
-                                          k_cache.data_ptr(), _strides(k_cache), v_cache.data_ptr(), _strides(v_cache),
-                                          int(position), rope_table.data_ptr(), rope_table.shape[0], o.data_ptr(),
-                                          _strides(o), lse.data_ptr() if lse is not None else None, ws_ptr, ws_bytes,
-                                          _stream()))
-    return o, lse
+    return _native().decode_step_rope(plan.handle, q_new, k_new, v_new, k_cache, v_cache, int(position), scale, rope_table,
+                                      out, want_lse, workspace)
 
 
 def cascade_attn_sharded_host(plan: Plan, q_host: torch.Tensor, k_host: torch.Tensor, v_host: torch.Tensor,
@@ -423,14 +371,7 @@ def cascade_attn_decode_static(plan: Plan, q: torch.Tensor, k: torch.Tensor, v: 
     """Decode step (one query row per sequence) that uses the library's built-in 16 MiB scratch array instead of
     a workspace: for callers that can neither pass nor allocate scratch memory.  Only the output tensors are
     created here; the C call itself allocates nothing.  Returns (o [B, 1, H, 128], lse or None)."""
-    B, n_q, H, d = q.shape
-    assert n_q == 1 and d == 128 and q.dtype == torch.bfloat16
-    o = out if out is not None else torch.empty((B, n_q, H, d), dtype=q.dtype, device=q.device)
-    lse = torch.empty((B, n_q, H), dtype=torch.float32, device=q.device) if want_lse else None
-    _check(lib().cascade_attn_decode_static(plan.handle, B, H, k.shape[2], scale, q.data_ptr(), _strides(q),
-                                            k.data_ptr(), _strides(k), v.data_ptr(), _strides(v), o.data_ptr(),
-                                            _strides(o), lse.data_ptr() if lse is not None else None, _stream()))
-    return o, lse
+    return _native().attn_decode_static(plan.handle, q, k, v, scale, out, want_lse)
 
 
 def _np_ptr(a: np.ndarray):

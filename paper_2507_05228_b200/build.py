@@ -13,6 +13,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcascade_b200.so")
+FASTCALL = os.path.join(HERE, "_fastcall.so")
 LIB_DEBUG = os.path.join(HERE, "libcascade_b200_debug.so")
 SOURCES = ["cascade_api.cu", "merge.cu", "attn_simt.cu", "attn_tc.cu", "gather.cu", "decode.cu", "decode_static.cu",
            "shard_maps.cu", "rope.cu", "plan_advance.cu"]
@@ -33,12 +34,35 @@ def _stale(lib: str = LIB) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "cascade.h"), __file__]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != "fastcall.cpp"] + [os.path.join(ROOT, "include", "cascade.h"), __file__]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _build_fastcall(force: bool) -> None:
+    """Compile csrc/fastcall.cpp (the native side of binding.py) against this interpreter and torch."""
+    src = os.path.join(CSRC, "fastcall.cpp")
+    if not force and os.path.exists(FASTCALL):
+        t = os.path.getmtime(FASTCALL)
+        if all(os.path.getmtime(d) <= t for d in (src, os.path.join(ROOT, "include", "cascade.h"), __file__)):
+            return
+    import sysconfig
+
+    import torch
+    base = os.path.dirname(torch.__file__)
+    inc = [sysconfig.get_paths()["include"], os.path.join(base, "include"),
+           os.path.join(base, "include", "torch", "csrc", "api", "include"),
+           os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"), os.path.join(ROOT, "include")]
+    tmp = FASTCALL + f".{os.getpid()}.tmp"
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-w",
+                           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+                           *[f"-I{i}" for i in inc], src, "-o", tmp, f"-L{os.path.join(base, 'lib')}",
+                           "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-ldl"])
+    os.replace(tmp, FASTCALL)
 
 
 def build_library(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
     """Compile every .cu file for sm_100a and link libcascade_b200.so (or the _debug variant) next to this file."""
+    _build_fastcall(force and not debug)
     lib = LIB_DEBUG if debug else LIB
     if not force and not _stale(lib):
         return lib
