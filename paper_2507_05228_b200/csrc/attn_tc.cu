@@ -92,7 +92,7 @@ struct Cfg {
   static constexpr int kOffV = kOffK + kKStages * kTileBytes;
   static constexpr int kOffBar = kOffV + kVStages * kTileBytes;
   static_assert(2 * kM * kStageRowBytes <= kOffV, "the output staging area must fit in the Q and K tiles");
-  static constexpr int kNumBars = 28;
+  static constexpr int kNumBars = 30;
   static constexpr int kOffMisc = kOffBar + kNumBars * 8;   // tmem slot, abort flag, 12 progress words
   static constexpr int kOffShard = kOffMisc + 64;           // int32 [5][kMaxShards], see ShardTab
   static constexpr int kSmemBytes = kOffShard + 5 * kMaxShards * 4 + 1024;  // + alignment slack
@@ -106,8 +106,8 @@ enum Bar {
   V_FULL = K_EMPTY + kMaxStages,    // [kVStages]
   V_EMPTY = V_FULL + kMaxStages,    // [kVStages]
   S_FULL = V_EMPTY + kMaxStages,    // [2]; kRing: [2][2], see s_full
-  P_FULL = S_FULL + 4,              // [2]
-  O_FULL = P_FULL + 2,              // [1]
+  P_FULL = S_FULL + 4,              // [2]; kRing: [2][2], see p_full
+  O_FULL = P_FULL + 4,              // [1]
   O_RDY = O_FULL + 1                // [2]  kWalk: the accumulator of a sub-tile holds a finished shard;
                                     //      kRing: the product of a sub-tile's latest tile is in its accumulator
 };
@@ -391,6 +391,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   // Logits of sub-tile s, tile i.  With kRing they may be two tiles ahead of a softmax thread, which a phase parity cannot
   // tell from "not there yet": even and odd tiles have a barrier each (tile i + 2 is issued after the thread's P(i)).
   auto s_full = [&](int s, int i) { return bar(S_FULL + (kRing ? 2 * (i & 1) : 0) + s); };
+  // Weights of sub-tile s, tile i.  With kRing a warp can be done with tile i + 1 before another has arrived for tile i, and
+  // on one barrier its arrival would complete the other's phase; it cannot get to tile i + 2 (PV(i) waits for everyone).
+  auto p_full = [&](int s, int i) { return bar(P_FULL + (kRing ? 2 * (i & 1) : 0) + s); };
   auto s_parity = [&](int i) { return (uint32_t)((kRing ? i >> 1 : i) & 1); };
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kOffMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 4);
@@ -537,6 +540,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       mbar_init(bar(S_FULL + s), 1);
       mbar_init(bar(S_FULL + 2 + s), 1);
       mbar_init(bar(P_FULL + s), 128);
+      mbar_init(bar(P_FULL + 2 + s), 128);
     }
     mbar_init(bar(O_FULL), 1);
     mbar_init(bar(O_RDY), 1);
@@ -833,7 +837,7 @@ if constexpr (kRope) {
         }
         tmem_wait_st();
         tc_fence_before();
-        mbar_arrive(bar(P_FULL + s));
+        mbar_arrive(p_full(s, i));
         note(8 * i + 2);
       }
       note(8 * n_tiles + 3);
@@ -1009,7 +1013,7 @@ if constexpr (kRope) {
             wait_bar(wc, bar(V_FULL + i % kVStages), (uint32_t)((i / kVStages) & 1), 4, i);
             for (int s = 0; s < n_sub; ++s) {
               note(8 * i + 2 + s);
-              wait_bar(wc, bar(P_FULL + s), (uint32_t)(i & 1), 5, i);
+              wait_bar(wc, p_full(s, i), s_parity(i), 5, i);
               tc_fence_after();
               issue_pv(s, i, n_cur, opens_cur);
               if (s == last_sub && leader) mma_commit(bar(V_EMPTY + i % kVStages));
@@ -1040,7 +1044,7 @@ if constexpr (kRope) {
           wait_bar(wc, bar(V_FULL + i % kVStages), (uint32_t)((i / kVStages) & 1), 4, i);
           for (int s = 0; s < n_sub; ++s) {
             note(8 * i + 2 + s);
-            wait_bar(wc, bar(P_FULL + s), (uint32_t)(i & 1), 5, i);
+            wait_bar(wc, p_full(s, i), s_parity(i), 5, i);
             tc_fence_after();
             issue_pv(s, i, n_cur, opens_cur);
             if (kWalk && has_next && opens_next && leader) mma_commit(bar(O_RDY + s));

@@ -28,6 +28,22 @@ def test_head_dim_64_on_the_tensor_cores(gu, n, H, Hkv, shards, causal):
                                     causal=causal))
 
 
+def test_head_dim_64_warps_at_different_speeds(gu):
+    """Cold caches and many short shards let the warps of a sub-tile drift a tile apart; every run is the same."""
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload("d64_drift", 2, 1500, 1500, 6, 2, 64, "bf16", "random", "random", 40, 40, seed=1500)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    o_ref, lse_ref = oracle.attention_unsharded(w.q, w.k, w.v, w.scale)
+    flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
+    for i in range(20):
+        flush.fill_(i)
+        o, lse = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+        gu.check_output(o, lse, o_ref, lse_ref, w.tol, f"run {i}")
+    assert plan.device_status() == 0
+    plan.destroy()
+
+
 def test_head_dim_64_without_a_workspace_takes_the_alu_kernel(gu):
     from paper_2507_05228_b200 import binding as cb
     w = wl.make_workload("d64_nows", 1, 200, 200, 8, 2, 64, "bf16", "random", "random", 3, 3, seed=7)
