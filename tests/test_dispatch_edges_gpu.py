@@ -60,6 +60,19 @@ def test_head_dim_64_without_a_workspace_takes_the_alu_kernel(gu):
     plan.destroy()
 
 
+@pytest.mark.parametrize("n_q,n_kv,H,Hkv,d,B,shards,dtype,causal", [
+    (1, 1, 2, 2, 64, 1, 1, "f32", True),          # one key
+    (1, 300, 6, 2, 64, 2, 3, "bf16", True),       # one query row on the ALU route: key groups share the row
+    (17, 33, 3, 1, 128, 1, 2, "f32", False),      # one row and one key more than a piece / a tile
+    (640, 640, 8, 8, 64, 8, 4, "f32", True),      # wide form: 64-row tiles, masked and unmasked 64-key tiles
+    (512, 512, 4, 4, 128, 12, 4, "f32", False),   # wide form at head_dim 128
+    (300, 300, 8, 8, 64, 8, 60, "f32", True),     # five keys per shard: chunks of many shards in a tile
+])
+def test_alu_kernel_forms(gu, n_q, n_kv, H, Hkv, d, B, shards, dtype, causal):
+    gu.full_parity(wl.make_workload(f"alu_{n_q}_{d}", B, n_q, n_kv, H, Hkv, d, dtype, "random", "random",
+                                    1 if n_q == 1 else shards, shards, seed=n_q + d, causal=causal))
+
+
 @pytest.mark.parametrize("n_q,n_kv,P,causal", [(128, 128, 2, True), (129, 200, 2, True), (300, 900, 7, False), (40, 64, 64, True)])
 def test_new_plans_have_the_same_arrays_on_the_device(gu, n_q, n_kv, P, causal):
     """vis and pair_class come from the host up to 256 entries and from a kernel above; two plans alive at a time, and a
