@@ -238,8 +238,8 @@ cascade_status_t cascade_merge_peers(cascade_dtype_t dtype, int32_t batch, int32
  * (n, w, o) across shards, so no partial is written to memory; by the identity of Section 5.2.3 the
  * result equals cascade_merge(cascade_attn_partials(...)).  Output in token order:
  *   o_out [batch][n_q][n_heads][head_dim] with strides; lse_out optional fp32 [batch][n_q][n_heads].
- * For n_q == 1 (decode, Appendix F "Caching") the KV shards are processed as independent partials in
- * `workspace` and merged by a second launch.  The tensor-core route (bf16, head_dim 128) uses `workspace` for
+ * For n_q == 1 (decode, Appendix F "Caching") the KV shards are processed as independent partials that meet on chip, in
+ * one launch (`workspace` is checked but not used).  The tensor-core route (bf16, head_dim 128) uses `workspace` for
  * the shard-major K/V copies as cascade_attn_partials does.  Size: cascade_workspace_bytes(CASCADE_CALL_SHARDED).
  */
 cascade_status_t cascade_attn_sharded(const cascade_plan_t* plan, cascade_dtype_t dtype, int32_t batch,
@@ -365,10 +365,10 @@ cascade_status_t cascade_attn_sharded_host(const cascade_plan_t* plan, cascade_d
  * calls this function with the token's position: the causal mask (key token <= query position) then admits exactly
  * the cache rows written so far, and the new row belongs to its shard's list without any list being rebuilt.
  * Recomputes VIS and PAIR_CLASS for query position q_pos_offset + token index; the index lists do not change.  On a
- * device plan with more than 256 (query row, KV shard) entries two small kernels rewrite the device arrays in stream
+ * device plan with more than 256 (query row, KV shard) entries a small kernel rewrites the device arrays in stream
  * order from the plan's own index lists (no host computation, no upload; the host copies that cascade_plan_get and
  * cascade_plan_dense_mask return are brought up to date when they are next asked for).  Smaller plans (a decode
- * step), host-only plans and plans over resident K/V rows (kv_pos) recompute on the host and upload in stream order.  Works for any n_q (a prefill chunk that slides along the sequence);
+ * step), host-only plans and plans over resident K/V rows (kv_pos) recompute on the host and update the device in stream order.  Works for any n_q (a prefill chunk that slides along the sequence);
  * the work-sorted order of the plan's query tiles is left as it was built, which affects speed only.
  * Calls that use the plan before and after must be on `stream` or ordered with it.
  * Cache rows beyond the new position need not be initialised (see cascade_attn_partials); rows at or before it must be
@@ -384,18 +384,13 @@ cascade_status_t cascade_plan_advance(cascade_plan_t* plan, int32_t q_pos_offset
  *
  * Who it is for: callers that cannot hand over scratch memory and cannot allocate it either -- a server whose
  * cache manager already owns all free HBM, a decode loop that must not hit the device-wide synchronisation of
- * cudaMalloc / cudaFree, a plug-in that only receives raw pointers.  The per-shard partials that the merge
- * kernel combines live in a 16 MiB array compiled into the library (every GPU that loads the library carries
- * it until the process exits).  The call issues no cudaMalloc, cudaFree or other allocating routine.
+ * cudaMalloc / cudaFree, a plug-in that only receives raw pointers.  The per-shard partials meet on chip, so the call needs
+ * no scratch memory; it issues no cudaMalloc, cudaFree or other allocating routine.
  *
  *  - Limit: batch * n_kv_shards * n_heads * 264 bytes (rounded up per region to 256) must fit in 16 MiB,
  *    e.g. batch 64 x 16 shards x 32 heads = 8.3 MiB.  Larger problems return CASCADE_ERR_WORKSPACE with a
  *    message naming the sizes; use cascade_attn_sharded with a workspace for those.
- *  - The first call on each device looks up the array's device address (the device current at that moment).
- *    Make that first call during start-up, before any stream capture.
- *  - All calls share the one array.  Its contents are overwritten completely by each call before they are read,
- *    so results never depend on an earlier call; but two calls whose kernels overlap on the GPU (different
- *    streams, no ordering between them) race on it.  Keep calls on one stream or order them with events.
+ *  - Make the first call on each device during start-up, before any stream capture (it loads the kernel).
  *  - Inputs, outputs, strides, stream and results are exactly those of cascade_attn_sharded.
  */
 cascade_status_t cascade_attn_decode_static(const cascade_plan_t* plan, int32_t batch, int32_t n_heads,

@@ -368,9 +368,9 @@ def cascade_attn_sharded_host(plan: Plan, q_host: torch.Tensor, k_host: torch.Te
 
 def cascade_attn_decode_static(plan: Plan, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, scale: float, out=None,
                                want_lse: bool = True):
-    """Decode step (one query row per sequence) that uses the library's built-in 16 MiB scratch array instead of
-    a workspace: for callers that can neither pass nor allocate scratch memory.  Only the output tensors are
-    created here; the C call itself allocates nothing.  Returns (o [B, 1, H, 128], lse or None)."""
+    """Decode step (one query row per sequence) without a workspace: for callers that can neither pass nor allocate
+    scratch memory.  Only the output tensors are created here; the C call itself allocates nothing.
+    Returns (o [B, 1, H, 128], lse or None)."""
     return _native().attn_decode_static(plan.handle, q, k, v, scale, out, want_lse)
 
 

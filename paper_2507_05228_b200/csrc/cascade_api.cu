@@ -1,5 +1,6 @@
 // C ABI entry points: argument checks, plan construction (host) and kernel dispatch.
 #include <stdarg.h>
+#include <stddef.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -60,7 +61,7 @@ static cascade_status_t cuda_fail(cudaError_t e, const char* what) {
 }
 
 // Number of keys of all shards that a query at position `pos` sees.
-static int64_t visible_keys(const cascade_plan& pl, int map, int64_t pos) {
+int64_t visible_keys(const cascade_plan& pl, int map, int64_t pos) {
   const int n_kv = pl.dev.n_kv;
   if (!pl.dev.causal) return n_kv;
   if (!pl.kv_pos.empty()) {
@@ -122,10 +123,11 @@ static void fill_vis(const cascade_plan& pl, int mp, int q_pos_offset, int32_t* 
 }
 
 // Whether vis and pair_class of a device plan are computed on the host.  A decode step (one query row, a few KV shards) is
-// a handful of binary searches and a 64-byte upload: 3 us on the host against 12 us for a dependent-load kernel.  Anything
-// larger goes to the device, except with kv_pos, which the device arrays do not hold.
+// a handful of binary searches, and the result travels with a launch; anything larger is searched for by a kernel, except
+// with kv_pos, which the device arrays do not hold.
 static bool vis_from_host(const cascade_plan& pl) {
-  return !pl.kv_pos.empty() || (int64_t)pl.dev.n_maps * pl.dev.n_q * pl.dev.n_kv_shards <= 256;
+  return !pl.kv_pos.empty() || ((int64_t)pl.dev.n_maps * pl.dev.n_q * pl.dev.n_kv_shards <= kMaxGivenVis &&
+                                (int64_t)pl.dev.n_maps * pl.dev.n_q_shards * pl.dev.n_kv_shards <= kMaxGivenVis);
 }
 
 // EMPTY / PARTIAL / FULL per (query shard, KV shard) from the prefix lengths of the shard's first and last row
@@ -573,7 +575,11 @@ cascade_status_t cascade_plan_advance(cascade_plan_t* plan, int32_t q_pos_offset
   }
   plan->dev.q_pos_offset = q_pos_offset;
   refresh_host_vis(*plan, true);
-  if (plan->dev_blob) {
+  if (plan->dev_blob && plan->vis.size() <= kMaxGivenVis && plan->pair_class.size() <= kMaxGivenVis) {
+    cudaError_t e = launch_plan_set(d, plan->vis.data(), (int)plan->vis.size(), plan->pair_class.data(),
+                                    (int)plan->pair_class.size(), (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "cascade_plan_advance: launch");
+  } else if (plan->dev_blob) {
     // pageable source: the runtime stages it before the call returns, the device copy lands in stream order
     cudaError_t e = cudaMemcpyAsync(const_cast<int32_t*>(d.vis), plan->vis.data(), plan->vis.size() * 4,
                                     cudaMemcpyHostToDevice, (cudaStream_t)stream);
@@ -684,8 +690,15 @@ static AttnParams make_params(const cascade_plan_t* plan, int32_t batch, int32_t
   p.Hkv = Hkv;
   p.G = H / Hkv;
   p.d = d;
+  p.rule_kv_heads = Hkv;
   p.scale = scale;
   return p;
+}
+
+cudaError_t run_decode_fused(const cascade_plan& plan, const AttnParams& p, cudaStream_t stream) {
+  DecodeStep none;
+  memset(&none, 0, sizeof(none));
+  return launch_decode_fused(p, none, visible_keys(plan, 0, (int64_t)plan.q_idx[0] + plan.dev.q_pos_offset), stream);
 }
 
 static bool use_decode(const cascade_plan_t* plan, cascade_dtype_t dtype, int H, int Hkv, int d) {
@@ -963,7 +976,7 @@ static cascade_status_t attn_sharded_impl(const char* fn, const cascade_plan_t* 
                                           cascade_strides_t k_strides, const void* v, cascade_strides_t v_strides,
                                           const float* rope_table, int32_t n_positions, void* o_out,
                                           cascade_strides_t o_strides, float* lse_out, void* workspace,
-                                          size_t workspace_bytes, void* stream) {
+                                          size_t workspace_bytes, void* stream, int32_t rule_kv_heads = 0) {
   cascade_status_t s = check_attn_args(fn, plan, dtype, batch, n_heads, n_kv_heads, head_dim, scale, q, q_strides, k,
                                        k_strides, v, v_strides);
   if (s != CASCADE_OK) return s;
@@ -977,6 +990,7 @@ static cascade_status_t attn_sharded_impl(const char* fn, const cascade_plan_t* 
   }
   AttnParams p = make_params(plan, batch, n_heads, n_kv_heads, head_dim, scale, q, q_strides, k, k_strides, v,
                              v_strides);
+  if (rule_kv_heads) p.rule_kv_heads = rule_kv_heads;
   if (rope_table) {
     if (!aligned16(rope_table)) {
       set_error("%s: the positional table must be 16-byte aligned", fn);
@@ -1001,36 +1015,19 @@ static cascade_status_t attn_sharded_impl(const char* fn, const cascade_plan_t* 
   }
   cudaStream_t st = (cudaStream_t)stream;
   if (use_decode(plan, dtype, n_heads, n_kv_heads, head_dim)) {
-    // one query row per sequence: every KV shard is an independent partial, combined by the merge kernel
+    // One query row per sequence: partials and post-pass in one kernel.  (The workspace the interface asks for is checked but
+    // not used: the partials meet in distributed shared memory.)
     const size_t need = decode_ws_bytes(plan, dtype, batch, n_heads, head_dim);
     if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) {
       set_error("%s: workspace of %zu bytes (256-byte aligned) required, got %zu", fn, need, workspace_bytes);
       return CASCADE_ERR_WORKSPACE;
     }
-    const size_t rows = (size_t)batch * plan->dev.n_kv_shards * plan->dev.n_q * n_heads;
-    char* ws = (char*)workspace;
-    p.fused = 0;
-    p.o_part = ws;
-    p.m_part = (float*)(ws + align_up(rows * head_dim * elt_size(dtype), 256));
-    p.l_part = (float*)((char*)p.m_part + align_up(rows * 4, 256));
-    cudaError_t e = launch_decode(p, st);
+    p.fused = 1;
+    p.o_out = o_out;
+    p.os = {o_strides.batch, o_strides.token, o_strides.head};
+    p.lse_out = lse_out;
+    cudaError_t e = run_decode_fused(*plan, p, st);
     if (e != cudaSuccess) return cuda_fail(e, "attention (fused route): decode launch");
-    MergeParams mp;
-    mp.o_part = p.o_part;
-    mp.m_part = p.m_part;
-    mp.l_part = p.l_part;
-    mp.row_scatter = nullptr;  // a single query row: slot 0 is token 0
-    mp.row_scatter_batch_stride = 0;
-    mp.o_out = o_out;
-    mp.os = {o_strides.batch, o_strides.token, o_strides.head};
-    mp.lse_out = lse_out;
-    mp.batch = batch;
-    mp.n_parts = plan->dev.n_kv_shards;
-    mp.n_rows = plan->dev.n_q;
-    mp.H = n_heads;
-    mp.d = head_dim;
-    e = launch_merge(mp, dtype, st);
-    if (e != cudaSuccess) return cuda_fail(e, "attention (fused route): merge launch");
     return CASCADE_OK;
   }
   p.fused = 1;
@@ -1162,29 +1159,42 @@ cascade_status_t cascade_decode_step_rope(cascade_plan_t* plan, int32_t batch, i
     set_error("%s: pointers and row strides must be 16-byte aligned", fn);
     return CASCADE_ERR_INVALID_ARG;
   }
-  const size_t part_bytes = align_up(decode_ws_bytes(plan, CASCADE_BF16, batch, n_heads, kHeadDim), 256);
-  const size_t need = part_bytes + align_up((size_t)batch * n_heads * kHeadDim * 2, 256);
+  const size_t need = align_up(decode_ws_bytes(plan, CASCADE_BF16, batch, n_heads, kHeadDim), 256) + align_up((size_t)batch * n_heads * kHeadDim * 2, 256);
   if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) {
     set_error("%s: workspace of %zu bytes (256-byte aligned) required, got %zu", fn, need, workspace_bytes);
     return CASCADE_ERR_WORKSPACE;
   }
-  // the new token sits at `position`: it is the query position, and the mask admits the cache rows up to it
-  s = cascade_plan_advance(plan, position - plan->q_idx[0], stream);
-  if (s != CASCADE_OK) return s;
-  char* ws = (char*)workspace;
-  void* q_rot = ws + part_bytes;
+  // The new token sits at `position`: it is the query position, and the mask admits the cache rows up to it.  A plan with
+  // few prefixes gets them computed here and carried by the one launch of the step; otherwise a kernel moves them first.
+  DecodeStep step;
+  memset(&step, 0, offsetof(DecodeStep, vis));
   cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = launch_append_rope(batch, n_heads, n_kv_heads, q_new, {q_strides.batch, q_strides.token, q_strides.head},
-                                     k_new, {k_new_strides.batch, k_new_strides.token, k_new_strides.head}, v_new,
-                                     {v_new_strides.batch, v_new_strides.token, v_new_strides.head}, q_rot, k_cache,
-                                     {k_cache_strides.batch, k_cache_strides.token, k_cache_strides.head}, v_cache,
-                                     {v_cache_strides.batch, v_cache_strides.token, v_cache_strides.head}, position,
-                                     reinterpret_cast<const float2*>(rope_table), st);
-  if (e != cudaSuccess) return cuda_fail(e, "cascade_decode_step_rope: append launch");
-  const cascade_strides_t qr = {(int64_t)n_heads * kHeadDim, (int64_t)n_heads * kHeadDim, kHeadDim};
-  return attn_sharded_impl(fn, plan, CASCADE_BF16, batch, n_heads, n_kv_heads, kHeadDim, scale, q_rot, qr, k_cache,
-                           k_cache_strides, v_cache, v_cache_strides, nullptr, 0, o_out, o_strides, lse_out, ws, part_bytes,
-                           st);
+  cudaError_t e = cudaSuccess;
+  plan->dev.q_pos_offset = position - plan->q_idx[0];
+  if (vis_from_host(*plan)) {
+    refresh_host_vis(*plan, true);
+    step.n_vis = (int32_t)plan->vis.size();
+    memcpy(step.vis, plan->vis.data(), plan->vis.size() * 4);
+  } else {
+    plan->host_vis_stale = true;
+    e = launch_plan_advance(plan->dev, plan->dev.q_pos_offset, st);
+    if (e != cudaSuccess) return cuda_fail(e, "cascade_decode_step_rope: plan advance");
+  }
+  step.rope = reinterpret_cast<const float2*>(rope_table);
+  step.k_new = static_cast<const __nv_bfloat16*>(k_new);
+  step.v_new = static_cast<const __nv_bfloat16*>(v_new);
+  step.kns = {k_new_strides.batch, k_new_strides.token, k_new_strides.head};
+  step.vns = {v_new_strides.batch, v_new_strides.token, v_new_strides.head};
+  step.position = position;
+  AttnParams p = make_params(plan, batch, n_heads, n_kv_heads, kHeadDim, scale, q_new, q_strides, k_cache, k_cache_strides,
+                             v_cache, v_cache_strides);
+  p.fused = 1;
+  p.o_out = o_out;
+  p.os = {o_strides.batch, o_strides.token, o_strides.head};
+  p.lse_out = lse_out;
+  e = launch_decode_fused(p, step, visible_keys(*plan, 0, position), st);
+  if (e != cudaSuccess) return cuda_fail(e, "cascade_decode_step_rope: launch");
+  return CASCADE_OK;
 }
 
 cascade_status_t cascade_attn_sharded_host(const cascade_plan_t* plan, cascade_dtype_t dtype, int32_t batch,
@@ -1272,7 +1282,7 @@ cascade_status_t cascade_attn_sharded_host(const cascade_plan_t* plan, cascade_d
     cascade_status_t rc = attn_sharded_impl(fn, plan, dtype, batch, G * gs, gs, head_dim, scale, ws + L.q + q_off, qs,
                                             ws + L.k + kv_off, ks, ws + L.v + kv_off, ks, nullptr, 0,
                                             ws + L.o + q_off, qs, nullptr, L.inner_bytes ? ws + L.inner : nullptr,
-                                            L.inner_bytes, st);
+                                            L.inner_bytes, st, n_kv_heads);
     if (rc != CASCADE_OK) return rc;
     e = cudaEventRecord(hs.computed[g], st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(hs.d2h, hs.computed[g], 0);

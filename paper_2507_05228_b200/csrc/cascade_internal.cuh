@@ -45,6 +45,9 @@ struct AttnParams {
   const void* v;
   Strides qs, ks, vs;
   int32_t batch, H, Hkv, G, d;
+  // KV heads of the whole problem: more than Hkv where a call computes a part of the heads at a time.  Rules that decide how
+  // sums are split go by it, so that the parts get the same bits as one call would.
+  int32_t rule_kv_heads;
   float scale;
   int32_t fused;  // 0: one job per KV shard, write (u, m, l); 1: walk all KV shards, write o (+lse)
   void* o_part;
@@ -73,6 +76,17 @@ __device__ __forceinline__ int64_t cascade_checked_index(int64_t i, int64_t n, i
 #else
 #define CASCADE_CHECKED(i, n, status, code) (i)
 #endif
+
+// What a decode step adds to the fused decode kernel (cascade_decode_step_rope); all zero for a plain decode.
+constexpr int kMaxGivenVis = 256;
+struct DecodeStep {
+  const float2* rope;  // positional table, or null: no rotation, no append
+  const __nv_bfloat16 *k_new, *v_new;
+  Strides kns, vns;
+  int32_t position;  // row of the caches that takes the new token
+  int32_t n_vis;     // > 0: the prefix lengths of the plan for this position (n_maps * n_kv_shards of them) come along
+  int32_t vis[kMaxGivenVis];
+};
 
 struct MergeParams {
   const void* o_part;
@@ -140,10 +154,16 @@ cudaError_t launch_rope_table(int32_t n_positions, int32_t head_dim, double base
 cudaError_t launch_rope_apply(cascade_dtype_t dtype, int32_t batch, int32_t n_rows, int32_t n_heads, int32_t head_dim,
                               const void* x, Strides xs, int32_t first_position, const float2* table, void* y, Strides ys,
                               cudaStream_t stream);
-cudaError_t launch_append_rope(int32_t batch, int32_t H, int32_t Hkv, const void* q_new, Strides qs, const void* k_new,
-                               Strides kns, const void* v_new, Strides vns, void* q_rot, void* k_cache, Strides kcs,
-                               void* v_cache, Strides vcs, int32_t position, const float2* table, cudaStream_t stream);
 cudaError_t launch_decode(const AttnParams& p, cudaStream_t stream);
+// decode of all shards with the post-pass in the same kernel; n_visible = keys the (longest) query row sees
+cudaError_t launch_decode_fused(const AttnParams& p, const DecodeStep& step, int64_t n_visible, cudaStream_t stream);
+// vis (n_vis values) and pair_class (n_cls) of a small plan written from the launch's own arguments
+cudaError_t launch_plan_set(const PlanDev& d, const int32_t* vis, int n_vis, const uint8_t* pair_class, int n_cls,
+                            cudaStream_t stream);
+// number of keys of all shards that a query at position `pos` sees
+int64_t visible_keys(const cascade_plan& pl, int map, int64_t pos);
+// the fused decode of a checked call: cascade_attn_sharded, cascade_attn_decode_static
+cudaError_t run_decode_fused(const cascade_plan& plan, const AttnParams& p, cudaStream_t stream);
 // vis and pair_class of a device plan recomputed for a new q_pos_offset (plans without kv_pos)
 cudaError_t launch_plan_advance(const PlanDev& d, int32_t q_pos_offset, cudaStream_t stream);
 cudaError_t launch_merge(const MergeParams& p, cascade_dtype_t dtype, cudaStream_t stream);

@@ -1,17 +1,26 @@
 // Decode step with a token-sharded KV cache (Appendix F, "Caching"): one new query row per sequence against
 // every KV shard.  Each shard is an independent partial (the Attention-Pass algorithm with a single query row) and the K/V rows
-// of the cache are read exactly once, so the kernel must be bound by HBM reads of gathered 256-byte rows.
+// of the cache are read exactly once, so the kernels must be bound by HBM reads of gathered 256-byte rows.
 //
-// One CTA = (KV shard, KV head, sequence); each of its 4 warps walks blocks of 16 gathered keys.  The G query
-// heads that share the KV head ("repeat_kv") form the M rows of warp-level mma.m16n8k16 products, which keeps the
-// instruction count per loaded byte low enough for the memory system to be the limit (plain FMA code was
-// issue-bound at ~60 % of the HBM rate).  No shared-memory staging is needed because the contraction order is
-// free: the k index of an MMA may be any fixed permutation of head_dim / of the keys as long as both operands
-// use the same one, so every thread loads contiguous 16-byte pieces straight from global memory into fragments:
-//   logits  S[head, key]   : A = Q (heads x d), B = K (keys x d);   thread (x = lane/4, j = lane%4) holds
-//                            d = 32j .. 32j+31 of Q row x and of K row x of the 8-key block
-//   output  O[head, d]     : A = P (heads x 16 keys, taken directly from two S accumulators), B = V; the thread
-//                            holds d = 16x .. 16x+15 of V rows 2j, 2j+1, 2j+8, 2j+9 and pairs them with PRMT
+// decode_kernel (partials): one CTA = (KV shard, KV head, sequence); decode_fused_kernel: all shards, post-pass included.
+// In both, a warp walks blocks of 16 gathered keys with warp-level mma.m16n8k16 products, which keeps the instruction count
+// per loaded byte low enough for the memory system to be the limit (plain FMA code was issue-bound at ~60 % of the HBM
+// rate).  Keys are the M rows of the logits and head_dim the M rows of the output, so that the G query heads that share the
+// KV head ("repeat_kv") are the 8 columns and no row is padding: 16 products and 32 accumulators per block (with the heads as
+// M rows it was 32 products, and 8 registers for rows that do not exist).  No staging of K or V is needed because the
+// contraction order is free: the k index of an MMA may be any fixed permutation of head_dim / of the keys as long as both
+// operands use the same one, so every thread loads 16-byte pieces straight from global memory into fragments
+// (x = lane / 4, j = lane % 4):
+//   logits  S^T[key, head] : A = K, rows x and x + 8 of the block; B = Q^T; pieces d = 64c + 16j .. + 15 (c < 2)
+//   output  O^T[d, head]   : A = V^T, pieces d = 16x .. + 15 of V rows 2j, 2j+1, 2j+8, 2j+9, paired with PRMT;
+//                            B = P^T, the bf16 weights of S^T transposed with movmatrix
+// so that the loads of a row cover whole 128-byte lines.  (One 32-byte load per piece was 2 to 4 % slower than two of 16
+// bytes at every size.)
+// 64 registers hold the loads in flight.  Anything else kept through the loop ends up spilled, and a spilled value comes back
+// from L2, because the streaming loads evict it from L1: the query fragments therefore live in shared memory.
+#include <algorithm>
+#include <type_traits>
+
 #include "cascade_internal.cuh"
 
 namespace cascade {
@@ -30,14 +39,11 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Same product when rows 8-15 of A are zero: their accumulators never change, so a few shared dummy registers can
-// stand in for them (saves registers; callers rotate the dummies to keep the dependency chains short).
-__device__ __forceinline__ void mma_16816_top(float& c0, float& c1, float& z0, float& z1, uint32_t a0, uint32_t a2,
-                                              uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c0), "+f"(c1), "+f"(z0), "+f"(z1)
-      : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
+// 8 x 8 transpose of 16-bit elements across a warp (lane (x, j) holds row x, columns 2j and 2j + 1)
+__device__ __forceinline__ uint32_t transpose8(uint32_t v) {
+  uint32_t r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+  return r;
 }
 
 __device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
@@ -45,22 +51,190 @@ __device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-__device__ __forceinline__ void load64(const __nv_bfloat16* p, uint32_t (&r)[16], int o) {
+// 32 bytes, streaming; volatile so that the loads stay where the pipeline below puts them
+__device__ __forceinline__ void load32(const __nv_bfloat16* p, uint32_t* r) {
+#pragma unroll
+  for (int i = 0; i < 8; i += 4)
+    asm volatile("ld.global.cs.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[i]), "=r"(r[i + 1]), "=r"(r[i + 2]), "=r"(r[i + 3])
+                 : "l"(p + 2 * i)
+                 : "memory");
+}
+
+// Query fragments of a CTA in shared memory: B operand of k-step s, lane (x = head, j) -> its two registers.
+struct DecodeQuery {
+  uint2 frag[8][32];
+};
+// Filled by one warp from the thread's pieces qf[8 c + e] = columns 64c + 16j + 2e, + 1 of head x (zero from G on).
+__device__ __forceinline__ void publish_query(DecodeQuery& q, const uint32_t (&qf)[16], int lane) {
+#pragma unroll
+  for (int s = 0; s < 8; ++s) q.frag[s][lane] = make_uint2(qf[2 * s], qf[2 * s + 1]);
+}
+// The pieces of one head vector.
+__device__ __forceinline__ void load_query(const __nv_bfloat16* row, int j, uint32_t (&qf)[16]) {
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    const uint4 t = __ldcs(reinterpret_cast<const uint4*>(p) + c);
-    r[o + 4 * c] = t.x; r[o + 4 * c + 1] = t.y; r[o + 4 * c + 2] = t.z; r[o + 4 * c + 3] = t.w;
+    const uint4 t = __ldg(reinterpret_cast<const uint4*>(row + 64 * (c >> 1) + 16 * j + 8 * (c & 1)));
+    qf[4 * c] = t.x; qf[4 * c + 1] = t.y; qf[4 * c + 2] = t.z; qf[4 * c + 3] = t.w;
   }
 }
 
+struct DecodeState {
+  float o[8][4];     // o[e][2 r + h]: head 2j + h, column 16x + 2e + r
+  float m[2], l[2];  // heads 2j, 2j + 1 (log2 units); l is this thread's share (its key rows x, x + 8)
+};
+__device__ __forceinline__ void decode_init(DecodeState& st) {
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) st.o[e][i] = 0.f;
+  st.m[0] = st.m[1] = -INFINITY;
+  st.l[0] = st.l[1] = 0.f;
+}
+
+// Walks `count` blocks of 16 keys; block t is the keys kv_idx[at .. at + n - 1] (n >= 1; 16 at most are taken) with
+// (at, n) = get(t).
+// kAhead: the key rows of block t + 1 are requested as soon as the logits of block t are formed, its value rows after the
+// product of block t, its tokens a block earlier still, all into registers that have just come free: one memory latency per
+// block instead of two and the arithmetic (a block took 3200 cycles one after another).  Without it nothing is spilled,
+// which is the better trade where 16 warps per SM cover the latencies anyway (partials of 64 sequences of 16384 tokens: 630
+// us without, 820 with; all shards in one kernel: 711 without, 620 with).
+template <bool kAhead, typename Get>
+__device__ __forceinline__ void decode_walk(DecodeState& st, const DecodeQuery& q, const PlanDev& pl, const int32_t* kv_idx,
+                                            int count, Get get, const __nv_bfloat16* kp, int64_t k_token,
+                                            const __nv_bfloat16* vp, int64_t v_token, int lane, float cs) {
+  if (count <= 0) return;
+  const int x = lane >> 2, j = lane & 3;
+  uint32_t ka[16], kb[16], vr[4][8];
+  auto token = [&](int2 e) {  // lane l: token of key l (clamped to the last key; masked below)
+    return (int)CASCADE_CHECKED((int64_t)__ldg(kv_idx + e.x + min(lane & 15, e.y - 1)), pl.n_kv, pl.status, 106);
+  };
+  auto load_k = [&](int tok) {  // rows x and x + 8
+    const __nv_bfloat16* r0 = kp + (int64_t)__shfl_sync(0xffffffffu, tok, x) * k_token;
+    const __nv_bfloat16* r1 = kp + (int64_t)__shfl_sync(0xffffffffu, tok, x + 8) * k_token;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      load32(r0 + 64 * c, ka + 8 * c);
+      load32(r1 + 64 * c, kb + 8 * c);
+    }
+  };
+  auto load_v = [&](int tok) {  // rows 2j, 2j + 1, 2j + 8, 2j + 9
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr)
+      load32(vp + (int64_t)__shfl_sync(0xffffffffu, tok, 2 * j + (rr & 1) + (rr >> 1) * 8) * v_token, vr[rr]);
+  };
+  int2 e;
+  int tok;
+  if constexpr (kAhead) {
+    e = get(0);
+    tok = token(e);
+    load_k(tok);
+    load_v(tok);
+    if (count > 1) tok = token(get(1));
+  }
+#pragma unroll 1
+  for (int t = 0; t < count; ++t) {
+    if constexpr (!kAhead) {
+      e = get(t);
+      tok = token(e);
+      load_k(tok);
+      load_v(tok);
+    }
+    const int n_keys = e.y;
+    const bool more = kAhead && t + 1 < count;
+    float sc[4] = {0.f, 0.f, 0.f, 0.f};  // (key x, head 2j), (x, 2j + 1), (x + 8, 2j), (x + 8, 2j + 1)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint2 b = q.frag[i][lane];
+      mma_16816(sc, ka[2 * i], kb[2 * i], ka[2 * i + 1], kb[2 * i + 1], b.x, b.y);
+    }
+    if (more) {
+      e = get(t + 1);
+      load_k(tok);
+    }
+    float alpha[2], p0[2], p1[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float t0 = x < n_keys ? sc[h] * cs : -INFINITY, t1 = x + 8 < n_keys ? sc[2 + h] * cs : -INFINITY;
+      float mx = fmaxf(t0, t1);
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      const float m_new = fmaxf(st.m[h], mx);  // finite: key 0 of the block exists
+      alpha[h] = ex2f(st.m[h] - m_new);        // ex2(-inf) = 0 on the first block
+      p0[h] = ex2f(t0 - m_new);
+      p1[h] = ex2f(t1 - m_new);
+      st.l[h] = st.l[h] * alpha[h] + (p0[h] + p1[h]);
+      st.m[h] = m_new;
+    }
+    const uint32_t pa = transpose8(pack2_bf16(p0[0], p0[1]));  // -> head x, keys 2j, 2j + 1
+    const uint32_t pb = transpose8(pack2_bf16(p1[0], p1[1]));  // -> head x, keys 2j + 8, 2j + 9
+    if (__any_sync(0xffffffffu, alpha[0] != 1.f || alpha[1] != 1.f)) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) st.o[i][c] *= alpha[c & 1];
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      mma_16816(st.o[i], __byte_perm(vr[0][i], vr[1][i], 0x5410), __byte_perm(vr[0][i], vr[1][i], 0x7632),
+                __byte_perm(vr[2][i], vr[3][i], 0x5410), __byte_perm(vr[2][i], vr[3][i], 0x7632), pa, pb);
+    if (more) {
+      load_v(tok);
+      if (t + 2 < count) tok = token(get(t + 2));
+    }
+  }
+}
+
+// Combines the warps of a CTA (each saw disjoint keys) through shared memory.
+template <int G, int NW>
+struct DecodeShared {
+  float m[NW][G], l[NW][G];
+  float o[NW][G][132];
+};
+template <int G, int NW>
+__device__ __forceinline__ void decode_publish(DecodeShared<G, NW>& sh, DecodeState& st, int warp, int lane) {
+  const int x = lane >> 2, j = lane & 3;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float l = st.l[h];  // this thread's share of the sum of exponentials -> whole row
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    const int head = 2 * j + h;
+    if (head < G) {
+      if (x == 0) {
+        sh.m[warp][head] = st.m[h];
+        sh.l[warp][head] = l;
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        *reinterpret_cast<float2*>(&sh.o[warp][head][16 * x + 2 * e]) = make_float2(st.o[e][h], st.o[e][2 + h]);
+    }
+  }
+}
+// Output column `col` of head gg: the maximum n, the weight w and the weighted sum, relative to n.
+template <int G, int NW>
+__device__ __forceinline__ void decode_combine(const DecodeShared<G, NW>& sh, int gg, int col, float& n, float& w, float& acc) {
+  n = -INFINITY;
+#pragma unroll
+  for (int w2 = 0; w2 < NW; ++w2) n = fmaxf(n, sh.m[w2][gg]);
+  const float n_use = n == -INFINITY ? 0.f : n;
+  w = 0.f;
+  acc = 0.f;
+#pragma unroll
+  for (int w2 = 0; w2 < NW; ++w2) {
+    const float f = ex2f(sh.m[w2][gg] - n_use);  // 0 for a warp that saw no key
+    w = fmaf(f, sh.l[w2][gg], w);
+    acc = fmaf(f, sh.o[w2][gg][col], acc);
+  }
+}
+
+// Partials.  Four CTAs per SM at 128 registers per thread (no spills).
 template <int G>
-// Four CTAs per SM (128 registers per thread, a few spilled values): 5.78 TB/s on the decode workload against 5.59 with
-// three (168 registers); five or six spill too much (3.9 / 3.6 TB/s).
-__global__ void __launch_bounds__(128, 4) decode_kernel(AttnParams p) {
+__global__ void __launch_bounds__(128, 4) decode_kernel(const __grid_constant__ AttnParams p) {
   constexpr int D = 128;
   constexpr int NW = 4;  // warps per CTA
-  __shared__ float s_m[NW][8], s_l[NW][8];
-  __shared__ float s_o[NW][G * 4][33];  // [warp][head * 4 + j][32 columns + 1 pad]: conflict-free both ways
+  __shared__ DecodeShared<G, NW> sh;
+  __shared__ DecodeQuery s_q;
 
   const PlanDev& pl = p.plan;
   const int P = pl.n_kv_shards;
@@ -84,135 +258,317 @@ __global__ void __launch_bounds__(128, 4) decode_kernel(AttnParams p) {
   }
   const int tok_q = (int)CASCADE_CHECKED((int64_t)pl.q_idx[(size_t)map * pl.n_q], pl.n_q, pl.status, 107);
   const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(p.k) + (int64_t)b * p.ks.batch +
-                            (int64_t)g * p.ks.head + 32 * j;
+                            (int64_t)g * p.ks.head + 16 * j;
   const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(p.v) + (int64_t)b * p.vs.batch +
                             (int64_t)g * p.vs.head + 16 * x;
-
-  // A fragments of Q: row x = head g*G + x (rows >= G are zero), this thread's 32 d-values
-  uint32_t qf[16];
-  if (x < G) {
-    const __nv_bfloat16* qp = static_cast<const __nv_bfloat16*>(p.q) + (int64_t)b * p.qs.batch +
-                              (int64_t)tok_q * p.qs.token + (int64_t)(g * G + x) * p.qs.head + 32 * j;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const uint4 t = __ldg(reinterpret_cast<const uint4*>(qp) + c);
-      qf[4 * c] = t.x; qf[4 * c + 1] = t.y; qf[4 * c + 2] = t.z; qf[4 * c + 3] = t.w;
-    }
-  } else {
+  if (warp == 0) {
+    uint32_t qf[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) qf[c] = 0u;
-  }
-  const float cs = p.scale * 1.4426950408889634f;  // logits in log2 units
-
-  float o[16][2];
-#pragma unroll
-  for (int t = 0; t < 16; ++t) o[t][0] = o[t][1] = 0.f;
-  float zz[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};  // accumulators of the unused rows 8-15
-  float m_run = -INFINITY, l_run = 0.f;  // for head x; l is this thread's share (its 4 key columns)
-
-  for (int k0 = warp * 16; k0 < n_vis; k0 += NW * 16) {
-    const int last = n_vis - 1;
-    // gathered rows: K rows x and x+8 of the block, V rows 2j, 2j+1, 2j+8, 2j+9 (clamped; masked below)
-    uint32_t ka[16], kbv[16];
-    load64(kb + CASCADE_CHECKED((int64_t)__ldg(kv_idx + min(k0 + x, last)), pl.n_kv, pl.status, 106) * p.ks.token, ka, 0);
-    load64(kb + CASCADE_CHECKED((int64_t)__ldg(kv_idx + min(k0 + 8 + x, last)), pl.n_kv, pl.status, 106) * p.ks.token, kbv, 0);
-    uint32_t vr[4][8];
-#pragma unroll
-    for (int rr = 0; rr < 4; ++rr) {
-      const int key = k0 + 2 * j + (rr & 1) + (rr >> 1) * 8;
-      const uint4* src = reinterpret_cast<const uint4*>(vb + CASCADE_CHECKED((int64_t)__ldg(kv_idx + min(key, last)), pl.n_kv, pl.status, 106) * p.vs.token);
-      const uint4 t0 = __ldcs(src), t1 = __ldcs(src + 1);
-      vr[rr][0] = t0.x; vr[rr][1] = t0.y; vr[rr][2] = t0.z; vr[rr][3] = t0.w;
-      vr[rr][4] = t1.x; vr[rr][5] = t1.y; vr[rr][6] = t1.z; vr[rr][7] = t1.w;
-    }
-    // S = Q K^T for the two 8-key blocks; 8 k-steps of 16 over the (permuted) head_dim
-    float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      mma_16816(sa, qf[2 * i], 0u, qf[2 * i + 1], 0u, ka[2 * i], ka[2 * i + 1]);
-      mma_16816(sb, qf[2 * i], 0u, qf[2 * i + 1], 0u, kbv[2 * i], kbv[2 * i + 1]);
-    }
-    // this thread: head x, keys k0 + 2j, +1 (block a) and k0 + 8 + 2j, +1 (block b)
-    float t[4];
-    t[0] = (k0 + 2 * j < n_vis) ? sa[0] * cs : -INFINITY;
-    t[1] = (k0 + 2 * j + 1 < n_vis) ? sa[1] * cs : -INFINITY;
-    t[2] = (k0 + 8 + 2 * j < n_vis) ? sb[0] * cs : -INFINITY;
-    t[3] = (k0 + 9 + 2 * j < n_vis) ? sb[1] * cs : -INFINITY;
-    float mx = fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3]));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const float m_new = fmaxf(m_run, mx);  // finite: key k0 is visible
-    const float alpha = ex2f(m_run - m_new);  // ex2(-inf) = 0 on the first block
-    const float p0 = ex2f(t[0] - m_new), p1 = ex2f(t[1] - m_new), p2 = ex2f(t[2] - m_new), p3 = ex2f(t[3] - m_new);
-    l_run = l_run * alpha + (p0 + p1) + (p2 + p3);
-    m_run = m_new;
-    const uint32_t pa = pack2_bf16(p0, p1), pb = pack2_bf16(p2, p3);
-    if (__any_sync(0xffffffffu, alpha != 1.f)) {
-#pragma unroll
-      for (int tt = 0; tt < 16; ++tt) {
-        o[tt][0] *= alpha;
-        o[tt][1] *= alpha;
-      }
-    }
-    // O += P V : 16 n-tiles of 8 columns; column n of tile tt is d = 16 n + tt
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const uint32_t b0lo = __byte_perm(vr[0][e], vr[1][e], 0x5410), b1lo = __byte_perm(vr[2][e], vr[3][e], 0x5410);
-      const uint32_t b0hi = __byte_perm(vr[0][e], vr[1][e], 0x7632), b1hi = __byte_perm(vr[2][e], vr[3][e], 0x7632);
-      mma_16816_top(o[2 * e][0], o[2 * e][1], zz[(2 * e) & 3][0], zz[(2 * e) & 3][1], pa, pb, b0lo, b1lo);
-      mma_16816_top(o[2 * e + 1][0], o[2 * e + 1][1], zz[(2 * e + 1) & 3][0], zz[(2 * e + 1) & 3][1], pa, pb, b0hi,
-                    b1hi);
-    }
-  }
-  // this thread's share of the sum of exponentials -> whole row
-  l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
-  l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
-  if (x < G) {
-    if (j == 0) {
-      s_m[warp][x] = m_run;
-      s_l[warp][x] = l_run;
-    }
-    // accumulator (tile tt, c0) is column n = 2j -> d = 32j + tt; (tile tt, c1) is n = 2j+1 -> d = 32j + 16 + tt
-#pragma unroll
-    for (int tt = 0; tt < 16; ++tt) {
-      s_o[warp][x * 4 + j][tt] = o[tt][0];
-      s_o[warp][x * 4 + j][16 + tt] = o[tt][1];
-    }
+    if (x < G)
+      load_query(static_cast<const __nv_bfloat16*>(p.q) + (int64_t)b * p.qs.batch + (int64_t)tok_q * p.qs.token +
+                     (int64_t)(g * G + x) * p.qs.head, j, qf);
+    publish_query(s_q, qf, lane);
   }
   __syncthreads();
-  // combine the warps (each saw a disjoint quarter of the keys); thread = output column
+  const float cs = p.scale * 1.4426950408889634f;  // logits in log2 units
+
+  DecodeState st;
+  decode_init(st);
+  decode_walk<false>(st, s_q, pl, kv_idx, (n_vis - warp * 16 + NW * 16 - 1) / (NW * 16),
+                     [&](int t) { const int k0 = (t * NW + warp) * 16; return make_int2(k0, n_vis - k0); }, kb, p.ks.token,
+                     vb, p.vs.token, lane, cs);
+  decode_publish<G, NW>(sh, st, warp, lane);
+  __syncthreads();
+  // thread = output column
 #pragma unroll
   for (int gg = 0; gg < G; ++gg) {
-    float n = -INFINITY;
-#pragma unroll
-    for (int w2 = 0; w2 < NW; ++w2) n = fmaxf(n, s_m[w2][gg]);
-    float wsum = 0.f, acc = 0.f;
-#pragma unroll
-    for (int w2 = 0; w2 < NW; ++w2) {
-      const float f = ex2f(s_m[w2][gg] - n);  // 0 for a warp that saw no key
-      wsum = fmaf(f, s_l[w2][gg], wsum);
-      acc = fmaf(f, s_o[w2][gg * 4 + (tid >> 5)][tid & 31], acc);
-    }
-    o_part[(stat0 + gg) * D + tid] = __float2bfloat16_rn(acc / wsum);
+    float n, w, acc;
+    decode_combine<G, NW>(sh, gg, tid, n, w, acc);
+    o_part[(stat0 + gg) * D + tid] = __float2bfloat16_rn(acc / w);
     if (tid == 0) {
       p.m_part[stat0 + gg] = n * 0.6931471805599453f;  // back to natural-log units
-      p.l_part[stat0 + gg] = wsum;
+      p.l_part[stat0 + gg] = w;
     }
   }
+}
+
+// ---------------------------------------------------------------------------------------------------------------------
+// Decode with the post-pass in the same kernel (the fused route): a cluster of CTAs owns one (KV head, sequence), its warps
+// share the 16-key blocks of all shards' visible prefixes, and the partial (m, l, o) meet in distributed shared memory, so
+// no partial goes to memory and nothing is launched after it.  Bound by HBM reads for large batches and by latency for small
+// ones; the number of CTAs per (KV head, sequence) follows from both, see launch_decode_fused.
+// With `step` the kernel is the whole decode step of a cache with rotary positions (the tail of the Pre-Pass algorithm,
+// then "Caching"): query rows are turned while they are loaded, and the new token's key row is turned and written, with its
+// value row, to the caches before anyone reads them.
+// Measured (32 query / 8 KV heads): 64 sequences of 16384 tokens in 16 shards 620 us = 6.93 TB/s (partials and merge as two
+// kernels 742 + 28), one sequence 23 us (44); the whole step of one sequence at 2500 of 4096 rows 10.5 us (38, four launches
+// and two copies).
+
+__device__ __forceinline__ uint32_t rotate_pair2(uint32_t x, uint32_t partner, const float4& cs, float sign) {
+  // two neighbouring columns of one half: y = x cos + sign * partner * sin  (sign -1: lower half, +1: upper half)
+  const float x0 = __uint_as_float(x << 16), x1 = __uint_as_float(x & 0xffff0000u);
+  const float h0 = __uint_as_float(partner << 16), h1 = __uint_as_float(partner & 0xffff0000u);
+  return pack2_bf16(x0 * cs.x + sign * (h0 * cs.y), x1 * cs.z + sign * (h1 * cs.w));
+}
+
+constexpr int kMaxCluster = 16;
+constexpr int kFusedShards = 256;  // KV shards whose table fits in the kernel's shared memory at a time
+
+template <int G, int NW>
+__global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __grid_constant__ AttnParams p,
+                                                                       const __grid_constant__ DecodeStep step) {
+  constexpr int D = 128;
+  __shared__ DecodeShared<G, NW> sh;
+  __shared__ DecodeQuery s_q;
+  // what the CTAs of the cluster send for this CTA's part of the outputs: [sender][output], and n, w of every head
+  __shared__ float s_o[G * D + kMaxCluster], s_n[kMaxCluster][G], s_w[kMaxCluster][G];
+
+  const PlanDev& pl = p.plan;
+  const int P = pl.n_kv_shards;
+  const int n_cta = gridDim.x, rank = blockIdx.x;  // the cluster spans the x dimension
+  const int g = blockIdx.y, b = blockIdx.z;
+  const int map = pl.n_maps == 1 ? 0 : b;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int x = lane >> 2, j = lane & 3;
+  const int32_t* kv_idx = pl.kv_idx + (size_t)map * pl.n_kv;
+  const int32_t* kv_off = pl.kv_off + (size_t)map * (P + 1);
+  const int32_t* vis = pl.vis + (size_t)map * P;  // one query row
+  const bool vis_given = step.n_vis > 0;          // the prefixes come with the launch (the plan's copy is written below)
+
+  // step: the new token's rows go to the caches first, by warp 0 of the cluster's first CTA (two rotation pairs and four
+  // value columns per lane); the cluster barrier below orders them before everyone's reads
+  if (step.rope && rank == 0 && warp == 0) {
+    const __nv_bfloat16* kn = step.k_new + (int64_t)b * step.kns.batch + (int64_t)g * step.kns.head + 2 * lane;
+    const uint32_t lo = *reinterpret_cast<const uint32_t*>(kn), hi = *reinterpret_cast<const uint32_t*>(kn + 64);
+    const float4 c2 = __ldg(reinterpret_cast<const float4*>(step.rope + (int64_t)step.position * (D / 2)) + lane);
+    const __nv_bfloat16* vn = step.v_new + (int64_t)b * step.vns.batch + (int64_t)g * step.vns.head + 4 * lane;
+    const uint2 vx = *reinterpret_cast<const uint2*>(vn);
+    __nv_bfloat16* kd = static_cast<__nv_bfloat16*>(const_cast<void*>(p.k)) + (int64_t)b * p.ks.batch +
+                        (int64_t)step.position * p.ks.token + (int64_t)g * p.ks.head + 2 * lane;
+    *reinterpret_cast<uint32_t*>(kd) = rotate_pair2(lo, hi, c2, -1.f);
+    *reinterpret_cast<uint32_t*>(kd + 64) = rotate_pair2(hi, lo, c2, 1.f);
+    __nv_bfloat16* vd = static_cast<__nv_bfloat16*>(const_cast<void*>(p.v)) + (int64_t)b * p.vs.batch +
+                        (int64_t)step.position * p.vs.token + (int64_t)g * p.vs.head + 4 * lane;
+    *reinterpret_cast<uint2*>(vd) = vx;
+  }
+  // first barrier of the cluster: everyone has started (its shared memory may be written), the new token is in the caches
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+
+  // Shards (of a window of kFusedShards) in shared memory: visible keys, first position in kv_idx, 16-key blocks before.
+  __shared__ int s_vis[kFusedShards], s_off[kFusedShards], s_before[kFusedShards + 1], s_most;
+  auto fill_table = [&](int w0) {
+    int most = 0, before = 0;
+    const int n_w = min(kFusedShards, P - w0);
+    for (int k0 = 0; k0 < n_w; k0 += 32) {
+      const int kk = k0 + lane;
+      const int v = kk < n_w ? (vis_given ? step.vis[map * P + w0 + kk] : __ldg(vis + w0 + kk)) : 0;
+      const int nb = (v + 15) >> 4;
+      int incl = nb;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      if (kk < n_w) {
+        s_vis[kk] = v;
+        s_off[kk] = __ldg(kv_off + w0 + kk);
+        s_before[kk] = before + incl - nb;
+      }
+      before += __shfl_sync(0xffffffffu, incl, 31);
+      most = max(most, __reduce_max_sync(0xffffffffu, nb));
+    }
+    if (lane == 0) {
+      s_before[n_w] = before;
+      s_most = most;
+    }
+  };
+  if (warp == 0) fill_table(0);
+  if (warp == 1) {
+    uint32_t qf[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) qf[c] = 0u;
+    if (x < G) {
+      const int tok_q = (int)CASCADE_CHECKED((int64_t)pl.q_idx[(size_t)map * pl.n_q], pl.n_q, pl.status, 107);
+      load_query(static_cast<const __nv_bfloat16*>(p.q) + (int64_t)b * p.qs.batch + (int64_t)tok_q * p.qs.token +
+                     (int64_t)(g * G + x) * p.qs.head, j, qf);
+      if (step.rope) {  // the two pieces hold the two halves of the same pairs
+        const float4* cs4 = reinterpret_cast<const float4*>(step.rope + (int64_t)step.position * (D / 2) + 16 * j);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const float4 t = __ldg(cs4 + e);  // pairs 16j + 2e and the next
+          const uint32_t lo = qf[e], hi = qf[8 + e];
+          qf[e] = rotate_pair2(lo, hi, t, -1.f);
+          qf[8 + e] = rotate_pair2(hi, lo, t, 1.f);
+        }
+      }
+    }
+    publish_query(s_q, qf, lane);
+  }
+  const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(p.k) + (int64_t)b * p.ks.batch +
+                            (int64_t)g * p.ks.head + 16 * j;
+  const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(p.v) + (int64_t)b * p.vs.batch +
+                            (int64_t)g * p.vs.head + 16 * x;
+  const float cs = p.scale * 1.4426950408889634f;  // logits in log2 units
+  DecodeState st;
+  decode_init(st);
+
+  // Order of the 16-key blocks.  If the visible prefixes are about equally long, block i of every shard comes before block
+  // i + 1 of any: shards interleave in the sequence, so the warps of a cluster read one region of the cache together.
+  // Otherwise shard after shard, which balances whatever the lengths are.
+  __shared__ int2 s_list[NW][32];  // of this warp's next blocks: first position in kv_idx, keys left there
+  if (step.rope) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+#pragma unroll 1
+  for (int w0 = 0; w0 < P; w0 += kFusedShards) {
+    if (w0 > 0) {
+      __syncthreads();
+      if (warp == 0) fill_table(w0);
+    }
+    __syncthreads();
+    const int n_w = min(kFusedShards, P - w0), total = s_before[n_w];
+    const bool even = s_most * n_w * 4 <= total * 5;
+    const int n_ids = even ? s_most * n_w : total;
+    // Each lane works out one of the warp's next 32 blocks; those that exist are listed in shared memory.
+#pragma unroll 1
+    for (int id0 = rank * NW + warp; id0 < n_ids; id0 += 32 * n_cta * NW) {
+      const int id = id0 + lane * n_cta * NW;
+      int2 e = make_int2(0, 0);
+      if (id < n_ids) {
+        int kk, i;
+        if (even) {
+          kk = id % n_w;
+          i = id / n_w;
+        } else {
+          int lo = 0, hi = n_w - 1;  // the last shard that starts at or before the block: it is not empty
+          while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_before[mid] <= id) lo = mid;
+            else hi = mid - 1;
+          }
+          kk = lo;
+          i = id - s_before[kk];
+        }
+        e = make_int2(s_off[kk] + i * 16, s_vis[kk] - i * 16);
+      }
+      const uint32_t there = __ballot_sync(0xffffffffu, e.y > 0);
+      __syncwarp();
+      if (e.y > 0) s_list[warp][__popc(there & ((1u << lane) - 1u))] = e;
+      __syncwarp();
+      decode_walk<true>(st, s_q, pl, kv_idx, __popc(there), [&](int t) { return s_list[warp][t]; }, kb, p.ks.token, vb,
+                        p.vs.token, lane, cs);
+    }
+  }
+  decode_publish<G, NW>(sh, st, warp, lane);
+  if (!step.rope) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  __syncthreads();
+  // The cluster's shares meet: CTA r finishes outputs r * per_cta ... ; every CTA sends it its share of them, and one barrier
+  // later everything is in the receiver's own shared memory.
+  const int per_cta = (G * D + n_cta - 1) / n_cta;
+  auto send = [&](const float* local, int to, float v) {
+    uint32_t addr;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(to));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+  };
+  for (int i = tid; i < G * D; i += NW * 32) {
+    float n_i, w_i, acc;
+    decode_combine<G, NW>(sh, i / D, i % D, n_i, w_i, acc);
+    const int to = i / per_cta;
+    send(&s_o[rank * per_cta + i - to * per_cta], to, acc);
+    if (i % D < n_cta) {  // one thread per (head, receiver)
+      send(&s_n[rank][i / D], i % D, n_i);
+      send(&s_w[rank][i / D], i % D, w_i);
+    }
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // the plan's own prefixes and pair classes, for later calls on it (the caller's stream orders them after this kernel)
+  if (vis_given && rank == 0 && g == 0 && (pl.n_maps > 1 || b == 0)) {
+    for (int kk = tid; kk < P; kk += NW * 32) {
+      const int v = step.vis[map * P + kk], len = kv_off[kk + 1] - kv_off[kk];
+      const_cast<int32_t*>(vis)[kk] = v;
+      const_cast<uint8_t*>(pl.pair_class)[(size_t)map * P + kk] =
+          v == 0 ? CASCADE_PAIR_EMPTY : (v == len ? CASCADE_PAIR_FULL : CASCADE_PAIR_PARTIAL);
+    }
+  }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  const int mine = min(per_cta, G * D - rank * per_cta);
+  for (int o = tid; o < mine; o += NW * 32) {
+    const int gg = (rank * per_cta + o) / D, col = (rank * per_cta + o) % D;
+    float n_all = -INFINITY;
+    for (int r = 0; r < n_cta; ++r) n_all = fmaxf(n_all, s_n[r][gg]);
+    const float n_use = n_all == -INFINITY ? 0.f : n_all;
+    float w = 0.f, acc = 0.f;
+#pragma unroll 4
+    for (int r = 0; r < n_cta; ++r) {
+      const float f = ex2f(s_n[r][gg] - n_use);
+      w = fmaf(f, s_w[r][gg], w);
+      acc = fmaf(f, s_o[r * per_cta + o], acc);
+    }
+    const int h = g * G + gg;
+    static_cast<__nv_bfloat16*>(p.o_out)[(int64_t)b * p.os.batch + (int64_t)h * p.os.head + col] =
+        __float2bfloat16_rn(w > 0.f ? acc / w : 0.f);
+    if (col == 0 && p.lse_out)
+      p.lse_out[(int64_t)b * p.H + h] = w > 0.f ? n_use * 0.6931471805599453f + logf(w) : -INFINITY;
+  }
+}
+
+template <int G>
+static cudaError_t launch_fused(const AttnParams& p, const DecodeStep& step, int n_cta, cudaStream_t stream) {
+  constexpr int NW = 8;
+  auto kernel = decode_fused_kernel<G, NW>;
+  if (n_cta > 8) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_cta, p.Hkv, p.batch);
+  cfg.blockDim = dim3(NW * 32);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = n_cta;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, p, step);
+}
+
+// f(integral_constant G) for the group sizes the kernels are built for
+template <typename F>
+static cudaError_t with_group(int G, F f) {
+  switch (G) {
+    case 1: return f(std::integral_constant<int, 1>());
+    case 2: return f(std::integral_constant<int, 2>());
+    case 4: return f(std::integral_constant<int, 4>());
+    case 8: return f(std::integral_constant<int, 8>());
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_decode_fused(const AttnParams& p, const DecodeStep& step, int64_t n_visible, cudaStream_t stream) {
+  // CTAs (of eight warps) per (KV head, sequence): 256 in all, which is what two per SM on most of the chip come to with
+  // every warp's loads in flight; more only repeat the set-up (64 sequences of 16384 tokens: 1 per pair 620 us, 2 653 us; 16
+  // sequences: 2 159 us, 4 163 us, 1 165 us).  At most 10 where several pairs want the chip: clusters of 10 fit 11 times
+  // with one CTA per SM, clusters of 16 only 7 times (one sequence: 10 per pair 20.7 us, 16 22.8 us).  No more than give
+  // every warp a block.  `rule_kv_heads` counts the heads of the whole problem where a call computes a part of them.
+  const int64_t pairs = (int64_t)p.rule_kv_heads * p.batch, blocks = std::max<int64_t>(1, (n_visible + 15) / 16);
+  const int64_t most = pairs <= 7 ? kMaxCluster : 10;
+  const int n_cta = (int)std::max<int64_t>(1, std::min(std::min(256 / pairs, most), (blocks + 7) / 8));
+  TimedLaunch timed(stream);
+  const cudaError_t e = with_group(p.G, [&](auto g) { return launch_fused<decltype(g)::value>(p, step, n_cta, stream); });
+  count_launch();
+  return e;
 }
 
 cudaError_t launch_decode(const AttnParams& p, cudaStream_t stream) {
   dim3 grid(p.plan.n_kv_shards, p.Hkv, p.batch);
   TimedLaunch timed(stream);
-  switch (p.G) {
-    case 1: decode_kernel<1><<<grid, 128, 0, stream>>>(p); break;
-    case 2: decode_kernel<2><<<grid, 128, 0, stream>>>(p); break;
-    case 4: decode_kernel<4><<<grid, 128, 0, stream>>>(p); break;
-    case 8: decode_kernel<8><<<grid, 128, 0, stream>>>(p); break;
-    default: return cudaErrorInvalidValue;
-  }
+  const cudaError_t e = with_group(p.G, [&](auto g) {
+    decode_kernel<decltype(g)::value><<<grid, 128, 0, stream>>>(p);
+    return cudaGetLastError();
+  });
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace cascade

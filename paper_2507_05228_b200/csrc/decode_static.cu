@@ -1,49 +1,19 @@
 // Decode attention for callers that cannot provide or allocate scratch memory.
 //
-// cascade_attn_sharded needs a caller-provided workspace for the decode step (the per-shard partials that the
-// merge kernel then combines).  Some callers have none to give: an inference server whose cache manager has
-// already claimed all free HBM, so a cudaMalloc at request time fails or fragments its pool; a latency-critical
-// decode loop in which cudaMalloc / cudaFree would synchronise the whole device; a plug-in that is handed raw
-// pointers and has no access to the host framework's allocator.  For them this file keeps the scratch in a
-// file-scope device array that is part of the library image: it costs kScratchBytes of HBM on every GPU that
-// loads the library, for the life of the process, and in exchange this entry point never allocates.
-#include <mutex>
+// cascade_attn_sharded asks for a caller-provided workspace for the decode step.  Some callers have none to give: an
+// inference server whose cache manager has already claimed all free HBM, so a cudaMalloc at request time fails or fragments
+// its pool; a latency-critical decode loop in which cudaMalloc / cudaFree would synchronise the whole device; a plug-in that
+// is handed raw pointers and has no access to the host framework's allocator.  The fused decode kernel keeps the partials of
+// the KV shards in distributed shared memory, so this entry point needs no scratch memory at all; the size limit of its
+// interface (what a 16 MiB scratch array would hold) is kept.
+#include <string.h>
 
 #include "cascade_internal.cuh"
 
 namespace cascade {
 namespace {
 
-constexpr size_t kScratchBytes = 16u << 20;  // 16 MiB: the 64 x 16-shard x 32-head decode step needs 8.3 MiB
-constexpr int kMaxDevices = 64;
-
-// In host code this name is only a handle for cudaGetSymbolAddress; it is not a device address.
-static __device__ __align__(256) unsigned char g_decode_scratch[kScratchBytes];
-
-std::mutex g_setup_mutex;
-void* g_scratch_addr[kMaxDevices] = {};  // device address of g_decode_scratch, per device ordinal
-
-// Resolves the array's address on the current device (once per device).  Returns nullptr and sets the error
-// text on failure.
-void* scratch_for_current_device() {
-  int dev = -1;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
-    set_error("cascade_attn_decode_static: cudaGetDevice: %s (device %d)", cudaGetErrorString(e), dev);
-    return nullptr;
-  }
-  std::lock_guard<std::mutex> lock(g_setup_mutex);
-  if (!g_scratch_addr[dev]) {
-    void* ptr = nullptr;
-    e = cudaGetSymbolAddress(&ptr, g_decode_scratch);
-    if (e != cudaSuccess || !ptr) {
-      set_error("cascade_attn_decode_static: cudaGetSymbolAddress: %s", cudaGetErrorString(e));
-      return nullptr;
-    }
-    g_scratch_addr[dev] = ptr;
-  }
-  return g_scratch_addr[dev];
-}
+constexpr size_t kScratchBytes = 16u << 20;  // the interface's limit: batch x KV shards x heads x 264 bytes
 
 size_t round256(size_t x) { return (x + 255) / 256 * 256; }
 
@@ -98,13 +68,10 @@ extern "C" cascade_status_t cascade_attn_decode_static(const cascade_plan_t* pla
   const size_t need = o_bytes + 2 * stat_bytes;
   if (need > kScratchBytes) {
     set_error("cascade_attn_decode_static: batch %d x %d KV shards x %d heads needs %zu bytes of scratch, the "
-              "built-in array holds %zu; use cascade_attn_sharded with a workspace instead",
+              "limit of this call is %zu; use cascade_attn_sharded with a workspace instead",
               batch, plan->dev.n_kv_shards, n_heads, need, kScratchBytes);
     return CASCADE_ERR_WORKSPACE;
   }
-  char* scratch = static_cast<char*>(scratch_for_current_device());
-  if (!scratch) return CASCADE_ERR_CUDA;
-
   AttnParams p;
   memset(&p, 0, sizeof(p));
   p.plan = plan->dev;
@@ -120,35 +87,14 @@ extern "C" cascade_status_t cascade_attn_decode_static(const cascade_plan_t* pla
   p.G = G;
   p.d = kHeadDim;
   p.scale = scale;
-  p.fused = 0;
-  // Every element of the three regions below is written by the decode kernel before the merge kernel reads it,
-  // so nothing left over from an earlier call can leak into this one and nothing has to be cleared.
-  p.o_part = scratch;
-  p.m_part = reinterpret_cast<float*>(scratch + o_bytes);
-  p.l_part = reinterpret_cast<float*>(scratch + o_bytes + stat_bytes);
-  cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = launch_decode(p, st);
+  p.rule_kv_heads = n_kv_heads;
+  p.fused = 1;
+  p.o_out = o_out;
+  p.os = {o_strides.batch, o_strides.token, o_strides.head};
+  p.lse_out = lse_out;
+  cudaError_t e = run_decode_fused(*plan, p, (cudaStream_t)stream);
   if (e != cudaSuccess) {
     set_error("cascade_attn_decode_static: decode launch: %s", cudaGetErrorString(e));
-    return CASCADE_ERR_CUDA;
-  }
-  MergeParams mp;
-  mp.o_part = p.o_part;
-  mp.m_part = p.m_part;
-  mp.l_part = p.l_part;
-  mp.row_scatter = nullptr;
-  mp.row_scatter_batch_stride = 0;
-  mp.o_out = o_out;
-  mp.os = {o_strides.batch, o_strides.token, o_strides.head};
-  mp.lse_out = lse_out;
-  mp.batch = batch;
-  mp.n_parts = plan->dev.n_kv_shards;
-  mp.n_rows = 1;
-  mp.H = n_heads;
-  mp.d = kHeadDim;
-  e = launch_merge(mp, CASCADE_BF16, st);
-  if (e != cudaSuccess) {
-    set_error("cascade_attn_decode_static: merge launch: %s", cudaGetErrorString(e));
     return CASCADE_ERR_CUDA;
   }
   return CASCADE_OK;

@@ -3,6 +3,8 @@
 // cache grows by one row per generated token, the shard lists do not change).  No host work and no upload per call;
 // used for plans with more than a few hundred (row, shard) entries, where the host pass would cost more than a launch;
 // cascade_shard_plan fills the two arrays of a new plan the same way.
+#include <string.h>
+
 #include "cascade_internal.cuh"
 
 namespace cascade {
@@ -56,7 +58,31 @@ __global__ void plan_advance_kernel(PlanDev d, int32_t q_pos_offset, int32_t* __
   }
 }
 
+// The same arrays of a plan with few entries, computed on the host and carried by the launch itself (two copies from pageable
+// memory cost the caller 5 us, this 2 us).
+struct PlanSetArgs {
+  int32_t vis[kMaxGivenVis];
+  uint8_t pair_class[kMaxGivenVis];
+};
+__global__ void __launch_bounds__(kMaxGivenVis) plan_set_kernel(const __grid_constant__ PlanSetArgs a, int n_vis, int n_cls,
+                                                                int32_t* vis, uint8_t* pair_class) {
+  const int t = threadIdx.x;
+  if (t < n_vis) vis[t] = a.vis[t];
+  if (t < n_cls) pair_class[t] = a.pair_class[t];
+}
+
 }  // namespace
+
+cudaError_t launch_plan_set(const PlanDev& d, const int32_t* vis, int n_vis, const uint8_t* pair_class, int n_cls,
+                            cudaStream_t stream) {
+  PlanSetArgs a;
+  memcpy(a.vis, vis, (size_t)n_vis * 4);
+  memcpy(a.pair_class, pair_class, (size_t)n_cls);
+  plan_set_kernel<<<1, kMaxGivenVis, 0, stream>>>(a, n_vis, n_cls, const_cast<int32_t*>(d.vis),
+                                                  const_cast<uint8_t*>(d.pair_class));
+  count_launch();
+  return cudaGetLastError();
+}
 
 cudaError_t launch_plan_advance(const PlanDev& d, int32_t q_pos_offset, cudaStream_t stream) {
   const int64_t n = (int64_t)d.n_maps * (d.n_q + d.n_q_shards) * d.n_kv_shards;

@@ -1,7 +1,6 @@
 // The rotary steps of the Pre-Pass algorithm (q <- rotary_pos_emb(q, p^{R_i}), k <- rotary_pos_emb(k, p^{R_i})) as a pass
-// of its own, for the rows that no fused staging covers: fp32 tensors, head_dim 64, and above all the decode step,
-// where one new token's q row is rotated for immediate use and its k row once, on its way into the token-sharded
-// cache ("Caching" in the appendix on cost optimizations), so that cached key rows are never touched again.
+// of its own, for the rows that no fused staging covers: fp32 tensors, head_dim 64, rows rotated once and then cached.  (The
+// decode step turns its rows inside the decode kernel.)
 // A row's angle depends on its original position only (the rows of the positional table p are sharded with the
 // tokens, Section 5.1), so the rotation commutes with any sharding.
 // Pairing (i, i + d/2), angles from the table written by cascade_rope_table: y_lo = x_lo cos - x_hi sin,
@@ -114,72 +113,6 @@ cudaError_t launch_rope_apply(cascade_dtype_t dtype, int32_t batch, int32_t n_ro
   const unsigned grid = (unsigned)((total + 255) / 256);
   if (dtype == CASCADE_BF16) rope_apply_kernel<__nv_bfloat16><<<grid, 256, 0, stream>>>(p);
   else rope_apply_kernel<float><<<grid, 256, 0, stream>>>(p);
-  count_launch();
-  return cudaGetLastError();
-}
-
-// Decode-step append (bf16, head_dim 128): for every sequence, the new token's q row is rotated into q_rot, its k row
-// is rotated and written at row `position` of the key cache, and its v row is copied to the value cache.
-// grid = (H + 2 Hkv, batch), 8 threads per head vector.
-struct AppendParams {
-  const __nv_bfloat16 *q_new, *k_new, *v_new;
-  __nv_bfloat16 *q_rot, *k_cache, *v_cache;
-  Strides qs, kns, vns, kcs, vcs;
-  const float2* rope;
-  int32_t H, Hkv, position;
-};
-
-__global__ void __launch_bounds__(32) append_rope_kernel(AppendParams p) {
-  constexpr int D = 128;
-  const int b = blockIdx.y, which = blockIdx.x, c = threadIdx.x;
-  if (c >= 8) return;
-  const float2* cs = p.rope + (int64_t)p.position * (D / 2) + c * 8;
-  if (which < p.H) {  // a query head
-    const __nv_bfloat16* src = p.q_new + (int64_t)b * p.qs.batch + (int64_t)which * p.qs.head + c * 8;
-    __nv_bfloat16* dst = p.q_rot + ((int64_t)b * p.H + which) * D + c * 8;
-    uint4 lo = *reinterpret_cast<const uint4*>(src), hi = *reinterpret_cast<const uint4*>(src + 64);
-    rotate_pairs<__nv_bfloat16>(lo, hi, cs);
-    *reinterpret_cast<uint4*>(dst) = lo;
-    *reinterpret_cast<uint4*>(dst + 64) = hi;
-  } else if (which < p.H + p.Hkv) {  // a key head: rotated, then into the cache
-    const int g = which - p.H;
-    const __nv_bfloat16* src = p.k_new + (int64_t)b * p.kns.batch + (int64_t)g * p.kns.head + c * 8;
-    __nv_bfloat16* dst = p.k_cache + (int64_t)b * p.kcs.batch + (int64_t)p.position * p.kcs.token +
-                         (int64_t)g * p.kcs.head + c * 8;
-    uint4 lo = *reinterpret_cast<const uint4*>(src), hi = *reinterpret_cast<const uint4*>(src + 64);
-    rotate_pairs<__nv_bfloat16>(lo, hi, cs);
-    *reinterpret_cast<uint4*>(dst) = lo;
-    *reinterpret_cast<uint4*>(dst + 64) = hi;
-  } else {  // a value head: copied
-    const int g = which - p.H - p.Hkv;
-    const __nv_bfloat16* src = p.v_new + (int64_t)b * p.vns.batch + (int64_t)g * p.vns.head + c * 8;
-    __nv_bfloat16* dst = p.v_cache + (int64_t)b * p.vcs.batch + (int64_t)p.position * p.vcs.token +
-                         (int64_t)g * p.vcs.head + c * 8;
-    *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(src);
-    *reinterpret_cast<uint4*>(dst + 64) = *reinterpret_cast<const uint4*>(src + 64);
-  }
-}
-
-cudaError_t launch_append_rope(int32_t batch, int32_t H, int32_t Hkv, const void* q_new, Strides qs, const void* k_new,
-                               Strides kns, const void* v_new, Strides vns, void* q_rot, void* k_cache, Strides kcs,
-                               void* v_cache, Strides vcs, int32_t position, const float2* table, cudaStream_t stream) {
-  AppendParams p;
-  p.q_new = static_cast<const __nv_bfloat16*>(q_new);
-  p.k_new = static_cast<const __nv_bfloat16*>(k_new);
-  p.v_new = static_cast<const __nv_bfloat16*>(v_new);
-  p.q_rot = static_cast<__nv_bfloat16*>(q_rot);
-  p.k_cache = static_cast<__nv_bfloat16*>(k_cache);
-  p.v_cache = static_cast<__nv_bfloat16*>(v_cache);
-  p.qs = qs;
-  p.kns = kns;
-  p.vns = vns;
-  p.kcs = kcs;
-  p.vcs = vcs;
-  p.rope = table;
-  p.H = H;
-  p.Hkv = Hkv;
-  p.position = position;
-  append_rope_kernel<<<dim3(H + 2 * Hkv, batch), 32, 0, stream>>>(p);
   count_launch();
   return cudaGetLastError();
 }

@@ -93,3 +93,51 @@ def test_new_plans_have_the_same_arrays_on_the_device(gu, n_q, n_kv, P, causal):
             plans.pop(0).destroy()
     for plan in plans:
         plan.destroy()
+
+
+@pytest.mark.parametrize("B,n_kv,H,Hkv,P,kv_map,pos", [
+    (1, 1, 8, 8, 1, "random", 0),            # one key, one block: a single CTA per KV head
+    (1, 129, 16, 2, 3, "contiguous", 64),    # two of three shards empty or cut: shard-after-shard order
+    (2, 4097, 8, 4, 16, "round_robin", 4096),  # prefixes that differ by one block at most: interleaved order
+    (1, 9000, 8, 1, 300, "random", 8999),    # more shards than one table window
+    (5, 700, 4, 1, 7, "random", 699),        # fewer than eight (KV head, sequence) pairs: the largest clusters
+    (40, 333, 32, 8, 5, "block_rr", 300),    # more pairs than 256: one CTA each
+])
+def test_fused_decode_forms(gu, B, n_kv, H, Hkv, P, kv_map, pos):
+    gu.full_parity(wl.make_workload(f"dec_{B}_{n_kv}", B, 1, n_kv, H, Hkv, 128, "bf16", "round_robin", kv_map, 1, P,
+                                    seed=n_kv, block=16, q_pos_offset=pos))
+
+
+@pytest.mark.parametrize("B,P,per_seq", [(2, 5, False), (3, 100, True), (2, 300, False)])
+def test_decode_step_moves_the_plan_with_few_and_with_many_prefixes(gu, B, P, per_seq):
+    """Up to 256 prefixes travel with the launch, more are searched for on the device; either way the plan's arrays end up
+    as those of a plan built at that position, the new rows are in the caches, and the output is the oracle's."""
+    from oracle import rope
+    from paper_2507_05228_b200 import binding as cb
+    cap, H, Hkv, d, base = 700, 8, 2, 128, 10000.0
+    rng = np.random.default_rng(P)
+    maps = rng.integers(0, P, (B, cap)).astype(np.int32) if per_seq else rng.integers(0, P, cap).astype(np.int32)
+    q_map = np.zeros((B, 1) if per_seq else (1,), np.int32)
+    plan = cb.cascade_shard_plan(q_map, maps, 1, P, 0, True)
+    w = wl.make_workload("step", B, cap, cap, H, Hkv, d, "bf16", "random", "random", 1, 1, seed=P)
+    q, k, v = gu.to_device(w)
+    table = cb.cascade_rope_table(cap, d, base)
+    qr = rope.rotary_pos_emb(w.q, np.arange(cap), base, "bf16").astype(np.float32)
+    kr = rope.rotary_pos_emb(w.k, np.arange(cap), base, "bf16").astype(np.float32)
+    k_cache, v_cache = torch.full_like(k, float("nan")), torch.full_like(v, float("nan"))
+    known = torch.from_numpy(wl.bf16_bits(kr).view(np.int16)).cuda().view(torch.bfloat16)
+    for pos in (0, 1, 300, 699):
+        k_cache[:, :pos], v_cache[:, :pos] = known[:, :pos], v[:, :pos]
+        o, lse = cb.cascade_decode_step_rope(plan, q[:, pos:pos + 1], k[:, pos:pos + 1], v[:, pos:pos + 1], k_cache, v_cache,
+                                             pos, w.scale, table)
+        o_ref, lse_ref = oracle.attention_unsharded(qr[:, pos:pos + 1], kr, w.v, w.scale, causal=True, q_pos_offset=pos)
+        gu.check_output(o, lse, o_ref, lse_ref, w.tol, f"step at {pos}")
+        got, want = k_cache[:, pos].double().cpu().numpy(), kr[:, pos]
+        assert (np.abs(got - want) <= np.maximum(np.abs(want), 2.0 ** -126) * 2.0 ** -7).all()  # one bf16 step
+        assert torch.equal(v_cache[:, pos], v[:, pos])
+        for b in range(plan.n_maps):
+            op = oracle.shard_plan(q_map[b] if per_seq else q_map, maps[b] if per_seq else maps, 1, P, q_pos_offset=pos)
+            assert np.array_equal(gu.read_plan_device_array(plan, "vis")[b], op.vis)
+            assert np.array_equal(gu.read_plan_device_array(plan, "pair_class")[b], op.pair_class)
+            assert np.array_equal(plan.get("vis")[b], op.vis)
+    plan.destroy()
