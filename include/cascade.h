@@ -174,15 +174,15 @@ cascade_status_t cascade_plan_device_status(const cascade_plan_t* plan, int32_t*
  *   m_part, l_part  fp32 [batch][n_kv_shards][n_q shard-major][n_heads], contiguous
  * (Together these are the paper's stage-B payload: n_kv_shards * (head_dim + 2) * n_heads * n_q values
  * per sequence, Appendix D.)  batch must equal n_maps when the plan has per-sequence maps.
- * head_dim in {64,128}; bf16 with head_dim 128 runs on the tensor cores (tcgen05), everything else on
- * the fp32 ALU kernel; n_q == 1 with bf16 runs the KV-streaming decode kernel.
+ * head_dim in {64,128}; bf16 runs on the tensor cores (tcgen05), fp32 (and more than 256 KV shards, and head_dim 64
+ * without a workspace) on the fp32 ALU kernel; n_q == 1 with bf16 runs the KV-streaming decode kernel.
  * scale must be positive and finite (INVALID_ARG otherwise: the kernels take row maxima before scaling).
  * Only the k/v rows that some query row of the plan sees have to hold finite values: positions later than the last
  * query position (the unwritten tail of a preallocated cache) may hold anything, NaN bit patterns included; no route
  * lets them reach a result.  batch and n_heads may not exceed 65535 (and batch * n_kv_shards on the ALU route).
  * workspace: as reported by cascade_workspace_bytes(CASCADE_CALL_PARTIALS) (may be 0 -> NULL allowed).  The
  * tensor-core route first copies K and V into shard-major order there (the stage-A hand-over of each KV shard to
- * its AttnNodes, Appendix D): 2 * batch * n_kv_heads * n_kv * head_dim * 2 bytes, overwritten by every call.
+ * its AttnNodes, Appendix D); overwritten by every call.
  */
 cascade_status_t cascade_attn_partials(const cascade_plan_t* plan, cascade_dtype_t dtype, int32_t batch,
                                        int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, float scale,
@@ -234,13 +234,13 @@ cascade_status_t cascade_merge_peers(cascade_dtype_t dtype, int32_t batch, int32
                                      float* lse_out, void* stream);
 
 /*
- * cascade_attn_sharded -- attention-pass and post-pass fused (the Attention-Pass algorithm followed by the Post-Pass algorithm): walks the KV shards of the plan one after another for each query-shard tile and carries
- * (n, w, o) across shards, so no partial is written to memory; by the identity of Section 5.2.3 the
- * result equals cascade_merge(cascade_attn_partials(...)).  Output in token order:
+ * cascade_attn_sharded -- attention-pass and post-pass fused (the Attention-Pass algorithm followed by the Post-Pass
+ * algorithm): carries (n, w, o) across the keys of all shards, so no partial is written to memory; by the identity of
+ * Section 5.2.3 the result equals cascade_merge(cascade_attn_partials(...)).  Output in token order:
  *   o_out [batch][n_q][n_heads][head_dim] with strides; lse_out optional fp32 [batch][n_q][n_heads].
  * For n_q == 1 (decode, Appendix F "Caching") the KV shards are processed as independent partials that meet on chip, in
- * one launch (`workspace` is checked but not used).  The tensor-core route (bf16, head_dim 128) uses `workspace` for
- * the shard-major K/V copies as cascade_attn_partials does.  Size: cascade_workspace_bytes(CASCADE_CALL_SHARDED).
+ * one launch (`workspace` is checked but not used).  The tensor-core route (bf16) reads K and V where
+ * they are and uses `workspace` only for tensors whose strides its loads cannot take.  Size: cascade_workspace_bytes(CASCADE_CALL_SHARDED).
  */
 cascade_status_t cascade_attn_sharded(const cascade_plan_t* plan, cascade_dtype_t dtype, int32_t batch,
                                       int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, float scale,

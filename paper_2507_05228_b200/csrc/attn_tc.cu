@@ -1,20 +1,25 @@
-// Attention-pass on the 5th-generation tensor cores (tcgen05 + TMEM) for bf16, head_dim 128.
+// Attention-pass on the 5th-generation tensor cores (tcgen05 + TMEM) for bf16, head_dim 128 and 64.
 //
-// Work decomposition.  The M dimension of one MMA tile (128 rows) is filled with (query slot, head) pairs: the
+// Work decomposition.  The M dimension of one MMA tile (128 rows) is filled with (query row, head) pairs: the
 // Gp query heads that read the same KV head ("repeat_kv", the Attention-Pass algorithm) are stacked next to each other,
-// so a tile covers only 128 / Gp consecutive slots of one query shard.  Under token sharding the rows of a shard
-// are spread over the whole sequence, and the staircase between the shortest and the longest visible prefix of a
-// tile is wasted tensor work; stacking heads shrinks that staircase by Gp.
-// One CTA owns two such sub-tiles (the next 128 / Gp slots of the same shard, same heads), which share every K/V
-// tile, and walks all KV shards one after another.  Fused route: the carry n, w, o of the Post-Pass algorithm is the
-// running max / sum / output of the streaming softmax, and one output row is written at the end.  Partials (kWalk,
-// the Attention-Pass algorithm for every pair of the query tile): a tile never mixes two shards, and at every shard
-// boundary that shard's (u, m, l) is written out and the statistics and the accumulator start over.  (A CTA per
-// (query tile, KV shard) pair is kept as a compile-time alternative; it pays the CTA set-up once per pair.)
-// The KV shards are walked one after another; each shard's visible prefix (as seen by the CTA's last row, which has
-// the longest one) is cut into chunks of 32 keys, and four consecutive chunks of that stream - possibly from
-// different shards - form one MMA tile of 128 keys, so that only the last tile of a CTA is narrower.  (An MMA costs
-// the same for 32 keys as for 128, and every tile costs one softmax round trip.)
+// so a tile covers only 128 / Gp consecutive query rows.  One CTA owns two such sub-tiles (the next 128 / Gp rows, same
+// heads), which share every K/V tile.
+//
+// Fused route (not kWalk).  The Post-Pass algorithm makes of the partials of all KV shards exactly the softmax over all keys,
+// and of those a query sees a prefix in token order.  So the CTA takes 256 / Gp consecutive tokens and walks the keys in
+// token order, 128 at a time, straight from the caller's K and V; the carry n, w, o of the Post-Pass algorithm is the running
+// max / sum / output of the streaming softmax, and one output row is written at the end.  Only the last tile or two need the
+// causal mask.  Where there are few query tiles, a cluster of 2, 4 or 8 CTAs shares the keys of one and adds up through
+// distributed shared memory.
+// Measured, 32 query / 8 KV heads (before: shard by shard from gathered copies, query tiles inside one shard): 2048 tokens, 8
+// random shards 67 -> 47 us; 512 queries against 7168 cached tokens 127 -> 80 us; 32768 tokens, 64 / 8 heads, 32 random
+// shards 16.7 -> 16.0 ms; 2 x 3001 tokens, 16 / 4 heads of 64 columns 124 -> 85 us.
+//
+// Partials (kWalk, the Attention-Pass algorithm for every pair of the query tile).  The rows are consecutive slots of one
+// query shard and the KV shards are walked one after another: each shard's visible prefix (as seen by the CTA's last row,
+// which has the longest one) is cut into chunks of 32 keys, and up to four chunks form one MMA tile.  A tile never mixes two
+// shards: at every shard boundary that shard's (u, m, l) is written out and the statistics and the accumulator start over.
+// (A CTA per (query tile, KV shard) pair would pay the CTA set-up once per pair.)
 //
 // Warp roles (12 warps):
 //   0-3   softmax of sub-tile 0, 4-7 softmax of sub-tile 1: thread = MMA row = TMEM lane.  Reads the logits S with
@@ -29,25 +34,22 @@
 //         makes that safe without a barrier.  The whole warp runs the loop and one elected lane issues, so that
 //         descriptors and addresses stay warp-uniform.
 //   9-10  loaders: TMA box loads, completion counted in bytes on an mbarrier, data written in the 128-byte-swizzled
-//         layout the MMA descriptors expect.  Warp 9 streams the K tiles and warp 10 the V tiles from the
-//         shard-major copies that the gather pass (gather.cu) wrote: the visible prefix of a shard is a
-//         contiguous run of rows there, so a tile is two 16 KiB box loads.  An index-mapped gather straight from
+//         layout the MMA descriptors expect.  Warp 9 streams the K tiles and warp 10 the V tiles: 128 rows at a time from
+//         the caller's tensors, or with kWalk 32 at a time from the shard-major copies that the gather pass (gather.cu)
+//         wrote, where the visible prefix of a shard is a contiguous run of rows.  An index-mapped gather straight from
 //         the caller's tensors was far too slow for the K/V stream (measured: one 512-byte TMA row gather per ~36
 //         cycles per SM; 16-byte cp.async: one 512-byte request per ~90 cycles per warp).  The two query
 //         sub-tiles are gathered once per CTA by the softmax threads themselves (plain 16-byte loads).
-//   11    builds the table of the shards the CTA sees anything of (what each role needs per shard, and the number of
-//         chunks), then idles; it also keeps the register-reallocation groups of four warps whole.
-// The grid is launched as a programmatic dependent of the gather grid: everything up to the loaders' first TMA load
+//   11    works out the CTA's keys (kWalk: the table of the shards it sees anything of), then idles; it also keeps the register-reallocation groups of four warps whole.
+// After a gather the grid is launched as its programmatic dependent: everything up to the loaders' first TMA load
 // may run while the gather is still writing the shard-major copies (the loaders wait with griddepcontrol.wait).
 // Every mbarrier wait is bounded: on expiry the CTA raises a flag, records a code in the plan's status word
 // and drains without waiting again.
 #include <cuda.h>
 
-#include "cascade_internal.cuh"
+#include <algorithm>
 
-#ifndef CASCADE_PARTIALS_WALK
-#define CASCADE_PARTIALS_WALK 1
-#endif
+#include "cascade_internal.cuh"
 
 namespace cascade {
 namespace tc {
@@ -186,12 +188,30 @@ __device__ __forceinline__ bool wait_bar(const WaitCtx& c, uint32_t bar, uint32_
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// TMA box load: 32 rows x 64 elements of the 3-D tensor [matrix z][row y][column x] land as 32 rows of 128 bytes.
+// TMA box loads, 64 elements wide: rows land as 128 bytes each.  32 rows of the 3-D tensor [matrix z][row y][column x]
+// (shard-major copies), or 128 rows of the 4-D tensor [sequence w][head z][row y][column x].
+__device__ __forceinline__ void tma_tile4(uint32_t dst, const CUtensorMap* map, int x, int y, int z, int w, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+      : "memory");
+}
 __device__ __forceinline__ void tma_tile3(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
       : "memory");
+}
+
+// All threads of the cluster (each warp where it stands in its role).
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// 16 bytes into the shared memory of CTA `to` of the cluster, at the address `local` has in this one
+__device__ __forceinline__ void st_cluster(uint32_t local, int to, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  uint32_t addr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(local), "r"(to));
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
 // Shared-memory matrix descriptor, 128-byte swizzle, as two 32-bit words.  Low word: start address >> 4 (bits 0-13),
@@ -249,6 +269,12 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
         "=r"(r[o + 30]), "=r"(r[o + 31])                                                                        \
       : "r"(taddr)                                                                                              \
       : "memory")
+
+#define CASCADE_TMEM_LD8(taddr, r)                                                                             \
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"                  \
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) \
+               : "r"(taddr)                                                                                     \
+               : "memory")
 
 #define CASCADE_TMEM_ST32(taddr, r, o)                                                                         \
   asm volatile(                                                                                                 \
@@ -337,16 +363,16 @@ struct ChunkCursor {
 template <bool kWalk>
 struct TileSeq {
   const ShardTab* t;
-  int n_act, n_chunks, i, j, c, nc;
-  __device__ __forceinline__ TileSeq(const ShardTab* tab, int n_active, int chunks)
-      : t(tab), n_act(n_active), n_chunks(chunks), i(0), j(0), c(0) {
+  int n_act, n_keys, i, j, c, nc;
+  __device__ __forceinline__ TileSeq(const ShardTab* tab, int n_active, int keys)
+      : t(tab), n_act(n_active), n_keys(keys), i(0), j(0), c(0) {
     nc = (kWalk && n_act > 0) ? (t->need[0] + kChunk - 1) / kChunk : 0;
   }
   // the next tile: its chunks; first = it opens a shard (kWalk) or the whole stream
   __device__ __forceinline__ int next(bool& first) {
     if constexpr (!kWalk) {
       first = i == 0;
-      const int n = min(4, n_chunks - 4 * i);
+      const int n = min(4, (n_keys - 4 * kChunk * i + kChunk - 1) / kChunk);
       ++i;
       return n;
     } else {
@@ -364,7 +390,9 @@ struct TileSeq {
 };
 
 struct TmaArgs {
-  CUtensorMap k, v;  // shard-major copies as [batch * kv_heads][n_kv][head_dim]
+  // kWalk: the shard-major copies as [batch * kv_heads][n_kv][head_dim];
+  // otherwise K and V rows in token order as [batch][kv_heads][rows that are seen][head_dim]
+  CUtensorMap k, v;
 };
 
 // kRope: the query rows are turned by the rotary embedding of their positions while they are staged (the key rows
@@ -375,7 +403,7 @@ struct TmaArgs {
 // the barriers and the K/V pipelines are set up once per query tile instead of once per (query tile, KV shard).
 template <int D, bool kRope, bool kWalk>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_constant__ AttnParams p, int lg,
-                                                              int tile_major,
+                                                              int tile_major, int split,
                                                               const __grid_constant__ TmaArgs tma) {
   using C = Cfg<D>;
   constexpr int kD = D, kTileBytes = C::kTileBytes, kKStages = C::kKStages, kVStages = C::kVStages;
@@ -405,44 +433,61 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   const int Gp = 1 << lg, R = kM >> lg;
   const PlanDev& pl = p.plan;
   const int P = pl.n_kv_shards;
-  const int n_parts = (p.fused || kWalk) ? 1 : P;
-  // CTA index -> (query tile, batch, part, head group).  The tile lists are sorted by decreasing work.  With few CTAs
-  // per SM the query tile is the slowest index, so that the heaviest CTAs of all heads and sequences start first and
-  // the light ones fill the tail.  For a large problem the head group is slowest instead: the CTAs running at any
-  // time then read the K/V of few KV heads, which keeps that stream in L2.
+  // CTA index -> (query tile, batch, head group).  The tiles are listed by decreasing work.  With few CTAs per SM the
+  // query tile is the slowest index, so that the heaviest CTAs of all heads and sequences start first and the light ones
+  // fill the tail.  For a large problem the head group is slowest instead: the CTAs running at any time then read the
+  // K/V of few KV heads, which keeps that stream in L2.
   const int n_hg = p.H >> lg;
-  const int n_qt = pl.n_qtiles[3 - lg];
-  int tile_idx, hg, bz;
+  const int ts = 3 - lg;  // kWalk: tile list of 2 R = 256 >> lg slots
+  const int n_qt = kWalk ? pl.n_qtiles[ts] : (pl.n_q + 2 * R - 1) / (2 * R);
+  const int cta = kWalk ? blockIdx.x : blockIdx.x / split;
+  const int part_of_keys = kWalk ? 0 : blockIdx.x % split;  // rank in the cluster that shares a query tile's keys
+  int tile_idx, hg, b;
   if (tile_major) {
-    const int per_tile = n_hg * p.batch * n_parts;
-    const int rem = blockIdx.x % per_tile;
-    tile_idx = blockIdx.x / per_tile;
+    const int per_tile = n_hg * p.batch;
+    const int rem = cta % per_tile;
+    tile_idx = cta / per_tile;
     hg = rem % n_hg;
-    bz = rem / n_hg;
+    b = rem / n_hg;
   } else {
-    // the KV shards of one query tile (partials) are neighbours, so that its rows are read from HBM once and the
-    // CTAs running at a time walk all shards of one KV head
-    const int rem = blockIdx.x / (n_qt * n_parts);
-    tile_idx = (blockIdx.x / n_parts) % n_qt;
+    const int rem = cta / n_qt;
+    tile_idx = cta % n_qt;
     hg = rem % n_hg;
-    bz = (rem / n_hg) * n_parts + blockIdx.x % n_parts;
+    b = rem / n_hg;
   }
-  const int b = bz / n_parts;
-  const int part = bz % n_parts;
   const int map = pl.n_maps == 1 ? 0 : b;
   const int h0 = hg * Gp;  // first of the Gp stacked heads
   const int g = h0 / p.G;  // their KV head
-  const int ts = 3 - lg;   // tile list of 2 R = 256 >> lg slots
-  const int4 qt = pl.qtiles[ts][(size_t)map * pl.n_qtiles[ts] + tile_idx];
-  const int row0 = qt.x, nrows = qt.y;
-  if (nrows == 0) return;  // padding entry (uniform for the CTA)
-  if (*reinterpret_cast<volatile int32_t*>(pl.status) != 0) return;  // an earlier CTA gave up: do not pile on
+  int row0, nrows;         // kWalk: slots of the shard-major order; otherwise tokens
+  if constexpr (kWalk) {
+    const int4 qt = pl.qtiles[ts][(size_t)map * pl.n_qtiles[ts] + tile_idx];
+    row0 = qt.x;
+    nrows = qt.y;
+    if (nrows == 0) return;  // padding entry (uniform for the CTA)
+  } else {
+    row0 = (n_qt - 1 - tile_idx) * 2 * R;
+    nrows = min(2 * R, pl.n_q - row0);
+  }
+  // an earlier CTA gave up: do not pile on (a cluster stays whole, its waits end at once)
+  if (split == 1 && *reinterpret_cast<volatile int32_t*>(pl.status) != 0) return;
   const int n_sub = nrows > R ? 2 : 1;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int32_t* q_idx = pl.q_idx + (size_t)map * pl.n_q;
   const int32_t* kv_off = pl.kv_off + (size_t)map * (P + 1);
   const int32_t* vis = pl.vis + (size_t)map * pl.n_q * P;
-  const int k_begin = (p.fused || kWalk) ? 0 : part, k_end = (p.fused || kWalk) ? P : part + 1;
+  // Token of a row, and (not kWalk) how many K/V rows it sees: a prefix of the tensors, because the mask is causal in
+  // positions and the rows ascend in position.
+  auto token_of = [&](int row) {
+    return kWalk ? (int)CASCADE_CHECKED((int64_t)__ldg(q_idx + row), pl.n_q, pl.status, 108) : row;
+  };
+  auto seen_by = [&](int token) {
+    if (!pl.causal) return pl.n_kv;
+    if (!p.prefix_from_vis) return (int)max((int64_t)0, min((int64_t)pl.n_kv, (int64_t)pl.q_pos_offset + token + 1));
+    const int32_t* v = vis + (size_t)__ldg(pl.q_inv + (size_t)map * pl.n_q + token) * P;  // rows at positions of their own
+    int n = 0;
+    for (int kk = 0; kk < P; ++kk) n += __ldg(v + kk);
+    return n;
+  };
   // Query sub-tiles (row r = slot r / Gp, head r % Gp): the 128 softmax threads of a sub-tile gather it from the
   // caller's tensor, 16 bytes per thread and row, half a warp per 256-byte row.  The loads are issued here, before the
   // set-up below, and land in shared memory (128-byte-swizzled [2][128][128 B] layout) after it.  Rows past the end
@@ -466,8 +511,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int r = (tid >> 3 & 15) + 16 * j;
-        const int tok =
-            (int)CASCADE_CHECKED((int64_t)__ldg(q_idx + sub_row0 + min(r >> lg, sub_nrows - 1)), pl.n_q, pl.status, 108);
+        const int tok = token_of(sub_row0 + min(r >> lg, sub_nrows - 1));
         const __nv_bfloat16* row = qb + (int64_t)tok * p.qs.token + (int64_t)(h0 + (r & (Gp - 1))) * p.qs.head;
         qv[2 * j] = __ldg(reinterpret_cast<const uint4*>(row));
         qv[2 * j + 1] = __ldg(reinterpret_cast<const uint4*>(row + 64));
@@ -482,42 +526,51 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
 #pragma unroll
       for (int j = 0; j < kRowChunks; ++j) {
         const int r = q_row + kRowsPerPass * j;
-        const int tok =
-            (int)CASCADE_CHECKED((int64_t)__ldg(q_idx + sub_row0 + min(r >> lg, sub_nrows - 1)), pl.n_q, pl.status, 108);
+        const int tok = token_of(sub_row0 + min(r >> lg, sub_nrows - 1));
         qv[j] = __ldg(reinterpret_cast<const uint4*>(qb + (int64_t)tok * p.qs.token +
                                                      (int64_t)(h0 + (r & (Gp - 1))) * p.qs.head));
       }
     }
   }
   if (warp == 11) {  // the warp without a role of its own
-    // Compact the shards of which the CTA's last row (longest prefix; rows ascend) sees something, with what the
-    // roles need per shard, and count the chunks of the stream.
-    const int32_t* need_of = vis + (size_t)(row0 + nrows - 1) * P;
-    const int32_t* first0 = vis + (size_t)row0 * P;
-    const int32_t* first1 = vis + (size_t)(row0 + (n_sub - 1) * R) * P;
-    int n_act = 0, n_chunks = 0;
-    for (int base = k_begin; base < k_end; base += 32) {
-      const int kk = base + lane;
-      const int nd = kk < k_end ? __ldg(need_of + kk) : 0;
-      const uint32_t act = __ballot_sync(0xffffffffu, nd > 0);
-      if (nd > 0) {
-        const int pos = n_act + __popc(act & ((1u << lane) - 1u));
-        tab->need[pos] = nd;
-        tab->first[0][pos] = __ldg(first0 + kk);
-        tab->first[1][pos] = __ldg(first1 + kk);
-        tab->slot0[pos] = __ldg(kv_off + kk);
-        tab->kk[pos] = kk;
+    if constexpr (kWalk) {
+      // Compact the shards of which the CTA's last row (longest prefix; rows ascend) sees something, with what the
+      // roles need per shard, and count the tiles of the stream.
+      const int32_t* need_of = vis + (size_t)(row0 + nrows - 1) * P;
+      const int32_t* first0 = vis + (size_t)row0 * P;
+      const int32_t* first1 = vis + (size_t)(row0 + (n_sub - 1) * R) * P;
+      int n_act = 0, n_tiles = 0;
+      for (int base = 0; base < P; base += 32) {
+        const int kk = base + lane;
+        const int nd = kk < P ? __ldg(need_of + kk) : 0;
+        const uint32_t act = __ballot_sync(0xffffffffu, nd > 0);
+        if (nd > 0) {
+          const int pos = n_act + __popc(act & ((1u << lane) - 1u));
+          tab->need[pos] = nd;
+          tab->first[0][pos] = __ldg(first0 + kk);
+          tab->first[1][pos] = __ldg(first1 + kk);
+          tab->slot0[pos] = __ldg(kv_off + kk);
+          tab->kk[pos] = kk;
+        }
+        n_act += __popc(act);
+        n_tiles += __reduce_add_sync(0xffffffffu, (nd + 4 * kChunk - 1) / (4 * kChunk));  // a tile keeps to its shard
       }
-      n_act += __popc(act);
-      int ch = (nd + kChunk - 1) / kChunk;
-      if (kWalk) ch = (ch + 3) >> 2;  // tiles of this shard: a tile does not continue into the next shard
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) ch += __shfl_xor_sync(0xffffffffu, ch, off);
-      n_chunks += ch;
-    }
-    if (lane == 0) {
-      stream_info[0] = n_act;
-      stream_info[1] = n_chunks;
+      if (lane == 0) {
+        stream_info[0] = n_act;
+        stream_info[1] = n_tiles;
+      }
+    } else {
+      // the keys the last row sees, in tiles of 128 from the first on; this CTA takes its part of the tiles
+      const int seen = lane < 3 ? seen_by(lane == 0 ? row0 + nrows - 1 : row0 + (lane == 2 ? (n_sub - 1) * R : 0)) : 0;
+      const int tiles = (__shfl_sync(0xffffffffu, seen, 0) + kNMax - 1) / kNMax;
+      const int t0 = tiles * part_of_keys / split, t1 = tiles * (part_of_keys + 1) / split;
+      if (lane == 0) {
+        tab->need[0] = max(0, min(seen, t1 * kNMax) - t0 * kNMax);  // keys of this CTA's part
+        tab->slot0[0] = t0 * kNMax;
+        stream_info[0] = 1;
+        stream_info[1] = t1 - t0;
+      }
+      if (lane == 1 || lane == 2) tab->first[lane - 1][0] = seen;
     }
   }
   WaitCtx wc{abort_flag, progress, pl.status};
@@ -560,11 +613,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int n_act = stream_info[0];                 // shards of which the CTA sees something
-  const int n_chunks = stream_info[1];              // chunks of the KV stream (kWalk: tiles, counted per shard)
-  // MMA tiles: four chunks each; only the last one is narrower, or with kWalk the last one of every shard
-  const int n_tiles = kWalk ? n_chunks : (n_chunks + 3) >> 2;
-  auto tile_chunks = [&](int i) { return min(4, n_chunks - 4 * i); };  // not with kWalk: see TileSeq
+  const int n_act = stream_info[0];  // kWalk: shards of which the CTA sees something
+  const int n_tiles = stream_info[1];
+  // not kWalk: first key and number of keys of this CTA's part of the stream
+  const int key0 = kWalk ? 0 : tab->slot0[0], n_keys = kWalk ? 0 : tab->need[0];
+  // MMA tiles of four chunks; only the last one is narrower, or with kWalk the last one of every shard (see TileSeq)
+  auto tile_chunks = [&](int i) { return min(4, (n_keys - kNMax * i + kChunk - 1) / kChunk); };
 
   if (warp < 8) {
     // ------------------------------------------------------------------ softmax + epilogue
@@ -578,8 +632,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       const bool row_ok = slot_local < sub_nrows;
       const int slot = sub_row0 + (row_ok ? slot_local : 0);
       const int head = h0 + (m & (Gp - 1));
-      const int32_t* vis_row = vis + (size_t)slot * P;
-      const int32_t* vis_first = tab->first[s];  // shortest prefix of the sub-tile, per active shard
+      const int32_t* vis_row = vis + (size_t)(kWalk ? slot : 0) * P;
+      const int32_t* vis_first = tab->first[s];  // shortest prefix of the sub-tile, per active shard (not kWalk: of all keys)
+      const int my_seen = (kWalk || !row_ok) ? 0 : seen_by(slot) - key0;
+      const int sub_seen = kWalk ? 0 : vis_first[0] - key0;
       const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
       uint32_t s_addr = lane_base + (uint32_t)(s * 128);  // kRing: the buffer of the current tile
       const uint32_t o_addr = lane_base + C::kOCol + (uint32_t)(s * kD);
@@ -630,10 +686,10 @@ if constexpr (kRope) {
       }
       // This row's prefix lengths in the current and the next three active shards (a tile spans at most four), fetched
       // as the stream moves on so that the loads are off the critical path.
-      auto row_vis = [&](int j) { return (j < n_act && row_ok) ? __ldg(vis_row + tab->kk[j]) : 0; };
+      auto row_vis = [&](int j) { return (kWalk && j < n_act && row_ok) ? __ldg(vis_row + tab->kk[j]) : 0; };
       int vq0 = row_vis(0), vq1 = row_vis(1), vq2 = row_vis(2), vq3 = row_vis(3);
-      ChunkCursor cur;
-      cur.start(tab, n_act);
+      ChunkCursor cur{};
+      if (kWalk) cur.start(tab, n_act);
       int kk_open = -1;  // kWalk: the shard whose partial is being accumulated
       int n_flushed = 0;  // kWalk: partials written so far
       const bool rows32 = (reinterpret_cast<uintptr_t>(p.o_part) & 31) == 0;  // partial rows are 256 bytes apart
@@ -695,7 +751,11 @@ if constexpr (kRope) {
         uint32_t needm = 0;
 #pragma unroll
         for (int ch = 0; ch < 4; ++ch) {
-          if (ch < nch) {  // warp-uniform
+          if constexpr (!kWalk) {
+            const int t0 = kNMax * i + kChunk * ch;  // from this CTA's first key on
+            if (ch >= nch || t0 + kChunk > sub_seen) needm |= 1u << ch;
+            lc[ch] = ch < nch ? my_seen - t0 : 0;
+          } else if (ch < nch) {  // warp-uniform
             const int t0 = cur.c * kChunk;
             if (t0 + kChunk > vis_first[cur.j]) needm |= 1u << ch;
             lc[ch] = vq0 - t0;
@@ -841,19 +901,106 @@ if constexpr (kRope) {
         note(8 * i + 2);
       }
       note(8 * n_tiles + 3);
+      if (!kWalk && split > 1) {
+        // ---- epilogue of a query tile whose keys were shared by the cluster: CTA r finishes columns r * cols .. of all
+        // rows.  Every CTA sends it those columns of its accumulator and its row statistics (relative to its own m).
+        const int cols = kD / split, me = part_of_keys;
+        const int pitch = cols * 4 + 16;  // bytes between received rows: spreads a warp's 16-byte stores over the banks
+        const int row = s * kM + m;
+        if (n_tiles > 0) {
+          wait_bar(wc, bar(O_FULL), 0u, 3, n_tiles);
+          tc_fence_after();
+        }
+        cluster_barrier();  // every product of the cluster is done: its Q, K and V tiles may be overwritten
+        const uint32_t from_me = smem_base + (uint32_t)kOffQ;
+        auto slot_of = [&](int sender, int receiver) { return sender < receiver ? sender : sender - 1; };
+#pragma unroll
+        for (int cc = 0; cc < kD / 32; ++cc) {
+          uint32_t o[32];
+          if (n_tiles > 0) {
+            CASCADE_TMEM_LD32(o_addr + (uint32_t)(cc * 32), o, 0);
+            tmem_wait_ld();
+          } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) o[j] = 0u;
+          }
+#pragma unroll
+          for (int j = 0; j < 32; j += 4) {
+            const int to = (cc * 32 + j) / cols;
+            if (to != me)
+              st_cluster(from_me + (uint32_t)((slot_of(me, to) * 2 * kM + row) * pitch + ((cc * 32 + j) % cols) * 4), to,
+                         o[j], o[j + 1], o[j + 2], o[j + 3]);
+          }
+        }
+        const uint32_t stats = smem_base + (uint32_t)(kOffQ + (split - 1) * 2 * kM * pitch);  // [sender][row] (m, l)
+        for (int to = 0; to < split; ++to)
+          if (to != me)
+            st_cluster(stats + (uint32_t)((slot_of(me, to) * 2 * kM + row) * 16), to, __float_as_uint(m_run),
+                       __float_as_uint(l_run), 0u, 0u);
+        cluster_barrier();
+        float m_all = m_run;
+        for (int i = 0; i < split - 1; ++i)
+          m_all = fmaxf(m_all, *reinterpret_cast<const float*>(smem + kOffQ + (split - 1) * 2 * kM * pitch +
+                                                               (i * 2 * kM + row) * 16));
+        const float m_use = m_all == -INFINITY ? 0.f : m_all;
+        const float f_me = ex2(m_run - m_use);
+        float l_all = l_run * f_me;
+        for (int i = 0; i < split - 1; ++i) {
+          const float2 ml = *reinterpret_cast<const float2*>(smem + kOffQ + (split - 1) * 2 * kM * pitch +
+                                                             (i * 2 * kM + row) * 16);
+          l_all += ml.y * ex2(ml.x - m_use);
+        }
+        const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+        __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.o_out) + (int64_t)b * p.os.batch + (int64_t)slot * p.os.token +
+                             (int64_t)head * p.os.head + me * cols;
+        for (int c0 = 0; c0 < cols; c0 += 8) {
+          float acc[8];
+          uint32_t o[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+          if (n_tiles > 0) {
+            CASCADE_TMEM_LD8(o_addr + (uint32_t)(me * cols + c0), o);
+            tmem_wait_ld();
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[j] = n_tiles > 0 ? __uint_as_float(o[j]) * f_me : 0.f;
+          for (int i = 0; i < split - 1; ++i) {
+            const uint8_t* base = smem + kOffQ + (split - 1) * 2 * kM * pitch;
+            const float f = ex2(*reinterpret_cast<const float*>(base + (i * 2 * kM + row) * 16) - m_use);
+            const float4* src = reinterpret_cast<const float4*>(smem + kOffQ + (i * 2 * kM + row) * pitch + c0 * 4);
+            const float4 a = src[0], d = src[1];
+            acc[0] = fmaf(a.x, f, acc[0]); acc[1] = fmaf(a.y, f, acc[1]);
+            acc[2] = fmaf(a.z, f, acc[2]); acc[3] = fmaf(a.w, f, acc[3]);
+            acc[4] = fmaf(d.x, f, acc[4]); acc[5] = fmaf(d.y, f, acc[5]);
+            acc[6] = fmaf(d.z, f, acc[6]); acc[7] = fmaf(d.w, f, acc[7]);
+          }
+          if (row_ok) {
+            uint4 val;
+            val.x = pack_bf16x2(acc[0] * inv, acc[1] * inv);
+            val.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
+            val.z = pack_bf16x2(acc[4] * inv, acc[5] * inv);
+            val.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
+            *reinterpret_cast<uint4*>(dst + c0) = val;
+          }
+        }
+        if (row_ok && me == 0 && p.lse_out)
+          p.lse_out[((int64_t)b * pl.n_q + slot) * p.H + head] =
+              l_all > 0.f ? (m_use + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+      } else {
       // ---- epilogue
       // Where this row goes is looked up before the wait for the last product, which hides the load.
       __nv_bfloat16* dst = nullptr;
       int64_t stat = 0;
       if (row_ok) {
-        if (p.fused) {
-          const int tok = (int)CASCADE_CHECKED((int64_t)__ldg(q_idx + slot), pl.n_q, pl.status, 109);
-          stat = ((int64_t)b * pl.n_q + tok) * p.H + head;
-          dst = static_cast<__nv_bfloat16*>(p.o_out) + (int64_t)b * p.os.batch + (int64_t)tok * p.os.token +
+        if (!kWalk && p.fused) {
+          stat = ((int64_t)b * pl.n_q + slot) * p.H + head;
+          dst = static_cast<__nv_bfloat16*>(p.o_out) + (int64_t)b * p.os.batch + (int64_t)slot * p.os.token +
                 (int64_t)head * p.os.head;
         } else {
-          // kWalk: the last shard the CTA saw anything of; its other shards were written on the way
-          stat = (((int64_t)b * P + (kWalk ? max(kk_open, 0) : part)) * pl.n_q + slot) * p.H + head;
+          // kWalk: the last shard the CTA saw anything of; its other shards were written on the way.  Otherwise there is
+          // only one KV shard, and the row is a token.
+          const int row = kWalk ? slot
+                                : (int)CASCADE_CHECKED((int64_t)__ldg(pl.q_inv + (size_t)map * pl.n_q + slot), pl.n_q,
+                                                       pl.status, 109);
+          stat = (((int64_t)b * P + (kWalk ? max(kk_open, 0) : 0)) * pl.n_q + row) * p.H + head;
           dst = static_cast<__nv_bfloat16*>(p.o_part) + stat * kD;
         }
       }
@@ -907,6 +1054,7 @@ if constexpr (kRope) {
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the row has left shared memory
       }
+      }
       if constexpr (kWalk) {
         // the shards of which no row of the CTA sees anything were never walked: their partials are empty
         if (row_ok) {
@@ -927,6 +1075,9 @@ if constexpr (kRope) {
         }
       }
       tc_fence_before();
+    } else if (!kWalk && split > 1) {
+      cluster_barrier();
+      cluster_barrier();
     }
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
@@ -981,7 +1132,7 @@ if constexpr (kRope) {
             }
           }
         };
-        TileSeq<kWalk> seq(tab, n_act, n_chunks);
+        TileSeq<kWalk> seq(tab, n_act, n_keys);
         bool opens_cur = true, opens_next = false;
         int n_cur = kChunk * seq.next(opens_cur), n_next = 0;
         wait_bar(wc, bar(K_FULL), 0u, 7);
@@ -1073,13 +1224,13 @@ if constexpr (kRope) {
       if (n_tiles > 0 && lw < 2) {
         const bool is_k = lw == 0;
         const CUtensorMap* map = is_k ? &tma.k : &tma.v;
-        const int z = b * p.Hkv + g;  // which [n_kv][head_dim] matrix of the shard-major copy
+        const int z = b * p.Hkv + g;  // kWalk: which [n_kv][head_dim] matrix of the shard-major copy
         const int n_stages = is_k ? kKStages : kVStages;
         const int full0 = is_k ? K_FULL : V_FULL, empty0 = is_k ? K_EMPTY : V_EMPTY;
         const uint32_t tiles_s = smem_base + (is_k ? kOffK : kOffV);
         const bool leader = elect_one();
-        ChunkCursor cur;
-        cur.start(tab, n_act);
+        ChunkCursor cur{};
+        if (kWalk) cur.start(tab, n_act);
         // The shard-major copies are written by the gather grid launched just before this one; when this grid was
         // launched as its programmatic dependent it may have started early, so wait here for that grid to complete
         // (a no-op otherwise).  Nothing else in this kernel reads what the gather grid writes.
@@ -1090,21 +1241,33 @@ if constexpr (kRope) {
           note(8 * i + 1);
           wait_bar(wc, bar(empty0 + st), (uint32_t)(((i / n_stages) & 1) ^ 1), is_k ? 9 : 10, i);
           const uint32_t dst = tiles_s + (uint32_t)(st * kTileBytes), fb = bar(full0 + st);
-          if (leader) mbar_expect_tx(fb, (uint32_t)(nch * C::kHalves * kChunkBytes));
-          for (int ch = 0; ch < nch; ++ch) {
-            // A chunk is 32 consecutive rows of the shard-major copy.  Rows past the shard's visible prefix belong
-            // to later keys or, past the end of the matrix, are zero-filled: they are masked either way.
-            const int slot = tab->slot0[cur.j] + cur.c * kChunk;
-            if (leader) {
-              tma_tile3(dst + (uint32_t)(ch * kChunkBytes), map, 0, slot, z, fb);
-              if (C::kHalves == 2) tma_tile3(dst + (uint32_t)(kHalfBytes + ch * kChunkBytes), map, 64, slot, z, fb);
+          if constexpr (kWalk) {
+            if (leader) mbar_expect_tx(fb, (uint32_t)(nch * C::kHalves * kChunkBytes));
+            for (int ch = 0; ch < nch; ++ch) {
+              // A chunk is 32 consecutive rows of the shard-major copy.  Rows past the shard's visible prefix belong
+              // to later keys or, past the end of the matrix, are zero-filled: they are masked either way.
+              const int slot = tab->slot0[cur.j] + cur.c * kChunk;
+              if (leader) {
+                tma_tile3(dst + (uint32_t)(ch * kChunkBytes), map, 0, slot, z, fb);
+                if (C::kHalves == 2) tma_tile3(dst + (uint32_t)(kHalfBytes + ch * kChunkBytes), map, 64, slot, z, fb);
+              }
+              cur.advance(tab, n_act);
             }
-            cur.advance(tab, n_act);
+          } else if (leader) {
+            // 128 rows at a time; rows past what any query sees lie outside the tensor map and are zero-filled, so that
+            // whatever the unwritten tail of a cache holds stays out of the products
+            mbar_expect_tx(fb, (uint32_t)kTileBytes);
+            tma_tile4(dst, map, 0, key0 + kNMax * i, g, b, fb);
+            if (C::kHalves == 2) tma_tile4(dst + (uint32_t)kHalfBytes, map, 64, key0 + kNMax * i, g, b, fb);
           }
           __syncwarp();
           note(8 * i + 2);
         }
       }
+    }
+    if (!kWalk && split > 1) {
+      cluster_barrier();
+      cluster_barrier();
     }
   }
   __syncthreads();
@@ -1163,15 +1326,78 @@ int sm_count() {
 
 }  // namespace
 
-cudaError_t launch_attn_tc(const AttnParams& p, const void* k_sorted, const void* v_sorted, cudaStream_t stream) {
-  // the unfused route walks all KV shards of a query tile in one CTA (CASCADE_PARTIALS_WALK=0: a CTA per pair)
-  const bool walk = !p.fused && CASCADE_PARTIALS_WALK && p.plan.n_kv_shards > 1;
+namespace {
+
+// K or V rows in token order, [batch][kv_heads][rows][d] by strides; rows past `n_rows` read as zeros.
+bool encode_rows(CUtensorMap* map, const TcRows& r, int d, int64_t n_rows, int64_t n_heads, int64_t batch) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)std::max<int64_t>(1, n_rows), (cuuint64_t)n_heads,
+                              (cuuint64_t)batch};
+  auto stride = [&](int64_t elems, int64_t extent) { return (cuuint64_t)(extent > 1 ? elems * 2 : d * 2); };
+  const cuuint64_t strides[3] = {stride(r.strides.token, n_rows), stride(r.strides.head, n_heads),
+                                 stride(r.strides.batch, batch)};
+  const cuuint32_t box[4] = {64, (cuuint32_t)tc::kNMax, 1, 1};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(r.base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+struct TcLaunch {
+  int lg, tile_major, split;
+  bool after_gather;
+};
+
+cudaError_t launch_kernel(const AttnParams& p, bool walk, const TcLaunch& l, int64_t n_ctas, const tc::TmaArgs& tma,
+                          cudaStream_t stream) {
   auto kernel = p.d == 64 ? (walk ? tc::attn_tc_kernel<64, false, true> : tc::attn_tc_kernel<64, false, false>)
                 : p.rope  ? tc::attn_tc_kernel<128, true, false>
                           : (walk ? tc::attn_tc_kernel<128, false, true> : tc::attn_tc_kernel<128, false, false>);
   const int smem_bytes = p.d == 64 ? tc::Cfg<64>::kSmemBytes : tc::Cfg<128>::kSmemBytes;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
+  if (n_ctas * l.split >= (int64_t)1 << 31) return cudaErrorInvalidConfiguration;
+  TimedLaunch timed(stream);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n_ctas * l.split));
+  cfg.blockDim = dim3(tc::kThreads);
+  cfg.dynamicSmemBytes = smem_bytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  cfg.attrs = attr;
+  if (l.split > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = l.split;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs++].val.clusterDim.z = 1;
+  }
+  // Programmatic dependent launch on the gather grid that precedes it in the stream: the set-up of the CTAs overlaps
+  // the gather's tail.  Not while kernel timing is recording: the event between the two launches must separate them.
+  if (l.after_gather && !timing_recording()) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  e = cudaLaunchKernelEx(&cfg, kernel, p, l.lg, l.tile_major, l.split, tma);
+  count_launch();
+  return e;
+}
+
+// stack as many of the G heads of a KV head into one MMA tile as divide G (at most 8)
+int stacked_log2(int G) {
+  int lg = 0;
+  while (lg < 3 && G % (2 << lg) == 0) ++lg;
+  return lg;
+}
+
+}  // namespace
+
+bool tc_rows_loadable(const TcRows& r, int64_t n_rows, int64_t n_heads, int64_t batch) {
+  auto fine = [](int64_t stride, int64_t extent) { return extent <= 1 || (stride > 0 && stride < (int64_t)1 << 38); };
+  return fine(r.strides.token, n_rows) && fine(r.strides.head, n_heads) && fine(r.strides.batch, batch);
+}
+
+cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, const void* v_sorted, cudaStream_t stream) {
   tc::TmaArgs tma;
   const int64_t n_mats = (int64_t)p.batch * p.Hkv;
   if (!encode_sorted(&tma.k, k_sorted, p.d, p.plan.n_kv, n_mats) ||
@@ -1179,29 +1405,35 @@ cudaError_t launch_attn_tc(const AttnParams& p, const void* k_sorted, const void
     set_error("tensor-core attention: could not build the TMA descriptors of the shard-major K/V copies");
     return cudaErrorInvalidValue;
   }
-  // stack as many of the G heads of a KV head into one MMA tile as divide G (at most 8)
-  int lg = 0;
-  while (lg < 3 && p.G % (2 << lg) == 0) ++lg;
-  const int n_parts = (p.fused || walk) ? 1 : p.plan.n_kv_shards;
-  const int64_t n_ctas = (int64_t)p.plan.n_qtiles[3 - lg] * (p.H >> lg) * p.batch * n_parts;
-  if (n_ctas >= (int64_t)1 << 31) return cudaErrorInvalidConfiguration;
-  const int tile_major = n_ctas <= 8 * (int64_t)sm_count();  // few CTAs per SM: balance matters more than L2 locality
-  TimedLaunch timed(stream);
-  // Programmatic dependent launch on the gather grid that precedes it in the stream: the set-up of the CTAs overlaps
-  // the gather's tail.  Not while kernel timing is recording: the event between the two launches must separate them.
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)n_ctas);
-  cfg.blockDim = dim3(tc::kThreads);
-  cfg.dynamicSmemBytes = smem_bytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = timing_recording() ? 0 : 1;
-  e = cudaLaunchKernelEx(&cfg, kernel, p, lg, tile_major, tma);
-  count_launch();
-  return e;
+  const int lg = stacked_log2(p.G);
+  const int64_t n_ctas = (int64_t)p.plan.n_qtiles[3 - lg] * (p.H >> lg) * p.batch;
+  // few CTAs per SM: balance matters more than L2 locality
+  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), 1, true};
+  return launch_kernel(p, true, l, n_ctas, tma, stream);
+}
+
+cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v, int64_t n_seen, bool after_gather,
+                           cudaStream_t stream) {
+  tc::TmaArgs tma;
+  if (!encode_rows(&tma.k, k, p.d, n_seen, p.Hkv, p.batch) || !encode_rows(&tma.v, v, p.d, n_seen, p.Hkv, p.batch)) {
+    set_error("tensor-core attention: could not build the TMA descriptors of K and V");
+    return cudaErrorInvalidValue;
+  }
+  const int lg = stacked_log2(p.G);
+  const int64_t tile_slots = 256 >> lg, n_qt = (p.plan.n_q + tile_slots - 1) / tile_slots;
+  const int64_t n_ctas = n_qt * (p.H >> lg) * p.batch;
+  // Few query tiles (a chunk of a chunked prefill, a short prompt) leave SMs idle: a cluster then shares the keys of each
+  // tile, as far as its CTAs fit at once with one per SM (clusters of 2, 4 and 8: 148, 132 and 120 CTAs) and have two
+  // 128-key tiles each.  The rule counts the heads of the whole problem, see AttnParams.
+  const int64_t rule_ctas = n_qt * ((int64_t)p.rule_kv_heads * p.G >> lg) * p.batch, key_tiles = (n_seen + 127) / 128;
+  int split = 1;
+  if (p.fused) {
+    const int64_t fit[4] = {148, 148, 132, 120};
+    for (int i = 1; i < 4; ++i)
+      if (rule_ctas << i <= fit[i] && key_tiles >= 2 << i) split = 1 << i;
+  }
+  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), split, after_gather};
+  return launch_kernel(p, false, l, n_ctas, tma, stream);
 }
 
 }  // namespace cascade

@@ -720,18 +720,57 @@ static size_t decode_ws_bytes(const cascade_plan_t* plan, cascade_dtype_t dtype,
   return align_up(rows * d * elt_size(dtype), 256) + 2 * align_up(rows * 4, 256);
 }
 
-// Tensor-core route: shard gather of K and V into the workspace, then the attention kernel (two launches).
-static cascade_status_t run_tc(const AttnParams& p, const char* fn, const cascade_plan_t* plan, void* workspace,
+// Workspace of the tensor-core route: shard-major K and V copies, and for head_dim 128 a place for rotated keys in token
+// order (cascade_attn_sharded_rope).
+static size_t tc_ws_bytes(const cascade_plan_t* plan, int batch, int Hkv, int d) {
+  return (d == 128 ? 3 : 2) * sorted_kv_bytes(plan, batch, Hkv, d);
+}
+
+// Tensor-core route.
+// Partials of several KV shards: a gather of K and V into shard-major order, then a kernel that walks the shards.
+// Otherwise the shards are only different subsets of the same sum, in which a query sees a prefix of the K/V rows (all those
+// at positions up to its own), so the kernel takes tiles of consecutive tokens and reads the rows where they are: no copy,
+// no chunk of 32 keys left half empty at the end of every shard, and 64 queries of a tile that span 64 positions instead of
+// 64 times the number of shards (2048 tokens, 8 random shards: 1.32 times the causal work before, 1.09 now).
+static cascade_status_t run_tc(AttnParams p, const char* fn, const cascade_plan_t* plan, void* workspace,
                                size_t workspace_bytes, cudaStream_t st, cudaError_t* launch_error) {
-  const size_t each = sorted_kv_bytes(plan, p.batch, p.Hkv, p.d);
-  if (!workspace || workspace_bytes < 2 * each || ((uintptr_t)workspace & 255)) {
-    set_error("%s: workspace of %zu bytes (256-byte aligned) required for the shard-major K/V copies, got %zu", fn,
-              2 * each, workspace_bytes);
+  const size_t each = sorted_kv_bytes(plan, p.batch, p.Hkv, p.d), need = tc_ws_bytes(plan, p.batch, p.Hkv, p.d);
+  if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) {
+    set_error("%s: workspace of %zu bytes (256-byte aligned) required for copies of K and V, got %zu", fn, need,
+              workspace_bytes);
     return CASCADE_ERR_WORKSPACE;
   }
+  const PlanDev& d = plan->dev;
   char* ws = (char*)workspace;
-  *launch_error = launch_gather_kv(p, ws, ws + each, st);
-  if (*launch_error == cudaSuccess) *launch_error = launch_attn_tc(p, ws, ws + each, st);
+  if (!p.fused && d.n_kv_shards > 1) {
+    *launch_error = launch_gather_kv(p, ws, ws + each, nullptr, false, false, st);
+    if (*launch_error == cudaSuccess) *launch_error = launch_attn_tc_partials(p, ws, ws + each, st);
+    return CASCADE_OK;
+  }
+  p.prefix_from_vis = !plan->kv_pos.empty();
+  int64_t n_seen = 0;  // rows past what the last query sees may hold anything: the kernel does not load them
+  for (int mp = 0; mp < (p.prefix_from_vis ? d.n_maps : 1); ++mp)
+    n_seen = std::max(n_seen, visible_keys(*plan, mp, (int64_t)d.n_q - 1 + d.q_pos_offset));
+  TcRows k = {p.k, p.ks}, v = {p.v, p.vs};
+  const Strides dense = {(int64_t)p.Hkv * d.n_kv * p.d, p.d, (int64_t)d.n_kv * p.d};
+  const bool v_fits = tc_rows_loadable(v, n_seen, p.Hkv, p.batch);
+  bool gathered = false;
+  if (p.rope) {
+    // the rotated keys: in token order for the kernel, and shard-major with the values, as the call leaves them behind
+    *launch_error = launch_gather_kv(p, ws, ws + each, ws + 2 * each, false, !v_fits, st);
+    k = {ws + 2 * each, dense};
+    if (!v_fits) v = {ws + each, dense};
+    gathered = true;
+  } else if (!v_fits || !tc_rows_loadable(k, n_seen, p.Hkv, p.batch) || (p.prefix_from_vis && d.n_maps > 1)) {
+    // strides that a tensor map cannot hold (an expanded axis), or a different last visible row per sequence
+    *launch_error = launch_gather_kv(p, ws, ws + each, nullptr, true, true, st);
+    k = {ws, dense};
+    v = {ws + each, dense};
+    gathered = true;
+  } else {
+    *launch_error = cudaSuccess;
+  }
+  if (*launch_error == cudaSuccess) *launch_error = launch_attn_tc(p, k, v, n_seen, gathered, st);
   return CASCADE_OK;
 }
 
@@ -766,7 +805,7 @@ static HostCallLayout host_call_layout(const cascade_plan_t* plan, cascade_dtype
   // gs KV heads and their query heads per inner call
   const bool decode = use_decode(plan, dtype, G * gs, gs, d);
   L.inner_bytes = decode ? decode_ws_bytes(plan, dtype, batch, G * gs, d)
-                         : (use_tc(plan, dtype, d) ? 2 * sorted_kv_bytes(plan, batch, gs, d) : 0);
+                         : (use_tc(plan, dtype, d) ? tc_ws_bytes(plan, batch, gs, d) : 0);
   L.total = L.inner + align_up(L.inner_bytes, 256);
   return L;
 }
@@ -796,7 +835,7 @@ cascade_status_t cascade_workspace_bytes(const cascade_plan_t* plan, int32_t whi
     return CASCADE_ERR_INVALID_ARG;
   }
   const bool decode = use_decode(plan, dtype, n_heads, n_kv_heads, head_dim);
-  const size_t tc_bytes = !decode && use_tc(plan, dtype, head_dim) ? 2 * sorted_kv_bytes(plan, batch, n_kv_heads, head_dim) : 0;
+  const size_t tc_bytes = !decode && use_tc(plan, dtype, head_dim) ? tc_ws_bytes(plan, batch, n_kv_heads, head_dim) : 0;
   if (which_call == CASCADE_CALL_PARTIALS) {
     *out_bytes = tc_bytes;
   } else if (which_call == CASCADE_CALL_SHARDED) {

@@ -48,6 +48,7 @@ struct AttnParams {
   // KV heads of the whole problem: more than Hkv where a call computes a part of the heads at a time.  Rules that decide how
   // sums are split go by it, so that the parts get the same bits as one call would.
   int32_t rule_kv_heads;
+  int32_t prefix_from_vis;  // the K/V rows have positions of their own: a query's prefix is the sum of its row of vis
   float scale;
   int32_t fused;  // 0: one job per KV shard, write (u, m, l); 1: walk all KV shards, write o (+lse)
   void* o_part;
@@ -147,9 +148,21 @@ struct TimedLaunch {  // RAII: events around the launches issued while it lives
 
 // Launchers; each returns a cudaError_t from the launch.
 cudaError_t launch_attn_simt(const AttnParams& p, cascade_dtype_t dtype, cudaStream_t stream);
-// k_sorted / v_sorted: the shard-major copies written by launch_gather_kv, [batch][kv_head][n_kv][128] bf16
-cudaError_t launch_attn_tc(const AttnParams& p, const void* k_sorted, const void* v_sorted, cudaStream_t stream);
-cudaError_t launch_gather_kv(const AttnParams& p, void* k_out, void* v_out, cudaStream_t stream);
+// K or V rows [batch][kv_heads][rows][d] for the tensor-core kernel (strides in elements)
+struct TcRows {
+  const void* base;
+  Strides strides;
+};
+bool tc_rows_loadable(const TcRows& r, int64_t n_rows, int64_t n_heads, int64_t batch);
+// all keys of a query in one go, K and V in token order; rows from n_seen on are not looked at
+cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v, int64_t n_seen, bool after_gather,
+                           cudaStream_t stream);
+// the partials of every KV shard; k_sorted / v_sorted: shard-major copies, [batch][kv_head][n_kv][d] bf16
+cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, const void* v_sorted, cudaStream_t stream);
+// Copies of K and V for the above, [batch][kv_head][n_kv][d]: shard-major, or with token_order as the rows are.  With
+// p.rope the key rows are turned on the way, and k_tokens (if not null) gets them in token order as well.
+cudaError_t launch_gather_kv(const AttnParams& p, void* k_out, void* v_out, void* k_tokens, bool token_order, bool v_token_order,
+                             cudaStream_t stream);
 cudaError_t launch_rope_table(int32_t n_positions, int32_t head_dim, double base, float2* table, cudaStream_t stream);
 cudaError_t launch_rope_apply(cascade_dtype_t dtype, int32_t batch, int32_t n_rows, int32_t n_heads, int32_t head_dim,
                               const void* x, Strides xs, int32_t first_position, const float2* table, void* y, Strides ys,

@@ -27,7 +27,8 @@ __device__ __forceinline__ bool slot_is_visible(const PlanDev& pl, int map, int 
 }
 
 template <int D>
-__global__ void __launch_bounds__(256) gather_kv_kernel(AttnParams p, __nv_bfloat16* k_out, __nv_bfloat16* v_out) {
+__global__ void __launch_bounds__(256) gather_kv_kernel(const __grid_constant__ AttnParams p, __nv_bfloat16* k_out,
+                                                        __nv_bfloat16* v_out, bool token_order) {
   constexpr int kLanes = D / 8;              // 16 bytes per thread
   constexpr int kRows = 256 / kLanes;        // rows per pass
   constexpr int kPasses = kGatherRowsPerCta / kRows;
@@ -44,22 +45,25 @@ __global__ void __launch_bounds__(256) gather_kv_kernel(AttnParams p, __nv_bfloa
   const int64_t out_base = ((int64_t)b * p.Hkv + g) * pl.n_kv;
   const int slot0 = blockIdx.x * kGatherRowsPerCta;
   uint4 kr[kPasses], vr[kPasses];
+  int row[kPasses];  // of the copies
 #pragma unroll
   for (int i = 0; i < kPasses; ++i) {
     const int slot = slot0 + kRows * i + r0;
+    row[i] = slot;
     kr[i] = vr[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (slot < pl.n_kv && slot_is_visible(pl, map, slot)) {
-      const int64_t tok = CASCADE_CHECKED((int64_t)__ldg(kv_idx + slot), pl.n_kv, pl.status, 101);
+    if (slot >= pl.n_kv) continue;
+    const int64_t tok = CASCADE_CHECKED((int64_t)__ldg(kv_idx + slot), pl.n_kv, pl.status, 101);
+    if (token_order) row[i] = (int)tok;
+    if (slot_is_visible(pl, map, slot)) {
       kr[i] = __ldcs(reinterpret_cast<const uint4*>(kb + tok * p.ks.token + chunk * 8));
       vr[i] = __ldcs(reinterpret_cast<const uint4*>(vb + tok * p.vs.token + chunk * 8));
     }
   }
 #pragma unroll
   for (int i = 0; i < kPasses; ++i) {
-    const int slot = slot0 + kRows * i + r0;
-    if (slot < pl.n_kv) {
-      *reinterpret_cast<uint4*>(k_out + (out_base + slot) * D + chunk * 8) = kr[i];
-      *reinterpret_cast<uint4*>(v_out + (out_base + slot) * D + chunk * 8) = vr[i];
+    if (slot0 + kRows * i + r0 < pl.n_kv) {
+      *reinterpret_cast<uint4*>(k_out + (out_base + row[i]) * D + chunk * 8) = kr[i];
+      *reinterpret_cast<uint4*>(v_out + (out_base + row[i]) * D + chunk * 8) = vr[i];
     }
   }
 }
@@ -83,7 +87,9 @@ __device__ __forceinline__ void rotate8(uint4& lo, uint4& hi, const float2* __re
 // key rows on the way: a key row is turned by the angles of its own token index, so the rotation needs nothing but
 // the row and its row of the positional table.  A thread holds both halves of 8 rotation pairs (columns 8c.. and
 // 64 + 8c..), 8 threads per row; V rows are copied as they are.
-__global__ void __launch_bounds__(256) gather_kv_rope_kernel(AttnParams p, __nv_bfloat16* k_out, __nv_bfloat16* v_out) {
+__global__ void __launch_bounds__(256) gather_kv_rope_kernel(const __grid_constant__ AttnParams p, __nv_bfloat16* k_out,
+                                                             __nv_bfloat16* v_out, __nv_bfloat16* k_tokens,
+                                                             bool v_token_order) {
   constexpr int D = 128;
   constexpr int kPasses = kGatherRowsPerCta / 32;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // as in gather_kv_kernel
@@ -102,9 +108,10 @@ __global__ void __launch_bounds__(256) gather_kv_rope_kernel(AttnParams p, __nv_
   for (int i = 0; i < kPasses; ++i) {
     const int slot = slot0 + 32 * i + r0;
     klo[i] = khi[i] = vlo[i] = vhi[i] = make_uint4(0u, 0u, 0u, 0u);
-    tok[i] = -1;
-    if (slot < pl.n_kv && slot_is_visible(pl, map, slot)) {
-      tok[i] = (int)CASCADE_CHECKED((int64_t)__ldg(kv_idx + slot), pl.n_kv, pl.status, 101);
+    tok[i] = 0;
+    if (slot >= pl.n_kv) continue;
+    tok[i] = (int)CASCADE_CHECKED((int64_t)__ldg(kv_idx + slot), pl.n_kv, pl.status, 101);
+    if (slot_is_visible(pl, map, slot)) {
       const __nv_bfloat16* kr = kb + (int64_t)tok[i] * p.ks.token + chunk * 8;
       const __nv_bfloat16* vr = vb + (int64_t)tok[i] * p.vs.token + chunk * 8;
       klo[i] = __ldcs(reinterpret_cast<const uint4*>(kr));
@@ -117,25 +124,29 @@ __global__ void __launch_bounds__(256) gather_kv_rope_kernel(AttnParams p, __nv_
   for (int i = 0; i < kPasses; ++i) {
     const int slot = slot0 + 32 * i + r0;
     if (slot < pl.n_kv) {
-      if (tok[i] >= 0) rotate8(klo[i], khi[i], p.rope + (int64_t)tok[i] * (D / 2) + chunk * 8);
+      rotate8(klo[i], khi[i], p.rope + (int64_t)tok[i] * (D / 2) + chunk * 8);  // zeros stay zeros
       __nv_bfloat16* ko = k_out + (out_base + slot) * D + chunk * 8;
-      __nv_bfloat16* vo = v_out + (out_base + slot) * D + chunk * 8;
+      __nv_bfloat16* kt = k_tokens + (out_base + tok[i]) * D + chunk * 8;
+      __nv_bfloat16* vo = v_out + (out_base + (v_token_order ? tok[i] : slot)) * D + chunk * 8;
       *reinterpret_cast<uint4*>(ko) = klo[i];
       *reinterpret_cast<uint4*>(ko + 64) = khi[i];
+      *reinterpret_cast<uint4*>(kt) = klo[i];
+      *reinterpret_cast<uint4*>(kt + 64) = khi[i];
       *reinterpret_cast<uint4*>(vo) = vlo[i];
       *reinterpret_cast<uint4*>(vo + 64) = vhi[i];
     }
   }
 }
 
-cudaError_t launch_gather_kv(const AttnParams& p, void* k_out, void* v_out, cudaStream_t stream) {
+cudaError_t launch_gather_kv(const AttnParams& p, void* k_out, void* v_out, void* k_tokens, bool token_order, bool v_token_order,
+                             cudaStream_t stream) {
   dim3 grid((p.plan.n_kv + kGatherRowsPerCta - 1) / kGatherRowsPerCta, p.Hkv, p.batch);
+  __nv_bfloat16 *ko = static_cast<__nv_bfloat16*>(k_out), *vo = static_cast<__nv_bfloat16*>(v_out);
   if (p.rope) {
-    gather_kv_rope_kernel<<<grid, 256, 0, stream>>>(p, static_cast<__nv_bfloat16*>(k_out),
-                                                    static_cast<__nv_bfloat16*>(v_out));
+    gather_kv_rope_kernel<<<grid, 256, 0, stream>>>(p, ko, vo, static_cast<__nv_bfloat16*>(k_tokens), v_token_order);
   } else {
     auto kernel = p.d == 64 ? gather_kv_kernel<64> : gather_kv_kernel<128>;
-    kernel<<<grid, 256, 0, stream>>>(p, static_cast<__nv_bfloat16*>(k_out), static_cast<__nv_bfloat16*>(v_out));
+    kernel<<<grid, 256, 0, stream>>>(p, ko, vo, token_order);
   }
   count_launch();
   return cudaGetLastError();

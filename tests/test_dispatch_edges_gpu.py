@@ -141,3 +141,69 @@ def test_decode_step_moves_the_plan_with_few_and_with_many_prefixes(gu, B, P, pe
             assert np.array_equal(gu.read_plan_device_array(plan, "pair_class")[b], op.pair_class)
             assert np.array_equal(plan.get("vis")[b], op.vis)
     plan.destroy()
+
+
+@pytest.mark.parametrize("n_q,n_kv,H,Hkv,d,B,off,causal", [
+    (2, 2, 8, 8, 128, 1, 0, True),           # one tile; the rows see one and two keys
+    (65, 1025, 32, 8, 128, 1, 960, True),    # keys shared by clusters of 8; a second query tile of one row, one key past a tile
+    (200, 640, 8, 4, 128, 2, 0, True),       # clusters of 8 where the first tiles see fewer than 8 key tiles: idle ranks
+    (300, 700, 16, 4, 64, 2, 400, True),     # clusters of 4 at head_dim 64
+    (512, 900, 32, 8, 128, 1, 100, True),    # clusters of 2; keys past the last query position are not looked at
+    (130, 300, 12, 3, 128, 1, 0, False),     # every key for every row, shared
+    (40, 500, 4, 2, 128, 1, -20, True),      # the first rows see nothing
+])
+def test_fused_route_in_token_order(gu, n_q, n_kv, H, Hkv, d, B, off, causal):
+    w = wl.make_workload(f"tok_{n_q}_{n_kv}", B, n_q, n_kv, H, Hkv, d, "bf16", "random", "random", 3, 5, seed=n_q + n_kv,
+                         causal=causal, q_pos_offset=off, symmetric=False)
+    gu.full_parity(w)
+
+
+@pytest.mark.parametrize("n_q", [70, 700])
+def test_fused_route_with_strides_a_tensor_map_cannot_hold(gu, n_q):
+    """K and V of one sequence expanded over the batch (stride 0) go through a copy; the result is the same, bit for bit."""
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload("expanded", 2, n_q, 700, 8, 2, 128, "bf16", "random", "random", 2, 3, seed=n_q, symmetric=False)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    k1, v1 = k[:1].expand(2, -1, -1, -1), v[:1].expand(2, -1, -1, -1)
+    o_a, lse_a = cb.cascade_attn_sharded(plan, q, k1, v1, w.scale)
+    o_b, lse_b = cb.cascade_attn_sharded(plan, q, k1.contiguous(), v1.contiguous(), w.scale)
+    assert torch.equal(o_a, o_b) and torch.equal(lse_a, lse_b)
+    table = cb.cascade_rope_table(700, 128, 10000.0)
+    o_a, _ = cb.cascade_attn_sharded_rope(plan, q, k1, v1, w.scale, table)
+    o_b, _ = cb.cascade_attn_sharded_rope(plan, q, k1.contiguous(), v1.contiguous(), w.scale, table)
+    assert torch.equal(o_a, o_b)
+    plan.destroy()
+
+
+@pytest.mark.parametrize("n_maps", [1, 2])
+def test_fused_route_over_resident_rows(gu, n_maps):
+    """Rows with positions of their own: a query sees those at positions up to its own, and what lies behind may be NaN."""
+    from paper_2507_05228_b200 import binding as cb
+    rng = np.random.default_rng(n_maps)
+    n, n_q, n_kv, B = 600, 90, 250, 2
+    w = wl.make_workload("resident", B, n, n, 8, 2, 128, "bf16", "random", "random", 2, 2, seed=61)
+    q, k, v = gu.to_device(w)
+    pos = np.sort(np.stack([rng.choice(n, n_kv, replace=False) for _ in range(n_maps)]), axis=1).astype(np.int32)
+    off, q_of, kv_of = 300, rng.integers(0, 2, (n_maps, n_q)).astype(np.int32), rng.integers(0, 4, (n_maps, n_kv)).astype(np.int32)
+    plan = cb.cascade_shard_plan_resident(q_of, kv_of, pos, 2, 4, off)
+    sel = [torch.from_numpy(pos[b % n_maps].astype(np.int64)).cuda() for b in range(B)]
+    kr, vr = torch.stack([k[b, sel[b]] for b in range(B)]), torch.stack([v[b, sel[b]] for b in range(B)])
+    qr = q[:, off:off + n_q].contiguous()
+    for b in range(B):
+        hidden = sel[b] > off + n_q - 1
+        kr[b, hidden], vr[b, hidden] = float("nan"), float("nan")
+    o, lse = cb.cascade_attn_sharded(plan, qr, kr, vr, w.scale)
+    keep = np.full((B, n), -np.inf)
+    for b in range(B):
+        keep[b, pos[b % n_maps]] = 0.0
+    G = 4
+    logits = np.einsum("bqhd,bkhd->bhqk", w.q[:, off:off + n_q].astype(np.float64), np.repeat(w.k, G, 2).astype(np.float64)) * w.scale
+    causal = np.where(np.arange(n)[None, :] <= np.arange(off, off + n_q)[:, None], 0.0, -np.inf)
+    logits = logits + keep[:, None, None, :] + causal[None, None]
+    m = logits.max(-1, keepdims=True)
+    e = np.exp(logits - m)
+    o_ref = np.einsum("bhqk,bkhd->bqhd", e / e.sum(-1, keepdims=True), np.repeat(w.v, G, 2).astype(np.float64))
+    lse_ref = (m[..., 0] + np.log(e.sum(-1))).transpose(0, 2, 1)
+    gu.check_output(o, lse, o_ref, lse_ref, w.tol, "resident rows, fused")
+    plan.destroy()
