@@ -23,9 +23,9 @@
 //
 // Warp roles (12 warps):
 //   0-3   softmax of sub-tile 0, 4-7 softmax of sub-tile 1: thread = MMA row = TMEM lane.  Reads the logits S with
-//         tcgen05.ld, applies the shard mask (the row sees the first vis[slot][k] keys of the shard), keeps the running
-//         max / sum, writes the probabilities P as bf16 back into the TMEM columns of S, rescales the output
-//         accumulator in TMEM when the running max moved by more than 2^8, and runs the epilogue: the scaled output
+//         tcgen05.ld, applies the mask (the row sees a prefix of the keys), writes the weights P as bf16 back into the TMEM
+//         columns of S, keeps the running max / sum while the products run, rescales the output accumulator in TMEM in
+//         the rare case that a weight is far above the reference maximum, and runs the epilogue: the scaled output
 //         row goes through shared memory (the Q / K tiles are free by then) to the copy engine, one 256-byte bulk
 //         copy per row.
 //   8     MMA issuer: S_s = Q_s K^T (operands in shared memory) and O_s += P_s V (P from TMEM), issued as
@@ -59,7 +59,11 @@ constexpr int kM = 128;                  // MMA rows per sub-tile
 constexpr int kNMax = 128;               // keys per KV tile (upper bound)
 constexpr int kHalfBytes = kM * 128;     // one 64-column half of a 128-row tile: 128 rows of 128 bytes
 constexpr uint32_t kTmemCols = 512;
-constexpr float kRescaleThreshold = 8.f;  // log2 units
+// How far a row may rise above its reference maximum before it is rescaled: by its logits (log2 units), or by the sum of a
+// tile's weights.  (bf16 and fp32 keep their relative precision at any scale; the sums of 2^20 tiles and the products with
+// values below 2^40 stay in range.)
+constexpr float kRescaleThreshold = 60.f;
+constexpr float kRescaleSum = 1.1529215e18f;  // 2^60
 // setmaxnreg only redistributes the registers the CTA was launched with (168 per thread x 384 threads = 64512), and
 // all four warps of an allocation group execute the same instruction: 8 warps x 32 x 216 + 4 warps x 32 x 72 = 64512.
 // An increase that asks for more than the launch grant never returns.
@@ -806,25 +810,42 @@ if constexpr (kRope) {
             }
           }
         }
-        float mx[4];
+        auto row_max = [&]() {  // raw logit
+          float mx[4];
 #pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4) {
-          mx[q4] = __uint_as_float(sr[32 * q4]);
+          for (int q4 = 0; q4 < 4; ++q4) {
+            mx[q4] = __uint_as_float(sr[32 * q4]);
 #pragma unroll
-          for (int j = 1; j < 31; j += 2)
-            mx[q4] = fmax3(mx[q4], __uint_as_float(sr[32 * q4 + j]), __uint_as_float(sr[32 * q4 + j + 1]));
-          mx[q4] = fmaxf(mx[q4], __uint_as_float(sr[32 * q4 + 31]));
+            for (int j = 1; j < 31; j += 2)
+              mx[q4] = fmax3(mx[q4], __uint_as_float(sr[32 * q4 + j]), __uint_as_float(sr[32 * q4 + j + 1]));
+            mx[q4] = fmaxf(mx[q4], __uint_as_float(sr[32 * q4 + 31]));
+          }
+          return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+        };
+        // The reference the weights are scaled by is the maximum of the first tile, and stays that unless a later tile rises
+        // far above it.  kLateMax: that shows in the weights, so the maximum of this tile is not needed before its
+        // exponentials, and is taken while the products are under way (it was 320 of the 2200 cycles between the logits and
+        // the weights; 2048 tokens 47 -> 44 us, 4 x 8192 with rotary step 2.22 -> 2.06 ms).  Not with kWalk, where most tiles
+        // open a shard (434 -> 471 us on 4099 tokens in 16 shards), nor with kRing, whose next logits are there already.
+        constexpr bool kLateMax = !kWalk && !kRing;
+        float smax = 0.f, alpha = 1.f;
+        bool changed = false;
+        if constexpr (kLateMax) {
+          if (opens) {
+            smax = row_max();
+            m_true = m_run = smax * c;  // -inf: the row sees nothing of the stream (a prefix, so not later either)
+          }
+        } else {  // straight-line: branches here cost more than they save
+          smax = row_max();
+          m_true = fmaxf(m_true, smax * c);
+          float m_new = m_run;
+          if (m_run == -INFINITY || m_true > m_run + kRescaleThreshold) m_new = m_true;
+          alpha = (m_run == -INFINITY) ? 0.f : ex2(m_run - m_new);
+          changed = m_new != m_run;
+          m_run = m_new;
         }
-        const float smax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));  // raw logit
-        const float tmax = smax * c;
-        m_true = fmaxf(m_true, tmax);
-        float m_new = m_run;
-        if (m_run == -INFINITY || m_true > m_run + kRescaleThreshold) m_new = m_true;
-        const float alpha = (m_run == -INFINITY) ? 0.f : ex2(m_run - m_new);
-        const bool changed = m_new != m_run;
-        m_run = m_new;
-        const float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
-        const uint64_t neg_m2 = pack2(neg_m, neg_m);
+        float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
+        uint64_t neg_m2 = pack2(neg_m, neg_m);
         uint64_t psum2 = pack2(0.f, 0.f);
         auto exp_chunk = [&](int ch) {
           uint32_t pk[16], pr[kRing ? 16 : 1];
@@ -848,6 +869,7 @@ if constexpr (kRope) {
           CASCADE_TMEM_ST16(s_addr + (uint32_t)(16 * ch), pk);
           if constexpr (kRing) CASCADE_TMEM_ST16(s_addr + 64u + (uint32_t)(16 * ch), pr);
         };
+        auto exp_tile = [&]() {
         if (nch == 4) {
           // The full tile is one straight-line block, so that the scheduler can run the MUFU instructions of one chunk
           // (8 issue cycles each) under the FMA / convert / store work of its neighbours; with a branch per chunk the
@@ -861,29 +883,28 @@ if constexpr (kRope) {
           for (int ch = 0; ch < 3; ++ch)
             if (ch < nch) exp_chunk(ch);  // warp-uniform
         }
+        };
+        exp_tile();
         float psum0, psum1;
         unpack2(psum2, psum0, psum1);
         // The tensor core multiplies the weights after rounding them to bf16, while the sum above is taken before.
-        // With the lagging reference max even the largest weight of a row has an arbitrary mantissa, so when one key
+        // With the reference of another tile even the largest weight of a row has an arbitrary mantissa, so when one key
         // dominates a row its rounding error (up to 2^-9 relative) would go straight into O / l: 0.009 at |v| = 4.5.
         // The sum therefore takes the tile's largest weight as the tensor core sees it (same fma and ex2 as in the
         // loop above, so the same bits); the other weights' errors are small against l or average out.
         // (Not with kRing, whose weights keep 16 bits of mantissa.)
-        float top_err = 0.f;
-        if constexpr (!kRing) {
+        auto top_error = [&]() {
           const float p_top = ex2(fmaf(smax, c, neg_m));
-          top_err = __uint_as_float(pack_bf16x2(0.f, p_top) & 0xffff0000u) - p_top;
-        }
-        l_run = l_run * alpha + ((psum0 + psum1) + top_err);
-        // S_FULL(i) was committed after PV(i-1), so the output accumulator is quiescent until this thread's
-        // arrival on P_FULL(i) below.  With kRing the logits run ahead of the products, and O_RDY says when PV(i-1) is in
-        // (it cannot complete twice without this thread's arrival, so waiting only when needed keeps the parity exact).
-        if (!opens && __any_sync(0xffffffffu, changed)) {
+          return __uint_as_float(pack_bf16x2(0.f, p_top) & 0xffff0000u) - p_top;
+        };
+        // S_FULL(i) was committed after PV(i-1), so the output accumulator is quiescent until this thread's arrival on
+        // P_FULL(i) below.  With kRing the logits run ahead of the products, and O_RDY says when PV(i-1) is in (it cannot
+        // complete twice without this thread's arrival, so waiting only when needed keeps the parity).
+        auto rescale = [&]() {  // this warp's 32 rows
           if constexpr (kRing) {
             wait_bar(wc, bar(O_RDY + s), (uint32_t)((i - 1) & 1), 2, i);
             tc_fence_after();
           }
-          // rescale this warp's 32 rows of the output accumulator
           const float f = changed ? alpha : 1.f;
 #pragma unroll
           for (int cc = 0; cc < kD / 32; ++cc) {
@@ -894,17 +915,44 @@ if constexpr (kRope) {
             for (int j = 0; j < 32; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * f);
             CASCADE_TMEM_ST32(o_addr + (uint32_t)(cc * 32), o, 0);
           }
+        };
+        if constexpr (kLateMax) {
+          if (!opens && __any_sync(0xffffffffu, !(psum0 + psum1 < kRescaleSum))) {
+            smax = row_max();
+            const float m_new = fmaxf(m_run, smax * c);
+            alpha = (m_run == -INFINITY) ? 0.f : ex2(m_run - m_new);
+            changed = true;
+            m_run = m_new;
+            neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
+            neg_m2 = pack2(neg_m, neg_m);
+            l_run *= alpha;
+            rescale();
+            tmem_wait_st();  // the first weights, too: the second ones go to the same place
+            psum2 = pack2(0.f, 0.f);
+            exp_tile();
+            unpack2(psum2, psum0, psum1);
+          }
+        } else {
+          l_run = l_run * alpha + ((psum0 + psum1) + (kRing ? 0.f : top_error()));
+          if (!opens && __any_sync(0xffffffffu, changed)) rescale();
         }
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(p_full(s, i));
+        if constexpr (kLateMax) {
+          if (!opens) {
+            smax = row_max();
+            m_true = fmaxf(m_true, smax * c);
+          }
+          l_run += (psum0 + psum1) + top_error();
+        }
         note(8 * i + 2);
       }
       note(8 * n_tiles + 3);
       if (!kWalk && split > 1) {
         // ---- epilogue of a query tile whose keys were shared by the cluster: CTA r finishes columns r * cols .. of all
         // rows.  Every CTA sends it those columns of its accumulator and its row statistics (relative to its own m).
-        const int cols = kD / split, me = part_of_keys;
+        const int lcols = (kD == 64 ? 6 : 7) - (31 - __clz(split)), cols = 1 << lcols, me = part_of_keys;
         const int pitch = cols * 4 + 16;  // bytes between received rows: spreads a warp's 16-byte stores over the banks
         const int row = s * kM + m;
         if (n_tiles > 0) {
@@ -926,9 +974,9 @@ if constexpr (kRope) {
           }
 #pragma unroll
           for (int j = 0; j < 32; j += 4) {
-            const int to = (cc * 32 + j) / cols;
+            const int to = (cc * 32 + j) >> lcols;
             if (to != me)
-              st_cluster(from_me + (uint32_t)((slot_of(me, to) * 2 * kM + row) * pitch + ((cc * 32 + j) % cols) * 4), to,
+              st_cluster(from_me + (uint32_t)((slot_of(me, to) * 2 * kM + row) * pitch + ((cc * 32 + j) & (cols - 1)) * 4), to,
                          o[j], o[j + 1], o[j + 2], o[j + 3]);
           }
         }
@@ -938,17 +986,20 @@ if constexpr (kRope) {
             st_cluster(stats + (uint32_t)((slot_of(me, to) * 2 * kM + row) * 16), to, __float_as_uint(m_run),
                        __float_as_uint(l_run), 0u, 0u);
         cluster_barrier();
-        float m_all = m_run;
-        for (int i = 0; i < split - 1; ++i)
-          m_all = fmaxf(m_all, *reinterpret_cast<const float*>(smem + kOffQ + (split - 1) * 2 * kM * pitch +
-                                                               (i * 2 * kM + row) * 16));
+        const uint8_t* got_stats = smem + kOffQ + (split - 1) * 2 * kM * pitch + row * 16;
+        float f_of[7], m_all = m_run, l_all;  // the others' maxima, then their factors
+#pragma unroll
+        for (int i = 0; i < 7; ++i) {
+          f_of[i] = i < split - 1 ? *reinterpret_cast<const float*>(got_stats + i * 2 * kM * 16) : -INFINITY;
+          m_all = fmaxf(m_all, f_of[i]);
+        }
         const float m_use = m_all == -INFINITY ? 0.f : m_all;
         const float f_me = ex2(m_run - m_use);
-        float l_all = l_run * f_me;
-        for (int i = 0; i < split - 1; ++i) {
-          const float2 ml = *reinterpret_cast<const float2*>(smem + kOffQ + (split - 1) * 2 * kM * pitch +
-                                                             (i * 2 * kM + row) * 16);
-          l_all += ml.y * ex2(ml.x - m_use);
+        l_all = l_run * f_me;
+#pragma unroll
+        for (int i = 0; i < 7; ++i) {
+          f_of[i] = ex2(f_of[i] - m_use);
+          if (i < split - 1) l_all += f_of[i] * *reinterpret_cast<const float*>(got_stats + i * 2 * kM * 16 + 4);
         }
         const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
         __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.o_out) + (int64_t)b * p.os.batch + (int64_t)slot * p.os.token +
@@ -961,16 +1012,17 @@ if constexpr (kRope) {
             tmem_wait_ld();
           }
 #pragma unroll
-          for (int j = 0; j < 8; ++j) acc[j] = n_tiles > 0 ? __uint_as_float(o[j]) * f_me : 0.f;
-          for (int i = 0; i < split - 1; ++i) {
-            const uint8_t* base = smem + kOffQ + (split - 1) * 2 * kM * pitch;
-            const float f = ex2(*reinterpret_cast<const float*>(base + (i * 2 * kM + row) * 16) - m_use);
-            const float4* src = reinterpret_cast<const float4*>(smem + kOffQ + (i * 2 * kM + row) * pitch + c0 * 4);
-            const float4 a = src[0], d = src[1];
-            acc[0] = fmaf(a.x, f, acc[0]); acc[1] = fmaf(a.y, f, acc[1]);
-            acc[2] = fmaf(a.z, f, acc[2]); acc[3] = fmaf(a.w, f, acc[3]);
-            acc[4] = fmaf(d.x, f, acc[4]); acc[5] = fmaf(d.y, f, acc[5]);
-            acc[6] = fmaf(d.z, f, acc[6]); acc[7] = fmaf(d.w, f, acc[7]);
+          for (int j = 0; j < 8; ++j) acc[j] = __uint_as_float(o[j]) * f_me;
+#pragma unroll
+          for (int i = 0; i < 7; ++i) {
+            if (i < split - 1) {
+              const float4* src = reinterpret_cast<const float4*>(smem + kOffQ + (i * 2 * kM + row) * pitch + c0 * 4);
+              const float4 a = src[0], d = src[1];
+              acc[0] = fmaf(a.x, f_of[i], acc[0]); acc[1] = fmaf(a.y, f_of[i], acc[1]);
+              acc[2] = fmaf(a.z, f_of[i], acc[2]); acc[3] = fmaf(a.w, f_of[i], acc[3]);
+              acc[4] = fmaf(d.x, f_of[i], acc[4]); acc[5] = fmaf(d.y, f_of[i], acc[5]);
+              acc[6] = fmaf(d.z, f_of[i], acc[6]); acc[7] = fmaf(d.w, f_of[i], acc[7]);
+            }
           }
           if (row_ok) {
             uint4 val;
