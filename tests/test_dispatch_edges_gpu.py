@@ -44,6 +44,23 @@ def test_head_dim_64_warps_at_different_speeds(gu):
     plan.destroy()
 
 
+def test_head_dim_64_partials_with_cold_caches(gu):
+    """Shards of more than one tile, written out while the products of the last two tiles may be under way."""
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload("d64_cold", 1, 300, 700, 4, 4, 64, "bf16", "random", "random", 3, 5, seed=1000, q_pos_offset=400,
+                         symmetric=False)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    u, m, e = oracle.attn_pass(w.q, w.k, w.v, w.scale, gu.oracle_plan(w))
+    flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
+    for i in range(20):
+        flush.fill_(i)
+        parts = cb.cascade_attn_partials(plan, q, k, v, w.scale)
+        gu.check_partials(tuple(t.double().cpu().numpy() for t in parts), (u, m, e), w.tol, f"run {i}")
+    assert plan.device_status() == 0
+    plan.destroy()
+
+
 def test_head_dim_64_without_a_workspace_takes_the_alu_kernel(gu):
     from paper_2507_05228_b200 import binding as cb
     w = wl.make_workload("d64_nows", 1, 200, 200, 8, 2, 64, "bf16", "random", "random", 3, 3, seed=7)
