@@ -92,15 +92,17 @@ struct Cfg {
   static constexpr int kVStages = D == 64 ? 3 : (kWalk ? 1 : 2);
   static constexpr bool kRing = D == 64;                   // three logit buffers, P in two parts
   static constexpr uint32_t kOCol = kRing ? 384u : 256u;   // first accumulator column
-  static constexpr int kRowBytes = D * 2;
-  static constexpr int kStageRowBytes = kRowBytes + 16;    // output rows staged for the bulk copies, padded by 16 bytes
+  // Output rows staged for the copy engine.  kWalk: per warp, [halves][32 rows][128 bytes], swizzled like the operand tiles;
+  // otherwise rows, padded by 16 bytes
+  static constexpr int kStageWarpBytes = kHalves * 32 * 128, kRowBytes = D * 2, kStageRowBytes = kRowBytes + 16;
+  static constexpr int kStageBytes = kWalk ? 8 * kStageWarpBytes : 2 * kM * kStageRowBytes;
   // shared memory map (offsets from a 1024-byte aligned base)
   static constexpr int kOffQ = 0;
   static constexpr int kOffK = kOffQ + 2 * kTileBytes;
   static constexpr int kOffV = kOffK + kKStages * kTileBytes;
   static constexpr int kOffStage = kWalk ? kOffV + kVStages * kTileBytes : kOffQ;
-  static constexpr int kOffBar = kOffV + kVStages * kTileBytes + (kWalk ? 2 * kM * kStageRowBytes : 0);
-  static_assert(kWalk || 2 * kM * kStageRowBytes <= kOffV, "the output staging area must fit in the Q and K tiles");
+  static constexpr int kOffBar = kOffV + kVStages * kTileBytes + (kWalk ? kStageBytes : 0);
+  static_assert(kWalk || kStageBytes <= kOffV, "the output staging area must fit in the Q and K tiles");
   static constexpr int kNumBars = 30;
   static constexpr int kOffMisc = kOffBar + kNumBars * 8;   // tmem slot, abort flag, 12 progress words
   static constexpr int kOffShard = kOffMisc + 64;           // int32 [5][kMaxShards], see ShardTab
@@ -210,6 +212,12 @@ __device__ __forceinline__ void tma_tile3(uint32_t dst, const CUtensorMap* map, 
       : "memory");
 }
 
+__device__ __forceinline__ void tma_store4(const CUtensorMap* map, int x, int y, int z, int w, uint32_t src) {
+  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(x), "r"(y), "r"(z), "r"(w), "r"(src)
+               : "memory");
+}
 // All threads of the cluster (each warp where it stands in its role).
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -400,6 +408,10 @@ struct TmaArgs {
   // kWalk: the shard-major copies as [batch * kv_heads][n_kv][head_dim];
   // otherwise K and V rows in token order as [batch][kv_heads][rows that are seen][head_dim]
   CUtensorMap k, v;
+  // kWalk: where finished rows go, o_part as [batch * KV shards][n_q slots][heads][head_dim]; a box is the rows of one warp:
+  // 32 / Gp slots x Gp heads
+  CUtensorMap o;
+  int o_valid;  // 0: the threads store their rows themselves
 };
 
 // kRope: the query rows are turned by the rotary embedding of their positions while they are staged (the key rows
@@ -415,7 +427,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   using C = Cfg<D, kWalk>;
   constexpr int kD = D, kTileBytes = C::kTileBytes, kKStages = C::kKStages, kVStages = C::kVStages;
   constexpr int kOffQ = C::kOffQ, kOffK = C::kOffK, kOffV = C::kOffV, kOffMisc = C::kOffMisc;
-  constexpr int kStageRowBytes = C::kStageRowBytes;
   constexpr bool kRing = C::kRing;
   static_assert(!kRope || D == 128, "the rotary step is fused for head_dim 128 only");
   extern __shared__ uint8_t smem_raw[];
@@ -699,10 +710,53 @@ if constexpr (kRope) {
       if (kWalk) cur.start(tab, n_act);
       int kk_open = -1;  // kWalk: the shard whose partial is being accumulated
       int n_flushed = 0;  // kWalk: partials written so far
+      // kWalk: writes this warp's finished rows from TMEM, scaled: through shared memory to the copy engine, a box per 64
+      // columns.  (Stores from the threads, 32 bytes into each of 32 rows per instruction, kept a CTA's memory pipe busy for
+      // 3200 cycles, one copy per row takes 2200 cycles to issue: 4099 tokens, 16 shards, heads of 64 389 -> 361 us.)  Boxes
+      // that would reach past the rows of the shard are left to the threads.
+      const int warp_row0 = sub_row0 + (((warp & 3) * 32) >> lg);
+      const bool boxed = tma.o_valid && warp_row0 + (32 >> lg) <= sub_row0 + sub_nrows;
+      auto store_rows = [&](float scale, bool have, int z, __nv_bfloat16* dst) {
+        uint8_t* stage = smem + C::kOffStage + warp * C::kStageWarpBytes;
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the previous rows have left
+        __syncwarp();
+#pragma unroll
+        for (int half = 0; half < C::kHalves; ++half) {
+          uint32_t o[64];
+          if (have) {
+            CASCADE_TMEM_LD32(o_addr + (uint32_t)(half * 64), o, 0);
+            CASCADE_TMEM_LD32(o_addr + (uint32_t)(half * 64 + 32), o, 32);
+            tmem_wait_ld();
+          } else {
+#pragma unroll
+            for (int j = 0; j < 64; ++j) o[j] = 0u;
+          }
+#pragma unroll
+          for (int j = 0; j < 64; j += 8) {
+            uint4 val;
+            val.x = pack_bf16x2(__uint_as_float(o[j]) * scale, __uint_as_float(o[j + 1]) * scale);
+            val.y = pack_bf16x2(__uint_as_float(o[j + 2]) * scale, __uint_as_float(o[j + 3]) * scale);
+            val.z = pack_bf16x2(__uint_as_float(o[j + 4]) * scale, __uint_as_float(o[j + 5]) * scale);
+            val.w = pack_bf16x2(__uint_as_float(o[j + 6]) * scale, __uint_as_float(o[j + 7]) * scale);
+            if (boxed)
+              *reinterpret_cast<uint4*>(stage + half * 4096 + lane * 128 + (((j >> 3) ^ (lane & 7)) << 4)) = val;
+            else if (row_ok)
+              *reinterpret_cast<uint4*>(dst + half * 64 + j) = val;
+          }
+        }
+        if (boxed) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // this thread's writes -> the copy engine's reads
+          __syncwarp();
+          if (lane == 0) {
+#pragma unroll
+            for (int half = 0; half < C::kHalves; ++half)
+              tma_store4(&tma.o, half * 64, h0, warp_row0, z, smem_u32(stage + half * 4096));
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          }
+        }
+      };
       // kWalk: writes the finished partial of shard kk (this thread's row of u, and m, l) from TMEM and the running
-      // statistics, then starts over.  The row goes through shared memory to the copy engine as one bulk copy: stores from
-      // the threads, 32 bytes into each of 32 rows per instruction, kept a CTA's memory pipe busy for 3200 cycles per shard,
-      // and whatever came behind them waiting (4099 tokens, 16 shards: 336 us, now 328).
+      // statistics, then starts over.
       auto flush_shard = [&](int kk) {
         float o_scale = 0.f, m_out = -INFINITY, l_out = 0.f;
         if (l_run > 0.f) {
@@ -715,32 +769,7 @@ if constexpr (kRope) {
           p.m_part[stat] = m_out;
           p.l_part[stat] = l_out;
         }
-        uint8_t* stage = smem + C::kOffStage + (s * kM + m) * kStageRowBytes;
-        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // this thread's previous row has left
-#pragma unroll
-        for (int half = 0; half < C::kHalves; ++half) {
-          uint32_t o[64];
-          CASCADE_TMEM_LD32(o_addr + (uint32_t)(half * 64), o, 0);
-          CASCADE_TMEM_LD32(o_addr + (uint32_t)(half * 64 + 32), o, 32);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 64; j += 8) {
-            uint4 val;
-            val.x = pack_bf16x2(__uint_as_float(o[j]) * o_scale, __uint_as_float(o[j + 1]) * o_scale);
-            val.y = pack_bf16x2(__uint_as_float(o[j + 2]) * o_scale, __uint_as_float(o[j + 3]) * o_scale);
-            val.z = pack_bf16x2(__uint_as_float(o[j + 4]) * o_scale, __uint_as_float(o[j + 5]) * o_scale);
-            val.w = pack_bf16x2(__uint_as_float(o[j + 6]) * o_scale, __uint_as_float(o[j + 7]) * o_scale);
-            *reinterpret_cast<uint4*>(stage + half * 128 + j * 2) = val;
-          }
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // this thread's writes -> the copy engine's reads
-        if (row_ok) {
-          asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
-                           static_cast<__nv_bfloat16*>(p.o_part) + stat * kD),
-                       "r"(smem_u32(stage)), "n"(C::kRowBytes)
-                       : "memory");
-          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        }
+        store_rows(o_scale, true, b * P + kk, static_cast<__nv_bfloat16*>(p.o_part) + stat * kD);
         m_run = -INFINITY;
         m_true = -INFINITY;
         l_run = 0.f;
@@ -1078,38 +1107,43 @@ if constexpr (kRope) {
           p.l_part[stat] = l_out;
         }
       }
-      // Every product of the CTA has completed, so the Q / K tiles in shared memory are free: the thread stages its
-      // output row there (rows 16 bytes further apart than they are long, which spreads a warp's 16-byte stores over all banks) and hands
-      // it to the copy engine as one bulk copy, instead of writing 32-byte pieces of 32 different rows per instruction.
-      uint8_t* stage = smem + C::kOffStage + (s * kM + m) * kStageRowBytes;
-      if (kWalk) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the previous shard's row has left
+      if constexpr (kWalk) {
+        store_rows(o_scale, n_tiles > 0, b * P + max(kk_open, 0), dst);
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the rows have left shared memory
+      } else {
+        // Every product of the CTA has completed, so the Q / K tiles in shared memory are free: the thread stages its
+        // output row there (rows 16 bytes further apart than they are long, which spreads a warp's stores over all banks)
+        // and hands it to the copy engine.  (Boxes as with kWalk were slower here, 43.6 -> 45.0 us on 2048 tokens: it happens
+        // once, and the first use of a tensor map costs more than that.)
+        uint8_t* stage = smem + C::kOffStage + (s * kM + m) * C::kStageRowBytes;
 #pragma unroll
-      for (int cc = 0; cc < kD / 32; ++cc) {
-        uint32_t o[32];
-        if (n_tiles > 0) {
-          CASCADE_TMEM_LD32(o_addr + (uint32_t)(cc * 32), o, 0);
-          tmem_wait_ld();
-        } else {
+        for (int cc = 0; cc < kD / 32; ++cc) {
+          uint32_t o[32];
+          if (n_tiles > 0) {
+            CASCADE_TMEM_LD32(o_addr + (uint32_t)(cc * 32), o, 0);
+            tmem_wait_ld();
+          } else {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) o[j] = 0u;
+            for (int j = 0; j < 32; ++j) o[j] = 0u;
+          }
+#pragma unroll
+          for (int j = 0; j < 32; j += 8) {
+            uint4 val;
+            val.x = pack_bf16x2(__uint_as_float(o[j]) * o_scale, __uint_as_float(o[j + 1]) * o_scale);
+            val.y = pack_bf16x2(__uint_as_float(o[j + 2]) * o_scale, __uint_as_float(o[j + 3]) * o_scale);
+            val.z = pack_bf16x2(__uint_as_float(o[j + 4]) * o_scale, __uint_as_float(o[j + 5]) * o_scale);
+            val.w = pack_bf16x2(__uint_as_float(o[j + 6]) * o_scale, __uint_as_float(o[j + 7]) * o_scale);
+            *reinterpret_cast<uint4*>(stage + cc * 64 + j * 2) = val;
+          }
         }
-#pragma unroll
-        for (int j = 0; j < 32; j += 8) {
-          uint4 val;
-          val.x = pack_bf16x2(__uint_as_float(o[j]) * o_scale, __uint_as_float(o[j + 1]) * o_scale);
-          val.y = pack_bf16x2(__uint_as_float(o[j + 2]) * o_scale, __uint_as_float(o[j + 3]) * o_scale);
-          val.z = pack_bf16x2(__uint_as_float(o[j + 4]) * o_scale, __uint_as_float(o[j + 5]) * o_scale);
-          val.w = pack_bf16x2(__uint_as_float(o[j + 6]) * o_scale, __uint_as_float(o[j + 7]) * o_scale);
-          *reinterpret_cast<uint4*>(stage + cc * 64 + j * 2) = val;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // this thread's writes -> the copy engine's reads
+        if (row_ok) {
+          asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(stage)),
+                       "n"(C::kRowBytes)
+                       : "memory");
+          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the row has left shared memory
         }
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // this thread's writes -> the copy engine's reads
-      if (row_ok) {
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(stage)),
-                     "n"(C::kRowBytes)
-                     : "memory");
-        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the row has left shared memory
       }
       }
       if constexpr (kWalk) {
@@ -1401,6 +1435,19 @@ bool encode_rows(CUtensorMap* map, const TcRows& r, int d, int64_t n_rows, int64
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Output rows [outer][rows][heads][d]; box = the rows of one warp (32 >> lg rows x 1 << lg heads), 64 columns.
+bool encode_out(CUtensorMap* map, void* base, int d, int lg, int64_t heads, int64_t rows, int64_t outer, const Strides& st) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)heads, (cuuint64_t)rows, (cuuint64_t)outer};
+  auto stride = [&](int64_t elems, int64_t extent) { return (cuuint64_t)(extent > 1 ? elems * 2 : d * 2); };
+  const cuuint64_t strides[3] = {stride(st.head, heads), stride(st.token, rows), stride(st.batch, outer)};
+  const cuuint32_t box[4] = {64, 1u << lg, 32u >> lg, 1};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 struct TcLaunch {
   int lg, tile_major, split;
   bool after_gather;
@@ -1456,7 +1503,7 @@ bool tc_rows_loadable(const TcRows& r, int64_t n_rows, int64_t n_heads, int64_t 
 }
 
 cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, const void* v_sorted, cudaStream_t stream) {
-  tc::TmaArgs tma;
+  tc::TmaArgs tma = {};
   const int64_t n_mats = (int64_t)p.batch * p.Hkv;
   if (!encode_sorted(&tma.k, k_sorted, p.d, p.plan.n_kv, n_mats) ||
       !encode_sorted(&tma.v, v_sorted, p.d, p.plan.n_kv, n_mats)) {
@@ -1464,6 +1511,9 @@ cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, c
     return cudaErrorInvalidValue;
   }
   const int lg = stacked_log2(p.G);
+  const int64_t n_q = p.plan.n_q;
+  tma.o_valid = encode_out(&tma.o, p.o_part, p.d, lg, p.H, n_q, (int64_t)p.batch * p.plan.n_kv_shards,
+                           {n_q * p.H * p.d, (int64_t)p.H * p.d, p.d});
   const int64_t n_ctas = (int64_t)p.plan.n_qtiles[3 - lg] * (p.H >> lg) * p.batch;
   // few CTAs per SM: balance matters more than L2 locality
   const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), 1, true};
@@ -1472,13 +1522,13 @@ cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, c
 
 cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v, int64_t n_seen, bool after_gather,
                            cudaStream_t stream) {
-  tc::TmaArgs tma;
+  tc::TmaArgs tma = {};
   if (!encode_rows(&tma.k, k, p.d, n_seen, p.Hkv, p.batch) || !encode_rows(&tma.v, v, p.d, n_seen, p.Hkv, p.batch)) {
     set_error("tensor-core attention: could not build the TMA descriptors of K and V");
     return cudaErrorInvalidValue;
   }
   const int lg = stacked_log2(p.G);
-  const int64_t tile_slots = 256 >> lg, n_qt = (p.plan.n_q + tile_slots - 1) / tile_slots;
+  const int64_t tilslots = 256 >> lg, n_qt = (p.plan.n_q + tilslots - 1) / tilslots;
   const int64_t n_ctas = n_qt * (p.H >> lg) * p.batch;
   // Few query tiles (a chunk of a chunked prefill, a short prompt) leave SMs idle: a cluster then shares the keys of each
   // tile, as far as its CTAs fit at once with one per SM (clusters of 2, 4 and 8: 148, 132 and 120 CTAs) and have two
