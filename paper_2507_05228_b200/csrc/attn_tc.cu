@@ -1112,9 +1112,9 @@ if constexpr (kRope) {
         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the rows have left shared memory
       } else {
         // Every product of the CTA has completed, so the Q / K tiles in shared memory are free: the thread stages its
-        // output row there (rows 16 bytes further apart than they are long, which spreads a warp's stores over all banks)
-        // and hands it to the copy engine.  (Boxes as with kWalk were slower here, 43.6 -> 45.0 us on 2048 tokens: it happens
-        // once, and the first use of a tensor map costs more than that.)
+        // output row there (rows 16 bytes further apart than they are long, which spreads a warp's accesses over all banks)
+        // and the warp stores whole rows, 512 bytes per instruction.  (A bulk copy per row took 2200 cycles to issue; boxes as
+        // with kWalk are issued once here, and the first use of a tensor map costs more: 2048 tokens 43.6 -> 45.0 us.)
         uint8_t* stage = smem + C::kOffStage + (s * kM + m) * C::kStageRowBytes;
 #pragma unroll
         for (int cc = 0; cc < kD / 32; ++cc) {
@@ -1136,13 +1136,16 @@ if constexpr (kRope) {
             *reinterpret_cast<uint4*>(stage + cc * 64 + j * 2) = val;
           }
         }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // this thread's writes -> the copy engine's reads
-        if (row_ok) {
-          asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(stage)),
-                       "n"(C::kRowBytes)
-                       : "memory");
-          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-          asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the row has left shared memory
+        __syncwarp();
+        const uint64_t dst_or_null = reinterpret_cast<uint64_t>(dst);  // null past the end of the sub-tile
+        constexpr int kLanesPerRow = C::kRowBytes / 16, kRowsAtOnce = 32 / kLanesPerRow;
+        const uint8_t* rows = smem + C::kOffStage + (s * kM + m - lane) * C::kStageRowBytes + (lane % kLanesPerRow) * 16;
+#pragma unroll
+        for (int r0 = 0; r0 < 32; r0 += kRowsAtOnce) {
+          const int r = r0 + lane / kLanesPerRow;
+          const uint64_t to = __shfl_sync(0xffffffffu, dst_or_null, r);
+          const uint4 val = *reinterpret_cast<const uint4*>(rows + r * C::kStageRowBytes);
+          if (to) *reinterpret_cast<uint4*>(to + (lane % kLanesPerRow) * 16) = val;
         }
       }
       }
