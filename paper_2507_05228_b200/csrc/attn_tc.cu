@@ -422,7 +422,7 @@ struct TmaArgs {
 // the barriers and the K/V pipelines are set up once per query tile instead of once per (query tile, KV shard).
 template <int D, bool kRope, bool kWalk>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_constant__ AttnParams p, int lg,
-                                                              int tile_major, int split,
+                                                              int tile_major, int split, int early,
                                                               const __grid_constant__ TmaArgs tma) {
   using C = Cfg<D, kWalk>;
   constexpr int kD = D, kTileBytes = C::kTileBytes, kKStages = C::kKStages, kVStages = C::kVStages;
@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     if (lane == 0) progress[warp] = v;
   };
 
-  if (tid == 0) {
+  if (tid == 9 * 32) {
     mbar_init(bar(Q_FULL), 128);  // every thread of the sub-tile's softmax group brings a share of the rows
     mbar_init(bar(Q_FULL + 1), 128);
     for (int s = 0; s < kKStages; ++s) {
@@ -619,6 +619,23 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     *abort_flag = 0;
     for (int w = 0; w < kThreads / 32; ++w) progress[w] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if constexpr (!kWalk) {
+      // early (bit 0: K, bit 1: V; not what a gather in front of this grid writes): the first tile is requested here, under
+      // the query rows and the rest of the set-up, instead of after them
+      const int tiles = early ? (seen_by(row0 + nrows - 1) + kNMax - 1) / kNMax : 0;
+      const int t0 = tiles * part_of_keys / split;
+      if (tiles * (part_of_keys + 1) / split > t0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        for (int kv = 0; kv < 2; ++kv)
+          if ((early >> kv) & 1) {
+            const CUtensorMap* map = kv == 0 ? &tma.k : &tma.v;
+            const uint32_t dst = smem_base + (kv == 0 ? kOffK : kOffV), fb = bar(kv == 0 ? K_FULL : V_FULL);
+            mbar_expect_tx(fb, (uint32_t)kTileBytes);
+            tma_tile4(dst, map, 0, t0 * kNMax, g, b, fb);
+            if (C::kHalves == 2) tma_tile4(dst + (uint32_t)kHalfBytes, map, 64, t0 * kNMax, g, b, fb);
+          }
+      }
+    }
   }
   if (warp == 8) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -1347,7 +1364,7 @@ if constexpr (kRope) {
               }
               cur.advance(tab, n_act);
             }
-          } else if (leader) {
+          } else if (leader && !(i == 0 && ((early >> lw) & 1))) {
             // 128 rows at a time; rows past what any query sees lie outside the tensor map and are zero-filled, so that
             // whatever the unwritten tail of a cache holds stays out of the products
             mbar_expect_tx(fb, (uint32_t)kTileBytes);
@@ -1452,7 +1469,7 @@ bool encode_out(CUtensorMap* map, void* base, int d, int lg, int64_t heads, int6
 }
 
 struct TcLaunch {
-  int lg, tile_major, split;
+  int lg, tile_major, split, early;
   bool after_gather;
 };
 
@@ -1486,7 +1503,7 @@ cudaError_t launch_kernel(const AttnParams& p, bool walk, const TcLaunch& l, int
     attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
   }
-  e = cudaLaunchKernelEx(&cfg, kernel, p, l.lg, l.tile_major, l.split, tma);
+  e = cudaLaunchKernelEx(&cfg, kernel, p, l.lg, l.tile_major, l.split, l.early, tma);
   count_launch();
   return e;
 }
@@ -1519,11 +1536,11 @@ cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, c
                            {n_q * p.H * p.d, (int64_t)p.H * p.d, p.d});
   const int64_t n_ctas = (int64_t)p.plan.n_qtiles[3 - lg] * (p.H >> lg) * p.batch;
   // few CTAs per SM: balance matters more than L2 locality
-  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), 1, true};
+  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), 1, 0, true};
   return launch_kernel(p, true, l, n_ctas, tma, stream);
 }
 
-cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v, int64_t n_seen, bool after_gather,
+cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v, int64_t n_seen, bool k_gathered, bool v_gathered,
                            cudaStream_t stream) {
   tc::TmaArgs tma = {};
   if (!encode_rows(&tma.k, k, p.d, n_seen, p.Hkv, p.batch) || !encode_rows(&tma.v, v, p.d, n_seen, p.Hkv, p.batch)) {
@@ -1543,7 +1560,8 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
     for (int i = 1; i < 4; ++i)
       if (rule_ctas << i <= fit[i] && key_tiles >= 2 << i) split = 1 << i;
   }
-  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), split, after_gather};
+  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), split,
+                      p.prefix_from_vis ? 0 : (k_gathered ? 0 : 1) | (v_gathered ? 0 : 2), k_gathered || v_gathered};
   return launch_kernel(p, false, l, n_ctas, tma, stream);
 }
 

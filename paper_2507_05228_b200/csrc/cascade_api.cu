@@ -754,23 +754,24 @@ static cascade_status_t run_tc(AttnParams p, const char* fn, const cascade_plan_
   TcRows k = {p.k, p.ks}, v = {p.v, p.vs};
   const Strides dense = {(int64_t)p.Hkv * d.n_kv * p.d, p.d, (int64_t)d.n_kv * p.d};
   const bool v_fits = tc_rows_loadable(v, n_seen, p.Hkv, p.batch);
-  bool gathered = false;
+  bool k_gathered = false, v_gathered = false;
   if (p.rope) {
     // the rotated keys: in token order for the kernel, and shard-major with the values, as the call leaves them behind
     *launch_error = launch_gather_kv(p, ws, ws + each, ws + 2 * each, false, !v_fits, st);
     k = {ws + 2 * each, dense};
-    if (!v_fits) v = {ws + each, dense};
-    gathered = true;
+    k_gathered = true;
+    v_gathered = !v_fits;
+    if (v_gathered) v = {ws + each, dense};
   } else if (!v_fits || !tc_rows_loadable(k, n_seen, p.Hkv, p.batch) || (p.prefix_from_vis && d.n_maps > 1)) {
     // strides that a tensor map cannot hold (an expanded axis), or a different last visible row per sequence
     *launch_error = launch_gather_kv(p, ws, ws + each, nullptr, true, true, st);
     k = {ws, dense};
     v = {ws + each, dense};
-    gathered = true;
+    k_gathered = v_gathered = true;
   } else {
     *launch_error = cudaSuccess;
   }
-  if (*launch_error == cudaSuccess) *launch_error = launch_attn_tc(p, k, v, n_seen, gathered, st);
+  if (*launch_error == cudaSuccess) *launch_error = launch_attn_tc(p, k, v, n_seen, k_gathered, v_gathered, st);
   return CASCADE_OK;
 }
 

@@ -154,9 +154,10 @@ struct TcRows {
   Strides strides;
 };
 bool tc_rows_loadable(const TcRows& r, int64_t n_rows, int64_t n_heads, int64_t batch);
-// all keys of a query in one go, K and V in token order; rows from n_seen on are not looked at
-cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v, int64_t n_seen, bool after_gather,
-                           cudaStream_t stream);
+// all keys of a query in one go, K and V in token order; rows from n_seen on are not looked at; k_gathered / v_gathered: the
+// rows are written by a gather launched just before
+cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v, int64_t n_seen, bool k_gathered,
+                           bool v_gathered, cudaStream_t stream);
 // the partials of every KV shard; k_sorted / v_sorted: shard-major copies, [batch][kv_head][n_kv][d] bf16
 cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, const void* v_sorted, cudaStream_t stream);
 // Copies of K and V for the above, [batch][kv_head][n_kv][d]: shard-major, or with token_order as the rows are.  With
