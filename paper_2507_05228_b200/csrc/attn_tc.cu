@@ -41,8 +41,9 @@
 //         cycles per SM; 16-byte cp.async: one 512-byte request per ~90 cycles per warp).  The two query
 //         sub-tiles are gathered once per CTA by the softmax threads themselves (plain 16-byte loads).
 //   11    works out the CTA's keys (kWalk: the table of the shards it sees anything of), then idles; it also keeps the register-reallocation groups of four warps whole.
-// After a gather the grid is launched as its programmatic dependent: everything up to the loaders' first TMA load
-// may run while the gather is still writing the shard-major copies (the loaders wait with griddepcontrol.wait).
+// The grid is launched as a programmatic dependent (partials: only after a gather).  After a gather everything up to the
+// loaders' first TMA load may run while the copies are still being written; otherwise the set-up of the block scheduler
+// and of the parameters overlaps the tail of whatever kernel comes before.
 // Every mbarrier wait is bounded: on expiry the CTA raises a flag, records a code in the plan's status word
 // and drains without waiting again.
 #include <cuda.h>
@@ -422,7 +423,7 @@ struct TmaArgs {
 // the barriers and the K/V pipelines are set up once per query tile instead of once per (query tile, KV shard).
 template <int D, bool kRope, bool kWalk>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_constant__ AttnParams p, int lg,
-                                                              int tile_major, int split, int early,
+                                                              int tile_major, int split, int early, int after_gather,
                                                               const __grid_constant__ TmaArgs tma) {
   using C = Cfg<D, kWalk>;
   constexpr int kD = D, kTileBytes = C::kTileBytes, kKStages = C::kKStages, kVStages = C::kVStages;
@@ -473,6 +474,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     hg = rem % n_hg;
     b = rem / n_hg;
   }
+  // A gather right before this grid runs after all that came before it, and writes only what the loaders read: they wait
+  // for it.
+  grid_go();
+  if (!after_gather) grid_wait();
   const int map = pl.n_maps == 1 ? 0 : b;
   const int h0 = hg * Gp;  // first of the Gp stacked heads
   const int g = h0 / p.G;  // their KV head
@@ -481,13 +486,19 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     const int4 qt = pl.qtiles[ts][(size_t)map * pl.n_qtiles[ts] + tile_idx];
     row0 = qt.x;
     nrows = qt.y;
-    if (nrows == 0) return;  // padding entry (uniform for the CTA)
+    if (nrows == 0) {  // padding entry (uniform for the CTA)
+      grid_wait();
+      return;
+    }
   } else {
     row0 = (n_qt - 1 - tile_idx) * 2 * R;
     nrows = min(2 * R, pl.n_q - row0);
   }
   // an earlier CTA gave up: do not pile on (a cluster stays whole, its waits end at once)
-  if (split == 1 && *reinterpret_cast<volatile int32_t*>(pl.status) != 0) return;
+  if (split == 1 && *reinterpret_cast<volatile int32_t*>(pl.status) != 0) {
+    grid_wait();
+    return;
+  }
   const int n_sub = nrows > R ? 2 : 1;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int32_t* q_idx = pl.q_idx + (size_t)map * pl.n_q;
@@ -1345,7 +1356,7 @@ if constexpr (kRope) {
         // The shard-major copies are written by the gather grid launched just before this one; when this grid was
         // launched as its programmatic dependent it may have started early, so wait here for that grid to complete
         // (a no-op otherwise).  Nothing else in this kernel reads what the gather grid writes.
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        grid_wait();
         for (int i = 0; i < n_tiles; ++i) {
           const int nch = kWalk ? min(4, cur.nc - cur.c) : tile_chunks(i);
           const int st = i % n_stages;
@@ -1381,6 +1392,7 @@ if constexpr (kRope) {
       cluster_barrier();
     }
   }
+  if (after_gather) grid_wait();
   __syncthreads();
   if (warp == 8) {
     tc_fence_after();
@@ -1484,28 +1496,8 @@ cudaError_t launch_kernel(const AttnParams& p, bool walk, const TcLaunch& l, int
   if (e != cudaSuccess) return e;
   if (n_ctas * l.split >= (int64_t)1 << 31) return cudaErrorInvalidConfiguration;
   TimedLaunch timed(stream);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(n_ctas * l.split));
-  cfg.blockDim = dim3(tc::kThreads);
-  cfg.dynamicSmemBytes = smem_bytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
-  cfg.attrs = attr;
-  if (l.split > 1) {
-    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
-    attr[cfg.numAttrs].val.clusterDim.x = l.split;
-    attr[cfg.numAttrs].val.clusterDim.y = 1;
-    attr[cfg.numAttrs++].val.clusterDim.z = 1;
-  }
-  // Programmatic dependent launch on the gather grid that precedes it in the stream: the set-up of the CTAs overlaps
-  // the gather's tail.  Not while kernel timing is recording: the event between the two launches must separate them.
-  if (l.after_gather && !timing_recording()) {
-    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
-  }
-  e = cudaLaunchKernelEx(&cfg, kernel, p, l.lg, l.tile_major, l.split, l.early, tma);
-  count_launch();
-  return e;
+  return launch_dependent(kernel, dim3((unsigned)(n_ctas * l.split)), tc::kThreads, smem_bytes, l.split,
+                          !walk || l.after_gather, stream, p, l.lg, l.tile_major, l.split, l.early, (int)l.after_gather, tma);
 }
 
 // stack as many of the G heads of a KV head into one MMA tile as divide G (at most 8)

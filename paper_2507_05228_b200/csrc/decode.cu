@@ -334,6 +334,8 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __
   const int32_t* kv_idx = pl.kv_idx + (size_t)map * pl.n_kv;
   const int32_t* kv_off = pl.kv_off + (size_t)map * (P + 1);
   const int32_t* vis = pl.vis + (size_t)map * P;  // one query row
+  grid_go();
+  grid_wait();
   const bool vis_given = step.n_vis > 0;          // the prefixes come with the launch (the plan's copy is written below)
 
   // step: the new token's rows go to the caches first, by warp 0 of the cluster's first CTA (two rotation pairs and four
@@ -519,18 +521,7 @@ static cudaError_t launch_fused(const AttnParams& p, const DecodeStep& step, int
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_cta, p.Hkv, p.batch);
-  cfg.blockDim = dim3(NW * 32);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = n_cta;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, p, step);
+  return launch_dependent(kernel, dim3(n_cta, p.Hkv, p.batch), NW * 32, 0, n_cta, true, stream, p, step);
 }
 
 // f(integral_constant G) for the group sizes the kernels are built for
@@ -555,9 +546,7 @@ cudaError_t launch_decode_fused(const AttnParams& p, const DecodeStep& step, int
   const int64_t most = pairs <= 7 ? kMaxCluster : 10;
   const int n_cta = (int)std::max<int64_t>(1, std::min(std::min(256 / pairs, most), (blocks + 7) / 8));
   TimedLaunch timed(stream);
-  const cudaError_t e = with_group(p.G, [&](auto g) { return launch_fused<decltype(g)::value>(p, step, n_cta, stream); });
-  count_launch();
-  return e;
+  return with_group(p.G, [&](auto g) { return launch_fused<decltype(g)::value>(p, step, n_cta, stream); });
 }
 
 cudaError_t launch_decode(const AttnParams& p, cudaStream_t stream) {
