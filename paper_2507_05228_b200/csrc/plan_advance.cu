@@ -34,6 +34,8 @@ __device__ __forceinline__ int32_t visible_prefix(const PlanDev& d, int32_t q_po
 // last the longest; both are searched for again here, so that one launch does everything: the launch is what costs).
 __global__ void plan_advance_kernel(PlanDev d, int32_t q_pos_offset, int32_t* __restrict__ vis,
                                     uint8_t* __restrict__ pair_class) {
+  grid_go();
+  grid_wait();
   const int J = d.n_q_shards, P = d.n_kv_shards;
   const int64_t n_vis = (int64_t)d.n_maps * d.n_q * P, n = n_vis + (int64_t)d.n_maps * J * P;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
@@ -66,6 +68,8 @@ struct PlanSetArgs {
 };
 __global__ void __launch_bounds__(kMaxGivenVis) plan_set_kernel(const __grid_constant__ PlanSetArgs a, int n_vis, int n_cls,
                                                                 int32_t* vis, uint8_t* pair_class) {
+  grid_go();
+  grid_wait();
   const int t = threadIdx.x;
   if (t < n_vis) vis[t] = a.vis[t];
   if (t < n_cls) pair_class[t] = a.pair_class[t];
@@ -78,20 +82,17 @@ cudaError_t launch_plan_set(const PlanDev& d, const int32_t* vis, int n_vis, con
   PlanSetArgs a;
   memcpy(a.vis, vis, (size_t)n_vis * 4);
   memcpy(a.pair_class, pair_class, (size_t)n_cls);
-  plan_set_kernel<<<1, kMaxGivenVis, 0, stream>>>(a, n_vis, n_cls, const_cast<int32_t*>(d.vis),
-                                                  const_cast<uint8_t*>(d.pair_class));
-  count_launch();
-  return cudaGetLastError();
+  return launch_dependent(plan_set_kernel, dim3(1), kMaxGivenVis, 0, 1, true, stream, a, n_vis, n_cls,
+                          const_cast<int32_t*>(d.vis), const_cast<uint8_t*>(d.pair_class));
 }
 
 cudaError_t launch_plan_advance(const PlanDev& d, int32_t q_pos_offset, cudaStream_t stream) {
   const int64_t n = (int64_t)d.n_maps * (d.n_q + d.n_q_shards) * d.n_kv_shards;
   const int threads = 256;
   const int blocks = (int)std::min<int64_t>((n + threads - 1) / threads, 8 * 1024);
-  plan_advance_kernel<<<blocks, threads, 0, stream>>>(d, q_pos_offset, const_cast<int32_t*>(d.vis),
-                                                      const_cast<uint8_t*>(d.pair_class));
-  count_launch();
-  return cudaGetLastError();
+  // a dependent too: the chain plan -> attention of a 512-token chunk at 8192 keys 70.3 -> 68.8 us back to back
+  return launch_dependent(plan_advance_kernel, dim3(blocks), threads, 0, 1, true, stream, d, q_pos_offset,
+                          const_cast<int32_t*>(d.vis), const_cast<uint8_t*>(d.pair_class));
 }
 
 }  // namespace cascade
