@@ -1361,7 +1361,9 @@ if constexpr (kRope) {
           const int nch = kWalk ? min(4, cur.nc - cur.c) : tile_chunks(i);
           const int st = i % n_stages;
           note(8 * i + 1);
-          wait_bar(wc, bar(empty0 + st), (uint32_t)(((i / n_stages) & 1) ^ 1), is_k ? 9 : 10, i);
+          // The first use of a stage waits for nothing, and must not: the products may have consumed a first tile that was
+          // requested early before this warp gets here, and a wait for the phase before that would never end.
+          if (i >= n_stages) wait_bar(wc, bar(empty0 + st), (uint32_t)(((i / n_stages) & 1) ^ 1), is_k ? 9 : 10, i);
           const uint32_t dst = tiles_s + (uint32_t)(st * kTileBytes), fb = bar(full0 + st);
           if constexpr (kWalk) {
             if (leader) mbar_expect_tx(fb, (uint32_t)(nch * C::kHalves * kChunkBytes));
