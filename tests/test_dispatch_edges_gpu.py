@@ -112,6 +112,22 @@ def test_new_plans_have_the_same_arrays_on_the_device(gu, n_q, n_kv, P, causal):
         plan.destroy()
 
 
+@pytest.mark.parametrize("n_q,n_kv,same,n_maps", [
+    (1, 1, True, 1), (333, 333, True, 2), (333, 333, False, 2), (65536, 65536, True, 1), (1, 65537, False, 1), (65537, 65537, True, 1)])
+def test_plan_lists_go_up_narrow_and_once(gu, n_q, n_kv, same, n_maps):
+    """Row ids travel as 16 bits up to 65536 rows and as 32 above, and once where both sides have the same lists."""
+    from paper_2507_05228_b200 import binding as cb
+    rng = np.random.default_rng(n_kv)
+    kv_of = rng.integers(0, 4, (n_maps, n_kv)).astype(np.int32)
+    q_of = kv_of if same else rng.integers(0, 4, (n_maps, n_q)).astype(np.int32)
+    plan = cb.cascade_shard_plan(q_of, kv_of, 4, 4, n_kv - n_q, True)
+    for mp in range(n_maps):
+        ref = oracle.shard_plan(q_of[mp], kv_of[mp], 4, 4, q_pos_offset=n_kv - n_q, causal=True)
+        for f in ("q_off", "q_idx", "q_inv", "kv_off", "kv_idx", "kv_inv", "vis", "pair_class"):
+            assert np.array_equal(gu.read_plan_device_array(plan, f)[mp], getattr(ref, f)), f
+    plan.destroy()
+
+
 @pytest.mark.parametrize("B,n_kv,H,Hkv,P,kv_map,pos", [
     (1, 1, 8, 8, 1, "random", 0),            # one key, one block: a single CTA per KV head
     (1, 129, 16, 2, 3, "contiguous", 64),    # two of three shards empty or cut: shard-after-shard order
