@@ -39,8 +39,11 @@
 //         wrote, where the visible prefix of a shard is a contiguous run of rows.  An index-mapped gather straight from
 //         the caller's tensors was far too slow for the K/V stream (measured: one 512-byte TMA row gather per ~36
 //         cycles per SM; 16-byte cp.async: one 512-byte request per ~90 cycles per warp).  The two query
-//         sub-tiles are gathered once per CTA by the softmax threads themselves (plain 16-byte loads).
-//   11    works out the CTA's keys (kWalk: the table of the shards it sees anything of), then idles; it also keeps the register-reallocation groups of four warps whole.
+//         sub-tiles come once per CTA, as boxes requested during the set-up; where their tokens are not consecutive (kWalk),
+//         where they are turned on the way (rotary step), or where their strides do not fit a tensor map, the softmax threads
+//         gather them themselves (plain 16-byte loads).
+//   11    works out the CTA's keys (kWalk: the table of the shards it sees anything of), then idles; it also keeps the
+//         register-reallocation groups of four warps whole.
 // The grid is launched as a programmatic dependent (partials: only after a gather).  After a gather everything up to the
 // loaders' first TMA load may run while the copies are still being written; otherwise the set-up of the block scheduler
 // and of the parameters overlaps the tail of whatever kernel comes before.
@@ -162,31 +165,47 @@ __device__ __forceinline__ bool elect_one() {  // true in exactly one lane of a 
   return pred != 0;
 }
 
+// The CTA's control words in shared memory: [1] abort flag, [2..] one progress word per warp (8 * tile + step, for the timeout
+// report).  By 32-bit shared address, which keeps registers free for the softmax loop (head_dim 64, 3001 tokens, 2
+// sequences: 78.7 -> 76.7 us); by pointer in the walk of the partials, where that is the faster code (421 -> 414 us on 4099 tokens in
+// 16 shards, with the post-pass).
+template <bool kPointer>
 struct WaitCtx {
-  volatile int* abort_flag;  // shared memory
-  volatile int* progress;    // shared memory, one word per warp: 8 * tile + step, for the timeout report
-  int32_t* status;           // global: [0] code, [1..3] block index, [4] tile of the waiter, [8..19] progress words
+  uint32_t misc;
+  volatile int* words;
+  int32_t* status;  // global: [0] code, [1..3] block index, [4] tile of the waiter, [8..19] progress words
+  __device__ __forceinline__ int load(int w) const {
+    if constexpr (kPointer) return words[w];
+    int v;
+    asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(v) : "r"(misc + 4 * w) : "memory");
+    return v;
+  }
+  __device__ __forceinline__ void store(int w, int v) const {
+    if constexpr (kPointer) words[w] = v;
+    else asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(misc + 4 * w), "r"(v) : "memory");
+  }
 };
 
 // Bounded wait: gives up after ~2 s, raises the CTA's abort flag and records `code`.
-__device__ __forceinline__ bool wait_bar(const WaitCtx& c, uint32_t bar, uint32_t parity, int code, int tile = 0) {
-  if (*c.abort_flag) return false;
+template <bool kPointer>
+__device__ __forceinline__ bool wait_bar(const WaitCtx<kPointer>& c, uint32_t bar, uint32_t parity, int code, int tile = 0) {
+  if (c.load(1)) return false;
   if (mbar_try_wait(bar, parity)) return true;
   uint64_t t0 = 0;
   uint32_t spins = 0;
   while (!mbar_try_wait(bar, parity)) {
     if ((++spins & 1023u) == 0) {
-      if (*c.abort_flag || *reinterpret_cast<volatile int32_t*>(c.status) != 0) return false;
+      if (c.load(1) || *reinterpret_cast<volatile int32_t*>(c.status) != 0) return false;
       const uint64_t now = global_timer_ns();
       if (t0 == 0) t0 = now;
       if (now - t0 > 2000000000ull) {
-        *c.abort_flag = 1;
+        c.store(1, 1);
         if (atomicCAS(c.status, 0, code) == 0) {  // first CTA to give up: leave a report
           c.status[1] = (int32_t)blockIdx.x;
           c.status[2] = (int32_t)blockIdx.y;
           c.status[3] = (int32_t)blockIdx.z;
           c.status[4] = tile;
-          for (int w = 0; w < kThreads / 32; ++w) c.status[8 + w] = c.progress[w];
+          for (int w = 0; w < kThreads / 32; ++w) c.status[8 + w] = c.load(2 + w);
         }
         return false;
       }
@@ -305,6 +324,10 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
         "r"(r[o + 30]), "r"(r[o + 31]), "r"(taddr)                                                              \
       : "memory")
 
+#define CASCADE_TMEM_ST8(taddr, r)                                                                             \
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"r"(r[0]),    \
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(taddr)         \
+               : "memory")
 #define CASCADE_TMEM_ST16(taddr, r)                                                                            \
   asm volatile(                                                                                                 \
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], "                                                          \
@@ -413,6 +436,10 @@ struct TmaArgs {
   // 32 / Gp slots x Gp heads
   CUtensorMap o;
   int o_valid;  // 0: the threads store their rows themselves
+  // Fused route without a rotary step: the query rows as [batch][tokens][heads][head_dim]; a box is one sub-tile, 128 / Gp
+  // tokens x Gp heads, 64 columns
+  int q_valid;  // 0: the threads load them
+  CUtensorMap q;
 };
 
 // kRope: the query rows are turned by the rotary embedding of their positions while they are staged (the key rows
@@ -443,8 +470,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   auto p_full = [&](int s, int i) { return bar(P_FULL + (kRing ? 2 * (i & 1) : 0) + s); };
   auto s_parity = [&](int i) { return (uint32_t)((kRing ? i >> 1 : i) & 1); };
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kOffMisc);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 4);
-  volatile int* progress = reinterpret_cast<volatile int*>(smem + kOffMisc + 8);  // [12]
   ShardTab* tab = reinterpret_cast<ShardTab*>(smem + C::kOffShard);
   volatile int* stream_info = reinterpret_cast<volatile int*>(smem + kOffMisc + 56);  // [0] active shards, [1] chunks
 
@@ -494,11 +519,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     row0 = (n_qt - 1 - tile_idx) * 2 * R;
     nrows = min(2 * R, pl.n_q - row0);
   }
-  // an earlier CTA gave up: do not pile on (a cluster stays whole, its waits end at once)
-  if (split == 1 && *reinterpret_cast<volatile int32_t*>(pl.status) != 0) {
-    grid_wait();
-    return;
-  }
   const int n_sub = nrows > R ? 2 : 1;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int32_t* q_idx = pl.q_idx + (size_t)map * pl.n_q;
@@ -528,7 +548,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   const int q_row = (tid & 127) / kRowChunks;
   const float4* rope_row[kRope ? 8 : 1];  // this thread's slice of the table row of each of its query rows
   float4 cs[kRope ? 4 : 1][4];            // (cos, sin) of four rows: 8 pairs each
-  if (warp < 8 && (warp >> 2) < n_sub) {
+  const bool q_boxes = !kWalk && !kRope && tma.q_valid;
+  if (!q_boxes && warp < 8 && (warp >> 2) < n_sub) {
     const int s = warp >> 2;
     const int sub_row0 = row0 + s * R;
     const int sub_nrows = min(R, nrows - s * R);
@@ -602,14 +623,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       if (lane == 1 || lane == 2) tab->first[lane - 1][0] = seen;
     }
   }
-  WaitCtx wc{abort_flag, progress, pl.status};
+  const WaitCtx<kWalk> wc{smem_base + (uint32_t)kOffMisc, reinterpret_cast<volatile int*>(smem + kOffMisc), pl.status};
   auto note = [&](int v) {
-    if (lane == 0) progress[warp] = v;
+    if (lane == 0) wc.store(2 + warp, v);
   };
 
   if (tid == 9 * 32) {
-    mbar_init(bar(Q_FULL), 128);  // every thread of the sub-tile's softmax group brings a share of the rows
-    mbar_init(bar(Q_FULL + 1), 128);
+    mbar_init(bar(Q_FULL), q_boxes ? 1 : 128);  // 128: every thread of the sub-tile's softmax group brings a share of the rows
+    mbar_init(bar(Q_FULL + 1), q_boxes ? 1 : 128);
     for (int s = 0; s < kKStages; ++s) {
       mbar_init(bar(K_FULL + s), 1);  // TMA: one arrival that announces the byte count, then the bytes
       mbar_init(bar(K_EMPTY + s), 1);
@@ -627,24 +648,32 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     mbar_init(bar(O_FULL), 1);
     mbar_init(bar(O_RDY), 1);
     mbar_init(bar(O_RDY + 1), 1);
-    *abort_flag = 0;
-    for (int w = 0; w < kThreads / 32; ++w) progress[w] = 0;
+    wc.store(1, 0);
+    for (int w = 0; w < kThreads / 32; ++w) wc.store(2 + w, 0);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if constexpr (!kWalk) {
-      // early (bit 0: K, bit 1: V; not what a gather in front of this grid writes): the first tile is requested here, under
-      // the query rows and the rest of the set-up, instead of after them
-      const int tiles = early ? (seen_by(row0 + nrows - 1) + kNMax - 1) / kNMax : 0;
+      // The query rows and the first tiles of K and V (early, bit 0: K, bit 1: V; not what a gather in front of this grid
+      // writes) are requested here, under the rest of the set-up.  (Query rows loaded by the softmax threads cost a CTA 2700
+      // cycles before its first product: 2048 tokens 40.3 -> 38.5 us, 2 x 3001 tokens of head_dim 64 78.2 -> 76.7.)
+      const int tiles = (seen_by(row0 + nrows - 1) + kNMax - 1) / kNMax;
       const int t0 = tiles * part_of_keys / split;
       if (tiles * (part_of_keys + 1) / split > t0) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        for (int kv = 0; kv < 2; ++kv)
-          if ((early >> kv) & 1) {
-            const CUtensorMap* map = kv == 0 ? &tma.k : &tma.v;
-            const uint32_t dst = smem_base + (kv == 0 ? kOffK : kOffV), fb = bar(kv == 0 ? K_FULL : V_FULL);
-            mbar_expect_tx(fb, (uint32_t)kTileBytes);
-            tma_tile4(dst, map, 0, t0 * kNMax, g, b, fb);
-            if (C::kHalves == 2) tma_tile4(dst + (uint32_t)kHalfBytes, map, 64, t0 * kNMax, g, b, fb);
-          }
+        auto request_q = [&](int s) {
+          mbar_expect_tx(bar(Q_FULL + s), (uint32_t)kTileBytes);
+          for (int half = 0; half < C::kHalves; ++half)
+            tma_tile4(smem_base + (uint32_t)(kOffQ + s * kTileBytes + half * kHalfBytes), &tma.q, 64 * half, h0, row0 + s * R, b,
+                      bar(Q_FULL + s));
+        };
+        auto request_kv = [&](const CUtensorMap* map, uint32_t dst, uint32_t fb) {
+          mbar_expect_tx(fb, (uint32_t)kTileBytes);
+          tma_tile4(dst, map, 0, t0 * kNMax, g, b, fb);
+          if (C::kHalves == 2) tma_tile4(dst + (uint32_t)kHalfBytes, map, 64, t0 * kNMax, g, b, fb);
+        };
+        if (q_boxes) request_q(0);
+        if (early & 1) request_kv(&tma.k, smem_base + kOffK, bar(K_FULL));
+        if (q_boxes && n_sub == 2) request_q(1);
+        if (early & 2) request_kv(&tma.v, smem_base + kOffV, bar(V_FULL));
       }
     }
   }
@@ -680,17 +709,20 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       const int head = h0 + (m & (Gp - 1));
       const int32_t* vis_row = vis + (size_t)(kWalk ? slot : 0) * P;
       const int32_t* vis_first = tab->first[s];  // shortest prefix of the sub-tile, per active shard (not kWalk: of all keys)
-      const int my_seen = (kWalk || !row_ok) ? 0 : seen_by(slot) - key0;
-      const int sub_seen = kWalk ? 0 : vis_first[0] - key0;
+      // not kWalk: tiles that end at or before `unmasked` need no mask; how many of the CTA's keys this row sees is kept in
+      // shared memory (unused columns of the shard table) for the others
+      const int unmasked = kWalk ? 0 : min(vis_first[0] - key0, n_keys);
+      volatile int* const my_seen = tab->kk + s * kM + m;
+      if constexpr (!kWalk) *my_seen = row_ok ? seen_by(slot) - key0 : 0;
       const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
       uint32_t s_addr = lane_base + (uint32_t)(s * 128);  // kRing: the buffer of the current tile
-      const uint32_t o_addr = lane_base + C::kOCol + (uint32_t)(s * kD);
+      const uint32_t o_addr = kRing ? lane_base + C::kOCol + (uint32_t)(s * kD) : s_addr + C::kOCol;
       const float c = p.scale * 1.4426950408889634f;  // logits are kept in log2 units: x = s * scale * log2(e)
       const uint64_t c2 = pack2(c, c);
       float m_run = -INFINITY;   // reference max the accumulators are scaled by (may lag by < 2^8)
       float m_true = -INFINITY;  // exact running max
       float l_run = 0.f;
-      if (n_tiles > 0) {
+      if (n_tiles > 0 && !q_boxes) {
 if constexpr (kRope) {
           // q <- rotary_pos_emb(q, p): (lo, hi) = (x[i], x[i + 64]) -> (lo cos - hi sin, hi cos + lo sin) in fp32,
           // rounded once to bf16, then stored like the unrotated rows
@@ -807,30 +839,28 @@ if constexpr (kRope) {
         const int nch = kWalk ? min(4, cur.nc - cur.c) : tile_chunks(i);
         const bool opens = kWalk ? cur.c == 0 : i == 0;  // first tile of a shard (kWalk) or of the stream
         const int kk_tile = kWalk ? tab->kk[cur.j] : 0;
-        // Mask bookkeeping for the tile's four chunks, done before the wait so that it costs nothing: a chunk of shard
+        // kWalk: mask bookkeeping for the tile's four chunks, done before the wait so that it costs nothing: a chunk of shard
         // j starting at key t0 needs the mask only if it reaches past the shortest prefix of the sub-tile; this row
         // then sees its first lc = vis - t0 columns.  Chunks a narrow last tile does not have count as fully masked.
-        int lc[4];
+        int lc[kWalk ? 4 : 1];
         uint32_t needm = 0;
+        if constexpr (kWalk) {
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          if constexpr (!kWalk) {
-            const int t0 = kNMax * i + kChunk * ch;  // from this CTA's first key on
-            if (ch >= nch || t0 + kChunk > sub_seen) needm |= 1u << ch;
-            lc[ch] = ch < nch ? my_seen - t0 : 0;
-          } else if (ch < nch) {  // warp-uniform
-            const int t0 = cur.c * kChunk;
-            if (t0 + kChunk > vis_first[cur.j]) needm |= 1u << ch;
-            lc[ch] = vq0 - t0;
-            if (cur.advance(tab, n_act)) {
-              vq0 = vq1;
-              vq1 = vq2;
-              vq2 = vq3;
-              vq3 = row_vis(cur.j + 3);
+          for (int ch = 0; ch < 4; ++ch) {
+            if (ch < nch) {  // warp-uniform
+              const int t0 = cur.c * kChunk;
+              if (t0 + kChunk > vis_first[cur.j]) needm |= 1u << ch;
+              lc[ch] = vq0 - t0;
+              if (cur.advance(tab, n_act)) {
+                vq0 = vq1;
+                vq1 = vq2;
+                vq2 = vq3;
+                vq3 = row_vis(cur.j + 3);
+              }
+            } else {
+              needm |= 1u << ch;
+              lc[ch] = 0;
             }
-          } else {
-            needm |= 1u << ch;
-            lc[ch] = 0;
           }
         }
         note(8 * i + 1);
@@ -860,7 +890,19 @@ if constexpr (kRope) {
         if (nch > 3) CASCADE_TMEM_LD32(s_addr + 96, sr, 96);
         tmem_wait_ld();
         // The mask is applied through a bit mask so that the compiler can move several bits at a time into predicates.
-        if (needm != 0) {  // warp-uniform
+        if constexpr (!kWalk) {
+          if (kNMax * (i + 1) > unmasked) {  // warp-uniform
+            const int mine = min(*my_seen, n_keys) - kNMax * i;  // visible columns of the tile
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) {
+              const int lc_ch = mine - kChunk * ch;
+              const uint32_t mk = lc_ch >= 32 ? 0xffffffffu : (lc_ch <= 0 ? 0u : ((1u << lc_ch) - 1u));
+#pragma unroll
+              for (int j = 0; j < 32; ++j)
+                if (!((mk >> j) & 1u)) sr[32 * ch + j] = 0xff800000u;  // -inf
+            }
+          }
+        } else if (needm != 0) {  // warp-uniform
 #pragma unroll
           for (int ch = 0; ch < 4; ++ch) {
             if ((needm >> ch) & 1u) {  // warp-uniform
@@ -967,14 +1009,26 @@ if constexpr (kRope) {
             tc_fence_after();
           }
           const float f = changed ? alpha : 1.f;
+          if constexpr (kWalk) {
 #pragma unroll
-          for (int cc = 0; cc < kD / 32; ++cc) {
-            uint32_t o[32];
-            CASCADE_TMEM_LD32(o_addr + (uint32_t)(cc * 32), o, 0);
-            tmem_wait_ld();
+            for (int cc = 0; cc < kD / 32; ++cc) {
+              uint32_t o[32];
+              CASCADE_TMEM_LD32(o_addr + (uint32_t)(cc * 32), o, 0);
+              tmem_wait_ld();
 #pragma unroll
-            for (int j = 0; j < 32; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * f);
-            CASCADE_TMEM_ST32(o_addr + (uint32_t)(cc * 32), o, 0);
+              for (int j = 0; j < 32; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * f);
+              CASCADE_TMEM_ST32(o_addr + (uint32_t)(cc * 32), o, 0);
+            }
+          } else {  // few registers: the tile's logits are still needed
+#pragma unroll 1
+            for (int cc = 0; cc < kD / 8; ++cc) {
+              uint32_t o[8];
+              CASCADE_TMEM_LD8(o_addr + (uint32_t)(cc * 8), o);
+              tmem_wait_ld();
+#pragma unroll
+              for (int j = 0; j < 8; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * f);
+              CASCADE_TMEM_ST8(o_addr + (uint32_t)(cc * 8), o);
+            }
           }
         };
         if constexpr (kLateMax) {
@@ -1482,6 +1536,20 @@ bool encode_out(CUtensorMap* map, void* base, int d, int lg, int64_t heads, int6
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Query rows [batch][tokens][heads][d]; box = a sub-tile (128 >> lg tokens x 1 << lg heads), 64 columns.
+bool encode_queries(CUtensorMap* map, const AttnParams& p, int lg) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn || !tc_rows_loadable({p.q, p.qs}, p.plan.n_q, p.H, p.batch)) return false;
+  const cuuint64_t dims[4] = {(cuuint64_t)p.d, (cuuint64_t)p.H, (cuuint64_t)p.plan.n_q, (cuuint64_t)p.batch};
+  auto stride = [&](int64_t elems, int64_t extent) { return (cuuint64_t)(extent > 1 ? elems * 2 : p.d * 2); };
+  const cuuint64_t strides[3] = {stride(p.qs.head, p.H), stride(p.qs.token, p.plan.n_q), stride(p.qs.batch, p.batch)};
+  const cuuint32_t box[4] = {64, 1u << lg, 128u >> lg, 1};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(p.q), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 struct TcLaunch {
   int lg, tile_major, split, early;
   bool after_gather;
@@ -1542,6 +1610,7 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
     return cudaErrorInvalidValue;
   }
   const int lg = stacked_log2(p.G);
+  tma.q_valid = !p.rope && encode_queries(&tma.q, p, lg);
   const int64_t tilslots = 256 >> lg, n_qt = (p.plan.n_q + tilslots - 1) / tilslots;
   const int64_t n_ctas = n_qt * (p.H >> lg) * p.batch;
   // Few query tiles (a chunk of a chunked prefill, a short prompt) leave SMs idle: a cluster then shares the keys of each

@@ -191,6 +191,23 @@ def test_fused_route_in_token_order(gu, n_q, n_kv, H, Hkv, d, B, off, causal):
     gu.full_parity(w)
 
 
+@pytest.mark.parametrize("n,H,Hkv,d", [(1, 8, 8, 64), (15, 8, 1, 128), (17, 8, 1, 128), (129, 4, 4, 128), (257, 6, 3, 64)])
+@pytest.mark.parametrize("n_q_extra", [1, 40])
+def test_query_boxes_at_the_end_of_the_tensor(gu, n, H, Hkv, d, n_q_extra):
+    """The last box of query rows reaches past the tokens of the sequence (here into the next one's, and past the last)."""
+    from paper_2507_05228_b200 import binding as cb
+    n_q, n_kv = n + n_q_extra, n + 300
+    w = wl.make_workload(f"boxes_{n}_{d}", 3, n_q, n_kv, H, Hkv, d, "bf16", "random", "random", 2, 2, seed=n + d,
+                         q_pos_offset=n_kv - n_q, causal=True)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    o, lse = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+    o_ref, lse_ref = oracle.attention_unsharded(w.q, w.k, w.v, w.scale, causal=True, q_pos_offset=w.q_pos_offset)
+    gu.check_output(o, lse, o_ref, lse_ref, w.tol, w.name)
+    assert plan.device_status() == 0
+    plan.destroy()
+
+
 @pytest.mark.parametrize("n_q", [70, 700])
 def test_fused_route_with_strides_a_tensor_map_cannot_hold(gu, n_q):
     """K and V of one sequence expanded over the batch (stride 0) go through a copy; the result is the same, bit for bit."""
