@@ -172,18 +172,26 @@ __device__ __forceinline__ bool elect_one() {  // true in exactly one lane of a 
 template <bool kPointer>
 struct WaitCtx {
   uint32_t misc;
-  volatile int* words;
   int32_t* status;  // global: [0] code, [1..3] block index, [4] tile of the waiter, [8..19] progress words
   __device__ __forceinline__ int load(int w) const {
-    if constexpr (kPointer) return words[w];
     int v;
     asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(v) : "r"(misc + 4 * w) : "memory");
     return v;
   }
   __device__ __forceinline__ void store(int w, int v) const {
-    if constexpr (kPointer) words[w] = v;
-    else asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(misc + 4 * w), "r"(v) : "memory");
+    asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(misc + 4 * w), "r"(v) : "memory");
   }
+  __device__ __forceinline__ void note(int warp, int v) const {  // (added up in this order the address costs no register)
+    asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(misc + 8 + 4 * warp), "r"(v) : "memory");
+  }
+};
+template <>
+struct WaitCtx<true> {
+  volatile int* words;
+  int32_t* status;
+  __device__ __forceinline__ int load(int w) const { return words[w]; }
+  __device__ __forceinline__ void store(int w, int v) const { words[w] = v; }
+  __device__ __forceinline__ void note(int warp, int v) const { words[2 + warp] = v; }
 };
 
 // Bounded wait: gives up after ~2 s, raises the CTA's abort flag and records `code`.
@@ -623,9 +631,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       if (lane == 1 || lane == 2) tab->first[lane - 1][0] = seen;
     }
   }
-  const WaitCtx<kWalk> wc{smem_base + (uint32_t)kOffMisc, reinterpret_cast<volatile int*>(smem + kOffMisc), pl.status};
+  WaitCtx<kWalk> wc;
+  if constexpr (kWalk) wc.words = reinterpret_cast<volatile int*>(smem + kOffMisc);
+  else wc.misc = smem_base + (uint32_t)kOffMisc;
+  wc.status = pl.status;
   auto note = [&](int v) {
-    if (lane == 0) wc.store(2 + warp, v);
+    if (lane == 0) wc.note(warp, v);
   };
 
   if (tid == 9 * 32) {
