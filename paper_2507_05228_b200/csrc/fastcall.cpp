@@ -134,8 +134,10 @@ PyObject* pair(PyObject* given_out, const at::Tensor& o, const at::Tensor& lse) 
   return r;
 }
 
+// The C calls run without the interpreter lock.  `f` must not throw, which would leave the lock behind: sizes and data pointers
+// are taken before (a tensor without storage, as torch.func.vmap hands out, throws when asked for its pointer).
 template <typename F>
-cascade_status_t unlocked(F&& f) {  // the C calls run without the interpreter lock
+cascade_status_t unlocked(F&& f) {
   cascade_status_t status;
   Py_BEGIN_ALLOW_THREADS
   status = f();
@@ -171,21 +173,22 @@ PyObject* attn_sharded(PyObject* const* a) {
   const cascade_strides_t os = strides(o);
   const at::Tensor lse = lse_for(truth(a[7]), q);
   const Scratch ws = scratch(plan, CASCADE_CALL_SHARDED, code, q, Hkv, a[8]);
-  void* st = stream();
+  void *st = stream(), *qp = q.data_ptr(), *kp = k.data_ptr(), *vp = v.data_ptr(), *op = o.data_ptr();
+  float* lp = data_or_null(lse);
   if (a[5] == Py_None) {
     check(unlocked([&] {
-      return api.attn_sharded(plan, code, B, H, Hkv, d, scale, q.data_ptr(), qs, k.data_ptr(), ks, v.data_ptr(), vs,
-                              o.data_ptr(), os, data_or_null(lse), ws.ptr, ws.bytes, st);
+      return api.attn_sharded(plan, code, B, H, Hkv, d, scale, qp, qs, kp, ks, vp, vs, op, os, lp, ws.ptr, ws.bytes, st);
     }));
   } else {
     const at::Tensor& table = tensor(a[5]);
     if (table.scalar_type() != at::kFloat || !table.is_contiguous() || table.dim() != 3 || table.size(1) != d / 2 ||
         table.size(2) != 2)
       raise(PyExc_AssertionError, "the positional table is fp32 [positions, head_dim / 2, 2], contiguous");
+    const auto* tp = static_cast<const float*>(table.data_ptr());
+    const int32_t n_positions = size(table, 0);
     check(unlocked([&] {
-      return api.attn_sharded_rope(plan, code, B, H, Hkv, d, scale, q.data_ptr(), qs, k.data_ptr(), ks, v.data_ptr(), vs,
-                                   static_cast<const float*>(table.data_ptr()), size(table, 0), o.data_ptr(), os,
-                                   data_or_null(lse), ws.ptr, ws.bytes, st);
+      return api.attn_sharded_rope(plan, code, B, H, Hkv, d, scale, qp, qs, kp, ks, vp, vs, tp, n_positions, op, os, lp,
+                                   ws.ptr, ws.bytes, st);
     }));
   }
   return pair(a[6], o, lse);
@@ -223,12 +226,12 @@ PyObject* attn_partials(PyObject* const* a) {
     Py_DECREF(seq);
     if (!fine) raise(PyExc_TypeError, "out: three tensors are expected");
   }
-  const Scratch ws = scratch(plan, CASCADE_CALL_PARTIALS, code, q, size(k, 2), a[7]);
-  void* st = stream();
+  const int32_t B = size(q, 0), H = size(q, 2), Hkv = size(k, 2), d = size(q, 3);
+  const Scratch ws = scratch(plan, CASCADE_CALL_PARTIALS, code, q, Hkv, a[7]);
+  void *st = stream(), *qp = q.data_ptr(), *kp = k.data_ptr(), *vp = v.data_ptr(), *op = o.data_ptr();
+  float *mp = static_cast<float*>(m.data_ptr()), *lp = static_cast<float*>(l.data_ptr());
   check(unlocked([&] {
-    return api.attn_partials(plan, code, size(q, 0), size(q, 2), size(k, 2), size(q, 3), scale, q.data_ptr(), qs,
-                             k.data_ptr(), ks, v.data_ptr(), vs, o.data_ptr(), static_cast<float*>(m.data_ptr()),
-                             static_cast<float*>(l.data_ptr()), ws.ptr, ws.bytes, st);
+    return api.attn_partials(plan, code, B, H, Hkv, d, scale, qp, qs, kp, ks, vp, vs, op, mp, lp, ws.ptr, ws.bytes, st);
   }));
   PyObject* r = PyTuple_New(3);
   if (!r) throw PyFailure();
@@ -240,21 +243,23 @@ PyObject* attn_partials(PyObject* const* a) {
 
 // (o_part, m_part, l_part, row_scatter address, batch stride, out or None, want_lse) -> (o, lse or None)
 PyObject* merge(PyObject* const* a) {
-  const at::Tensor &op = tensor(a[0]), &mp = tensor(a[1]), &lp = tensor(a[2]);
-  need_dims(op, 5);
-  const cascade_dtype_t code = dtype_code(op);
-  const int64_t B = op.size(0), n = op.size(2), H = op.size(3), d = op.size(4);
+  const at::Tensor &parts = tensor(a[0]), &m = tensor(a[1]), &l = tensor(a[2]);
+  need_dims(parts, 5);
+  const cascade_dtype_t code = dtype_code(parts);
+  const int64_t B = parts.size(0), n = parts.size(2), H = parts.size(3), d = parts.size(4);
+  const int32_t n_parts = size(parts, 1);
   const auto* rows = address<const int32_t>(a[3]);
   const int64_t row_stride = integer(a[4]);
-  const at::Tensor o = output_or(a[5], op, {B, n, H, d});
+  const at::Tensor o = output_or(a[5], parts, {B, n, H, d});
   const cascade_strides_t os = strides(o);
   at::Tensor lse;
-  if (truth(a[6])) lse = at::empty({B, n, H}, op.options().dtype(at::kFloat));
-  void* st = stream();
+  if (truth(a[6])) lse = at::empty({B, n, H}, parts.options().dtype(at::kFloat));
+  void *st = stream(), *pp = parts.data_ptr(), *op = o.data_ptr();
+  const auto *mp = static_cast<const float*>(m.data_ptr()), *lp = static_cast<const float*>(l.data_ptr());
+  float* lse_p = data_or_null(lse);
   check(unlocked([&] {
-    return api.merge(code, (int32_t)B, size(op, 1), (int32_t)n, (int32_t)H, (int32_t)d, op.data_ptr(),
-                     static_cast<const float*>(mp.data_ptr()), static_cast<const float*>(lp.data_ptr()), rows, row_stride,
-                     o.data_ptr(), os, data_or_null(lse), st);
+    return api.merge(code, (int32_t)B, n_parts, (int32_t)n, (int32_t)H, (int32_t)d, pp, mp, lp, rows, row_stride, op, os,
+                     lse_p, st);
   }));
   return pair(a[5], o, lse);
 }
@@ -271,14 +276,15 @@ PyObject* decode_step_rope(PyObject* const* a) {
   const at::Tensor o = a[9] == Py_None ? at::empty_like(q) : tensor(a[9]);
   const cascade_strides_t os = strides(o);
   const at::Tensor lse = lse_for(truth(a[10]), q);
-  const int32_t Hkv = size(kn, 2);
+  const int32_t B = size(q, 0), H = size(q, 2), Hkv = size(kn, 2), n_positions = size(table, 0);
   const Scratch ws = scratch(plan, CASCADE_CALL_DECODE_STEP_ROPE, CASCADE_BF16, q, Hkv, a[11]);
-  void* st = stream();
+  void *st = stream(), *qp = q.data_ptr(), *knp = kn.data_ptr(), *vnp = vn.data_ptr(), *kcp = kc.data_ptr(),
+       *vcp = vc.data_ptr(), *op = o.data_ptr();
+  const auto* tp = static_cast<const float*>(table.data_ptr());
+  float* lp = data_or_null(lse);
   check(unlocked([&] {
-    return api.decode_step_rope(plan, size(q, 0), size(q, 2), Hkv, scale, q.data_ptr(), qs, kn.data_ptr(), kns,
-                                vn.data_ptr(), vns, kc.data_ptr(), kcs, vc.data_ptr(), vcs, position,
-                                static_cast<const float*>(table.data_ptr()), size(table, 0), o.data_ptr(), os,
-                                data_or_null(lse), ws.ptr, ws.bytes, st);
+    return api.decode_step_rope(plan, B, H, Hkv, scale, qp, qs, knp, kns, vnp, vns, kcp, kcs, vcp, vcs, position, tp,
+                                n_positions, op, os, lp, ws.ptr, ws.bytes, st);
   }));
   return pair(a[9], o, lse);
 }
@@ -295,10 +301,11 @@ PyObject* attn_decode_static(PyObject* const* a) {
   const at::Tensor o = output_or(a[5], q, q.sizes());
   const cascade_strides_t os = strides(o);
   const at::Tensor lse = lse_for(truth(a[6]), q);
-  void* st = stream();
+  const int32_t B = size(q, 0), H = size(q, 2), Hkv = size(k, 2);
+  void *st = stream(), *qp = q.data_ptr(), *kp = k.data_ptr(), *vp = v.data_ptr(), *op = o.data_ptr();
+  float* lp = data_or_null(lse);
   check(unlocked([&] {
-    return api.decode_static(plan, size(q, 0), size(q, 2), size(k, 2), scale, q.data_ptr(), qs, k.data_ptr(), ks,
-                             v.data_ptr(), vs, o.data_ptr(), os, data_or_null(lse), st);
+    return api.decode_static(plan, B, H, Hkv, scale, qp, qs, kp, ks, vp, vs, op, os, lp, st);
   }));
   return pair(a[5], o, lse);
 }

@@ -3,6 +3,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -85,3 +87,33 @@ def test_host_side_argument_checks(binding):
     assert L.cascade_workspace_bytes(plan.handle, 0, 1, 1, 4, 3, 128, ctypes.byref(nbytes)) == 1
     assert L.cascade_workspace_bytes(plan.handle, 9, 1, 1, 4, 2, 128, ctypes.byref(nbytes)) == 1
     plan.destroy()
+
+
+def test_tensors_without_storage_raise(binding):
+    """torch.func.vmap hands out tensors that throw when asked for their data pointer.  In a child process: an exception that
+    leaves the interpreter lock released takes the interpreter down with it."""
+    code = """
+import numpy as np, torch
+from paper_2507_05228_b200 import binding as cb
+plan = cb.cascade_shard_plan_host(np.zeros(4, np.int32), np.zeros(4, np.int32), 1, 1)
+one = cb.cascade_shard_plan_host(np.zeros(1, np.int32), np.zeros(4, np.int32), 1, 1)
+table = torch.zeros(8, 64, 2)
+calls = {
+    "sharded": lambda x: cb.cascade_attn_sharded(plan, x, x, x, 1.0, want_lse=False)[0],
+    "rope": lambda x: cb.cascade_attn_sharded_rope(plan, x, x, x, 1.0, table, want_lse=False)[0],
+    "partials": lambda x: cb.cascade_attn_partials(plan, x, x, x, 1.0)[0],
+    "merge": lambda x: cb.cascade_merge(x[None], x[None, ..., 0], x[None, ..., 0], want_lse=False)[0],
+    "step": lambda x: cb.cascade_decode_step_rope(one, x[:, :1], x[:, :1], x[:, :1], x, x, 0, 1.0, table, want_lse=False)[0],
+    "static": lambda x: cb.cascade_attn_decode_static(one, x[:, :1], x, x, 1.0, want_lse=False)[0],
+}
+for name, call in calls.items():
+    try:
+        torch.func.vmap(call)(torch.zeros(3, 1, 4, 2, 128, dtype=torch.bfloat16))
+    except RuntimeError as e:
+        assert "data pointer" in str(e), (name, e)
+    else:
+        raise AssertionError(name)
+print("all raised")
+"""
+    run = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=600)
+    assert run.returncode == 0 and "all raised" in run.stdout, (run.returncode, run.stderr[-2000:])
