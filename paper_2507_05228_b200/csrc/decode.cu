@@ -482,12 +482,17 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __
     }
   }
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  // the plan's own prefixes and pair classes, for later calls on it (the caller's stream orders them after this kernel)
+  // the plan's own prefixes and pair classes, for later calls on it (the caller's stream orders them after this kernel); of
+  // several query shards one owns the only row, and the classes of the others are EMPTY as they were built
   if (vis_given && rank == 0 && g == 0 && (pl.n_maps > 1 || b == 0)) {
-    for (int kk = tid; kk < P; kk += NW * 32) {
+    const int J = pl.n_q_shards;
+    const int32_t* q_off = pl.q_off + (size_t)map * (J + 1);
+    for (int e = tid; e < J * P; e += NW * 32) {
+      const int jj = e / P, kk = e - jj * P;
+      if (J > 1 && q_off[jj] == q_off[jj + 1]) continue;
       const int v = step.vis[map * P + kk], len = kv_off[kk + 1] - kv_off[kk];
       const_cast<int32_t*>(vis)[kk] = v;
-      const_cast<uint8_t*>(pl.pair_class)[(size_t)map * P + kk] =
+      const_cast<uint8_t*>(pl.pair_class)[((size_t)map * J + jj) * P + kk] =
           v == 0 ? CASCADE_PAIR_EMPTY : (v == len ? CASCADE_PAIR_FULL : CASCADE_PAIR_PARTIAL);
     }
   }

@@ -176,6 +176,29 @@ def test_decode_step_moves_the_plan_with_few_and_with_many_prefixes(gu, B, P, pe
     plan.destroy()
 
 
+@pytest.mark.parametrize("n_maps", [1, 3])
+def test_decode_step_of_a_token_in_one_of_several_query_shards(gu, n_maps):
+    """The prefixes travel with the launch; the pair classes that the step leaves behind are those of the shard that owns the
+    query row, in every map, and a second plan update finds them so."""
+    from paper_2507_05228_b200 import binding as cb
+    cap, H, Hkv, J, P, B = 300, 8, 2, 6, 5, 3
+    rng = np.random.default_rng(n_maps)
+    kv_of = rng.integers(0, P, (n_maps, cap)).astype(np.int32)
+    q_of = rng.integers(1, J, (n_maps, 1)).astype(np.int32)
+    plan = cb.cascade_shard_plan(q_of, kv_of, J, P, 0, True)
+    w = wl.make_workload("step_J", B, cap, cap, H, Hkv, 128, "bf16", "random", "random", 1, 1, seed=n_maps)
+    q, k, v = gu.to_device(w)
+    table = cb.cascade_rope_table(cap, 128, 10000.0)
+    for pos in (7, 299):
+        cb.cascade_decode_step_rope(plan, q[:, :1], k[:, :1], v[:, :1], k.clone(), v.clone(), pos, w.scale, table)
+        for m in range(n_maps):
+            ref = oracle.shard_plan(q_of[m], kv_of[m], J, P, q_pos_offset=pos, causal=True)
+            for f in ("vis", "pair_class"):
+                assert np.array_equal(gu.read_plan_device_array(plan, f)[m], getattr(ref, f)), (f, pos, m)
+                assert np.array_equal(plan.get(f)[m], getattr(ref, f)), (f, pos, m)
+    plan.destroy()
+
+
 @pytest.mark.parametrize("n_q,n_kv,H,Hkv,d,B,off,causal", [
     (2, 2, 8, 8, 128, 1, 0, True),           # one tile; the rows see one and two keys
     (65, 1025, 32, 8, 128, 1, 960, True),    # keys shared by clusters of 8; a second query tile of one row, one key past a tile
