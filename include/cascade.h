@@ -273,7 +273,8 @@ cascade_status_t cascade_rope_table(int32_t n_positions, int32_t head_dim, doubl
  * depends on its original index only, the result equals rotating the whole sequence first and calling
  * cascade_attn_sharded.
  *   rope_table   DEVICE table written by cascade_rope_table for head_dim 128, 16-byte aligned, read-only
- *   n_positions  its row count; must cover max(q_pos_offset + n_q, n_kv)
+ *   n_positions  its row count; must cover max(q_pos_offset + n_q, n_kv).  A negative q_pos_offset is taken with the causal
+ *                mask only (a row before position 0 sees nothing and yields zeros); INVALID_ARG without
  * All other arguments, the workspace and the outputs are those of cascade_attn_sharded.
  * Supported on the tensor-core route only (bf16, head_dim 128, n_q > 1, at most 256 KV shards); other shapes return
  * CASCADE_ERR_UNSUPPORTED and the caller rotates q and k beforehand.

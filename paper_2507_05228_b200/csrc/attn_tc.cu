@@ -573,7 +573,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         const __nv_bfloat16* row = qb + (int64_t)tok * p.qs.token + (int64_t)(h0 + (r & (Gp - 1))) * p.qs.head;
         qv[2 * j] = __ldg(reinterpret_cast<const uint4*>(row));
         qv[2 * j + 1] = __ldg(reinterpret_cast<const uint4*>(row + 64));
-        rope_row[j] = reinterpret_cast<const float4*>(p.rope + (int64_t)(pl.q_pos_offset + tok) * 64 + (tid & 7) * 8);
+        // (a row before position 0 sees nothing, so its angle is of no account; the table starts at 0)
+        rope_row[j] = reinterpret_cast<const float4*>(p.rope + (int64_t)max(0, pl.q_pos_offset + tok) * 64 + (tid & 7) * 8);
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j)

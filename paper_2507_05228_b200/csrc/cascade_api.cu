@@ -1058,6 +1058,11 @@ static cascade_status_t attn_sharded_impl(const char* fn, const cascade_plan_t* 
       set_error("%s: the positional table has %d rows, the plan needs %lld", fn, n_positions, (long long)need);
       return CASCADE_ERR_INVALID_ARG;
     }
+    if (plan->dev.q_pos_offset < 0 && !plan->dev.causal) {  // (with the causal mask such a row sees nothing)
+      set_error("%s: without a mask every query row needs a position in the table, and the first is at %d", fn,
+                plan->dev.q_pos_offset);
+      return CASCADE_ERR_INVALID_ARG;
+    }
     if (!plan->kv_pos.empty()) {
       set_error("%s: the rotary step takes a key row's position from its index, which a plan over resident K/V rows "
                 "(cascade_shard_plan_resident) does not have", fn);

@@ -132,6 +132,30 @@ def test_headline_size_sampled_rows(cb, gu):
     plan.destroy()
 
 
+@pytest.mark.parametrize("offset", [-1, -40, -200])
+def test_rows_before_position_zero(cb, gu, offset):
+    """A plan may start before the first position: such rows see nothing, and no angle is looked up for them.  Without the
+    mask they would need one, and the call is refused."""
+    base, n_q, n_kv = 10000.0, 130, 150
+    w = wl.make_workload("rope_neg", 1, n_q, n_kv, 8, 2, 128, "bf16", "random", "random", 2, 3, seed=25, symmetric=False,
+                         q_pos_offset=offset)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    table = cb.cascade_rope_table(n_kv, 128, base)
+    o, lse = cb.cascade_attn_sharded_rope(plan, q, k, v, w.scale, table)
+    qr = rope.rotary_pos_emb(w.q, np.maximum(0, offset + np.arange(n_q)), base, "bf16").astype(np.float32)
+    kr = rope.rotary_pos_emb(w.k, np.arange(n_kv), base, "bf16").astype(np.float32)
+    o_ref, lse_ref = oracle.attention_unsharded(qr, kr, w.v, w.scale, causal=True, q_pos_offset=offset)
+    gu.check_output(o, lse, o_ref, lse_ref, w.tol, "rows before position 0")
+    assert (o[:, :min(n_q, -offset)] == 0).all()
+    plan.destroy()
+    full = cb.cascade_shard_plan(w.q_shard_of, w.kv_shard_of, 2, 3, offset, False)
+    with pytest.raises(cb.CascadeError) as ei:
+        cb.cascade_attn_sharded_rope(full, q, k, v, w.scale, table)
+    assert ei.value.status == 1
+    full.destroy()
+
+
 def test_argument_checks(cb, gu):
     w = wl.make_workload("rope_err", 1, 64, 64, 4, 2, 128, "bf16", "random", "random", 2, 2, seed=23)
     q, k, v = gu.to_device(w)
