@@ -50,6 +50,7 @@
 // Every mbarrier wait is bounded: on expiry the CTA raises a flag, records a code in the plan's status word
 // and drains without waiting again.
 #include <cuda.h>
+#include <float.h>
 
 #include <algorithm>
 
@@ -948,7 +949,10 @@ if constexpr (kRope) {
         if constexpr (kLateMax) {
           if (opens) {
             smax = row_max();
-            m_true = m_run = smax * c;  // -inf: the row sees nothing of the stream (a prefix, so not later either)
+            m_true = smax * c;
+            // Finite also where the row sees nothing of the tile or only logits of -inf: the first finite logit then lies so far
+            // above that its weight overflows, and the tile is done again with a reference of its own.
+            m_run = fmaxf(m_true, -FLT_MAX);
           }
         } else {  // straight-line: branches here cost more than they save
           smax = row_max();

@@ -249,6 +249,28 @@ def test_fused_route_with_strides_a_tensor_map_cannot_hold(gu, n_q):
     plan.destroy()
 
 
+@pytest.mark.parametrize("n_q,n_kv,hidden", [
+    (300, 300, 200),    # the first tile, and a part of the second
+    (64, 1200, 1000),   # keys shared by a cluster: whole parts, and the start of the last one
+    (64, 1200, 130),    # only the first part's first tile
+])
+def test_logits_of_minus_infinity_before_finite_ones(gu, n_q, n_kv, hidden):
+    """Keys so long that their logits overflow to -inf have weight 0 (in the fp64 oracle exp(-1e40) is 0 too): the rows that
+    see others are the softmax over those, although a first tile leaves them without a finite maximum."""
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload(f"minus_inf_{hidden}", 1, n_q, n_kv, 8, 2, 128, "bf16", "random", "random", 2, 3, seed=hidden,
+                         symmetric=False, q_pos_offset=n_kv - n_q)
+    w.q[:] = np.abs(w.q)
+    w.k[:, :hidden] = -(2.0 ** 127)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    o, lse = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+    o_ref, lse_ref = oracle.attention_unsharded(w.q, w.k, w.v, w.scale, q_pos_offset=w.q_pos_offset)
+    rows = np.arange(n_q) + w.q_pos_offset >= hidden
+    gu.check_output(o[:, rows], lse[:, rows], o_ref[:, rows], lse_ref[:, rows], w.tol, "rows with finite logits")
+    plan.destroy()
+
+
 @pytest.mark.parametrize("n_maps", [1, 2])
 def test_fused_route_over_resident_rows(gu, n_maps):
     """Rows with positions of their own: a query sees those at positions up to its own, and what lies behind may be NaN."""
