@@ -737,10 +737,12 @@ static size_t decode_ws_bytes(const cascade_plan_t* plan, cascade_dtype_t dtype,
   return align_up(rows * d * elt_size(dtype), 256) + 2 * align_up(rows * 4, 256);
 }
 
-// Workspace of the tensor-core route: shard-major K and V copies, and for head_dim 128 a place for rotated keys in token
-// order (cascade_attn_sharded_rope).
+// Workspace of the tensor-core route: room for copies of K and V.
 static size_t tc_ws_bytes(const cascade_plan_t* plan, int batch, int Hkv, int d) {
-  return (d == 128 ? 3 : 2) * sorted_kv_bytes(plan, batch, Hkv, d);
+  return 2 * sorted_kv_bytes(plan, batch, Hkv, d);
+}
+static bool tc_ws_given(const cascade_plan_t* plan, int batch, int Hkv, int d, const void* workspace, size_t bytes) {
+  return workspace && bytes >= tc_ws_bytes(plan, batch, Hkv, d) && ((uintptr_t)workspace & 255) == 0;
 }
 
 // Tensor-core route.
@@ -751,16 +753,16 @@ static size_t tc_ws_bytes(const cascade_plan_t* plan, int batch, int Hkv, int d)
 // 64 times the number of shards (2048 tokens, 8 random shards: 1.32 times the causal work before, 1.09 now).
 static cascade_status_t run_tc(AttnParams p, const char* fn, const cascade_plan_t* plan, void* workspace,
                                size_t workspace_bytes, cudaStream_t st, cudaError_t* launch_error) {
-  const size_t each = sorted_kv_bytes(plan, p.batch, p.Hkv, p.d), need = tc_ws_bytes(plan, p.batch, p.Hkv, p.d);
-  if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) {
-    set_error("%s: workspace of %zu bytes (256-byte aligned) required for copies of K and V, got %zu", fn, need,
-              workspace_bytes);
+  const size_t each = sorted_kv_bytes(plan, p.batch, p.Hkv, p.d);
+  if (!tc_ws_given(plan, p.batch, p.Hkv, p.d, workspace, workspace_bytes)) {
+    set_error("%s: workspace of %zu bytes (256-byte aligned) required for copies of K and V, got %zu", fn,
+              tc_ws_bytes(plan, p.batch, p.Hkv, p.d), workspace_bytes);
     return CASCADE_ERR_WORKSPACE;
   }
   const PlanDev& d = plan->dev;
   char* ws = (char*)workspace;
   if (!p.fused && d.n_kv_shards > 1) {
-    *launch_error = launch_gather_kv(p, ws, ws + each, nullptr, false, false, st);
+    *launch_error = launch_gather_kv(p, ws, ws + each, false, st);
     if (*launch_error == cudaSuccess) *launch_error = launch_attn_tc_partials(p, ws, ws + each, st);
     return CASCADE_OK;
   }
@@ -772,16 +774,37 @@ static cascade_status_t run_tc(AttnParams p, const char* fn, const cascade_plan_
   const Strides dense = {(int64_t)p.Hkv * d.n_kv * p.d, p.d, (int64_t)d.n_kv * p.d};
   const bool v_fits = tc_rows_loadable(v, n_seen, p.Hkv, p.batch);
   bool k_gathered = false, v_gathered = false;
+  RopeCopies after = {};  // what the workspace of a rotary call holds when it is done, as far as it is not written before
   if (p.rope) {
-    // the rotated keys: in token order for the kernel, and shard-major with the values, as the call leaves them behind
-    *launch_error = launch_gather_kv(p, ws, ws + each, ws + 2 * each, false, !v_fits, st);
-    k = {ws + 2 * each, dense};
+    // The kernel reads the rotated keys in token order; the call leaves them behind in shard-major order, with the values
+    // after them.  Both orders are the same with one shard.  Otherwise the second region holds the keys in token order
+    // until the kernel is done with them, and the values follow.  (A third region for them would refuse every caller who
+    // brings the two that cascade_workspace_bytes has always asked for.)
+    RopeCopies before = {};
+    k = {ws + each, dense};
+    if (d.n_kv_shards == 1) {
+      before.k_sorted = ws;
+      before.v = ws + each;
+      k = {ws, dense};
+      if (!v_fits) v = {ws + each, dense};
+    } else {
+      before.k_tokens = ws + each;
+      if (v_fits) {
+        before.k_sorted = ws;
+      } else {
+        before.v = ws;
+        before.v_token_order = true;
+        v = {ws, dense};
+        after.k_sorted = ws;
+      }
+      after.v = ws + each;
+    }
+    *launch_error = launch_gather_kv_rope(p, before, false, st);
     k_gathered = true;
     v_gathered = !v_fits;
-    if (v_gathered) v = {ws + each, dense};
   } else if (!v_fits || !tc_rows_loadable(k, n_seen, p.Hkv, p.batch) || (p.prefix_from_vis && d.n_maps > 1)) {
     // strides that a tensor map cannot hold (an expanded axis), or a different last visible row per sequence
-    *launch_error = launch_gather_kv(p, ws, ws + each, nullptr, true, true, st);
+    *launch_error = launch_gather_kv(p, ws, ws + each, true, st);
     k = {ws, dense};
     v = {ws + each, dense};
     k_gathered = v_gathered = true;
@@ -789,6 +812,7 @@ static cascade_status_t run_tc(AttnParams p, const char* fn, const cascade_plan_
     *launch_error = cudaSuccess;
   }
   if (*launch_error == cudaSuccess) *launch_error = launch_attn_tc(p, k, v, n_seen, k_gathered, v_gathered, st);
+  if (*launch_error == cudaSuccess && after.v) *launch_error = launch_gather_kv_rope(p, after, true, st);
   return CASCADE_OK;
 }
 
@@ -902,7 +926,8 @@ cascade_status_t cascade_attn_partials(const cascade_plan_t* plan, cascade_dtype
   cudaError_t e;
   if (use_decode(plan, dtype, n_heads, n_kv_heads, head_dim)) {
     e = launch_decode(p, st);
-  } else if (use_tc(plan, dtype, head_dim) && !(head_dim == 64 && !workspace)) {
+  } else if (use_tc(plan, dtype, head_dim) &&
+             (head_dim == 128 || tc_ws_given(plan, batch, n_kv_heads, head_dim, workspace, workspace_bytes))) {
     cascade_status_t ws = run_tc(p, "cascade_attn_partials", plan, workspace, workspace_bytes, st, &e);
     if (ws != CASCADE_OK) return ws;
   } else {
@@ -1097,8 +1122,9 @@ static cascade_status_t attn_sharded_impl(const char* fn, const cascade_plan_t* 
   p.os = {o_strides.batch, o_strides.token, o_strides.head};
   p.lse_out = lse_out;
   cudaError_t e;
-  // (heads of 64 columns without a workspace take the ALU kernel, which needs none)
-  if (use_tc(plan, dtype, head_dim) && !(head_dim == 64 && !workspace)) {
+  // (heads of 64 columns without a sufficient workspace take the ALU kernel, which needs none)
+  if (use_tc(plan, dtype, head_dim) &&
+      (head_dim == 128 || tc_ws_given(plan, batch, n_kv_heads, head_dim, workspace, workspace_bytes))) {
     cascade_status_t ws = run_tc(p, fn, plan, workspace, workspace_bytes, st, &e);
     if (ws != CASCADE_OK) return ws;
   } else {
@@ -1285,8 +1311,11 @@ cascade_status_t cascade_attn_sharded_host(const cascade_plan_t* plan, cascade_d
     return CASCADE_ERR_UNSUPPORTED;
   }
   const HostCallLayout L = host_call_layout(plan, dtype, batch, n_heads, n_kv_heads, head_dim);
-  if (!workspace || workspace_bytes < L.total || ((uintptr_t)workspace & 255)) {
-    set_error("%s: workspace of %zu bytes (256-byte aligned) required, got %zu", fn, L.total, workspace_bytes);
+  // heads of 64 columns do without the part for the head groups (on the ALU kernel), so a workspace without it is taken
+  const bool inner = L.inner_bytes && (head_dim == 128 || workspace_bytes >= L.total);
+  const size_t need = head_dim == 128 ? L.total : L.inner;
+  if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) {
+    set_error("%s: workspace of %zu bytes (256-byte aligned) required, got %zu", fn, need, workspace_bytes);
     return CASCADE_ERR_WORKSPACE;
   }
   int dev = 0;
@@ -1343,8 +1372,8 @@ cascade_status_t cascade_attn_sharded_host(const cascade_plan_t* plan, cascade_d
     if (e != cudaSuccess) return cuda_fail(e, "cascade_attn_sharded_host: queuing a query copy");
     cascade_status_t rc = attn_sharded_impl(fn, plan, dtype, batch, G * gs, gs, head_dim, scale, ws + L.q + q_off, qs,
                                             ws + L.k + kv_off, ks, ws + L.v + kv_off, ks, nullptr, 0,
-                                            ws + L.o + q_off, qs, nullptr, L.inner_bytes ? ws + L.inner : nullptr,
-                                            L.inner_bytes, st, n_kv_heads);
+                                            ws + L.o + q_off, qs, nullptr, inner ? ws + L.inner : nullptr,
+                                            inner ? L.inner_bytes : 0, st, n_kv_heads);
     if (rc != CASCADE_OK) return rc;
     e = cudaEventRecord(hs.computed[g], st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(hs.d2h, hs.computed[g], 0);

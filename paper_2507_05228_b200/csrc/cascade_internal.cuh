@@ -198,10 +198,16 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
                            bool v_gathered, cudaStream_t stream);
 // the partials of every KV shard; k_sorted / v_sorted: shard-major copies, [batch][kv_head][n_kv][d] bf16
 cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, const void* v_sorted, cudaStream_t stream);
-// Copies of K and V for the above, [batch][kv_head][n_kv][d]: shard-major, or with token_order as the rows are.  With
-// p.rope the key rows are turned on the way, and k_tokens (if not null) gets them in token order as well.
-cudaError_t launch_gather_kv(const AttnParams& p, void* k_out, void* v_out, void* k_tokens, bool token_order, bool v_token_order,
-                             cudaStream_t stream);
+// Copies of K and V for the above, [batch][kv_head][n_kv][d]: shard-major, or with token_order as the rows are.
+cudaError_t launch_gather_kv(const AttnParams& p, void* k_out, void* v_out, bool token_order, cudaStream_t stream);
+// The same with the key rows turned (p.rope) on the way; null = not asked for.
+struct RopeCopies {
+  void *k_sorted, *k_tokens;  // keys in shard-major order, in token order
+  void* v;                    // values, shard-major or in token order
+  bool v_token_order;
+};
+// dependent: launched as a programmatic dependent of the kernel in front, which writes none of its inputs
+cudaError_t launch_gather_kv_rope(const AttnParams& p, const RopeCopies& c, bool dependent, cudaStream_t stream);
 cudaError_t launch_rope_table(int32_t n_positions, int32_t head_dim, double base, float2* table, cudaStream_t stream);
 cudaError_t launch_rope_apply(cascade_dtype_t dtype, int32_t batch, int32_t n_rows, int32_t n_heads, int32_t head_dim,
                               const void* x, Strides xs, int32_t first_position, const float2* table, void* y, Strides ys,

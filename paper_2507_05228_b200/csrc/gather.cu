@@ -86,13 +86,13 @@ __device__ __forceinline__ void rotate8(uint4& lo, uint4& hi, const float2* __re
 // The same gather with the rotary step of the pre-pass (the Pre-Pass algorithm: k <- rotary_pos_emb(k, p^{R_i})) applied to the
 // key rows on the way: a key row is turned by the angles of its own token index, so the rotation needs nothing but
 // the row and its row of the positional table.  A thread holds both halves of 8 rotation pairs (columns 8c.. and
-// 64 + 8c..), 8 threads per row; V rows are copied as they are.
-__global__ void __launch_bounds__(256) gather_kv_rope_kernel(const __grid_constant__ AttnParams p, __nv_bfloat16* k_out,
-                                                             __nv_bfloat16* v_out, __nv_bfloat16* k_tokens,
-                                                             bool v_token_order) {
+// 64 + 8c..), 8 threads per row; V rows are copied as they are.  Of the copies those that are asked for are made.
+// Launched as a dependent (of the attention kernel, which still reads what is overwritten here) it loads and turns its rows
+// under the end of that kernel and stores them when it has completed.
+__global__ void __launch_bounds__(256) gather_kv_rope_kernel(const __grid_constant__ AttnParams p, const RopeCopies c) {
   constexpr int D = 128;
   constexpr int kPasses = kGatherRowsPerCta / 32;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // as in gather_kv_kernel
+  grid_go();  // as in gather_kv_kernel
   const PlanDev& pl = p.plan;
   const int g = blockIdx.y, b = blockIdx.z;
   const int map = pl.n_maps == 1 ? 0 : b;
@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(256) gather_kv_rope_kernel(const __grid_consta
   const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(p.v) + (int64_t)b * p.vs.batch + (int64_t)g * p.vs.head;
   const int64_t out_base = ((int64_t)b * p.Hkv + g) * pl.n_kv;
   const int slot0 = blockIdx.x * kGatherRowsPerCta;
+  const bool want_k = c.k_sorted || c.k_tokens;
   uint4 klo[kPasses], khi[kPasses], vlo[kPasses], vhi[kPasses];
   int tok[kPasses];
 #pragma unroll
@@ -114,42 +115,53 @@ __global__ void __launch_bounds__(256) gather_kv_rope_kernel(const __grid_consta
     if (slot_is_visible(pl, map, slot)) {
       const __nv_bfloat16* kr = kb + (int64_t)tok[i] * p.ks.token + chunk * 8;
       const __nv_bfloat16* vr = vb + (int64_t)tok[i] * p.vs.token + chunk * 8;
-      klo[i] = __ldcs(reinterpret_cast<const uint4*>(kr));
-      khi[i] = __ldcs(reinterpret_cast<const uint4*>(kr + 64));
-      vlo[i] = __ldcs(reinterpret_cast<const uint4*>(vr));
-      vhi[i] = __ldcs(reinterpret_cast<const uint4*>(vr + 64));
+      if (want_k) {
+        klo[i] = __ldcs(reinterpret_cast<const uint4*>(kr));
+        khi[i] = __ldcs(reinterpret_cast<const uint4*>(kr + 64));
+      }
+      if (c.v) {
+        vlo[i] = __ldcs(reinterpret_cast<const uint4*>(vr));
+        vhi[i] = __ldcs(reinterpret_cast<const uint4*>(vr + 64));
+      }
     }
   }
+  auto put = [&](void* base, int64_t row, const uint4& lo, const uint4& hi) {
+    __nv_bfloat16* to = static_cast<__nv_bfloat16*>(base) + (out_base + row) * D + chunk * 8;
+    *reinterpret_cast<uint4*>(to) = lo;
+    *reinterpret_cast<uint4*>(to + 64) = hi;
+  };
+  if (want_k) {
+#pragma unroll
+    for (int i = 0; i < kPasses; ++i)
+      if (slot0 + 32 * i + r0 < pl.n_kv)
+        rotate8(klo[i], khi[i], p.rope + (int64_t)tok[i] * (D / 2) + chunk * 8);  // zeros stay zeros
+  }
+  grid_wait();  // (returns at once unless launched as a dependent)
 #pragma unroll
   for (int i = 0; i < kPasses; ++i) {
     const int slot = slot0 + 32 * i + r0;
     if (slot < pl.n_kv) {
-      rotate8(klo[i], khi[i], p.rope + (int64_t)tok[i] * (D / 2) + chunk * 8);  // zeros stay zeros
-      __nv_bfloat16* ko = k_out + (out_base + slot) * D + chunk * 8;
-      __nv_bfloat16* kt = k_tokens + (out_base + tok[i]) * D + chunk * 8;
-      __nv_bfloat16* vo = v_out + (out_base + (v_token_order ? tok[i] : slot)) * D + chunk * 8;
-      *reinterpret_cast<uint4*>(ko) = klo[i];
-      *reinterpret_cast<uint4*>(ko + 64) = khi[i];
-      *reinterpret_cast<uint4*>(kt) = klo[i];
-      *reinterpret_cast<uint4*>(kt + 64) = khi[i];
-      *reinterpret_cast<uint4*>(vo) = vlo[i];
-      *reinterpret_cast<uint4*>(vo + 64) = vhi[i];
+      if (c.k_sorted) put(c.k_sorted, slot, klo[i], khi[i]);
+      if (c.k_tokens) put(c.k_tokens, tok[i], klo[i], khi[i]);
+      if (c.v) put(c.v, c.v_token_order ? tok[i] : slot, vlo[i], vhi[i]);
     }
   }
 }
 
-cudaError_t launch_gather_kv(const AttnParams& p, void* k_out, void* v_out, void* k_tokens, bool token_order, bool v_token_order,
-                             cudaStream_t stream) {
-  dim3 grid((p.plan.n_kv + kGatherRowsPerCta - 1) / kGatherRowsPerCta, p.Hkv, p.batch);
-  __nv_bfloat16 *ko = static_cast<__nv_bfloat16*>(k_out), *vo = static_cast<__nv_bfloat16*>(v_out);
-  if (p.rope) {
-    gather_kv_rope_kernel<<<grid, 256, 0, stream>>>(p, ko, vo, static_cast<__nv_bfloat16*>(k_tokens), v_token_order);
-  } else {
-    auto kernel = p.d == 64 ? gather_kv_kernel<64> : gather_kv_kernel<128>;
-    kernel<<<grid, 256, 0, stream>>>(p, ko, vo, token_order);
-  }
+static dim3 gather_grid(const AttnParams& p) {
+  return dim3((p.plan.n_kv + kGatherRowsPerCta - 1) / kGatherRowsPerCta, p.Hkv, p.batch);
+}
+
+cudaError_t launch_gather_kv(const AttnParams& p, void* k_out, void* v_out, bool token_order, cudaStream_t stream) {
+  auto kernel = p.d == 64 ? gather_kv_kernel<64> : gather_kv_kernel<128>;
+  kernel<<<gather_grid(p), 256, 0, stream>>>(p, static_cast<__nv_bfloat16*>(k_out), static_cast<__nv_bfloat16*>(v_out),
+                                             token_order);
   count_launch();
   return cudaGetLastError();
+}
+
+cudaError_t launch_gather_kv_rope(const AttnParams& p, const RopeCopies& c, bool dependent, cudaStream_t stream) {
+  return launch_dependent(gather_kv_rope_kernel, gather_grid(p), 256, 0, 1, dependent, stream, p, c);
 }
 
 // Positional table p of the rotary embedding (Section 5.1: p is set up before inference; the Pre-Pass algorithm takes its rows

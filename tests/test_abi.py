@@ -89,6 +89,17 @@ def test_host_side_argument_checks(binding):
     plan.destroy()
 
 
+def test_workspace_of_the_tensor_core_route_is_two_copies(binding):
+    """A copy of K and one of V, each rounded up to 256 bytes, for every call: programs size it by this documented sum."""
+    plan = binding.cascade_shard_plan_host(np.zeros(77, np.int32), np.zeros(77, np.int32), 1, 1)
+    for B, H, Hkv in ((1, 4, 4), (3, 6, 2)):
+        for d in (64, 128):
+            copies = 2 * ((B * Hkv * 77 * d * 2 + 255) // 256 * 256)
+            for call in (binding.CALL_PARTIALS, binding.CALL_SHARDED):
+                assert binding.cascade_workspace_bytes(plan, call, binding.BF16, B, H, Hkv, d) == copies
+    plan.destroy()
+
+
 def test_tensors_without_storage_raise(binding):
     """torch.func.vmap hands out tensors that throw when asked for their data pointer.  In a child process: an exception that
     leaves the interpreter lock released takes the interpreter down with it."""

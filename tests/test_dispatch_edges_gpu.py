@@ -77,6 +77,37 @@ def test_head_dim_64_without_a_workspace_takes_the_alu_kernel(gu):
     plan.destroy()
 
 
+def test_head_dim_64_with_too_small_a_workspace(gu):
+    """Heads of 64 columns never needed scratch memory: what is too small or misaligned for the tensor-core route is left
+    alone, and the ALU kernel runs.  The host call's workspace without scratch for its head groups likewise."""
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload("d64_small_ws", 1, 200, 200, 8, 2, 64, "bf16", "random", "random", 3, 3, seed=8)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    u, m, e = oracle.attn_pass(w.q, w.k, w.v, w.scale, gu.oracle_plan(w))
+    o_ref, lse_ref = oracle.attention_unsharded(w.q, w.k, w.v, w.scale)
+    need = cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED, cb.BF16, 1, 8, 2, 64)
+    raw = torch.full((need + 16,), 0x5A, dtype=torch.uint8, device="cuda")
+    for ws in (raw[:need - 256], raw[16:], raw[:16]):
+        o, lse = cb.cascade_attn_sharded(plan, q, k, v, w.scale, workspace=ws)
+        gu.check_output(o, lse, o_ref, lse_ref, w.tol, "small workspace")
+        parts = cb.cascade_attn_partials(plan, q, k, v, w.scale, workspace=ws)
+        gu.check_partials(tuple(t.double().cpu().numpy() for t in parts), (u, m, e), w.tol, "small workspace")
+    assert (raw == 0x5A).all()
+    hq, hk, hv = (t.cpu().pin_memory() for t in (q, k, v))
+    ho = torch.empty_like(hq).pin_memory()
+    staging = sum((t.numel() * 2 + 255) // 256 * 256 for t in (hq, hk, hv, ho))
+    raw = torch.full((staging + 256,), 0x5A, dtype=torch.uint8, device="cuda")
+    cb.cascade_attn_sharded_host(plan, hq, hk, hv, w.scale, ho, raw[:staging])
+    torch.cuda.synchronize()
+    gu.check_output(ho.double().numpy(), None, o_ref, None, w.tol, "host call without scratch")
+    assert (raw[staging:] == 0x5A).all()
+    with pytest.raises(cb.CascadeError) as ei:
+        cb.cascade_attn_sharded_host(plan, hq, hk, hv, w.scale, ho, raw[:staging - 256])
+    assert ei.value.status == 4
+    plan.destroy()
+
+
 @pytest.mark.parametrize("n_q,n_kv,H,Hkv,d,B,shards,dtype,causal", [
     (1, 1, 2, 2, 64, 1, 1, "f32", True),          # one key
     (1, 300, 6, 2, 64, 2, 3, "bf16", True),       # one query row on the ALU route: key groups share the row
