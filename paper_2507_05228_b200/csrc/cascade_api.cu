@@ -745,6 +745,15 @@ static bool tc_ws_given(const cascade_plan_t* plan, int batch, int Hkv, int d, c
   return workspace && bytes >= tc_ws_bytes(plan, batch, Hkv, d) && ((uintptr_t)workspace & 255) == 0;
 }
 
+static bool is_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {  // (the default stream beside a capture: the launch will say so)
+    cudaGetLastError();
+    return false;
+  }
+  return status != cudaStreamCaptureStatusNone;
+}
+
 // Tensor-core route.
 // Partials of several KV shards: a gather of K and V into shard-major order, then a kernel that walks the shards.
 // Otherwise the shards are only different subsets of the same sum, in which a query sees a prefix of the K/V rows (all those
@@ -766,13 +775,17 @@ static cascade_status_t run_tc(AttnParams p, const char* fn, const cascade_plan_
     if (*launch_error == cudaSuccess) *launch_error = launch_attn_tc_partials(p, ws, ws + each, st);
     return CASCADE_OK;
   }
-  p.prefix_from_vis = !plan->kv_pos.empty();
-  int64_t n_seen = 0;  // rows past what the last query sees may hold anything: the kernel does not load them
-  for (int mp = 0; mp < (p.prefix_from_vis ? d.n_maps : 1); ++mp)
+  // A call captured into a graph is replayed against what cascade_plan_advance has made of the plan by then, so nothing may
+  // follow from the host's copy of the query position: the prefixes come from vis, and what no query sees is kept out of the
+  // products by copies that vis governs too.
+  const bool replayed = is_capturing(st);
+  p.prefix_from_vis = replayed || !plan->kv_pos.empty();
+  int64_t n_seen = replayed ? d.n_kv : 0;  // rows past what the last query sees may hold anything: the kernel does not load them
+  for (int mp = 0; mp < (plan->kv_pos.empty() ? 1 : d.n_maps); ++mp)
     n_seen = std::max(n_seen, visible_keys(*plan, mp, (int64_t)d.n_q - 1 + d.q_pos_offset));
   TcRows k = {p.k, p.ks}, v = {p.v, p.vs};
   const Strides dense = {(int64_t)p.Hkv * d.n_kv * p.d, p.d, (int64_t)d.n_kv * p.d};
-  const bool v_fits = tc_rows_loadable(v, n_seen, p.Hkv, p.batch);
+  const bool v_fits = !replayed && tc_rows_loadable(v, n_seen, p.Hkv, p.batch);
   bool k_gathered = false, v_gathered = false;
   RopeCopies after = {};  // what the workspace of a rotary call holds when it is done, as far as it is not written before
   if (p.rope) {

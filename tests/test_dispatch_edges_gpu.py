@@ -333,3 +333,43 @@ def test_fused_route_over_resident_rows(gu, n_maps):
     lse_ref = (m[..., 0] + np.log(e.sum(-1))).transpose(0, 2, 1)
     gu.check_output(o, lse, o_ref, lse_ref, w.tol, "resident rows, fused")
     plan.destroy()
+
+
+@pytest.mark.parametrize("d,n_maps,P", [(128, 1, 5), (128, 2, 5), (64, 1, 5), (128, 1, 1)])
+def test_captured_call_follows_the_plan(gu, d, n_maps, P):
+    """A call captured into a graph is replayed after plan updates outside the graph: it sees what the plan says then, and
+    what lies behind the new position may be NaN."""
+    from paper_2507_05228_b200 import binding as cb
+    n_q, n_kv, B = 64, 600, 2
+    w = wl.make_workload("captured", B, n_kv, n_kv, 8, 2, d, "bf16", "random", "random", 1, 1, seed=d + P)
+    q, k, v = gu.to_device(w)
+    rng = np.random.default_rng(P)
+    kv_of = rng.integers(0, P, (n_maps, n_kv)).astype(np.int32)
+    q_of = rng.integers(0, 3, (n_maps, n_q)).astype(np.int32)
+    plan = cb.cascade_shard_plan(q_of, kv_of, 3, P, 100, True)
+    qc, kc, vc = q[:, :n_q].clone(), torch.full_like(k, float("nan")), torch.full_like(v, float("nan"))
+    ws = torch.empty(cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED, cb.BF16, B, 8, 2, d), dtype=torch.uint8, device="cuda")
+    o = torch.zeros_like(qc)
+    parts = [t.clone() for t in cb.cascade_attn_partials(plan, qc, k, v, w.scale, workspace=ws)]
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        cb.cascade_attn_sharded(plan, qc, kc, vc, w.scale, out=o, want_lse=False, workspace=ws)
+        cb.cascade_attn_partials(plan, qc, kc, vc, w.scale, out=parts, workspace=ws)
+    for off in (100, 300, 536, 20):
+        seen = off + n_q
+        qc.copy_(q[:, off:seen])
+        kc.fill_(float("nan")), vc.fill_(float("nan"))
+        kc[:, :seen], vc[:, :seen] = k[:, :seen], v[:, :seen]
+        plan.advance(off)
+        graph.replay()
+        torch.cuda.synchronize()
+        o_ref, lse_ref = oracle.attention_unsharded(w.q[:, off:seen], w.k, w.v, w.scale, q_pos_offset=off)
+        gu.check_output(o, None, o_ref, None, w.tol, f"captured at 100, replayed at {off}")
+        for b in range(B):
+            op = oracle.shard_plan(q_of[b % n_maps], kv_of[b % n_maps], 3, P, q_pos_offset=off, causal=True)
+            u, m, e = oracle.attn_pass(w.q[b:b + 1, off:seen], w.k[b:b + 1], w.v[b:b + 1], w.scale, op)
+            gu.check_partials(tuple(t[b:b + 1].double().cpu().numpy() for t in parts), (u, m, e), w.tol, f"partials at {off}")
+    del graph
+    plan.destroy()
