@@ -593,6 +593,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     }
   }
   if (warp == 11) {  // the warp without a role of its own
+    // Whether a wait of an earlier call on this plan gave up: then this one writes nothing.  Looked up here, beside the set-up
+    // of the others, the load costs nothing (before the set-up, 1000 cycles).
+    const int32_t gave_up = *reinterpret_cast<volatile int32_t*>(pl.status);
     if constexpr (kWalk) {
       // Compact the shards of which the CTA's last row (longest prefix; rows ascend) sees something, with what the
       // roles need per shard, and count the tiles of the stream.
@@ -632,6 +635,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       }
       if (lane == 1 || lane == 2) tab->first[lane - 1][0] = seen;
     }
+    if (lane == 0 && gave_up) stream_info[1] = -1;
   }
   WaitCtx<kWalk> wc;
   if constexpr (kWalk) wc.words = reinterpret_cast<volatile int*>(smem + kOffMisc);
@@ -641,6 +645,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     if (lane == 0) wc.note(warp, v);
   };
 
+  uint32_t requested = 0;  // barriers of the boxes requested below (one bit each)
   if (tid == 9 * 32) {
     mbar_init(bar(Q_FULL), q_boxes ? 1 : 128);  // 128: every thread of the sub-tile's softmax group brings a share of the rows
     mbar_init(bar(Q_FULL + 1), q_boxes ? 1 : 128);
@@ -673,20 +678,23 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       if (tiles * (part_of_keys + 1) / split > t0) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         auto request_q = [&](int s) {
+          requested |= 1u << (Q_FULL + s);
           mbar_expect_tx(bar(Q_FULL + s), (uint32_t)kTileBytes);
           for (int half = 0; half < C::kHalves; ++half)
             tma_tile4(smem_base + (uint32_t)(kOffQ + s * kTileBytes + half * kHalfBytes), &tma.q, 64 * half, h0, row0 + s * R, b,
                       bar(Q_FULL + s));
         };
-        auto request_kv = [&](const CUtensorMap* map, uint32_t dst, uint32_t fb) {
+        auto request_kv = [&](const CUtensorMap* map, uint32_t dst, int full) {
+          const uint32_t fb = bar(full);
+          requested |= 1u << full;
           mbar_expect_tx(fb, (uint32_t)kTileBytes);
           tma_tile4(dst, map, 0, t0 * kNMax, g, b, fb);
           if (C::kHalves == 2) tma_tile4(dst + (uint32_t)kHalfBytes, map, 64, t0 * kNMax, g, b, fb);
         };
         if (q_boxes) request_q(0);
-        if (early & 1) request_kv(&tma.k, smem_base + kOffK, bar(K_FULL));
+        if (early & 1) request_kv(&tma.k, smem_base + kOffK, K_FULL);
         if (q_boxes && n_sub == 2) request_q(1);
-        if (early & 2) request_kv(&tma.v, smem_base + kOffV, bar(V_FULL));
+        if (early & 2) request_kv(&tma.v, smem_base + kOffV, V_FULL);
       }
     }
   }
@@ -702,13 +710,23 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const int n_act = stream_info[0];  // kWalk: shards of which the CTA sees something
-  const int n_tiles = stream_info[1];
+  const int n_tiles = stream_info[1];  // -1: write nothing
   // not kWalk: first key and number of keys of this CTA's part of the stream
   const int key0 = kWalk ? 0 : tab->slot0[0], n_keys = kWalk ? 0 : tab->need[0];
   // MMA tiles of four chunks; only the last one is narrower, or with kWalk the last one of every shard (see TileSeq)
   auto tile_chunks = [&](int i) { return min(4, (n_keys - kNMax * i + kChunk - 1) / kChunk); };
 
-  if (warp < 8) {
+  if (n_tiles < 0) {
+    // an earlier call gave up: what was requested lands, the cluster's other CTAs find this one's shared memory there
+    for (uint32_t left = requested; left; left &= left - 1)
+      for (int i = 0; i < 1 << 20 && !mbar_try_wait(bar(__ffs(left) - 1), 0u); ++i) {
+      }
+    __syncwarp();
+    if (!kWalk && split > 1) {
+      cluster_barrier();
+      cluster_barrier();
+    }
+  } else if (warp < 8) {
     // ------------------------------------------------------------------ softmax + epilogue
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
     const int s = warp >> 2;  // sub-tile

@@ -373,3 +373,34 @@ def test_captured_call_follows_the_plan(gu, d, n_maps, P):
             gu.check_partials(tuple(t[b:b + 1].double().cpu().numpy() for t in parts), (u, m, e), w.tol, f"partials at {off}")
     del graph
     plan.destroy()
+
+
+@pytest.mark.parametrize("n_q,n_kv", [(300, 300), (64, 1200)])
+def test_calls_on_a_plan_whose_status_word_is_set_write_nothing(gu, n_q, n_kv):
+    """Once a wait inside the tensor-core kernel has given up, later calls on the plan leave their outputs alone (here the
+    word is set from outside; the second size shares keys in clusters).  With the word cleared the plan works again."""
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload("gave_up", 1, n_q, n_kv, 8, 2, 128, "bf16", "random", "random", 2, 3, seed=n_q, symmetric=False,
+                         q_pos_offset=n_kv - n_q)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    table = cb.cascade_rope_table(n_kv, 128, 10000.0)
+    word = torch.as_tensor(gu._DevicePointer(plan.dev_ptr("q_off") - 256, 1, "<i4"), device="cuda")  # first in the plan's memory
+    assert word.item() == 0
+    word.fill_(5)
+    with pytest.raises(cb.CascadeError) as ei:
+        plan.device_status()
+    assert ei.value.status == 7
+    o = torch.full_like(q, 7.0)
+    parts = (torch.full((1, 3, n_q, 8, 128), 7.0, dtype=q.dtype, device="cuda"), torch.full((1, 3, n_q, 8), 7.0, device="cuda"),
+             torch.full((1, 3, n_q, 8), 7.0, device="cuda"))
+    cb.cascade_attn_sharded(plan, q, k, v, w.scale, out=o)
+    cb.cascade_attn_sharded_rope(plan, q, k, v, w.scale, table, out=o)
+    cb.cascade_attn_partials(plan, q, k, v, w.scale, out=parts)
+    torch.cuda.synchronize()
+    assert all((t == 7.0).all() for t in (o, *parts))
+    word.fill_(0)
+    cb.cascade_attn_sharded(plan, q, k, v, w.scale, out=o)
+    o_ref, _ = oracle.attention_unsharded(w.q, w.k, w.v, w.scale, q_pos_offset=w.q_pos_offset)
+    gu.check_output(o, None, o_ref, None, w.tol, "after the word was cleared")
+    plan.destroy()
