@@ -87,27 +87,27 @@ constexpr int kMaxStages = 4;
 //            (sub-tile s, tile i: buffer (2 i + s) mod 3), so the next logits of a sub-tile are computed while it is still
 //            in the softmax of the current tile.  P is kept to twice the precision there: a bf16 part and the bf16
 //            rest, which together fill the 128 columns of the buffer they overwrite.
-// kWalk (partials) has a staging area of its own for finished rows, which at D = 128 takes the place of the second K and V
-// stages: a tile step with the write-out of a shard is long enough to hide a load.
+// kWalk (partials) at D = 64 has a staging area of its own for finished rows.
 template <int D, bool kWalk>
 struct Cfg {
   static constexpr int kHalves = D / 64;
   static constexpr int kTileBytes = kHalves * kHalfBytes;  // [halves][128 rows][128 bytes]
-  static constexpr int kKStages = D == 64 ? 4 : (kWalk ? 1 : 2);  // (D = 128: a third stage bought nothing)
-  static constexpr int kVStages = D == 64 ? 3 : (kWalk ? 1 : 2);
+  static constexpr int kKStages = D == 64 ? 4 : 2;  // (D = 128: a third stage bought nothing)
+  static constexpr int kVStages = D == 64 ? 3 : 2;
   static constexpr bool kRing = D == 64;                   // three logit buffers, P in two parts
   static constexpr uint32_t kOCol = kRing ? 384u : 256u;   // first accumulator column
-  // Output rows staged for the copy engine.  kWalk: per warp, [halves][32 rows][128 bytes], swizzled like the operand tiles;
-  // otherwise rows, padded by 16 bytes
-  static constexpr int kStageWarpBytes = kHalves * 32 * 128, kRowBytes = D * 2, kStageRowBytes = kRowBytes + 16;
-  static constexpr int kStageBytes = kWalk ? 8 * kStageWarpBytes : 2 * kM * kStageRowBytes;
+  // Output rows.  The last ones of a CTA are staged where Q and K were, padded by 16 bytes; with kBoxes all of them in an area
+  // of their own, per warp [32 rows][128 bytes], swizzled like the operand tiles.
+  static constexpr bool kBoxes = kWalk && D == 64;
+  static constexpr int kStageWarpBytes = 32 * 128, kRowBytes = D * 2, kStageRowBytes = kRowBytes + 16;
+  static constexpr int kStageBytes = kBoxes ? 8 * kStageWarpBytes : 2 * kM * kStageRowBytes;
   // shared memory map (offsets from a 1024-byte aligned base)
   static constexpr int kOffQ = 0;
   static constexpr int kOffK = kOffQ + 2 * kTileBytes;
   static constexpr int kOffV = kOffK + kKStages * kTileBytes;
-  static constexpr int kOffStage = kWalk ? kOffV + kVStages * kTileBytes : kOffQ;
-  static constexpr int kOffBar = kOffV + kVStages * kTileBytes + (kWalk ? kStageBytes : 0);
-  static_assert(kWalk || kStageBytes <= kOffV, "the output staging area must fit in the Q and K tiles");
+  static constexpr int kOffStage = kBoxes ? kOffV + kVStages * kTileBytes : kOffQ;
+  static constexpr int kOffBar = kOffV + kVStages * kTileBytes + (kBoxes ? kStageBytes : 0);
+  static_assert(kBoxes || kStageBytes <= kOffV, "the output staging area must fit in the Q and K tiles");
   static constexpr int kNumBars = 30;
   static constexpr int kOffMisc = kOffBar + kNumBars * 8;   // tmem slot, abort flag, 12 progress words
   static constexpr int kOffShard = kOffMisc + 64;           // int32 [5][kMaxShards], see ShardTab
@@ -444,7 +444,7 @@ struct TmaArgs {
   // kWalk: where finished rows go, o_part as [batch * KV shards][n_q slots][heads][head_dim]; a box is the rows of one warp:
   // 32 / Gp slots x Gp heads
   CUtensorMap o;
-  int o_valid;  // 0: the threads store their rows themselves
+  int o_valid;  // 0 (always so at head_dim 128): the threads store their rows themselves
   // Fused route without a rotary step: the query rows as [batch][tokens][heads][head_dim]; a box is one sub-tile, 128 / Gp
   // tokens x Gp heads, 64 columns
   int q_valid;  // 0: the threads load them
@@ -801,16 +801,22 @@ if constexpr (kRope) {
       if (kWalk) cur.start(tab, n_act);
       int kk_open = -1;  // kWalk: the shard whose partial is being accumulated
       int n_flushed = 0;  // kWalk: partials written so far
-      // kWalk: writes this warp's finished rows from TMEM, scaled: through shared memory to the copy engine, a box per 64
-      // columns.  (Stores from the threads, 32 bytes into each of 32 rows per instruction, kept a CTA's memory pipe busy for
-      // 3200 cycles, one copy per row takes 2200 cycles to issue: 4099 tokens, 16 shards, heads of 64 389 -> 361 us.)  Boxes
-      // that would reach past the rows of the shard are left to the threads.
+      // kWalk: writes this warp's finished rows from TMEM, scaled.  kBoxes: through shared memory to the copy engine, as a box
+      // (4099 tokens in 16 shards, 32 / 8 heads of 64 columns: 389 -> 361 us); a box that would reach past the rows of the shard
+      // is left to the threads.  Otherwise every thread stores its own row, 32 bytes at a time.  (At D = 128 the staging area
+      // would have to take the place of the second K and V stages.  That gained 2 % at 4099 tokens in 16 shards of 8-token
+      // clusters and lost up to 25 % where shards are short or a KV head has few query heads, so that many boxes do not fit
+      // the rows of a shard: 500 tokens in 32 random shards, 8 / 8 heads, 146 us and 195 with boxes.  Staging half a row, with
+      // the second K stage back, still lost up to 16 %.)
       const int warp_row0 = sub_row0 + (((warp & 3) * 32) >> lg);
-      const bool boxed = tma.o_valid && warp_row0 + (32 >> lg) <= sub_row0 + sub_nrows;
+      const bool boxed = C::kBoxes && tma.o_valid && warp_row0 + (32 >> lg) <= sub_row0 + sub_nrows;
+      const bool rows32 = (reinterpret_cast<uint64_t>(p.o_part) & 31) == 0;  // rows are multiples of 128 bytes
       auto store_rows = [&](float scale, bool have, int z, __nv_bfloat16* dst) {
         uint8_t* stage = smem + C::kOffStage + warp * C::kStageWarpBytes;
-        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the previous rows have left
-        __syncwarp();
+        if constexpr (C::kBoxes) {
+          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the previous rows have left
+          __syncwarp();
+        }
 #pragma unroll
         for (int half = 0; half < C::kHalves; ++half) {
           uint32_t o[64];
@@ -822,26 +828,39 @@ if constexpr (kRope) {
 #pragma unroll
             for (int j = 0; j < 64; ++j) o[j] = 0u;
           }
-#pragma unroll
-          for (int j = 0; j < 64; j += 8) {
+          auto packed = [&](int j) {
             uint4 val;
             val.x = pack_bf16x2(__uint_as_float(o[j]) * scale, __uint_as_float(o[j + 1]) * scale);
             val.y = pack_bf16x2(__uint_as_float(o[j + 2]) * scale, __uint_as_float(o[j + 3]) * scale);
             val.z = pack_bf16x2(__uint_as_float(o[j + 4]) * scale, __uint_as_float(o[j + 5]) * scale);
             val.w = pack_bf16x2(__uint_as_float(o[j + 6]) * scale, __uint_as_float(o[j + 7]) * scale);
-            if (boxed)
-              *reinterpret_cast<uint4*>(stage + half * 4096 + lane * 128 + (((j >> 3) ^ (lane & 7)) << 4)) = val;
-            else if (row_ok)
-              *reinterpret_cast<uint4*>(dst + half * 64 + j) = val;
+            return val;
+          };
+          if (boxed) {
+#pragma unroll
+            for (int j = 0; j < 64; j += 8)
+              *reinterpret_cast<uint4*>(stage + lane * 128 + (((j >> 3) ^ (lane & 7)) << 4)) = packed(j);
+          } else if (row_ok) {
+#pragma unroll
+            for (int j = 0; j < 64; j += 16) {
+              const uint4 a = packed(j), b2 = packed(j + 8);
+              __nv_bfloat16* to = dst + half * 64 + j;
+              if (rows32) {
+                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(to), "r"(a.x), "r"(a.y), "r"(a.z),
+                             "r"(a.w), "r"(b2.x), "r"(b2.y), "r"(b2.z), "r"(b2.w)
+                             : "memory");
+              } else {
+                *reinterpret_cast<uint4*>(to) = a;
+                *reinterpret_cast<uint4*>(to + 8) = b2;
+              }
+            }
           }
         }
         if (boxed) {
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // this thread's writes -> the copy engine's reads
           __syncwarp();
           if (lane == 0) {
-#pragma unroll
-            for (int half = 0; half < C::kHalves; ++half)
-              tma_store4(&tma.o, half * 64, h0, warp_row0, z, smem_u32(stage + half * 4096));
+            tma_store4(&tma.o, 0, h0, warp_row0, z, smem_u32(stage));
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           }
         }
@@ -1223,7 +1242,7 @@ if constexpr (kRope) {
           p.l_part[stat] = l_out;
         }
       }
-      if constexpr (kWalk) {
+      if constexpr (C::kBoxes) {
         store_rows(o_scale, n_tiles > 0, b * P + max(kk_open, 0), dst);
         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the rows have left shared memory
       } else {
@@ -1628,7 +1647,8 @@ cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, c
   }
   const int lg = stacked_log2(p.G);
   const int64_t n_q = p.plan.n_q;
-  tma.o_valid = encode_out(&tma.o, p.o_part, p.d, lg, p.H, n_q, (int64_t)p.batch * p.plan.n_kv_shards,
+  tma.o_valid = tc::Cfg<64, true>::kBoxes && p.d == 64 &&
+                encode_out(&tma.o, p.o_part, p.d, lg, p.H, n_q, (int64_t)p.batch * p.plan.n_kv_shards,
                            {n_q * p.H * p.d, (int64_t)p.H * p.d, p.d});
   const int64_t n_ctas = (int64_t)p.plan.n_qtiles[3 - lg] * (p.H >> lg) * p.batch;
   // few CTAs per SM: balance matters more than L2 locality
