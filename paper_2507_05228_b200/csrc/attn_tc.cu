@@ -108,7 +108,7 @@ struct Cfg {
   static constexpr int kOffStage = kBoxes ? kOffV + kVStages * kTileBytes : kOffQ;
   static constexpr int kOffBar = kOffV + kVStages * kTileBytes + (kBoxes ? kStageBytes : 0);
   static_assert(kBoxes || kStageBytes <= kOffV, "the output staging area must fit in the Q and K tiles");
-  static constexpr int kNumBars = 30;
+  static constexpr int kNumBars = 32;
   static constexpr int kOffMisc = kOffBar + kNumBars * 8;   // tmem slot, abort flag, 12 progress words
   static constexpr int kOffShard = kOffMisc + 64;           // int32 [5][kMaxShards], see ShardTab
   static constexpr int kSmemBytes = kOffShard + 5 * kMaxShards * 4 + 1024;  // + alignment slack
@@ -124,7 +124,8 @@ enum Bar {
   S_FULL = V_EMPTY + kMaxStages,    // [2]; kRing: [2][2], see s_full
   P_FULL = S_FULL + 4,              // [2]; kRing: [2][2], see p_full
   O_FULL = P_FULL + 4,              // [1]
-  O_RDY = O_FULL + 1                // [2]  kWalk: the accumulator of a sub-tile holds a finished shard;
+  CHECKED = O_FULL + 1,             // [1] the plan's status word has been looked at
+  O_RDY = CHECKED + 1               // [2]  kWalk: the accumulator of a sub-tile holds a finished shard;
                                     //      kRing: the product of a sub-tile's latest tile is in its accumulator
 };
 static_assert(O_RDY + 2 <= Cfg<128, false>::kNumBars, "barrier table too small");
@@ -592,10 +593,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       }
     }
   }
-  if (warp == 11) {  // the warp without a role of its own
-    // Whether a wait of an earlier call on this plan gave up: then this one writes nothing.  Looked up here, beside the set-up
-    // of the others, the load costs nothing (before the set-up, 1000 cycles).
-    const int32_t gave_up = *reinterpret_cast<volatile int32_t*>(pl.status);
+  int32_t gave_up = 0;  // warp 11: whether a wait of an earlier call on this plan gave up; used after the set-up
+  if (warp == 11) {     // the warp without a role of its own
+    asm volatile("ld.volatile.global.s32 %0, [%1];" : "=r"(gave_up) : "l"(pl.status) : "memory");
     if constexpr (kWalk) {
       // Compact the shards of which the CTA's last row (longest prefix; rows ascend) sees something, with what the
       // roles need per shard, and count the tiles of the stream.
@@ -635,7 +635,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       }
       if (lane == 1 || lane == 2) tab->first[lane - 1][0] = seen;
     }
-    if (lane == 0 && gave_up) stream_info[1] = -1;
   }
   WaitCtx<kWalk> wc;
   if constexpr (kWalk) wc.words = reinterpret_cast<volatile int*>(smem + kOffMisc);
@@ -664,6 +663,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       mbar_init(bar(P_FULL + 2 + s), 128);
     }
     mbar_init(bar(O_FULL), 1);
+    mbar_init(bar(CHECKED), 1);
     mbar_init(bar(O_RDY), 1);
     mbar_init(bar(O_RDY + 1), 1);
     wc.store(1, 0);
@@ -710,27 +710,65 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const int n_act = stream_info[0];  // kWalk: shards of which the CTA sees something
-  const int n_tiles = stream_info[1];  // -1: write nothing
+  const int n_tiles = stream_info[1];
   // not kWalk: first key and number of keys of this CTA's part of the stream
   const int key0 = kWalk ? 0 : tab->slot0[0], n_keys = kWalk ? 0 : tab->need[0];
   // MMA tiles of four chunks; only the last one is narrower, or with kWalk the last one of every shard (see TileSeq)
   auto tile_chunks = [&](int i) { return min(4, (n_keys - kNMax * i + kChunk - 1) / kChunk); };
 
-  if (n_tiles < 0) {
-    // an earlier call gave up: what was requested lands, the cluster's other CTAs find this one's shared memory there
-    for (uint32_t left = requested; left; left &= left - 1)
-      for (int i = 0; i < 1 << 20 && !mbar_try_wait(bar(__ffs(left) - 1), 0u); ++i) {
-      }
-    __syncwarp();
-    if (!kWalk && split > 1) {
-      cluster_barrier();
-      cluster_barrier();
-    }
-  } else if (warp < 8) {
+  // Once a wait has given up, later calls on the plan write nothing.  Warp 11 looks the word up during the set-up and every role
+  // asks here before it goes to work; by then its first data are still on their way.  (Looked up by all before the set-up the
+  // word costs 1000 cycles, joined to the barrier above 500: 500 tokens, 32 / 8 heads, 15.4 -> 15.9 us.)
+  auto goes_on = [&]() {
+    wait_bar(wc, bar(CHECKED), 0u, 11);
+    return wc.load(1) == 0;
+  };
+
+  if (warp < 8) {
     // ------------------------------------------------------------------ softmax + epilogue
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
     const int s = warp >> 2;  // sub-tile
-    if (s < n_sub) {
+    if (s < n_sub && n_tiles > 0 && !q_boxes) {
+      if constexpr (kRope) {
+        // q <- rotary_pos_emb(q, p): (lo, hi) = (x[i], x[i + 64]) -> (lo cos - hi sin, hi cos + lo sin) in fp32,
+        // rounded once to bf16, then stored like the unrotated rows
+        uint8_t* q_tile = smem + kOffQ + s * kTileBytes;
+        const int c = tid & 7;
+        auto turn_and_store = [&](int j, const float4 (&t)[4]) {
+          __nv_bfloat162* lo = reinterpret_cast<__nv_bfloat162*>(&qv[2 * j]);
+          __nv_bfloat162* hi = reinterpret_cast<__nv_bfloat162*>(&qv[2 * j + 1]);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float2 a = __bfloat1622float2(lo[e]), h = __bfloat1622float2(hi[e]);
+            lo[e] = __floats2bfloat162_rn(a.x * t[e].x - h.x * t[e].y, a.y * t[e].z - h.y * t[e].w);
+            hi[e] = __floats2bfloat162_rn(h.x * t[e].x + a.x * t[e].y, h.y * t[e].z + a.y * t[e].w);
+          }
+          const int r = (tid >> 3 & 15) + 16 * j;
+          uint8_t* dst = q_tile + r * 128 + ((c ^ (r & 7)) << 4);
+          *reinterpret_cast<uint4*>(dst) = qv[2 * j];
+          *reinterpret_cast<uint4*>(dst + kHalfBytes) = qv[2 * j + 1];
+        };
+        float4 cs2[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) cs2[j][e] = __ldg(rope_row[4 + j] + e);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) turn_and_store(j, cs[j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) turn_and_store(4 + j, cs2[j]);
+      } else {
+        uint8_t* q_tile = smem + kOffQ + s * kTileBytes + (q_chunk >> 3) * kHalfBytes;
+#pragma unroll
+        for (int j = 0; j < kRowChunks; ++j) {
+          const int r = q_row + kRowsPerPass * j;
+          *reinterpret_cast<uint4*>(q_tile + r * 128 + (((q_chunk & 7) ^ (r & 7)) << 4)) = qv[j];
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> tensor-core reads
+      mbar_arrive(bar(Q_FULL + s));
+    }
+    if (s < n_sub && goes_on()) {
       const int m = tid & 127;  // MMA row = TMEM lane
       const int sub_row0 = row0 + s * R;
       const int sub_nrows = min(R, nrows - s * R);
@@ -753,46 +791,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       float m_run = -INFINITY;   // reference max the accumulators are scaled by (may lag by < 2^8)
       float m_true = -INFINITY;  // exact running max
       float l_run = 0.f;
-      if (n_tiles > 0 && !q_boxes) {
-if constexpr (kRope) {
-          // q <- rotary_pos_emb(q, p): (lo, hi) = (x[i], x[i + 64]) -> (lo cos - hi sin, hi cos + lo sin) in fp32,
-          // rounded once to bf16, then stored like the unrotated rows
-          uint8_t* q_tile = smem + kOffQ + s * kTileBytes;
-          const int c = tid & 7;
-          auto turn_and_store = [&](int j, const float4 (&t)[4]) {
-            __nv_bfloat162* lo = reinterpret_cast<__nv_bfloat162*>(&qv[2 * j]);
-            __nv_bfloat162* hi = reinterpret_cast<__nv_bfloat162*>(&qv[2 * j + 1]);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float2 a = __bfloat1622float2(lo[e]), h = __bfloat1622float2(hi[e]);
-              lo[e] = __floats2bfloat162_rn(a.x * t[e].x - h.x * t[e].y, a.y * t[e].z - h.y * t[e].w);
-              hi[e] = __floats2bfloat162_rn(h.x * t[e].x + a.x * t[e].y, h.y * t[e].z + a.y * t[e].w);
-            }
-            const int r = (tid >> 3 & 15) + 16 * j;
-            uint8_t* dst = q_tile + r * 128 + ((c ^ (r & 7)) << 4);
-            *reinterpret_cast<uint4*>(dst) = qv[2 * j];
-            *reinterpret_cast<uint4*>(dst + kHalfBytes) = qv[2 * j + 1];
-          };
-          float4 cs2[4][4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) cs2[j][e] = __ldg(rope_row[4 + j] + e);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) turn_and_store(j, cs[j]);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) turn_and_store(4 + j, cs2[j]);
-        } else {
-          uint8_t* q_tile = smem + kOffQ + s * kTileBytes + (q_chunk >> 3) * kHalfBytes;
-#pragma unroll
-          for (int j = 0; j < kRowChunks; ++j) {
-            const int r = q_row + kRowsPerPass * j;
-            *reinterpret_cast<uint4*>(q_tile + r * 128 + (((q_chunk & 7) ^ (r & 7)) << 4)) = qv[j];
-          }
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> tensor-core reads
-        mbar_arrive(bar(Q_FULL + s));
-      }
       // This row's prefix lengths in the current and the next three active shards (a tile spans at most four), fetched
       // as the stream moves on so that the loads are off the critical path.
       auto row_vis = [&](int j) { return (kWalk && j < n_act && row_ok) ? __ldg(vis_row + tab->kk[j]) : 0; };
@@ -1321,7 +1319,7 @@ if constexpr (kRope) {
       const uint32_t q_lo0 = desc_lo(smem_base + kOffQ, 16);
       const uint32_t k_lo0 = desc_lo(smem_base + kOffK, 16);
       const uint32_t v_lo0 = desc_lo(smem_base + kOffV, kHalfBytes);  // the two 64-column halves of d
-      if (n_tiles > 0) {
+      if (n_tiles > 0 && goes_on()) {
         auto s_col = [&](int s, int i) {  // logit buffer of sub-tile s, tile i
           return tmem + (uint32_t)((kRing ? (2 * i + s) % 3 : s) * 128);
         };
@@ -1450,7 +1448,18 @@ if constexpr (kRope) {
       // from "one phase ahead", so a warp must never skip a use of a stage.
       //   warp 9: the K tiles, warp 10: the V tiles (warp 11 has no work).
       const int lw = warp - 9;
-      if (n_tiles > 0 && lw < 2) {
+      if (lw == 2) {
+        if (lane == 0) {
+          if (gave_up) wc.store(1, 1);
+          mbar_arrive(bar(CHECKED));
+        }
+      } else if (!goes_on()) {
+        // what was requested during the set-up lands before the CTA ends
+        for (uint32_t left = requested; left; left &= left - 1)
+          for (int i = 0; i < 1 << 20 && !mbar_try_wait(bar(__ffs(left) - 1), 0u); ++i) {
+          }
+        __syncwarp();
+      } else if (n_tiles > 0) {
         const bool is_k = lw == 0;
         const CUtensorMap* map = is_k ? &tma.k : &tma.v;
         const int z = b * p.Hkv + g;  // kWalk: which [n_kv][head_dim] matrix of the shard-major copy
