@@ -1678,13 +1678,15 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
   const int64_t n_ctas = n_qt * (p.H >> lg) * p.batch;
   // Few query tiles (a chunk of a chunked prefill, a short prompt) leave SMs idle: a cluster then shares the keys of each
   // tile, as far as its CTAs fit at once with one per SM (clusters of 2, 4 and 8: 148, 132 and 120 CTAs) and have two
-  // 128-key tiles each.  The rule counts the heads of the whole problem, see AttnParams.
+  // 128-key tiles each.  Three with a rotary step, where every CTA of a cluster turns the query rows for itself (32 / 8 heads,
+  // 500 tokens: 22.5 us in clusters of two, 18.5 without; 8 / 8 heads, 1000 tokens: 32.2 in clusters of four, 26.9 without;
+  // 1500 tokens 32.8 and 36.9).  The rule counts the heads of the whole problem, see AttnParams.
   const int64_t rule_ctas = n_qt * ((int64_t)p.rule_kv_heads * p.G >> lg) * p.batch, key_tiles = (n_seen + 127) / 128;
   int split = 1;
   if (p.fused) {
     const int64_t fit[4] = {148, 148, 132, 120};
     for (int i = 1; i < 4; ++i)
-      if (rule_ctas << i <= fit[i] && key_tiles >= 2 << i) split = 1 << i;
+      if (rule_ctas << i <= fit[i] && key_tiles >= (p.rope ? 3 : 2) << i) split = 1 << i;
   }
   const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), split,
                       p.prefix_from_vis ? 0 : (k_gathered ? 0 : 1) | (v_gathered ? 0 : 2), k_gathered || v_gathered};
