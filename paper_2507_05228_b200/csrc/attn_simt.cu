@@ -438,7 +438,8 @@ cudaError_t launch_one(const AttnParams& p, cudaStream_t stream) {
   auto parts_for = [&](int64_t base) {
     return p.fused ? 1 : (int)std::max<int64_t>(1, P / std::min<int64_t>(P, (enough + base - 1) / base));
   };
-  const bool fills = wide * heads * (p.fused ? 1 : P) >= enough;
+  // (which form runs decides how sums are split: it goes by the heads of the whole problem, see AttnParams)
+  const bool fills = wide * ((int64_t)p.rule_kv_heads * p.G * p.batch) * (p.fused ? 1 : P) >= enough;
   if (fills && wide * R4 * 4 <= narrow_rows * 6) return launch_rows<T, D, 4>(p, parts_for(wide * heads), stream);
   return launch_rows<T, D, 1>(p, parts_for(std::max<int64_t>(1, narrow_rows / R1) * heads), stream);
 }

@@ -59,3 +59,20 @@ def test_host_call_matches_oracle_and_device_call(cb, gu, case):
     assert ei.value.status == 4
     assert plan.device_status() == 0
     plan.destroy()
+
+
+def test_head_groups_take_the_form_of_the_whole_problem(cb, gu):
+    """512 fp32 tokens, 8 sequences, 8 heads: enough tiles for four row warps a block as a whole, not per head group.  The
+    host call computes the groups one by one and still gives the same bits as the device call."""
+    w = wl.make_workload("host_wide", 8, 512, 512, 8, 8, 64, "f32", "random", "random", 4, 4, seed=33)
+    plan = gu.make_plan(w)
+    hq, hk, hv = _host(w, w.q), _host(w, w.k), _host(w, w.v)
+    ho = torch.empty_like(hq).pin_memory()
+    ws = torch.empty(cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED_HOST, cb.F32, w.B, w.H, w.Hkv, w.d), dtype=torch.uint8,
+                     device="cuda")
+    cb.cascade_attn_sharded_host(plan, hq, hk, hv, w.scale, ho, ws)
+    torch.cuda.current_stream().synchronize()
+    q, k, v = gu.to_device(w)
+    o_dev, _ = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+    assert torch.equal(o_dev.cpu(), ho)
+    plan.destroy()
