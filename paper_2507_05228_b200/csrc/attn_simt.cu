@@ -95,6 +95,8 @@ struct SimtCfg {
   static_assert(kCtas * (kBytes + 1024) <= 233472, "CTAs per SM");
 };
 
+constexpr int64_t kEnough = 2 * 148;  // CTAs that fill the chip, two per SM
+
 // A tile of the key stream: per chunk of 16 keys its shard, its first key in the shard's list and its keys.
 template <int NC>
 struct SimtTile {
@@ -424,29 +426,56 @@ cudaError_t launch_rows(const AttnParams& p, int parts_per_cta, cudaStream_t str
   return cudaGetLastError();
 }
 
+// Whether four row warps share a CTA: when that fills the chip (two CTAs per SM) and does not pad the rows by more than what the
+// narrow form's four times larger K/V traffic costs.  It decides how sums are split, so it goes by the heads of the whole
+// problem (see AttnParams).
+bool use_wide(const AttnParams& p) {
+  const int64_t tiles = p.plan.n_qtiles[1], heads = (int64_t)p.rule_kv_heads * p.G * p.batch;
+  const int64_t narrow_rows = (int64_t)p.plan.n_q + (int64_t)p.plan.n_q_shards * 8;  // padded by half a piece a shard
+  return tiles * heads * (p.fused ? 1 : p.plan.n_kv_shards) >= kEnough && tiles * 64 * 4 <= narrow_rows * 6;
+}
+
+// partials: a CTA walks as many shards of its rows as leaves enough CTAs
+int parts_per_cta(const AttnParams& p, int64_t ctas) {
+  const int P = p.plan.n_kv_shards;
+  return p.fused ? 1 : (int)std::max<int64_t>(1, P / std::min<int64_t>(P, (kEnough + ctas - 1) / ctas));
+}
+int64_t narrow_pieces(const AttnParams& p) {
+  return std::max<int64_t>(1, ((int64_t)p.plan.n_q + (int64_t)p.plan.n_q_shards * 8) / 16);
+}
+
 template <typename T, int D>
 cudaError_t launch_one(const AttnParams& p, cudaStream_t stream) {
-  // Four row warps per CTA when that fills the chip (two CTAs per SM) and does not pad the rows by more than what the
-  // narrow form's four times larger K/V traffic costs; otherwise one row warp per CTA.
-  constexpr int R4 = SimtCfg<D, 4>::R, R1 = SimtCfg<D, 1>::R;
-  const int P = p.plan.n_kv_shards;
-  const int64_t wide = (int64_t)p.plan.n_qtiles[1];
-  const int64_t narrow_rows = (int64_t)p.plan.n_q + (int64_t)p.plan.n_q_shards * (R1 / 2);  // padded by half a piece a shard
   const int64_t heads = (int64_t)p.H * p.batch;
-  const int64_t enough = 2 * 148;
-  // partials: a CTA walks as many shards of its rows as leaves enough CTAs
-  auto parts_for = [&](int64_t base) {
-    return p.fused ? 1 : (int)std::max<int64_t>(1, P / std::min<int64_t>(P, (enough + base - 1) / base));
-  };
-  // (which form runs decides how sums are split: it goes by the heads of the whole problem, see AttnParams)
-  const bool fills = wide * ((int64_t)p.rule_kv_heads * p.G * p.batch) * (p.fused ? 1 : P) >= enough;
-  if (fills && wide * R4 * 4 <= narrow_rows * 6) return launch_rows<T, D, 4>(p, parts_for(wide * heads), stream);
-  return launch_rows<T, D, 1>(p, parts_for(std::max<int64_t>(1, narrow_rows / R1) * heads), stream);
+  if (use_wide(p)) return launch_rows<T, D, 4>(p, parts_per_cta(p, p.plan.n_qtiles[1] * heads), stream);
+  return launch_rows<T, D, 1>(p, parts_per_cta(p, narrow_pieces(p) * heads), stream);
 }
 
 }  // namespace
 
+// Estimated time in us, see rows_time.  At head_dim 64 a shard costs an SM 2 us and 6.2 us per 64 keys for 64 rows in the wide
+// form, and 2.4 us and 0.45 us (from the fifth on, 0.71) per 32 keys for 16 rows in the narrow one.
+double tiles_time(const AttnParams& p) {
+  const CutSize c(p);
+  const bool d64 = p.d == 64;
+  if (use_wide(p)) {
+    const double list = p.plan.n_qtiles[1];
+    const double seen = c.seen_by_last(list), chunks = c.pieces(seen, 16) * c.shards;  // of 16 keys, fused route
+    const double cta = d64 ? 2 + 6.2 * (p.fused ? chunks / 4 : c.pieces(seen, 64))
+                           : 2 + 5 * (p.fused ? chunks / 2 : c.pieces(seen, 32));
+    return list * c.heads * cta * (p.fused ? 1 : c.shards) / kEstimateSms;
+  }
+  const double pieces = c.row_tiles(16), seen = c.seen_by_last(pieces);
+  const double tiles = p.fused ? c.pieces(seen, 16) * c.shards / 2 : c.pieces(seen, 32);
+  const double cta = d64 ? 2.4 + 0.45 * std::min(tiles, 4.0) + 0.71 * std::max(0.0, tiles - 4)
+                         : 1 + (p.fused ? 10 : 7.2) * std::max(1.0, tiles / 4);
+  const double parts = parts_per_cta(p, std::max<int64_t>(1, (int64_t)(narrow_pieces(p) * c.heads)));
+  const double ctas = pieces * c.heads * (p.fused ? 1 : std::ceil(c.shards / parts));
+  return cta * parts * std::max(1.0, ctas / kEstimateSms);
+}
+
 cudaError_t launch_attn_simt(const AttnParams& p, cascade_dtype_t dtype, cudaStream_t stream) {
+  if (rows_time(p) < tiles_time(p)) return launch_attn_rows(p, dtype, stream);
   if (dtype == CASCADE_BF16) {
     if (p.d == 128) return launch_one<__nv_bfloat16, 128>(p, stream);
     return launch_one<__nv_bfloat16, 64>(p, stream);

@@ -1646,6 +1646,18 @@ bool tc_rows_loadable(const TcRows& r, int64_t n_rows, int64_t n_heads, int64_t 
   return fine(r.strides.token, n_rows) && fine(r.strides.head, n_heads) && fine(r.strides.batch, batch);
 }
 
+// Estimated time in us of the partials of several shards at head_dim 64, see rows_time: a CTA takes 2 to 3.2 us a shard (by how
+// many of its rows exist) and 1.5 us for every further 128 keys of it.  It is the wrong kernel for a query or KV shard of a few
+// tokens: 130 tokens in 40 shards, 12 / 12 heads, 338 us and 99 on the ALUs; 500 tokens in 40 shards 345 and 238, with 16 / 4
+// heads 176 and 317.
+double tc_partials_time(const AttnParams& p) {
+  const CutSize c(p);
+  const int lg = stacked_log2(p.G);
+  const double tiles = p.plan.n_qtiles[3 - lg], rows = p.plan.n_q / tiles;
+  const double shard = 2 + 1.2 * rows / (256 >> lg) + 1.5 * (std::ceil(c.keys / 128) - 1);
+  return std::ceil(tiles * (c.heads / (1 << lg)) / kEstimateSms) * (4 + c.shards * shard);
+}
+
 cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, const void* v_sorted, cudaStream_t stream) {
   tc::TmaArgs tma = {};
   const int64_t n_mats = (int64_t)p.batch * p.Hkv;

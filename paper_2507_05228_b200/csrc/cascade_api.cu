@@ -745,6 +745,11 @@ static bool tc_ws_given(const cascade_plan_t* plan, int batch, int Hkv, int d, c
   return workspace && bytes >= tc_ws_bytes(plan, batch, Hkv, d) && ((uintptr_t)workspace & 255) == 0;
 }
 
+// Partials over short shards of heads of 64 columns, in bf16: whether the ALU kernels beat the tensor cores.
+static bool alu_partials_faster(const AttnParams& p) {
+  return p.plan.n_kv_shards > 1 && (int64_t)p.batch * p.plan.n_kv_shards <= 65535 && rows_time(p) < tc_partials_time(p);
+}
+
 static bool is_capturing(cudaStream_t st) {
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {  // (the default stream beside a capture: the launch will say so)
@@ -940,7 +945,8 @@ cascade_status_t cascade_attn_partials(const cascade_plan_t* plan, cascade_dtype
   if (use_decode(plan, dtype, n_heads, n_kv_heads, head_dim)) {
     e = launch_decode(p, st);
   } else if (use_tc(plan, dtype, head_dim) &&
-             (head_dim == 128 || tc_ws_given(plan, batch, n_kv_heads, head_dim, workspace, workspace_bytes))) {
+             (head_dim == 128 || (tc_ws_given(plan, batch, n_kv_heads, head_dim, workspace, workspace_bytes) &&
+                                  !alu_partials_faster(p)))) {
     cascade_status_t ws = run_tc(p, "cascade_attn_partials", plan, workspace, workspace_bytes, st, &e);
     if (ws != CASCADE_OK) return ws;
   } else {

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <cmath>
 #include <utility>
 #include <vector>
 
@@ -184,7 +186,44 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, unsigned block, si
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// How a problem is cut, for the estimates by which a kernel is chosen.  They go by the heads of the whole problem, see
+// AttnParams, and by the SMs of the GPU on which they were measured.
+constexpr double kEstimateSms = 148;
+struct CutSize {
+  double heads, shards, q_shards, keys;  // (query head, sequence) pairs; KV shards, query shards; keys per KV shard
+  double n_q, n_kv, first;               // first: position of the first query row
+  bool causal;
+  explicit CutSize(const AttnParams& p)
+      : heads((double)p.rule_kv_heads * p.G * p.batch), shards(p.plan.n_kv_shards),
+        q_shards(std::min(p.plan.n_q_shards, p.plan.n_q)), keys((double)p.plan.n_kv / p.plan.n_kv_shards), n_q(p.plan.n_q),
+        n_kv(p.plan.n_kv), first(p.plan.q_pos_offset), causal(p.plan.causal != 0) {}
+  // share of the keys that the query row at x n_q sees
+  double seen_at(double x) const { return causal ? std::max(0.0, std::min(1.0, (first + x * n_q + 1) / n_kv)) : 1.0; }
+  // the same for the last rows of tiles that do not cross shards, on average: rows ascend in a shard and spread over the sequence
+  double seen_by_last(double tiles) const {
+    const double per = std::max(1.0, tiles / q_shards), rows = n_q / q_shards;
+    return seen_at((per + 1) / (2 * per) * rows / (rows + 1));
+  }
+  // tiles of `height` rows that do not cross shards (of equal size)
+  double row_tiles(double height) const {
+    const double least = std::floor(n_q / q_shards), longer = n_q - least * q_shards;
+    return (q_shards - longer) * std::ceil(least / height) + longer * std::ceil((least + 1) / height);
+  }
+  // pieces of `width` keys in the visible prefix of a shard, on average
+  double pieces(double seen, double width) const {
+    const double all = std::ceil(keys / width);
+    if (seen >= 1) return all;
+    const double none = std::min(1.0, 2 * (1 - seen) / (keys + 1));
+    return std::min(all, keys <= width ? 1 - none : seen * keys / width + 0.5);
+  }
+};
+double rows_time(const AttnParams& p);         // attn_rows.cu
+double tiles_time(const AttnParams& p);        // attn_simt.cu
+double tc_partials_time(const AttnParams& p);  // attn_tc.cu, partials of several shards at head_dim 64
+
 // Launchers; each returns a cudaError_t from the launch.
+cudaError_t launch_attn_rows(const AttnParams& p, cascade_dtype_t dtype, cudaStream_t stream);
+// the faster of attn_simt.cu and attn_rows.cu
 cudaError_t launch_attn_simt(const AttnParams& p, cascade_dtype_t dtype, cudaStream_t stream);
 // K or V rows [batch][kv_heads][rows][d] for the tensor-core kernel (strides in elements)
 struct TcRows {

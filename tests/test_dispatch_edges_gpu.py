@@ -143,6 +143,21 @@ def test_new_plans_have_the_same_arrays_on_the_device(gu, n_q, n_kv, P, causal):
         plan.destroy()
 
 
+@pytest.mark.parametrize("n_q,n_kv,H,Hkv,d,B,J,P,dtype,causal", [
+    (64, 64, 16, 16, 64, 1, 32, 32, "f32", True),     # partials of two rows and two keys each
+    (64, 64, 4, 2, 64, 8, 64, 4, "f32", True),        # fused route, one row per shard: one row of a tile of 32
+    (333, 333, 8, 8, 64, 1, 32, 12, "f32", False),    # tiles of 10 rows, the last tile of a shard short of keys
+    (130, 130, 12, 12, 64, 1, 40, 40, "bf16", True),  # heads of 64 in bf16: partials on the ALUs, the fused call on the tensor cores
+    (128, 128, 8, 2, 128, 2, 128, 2, "f32", True),    # head_dim 128
+    (1, 1000, 16, 16, 64, 8, 1, 8, "bf16", True),     # one query row
+    (300, 300, 4, 2, 128, 1, 290, 280, "bf16", True), # more shards than the tensor cores take, some of them empty
+])
+def test_row_kernel_forms(gu, n_q, n_kv, H, Hkv, d, B, J, P, dtype, causal):
+    """Problems cut so fine that a query row at a time is the faster way."""
+    gu.full_parity(wl.make_workload(f"rows_{n_q}_{d}", B, n_q, n_kv, H, Hkv, d, dtype, "random", "random", J, P, seed=n_q + d,
+                                    causal=causal, symmetric=False, q_pos_offset=n_kv - n_q))
+
+
 @pytest.mark.parametrize("n_q,n_kv,same,n_maps", [
     (1, 1, True, 1), (333, 333, True, 2), (333, 333, False, 2), (65536, 65536, True, 1), (1, 65537, False, 1), (65537, 65537, True, 1)])
 def test_plan_lists_go_up_narrow_and_once(gu, n_q, n_kv, same, n_maps):
