@@ -541,15 +541,37 @@ static cudaError_t with_group(int G, F f) {
   }
 }
 
+// CTAs per (KV head, sequence) where there are more than 128 pairs: the cluster size of 1 to 6 with the least estimated time.
+// 296 CTAs fit at once (two per SM; about 280 in clusters that do not divide a GPC's share).  A round of them takes 8 us and
+// what its CTAs take: 2 us per 16-key block of a warp, or what the reads of the round need at 6.8 TB/s, whichever is more; a
+// last round with few CTAs is bound by the former.  (One CTA per pair left 24 CTAs to a second round at 320 pairs of 16000
+// keys: 568 us, 5 per pair 403; 160 pairs 259 us, 3 per pair 200; 512 pairs 606 us, 2 per pair 638.  At 61 numbers of pairs
+// from 144 to 600 and 500 to 16000 keys the choice is within 4 % of the fastest.)
+static int cluster_for_many(int64_t pairs, int64_t blocks, int64_t most) {
+  int best = 1;
+  double least = 0;
+  for (int n = 1; n <= std::min<int64_t>(6, most); ++n) {
+    const int64_t fit = n <= 2 ? 296 : 280, ctas = pairs * n, rest = ctas % fit;
+    const double alone = 2.0 * blocks / (8 * n), reads = fit * (blocks * 16 * 512.0) / n / 6.8e6;  // us
+    const double t = (double)(ctas / fit) * (std::max(alone, reads) + 8) +
+                     (rest ? std::max(alone, reads * rest / fit) + 8 : 0.0);
+    if (n == 1 || t < least) {
+      best = n;
+      least = t;
+    }
+  }
+  return best;
+}
+
 cudaError_t launch_decode_fused(const AttnParams& p, const DecodeStep& step, int64_t n_visible, cudaStream_t stream) {
   // CTAs (of eight warps) per (KV head, sequence): 256 in all, which is what two per SM on most of the chip come to with
-  // every warp's loads in flight; more only repeat the set-up (64 sequences of 16384 tokens: 1 per pair 620 us, 2 653 us; 16
-  // sequences: 2 159 us, 4 163 us, 1 165 us).  At most 10 where several pairs want the chip: clusters of 10 fit 11 times
-  // with one CTA per SM, clusters of 16 only 7 times (one sequence: 10 per pair 20.7 us, 16 22.8 us).  No more than give
-  // every warp a block.  `rule_kv_heads` counts the heads of the whole problem where a call computes a part of them.
+  // every warp's loads in flight; more only repeat the set-up (16 sequences of 16384 tokens: 2 per pair 159 us, 4 163 us, 1
+  // 165 us).  At most 10 where several pairs want the chip: clusters of 10 fit 11 times with one CTA per SM, clusters of 16
+  // only 7 times (one sequence: 10 per pair 20.7 us, 16 22.8 us).  No more than give every warp a block.  More than 128 pairs:
+  // see above.  `rule_kv_heads` counts the heads of the whole problem where a call computes a part of them.
   const int64_t pairs = (int64_t)p.rule_kv_heads * p.batch, blocks = std::max<int64_t>(1, (n_visible + 15) / 16);
-  const int64_t most = pairs <= 7 ? kMaxCluster : 10;
-  const int n_cta = (int)std::max<int64_t>(1, std::min(std::min(256 / pairs, most), (blocks + 7) / 8));
+  const int64_t most = std::min<int64_t>(pairs <= 7 ? kMaxCluster : 10, (blocks + 7) / 8);
+  const int n_cta = pairs > 128 ? cluster_for_many(pairs, blocks, most) : (int)std::max<int64_t>(1, std::min(256 / pairs, most));
   TimedLaunch timed(stream);
   return with_group(p.G, [&](auto g) { return launch_fused<decltype(g)::value>(p, step, n_cta, stream); });
 }

@@ -181,6 +181,8 @@ def test_plan_lists_go_up_narrow_and_once(gu, n_q, n_kv, same, n_maps):
     (1, 9000, 8, 1, 300, "random", 8999),    # more shards than one table window
     (5, 700, 4, 1, 7, "random", 699),        # fewer than eight (KV head, sequence) pairs: the largest clusters
     (40, 333, 32, 8, 5, "block_rr", 300),    # more pairs than 256: one CTA each
+    (20, 2000, 32, 8, 8, "random", 1999),    # more than 128 pairs: clusters of three or more, the last round partly filled
+    (45, 1500, 16, 8, 4, "random", 1400),    # clusters of four or five
 ])
 def test_fused_decode_forms(gu, B, n_kv, H, Hkv, P, kv_map, pos):
     gu.full_parity(wl.make_workload(f"dec_{B}_{n_kv}", B, 1, n_kv, H, Hkv, 128, "bf16", "round_robin", kv_map, 1, P,
