@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   }
   int32_t gave_up = 0;  // warp 11: whether a wait of an earlier call on this plan gave up; used after the set-up
   if (warp == 11) {     // the warp without a role of its own
-    asm volatile("ld.volatile.global.s32 %0, [%1];" : "=r"(gave_up) : "l"(pl.status) : "memory");
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(gave_up) : "l"(pl.status) : "memory");
     if constexpr (kWalk) {
       // Compact the shards of which the CTA's last row (longest prefix; rows ascend) sees something, with what the
       // roles need per shard, and count the tiles of the stream.
@@ -644,7 +644,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     if (lane == 0) wc.note(warp, v);
   };
 
-  uint32_t requested = 0;  // barriers of the boxes requested below (one bit each)
   if (tid == 9 * 32) {
     mbar_init(bar(Q_FULL), q_boxes ? 1 : 128);  // 128: every thread of the sub-tile's softmax group brings a share of the rows
     mbar_init(bar(Q_FULL + 1), q_boxes ? 1 : 128);
@@ -678,23 +677,20 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       if (tiles * (part_of_keys + 1) / split > t0) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         auto request_q = [&](int s) {
-          requested |= 1u << (Q_FULL + s);
           mbar_expect_tx(bar(Q_FULL + s), (uint32_t)kTileBytes);
           for (int half = 0; half < C::kHalves; ++half)
             tma_tile4(smem_base + (uint32_t)(kOffQ + s * kTileBytes + half * kHalfBytes), &tma.q, 64 * half, h0, row0 + s * R, b,
                       bar(Q_FULL + s));
         };
-        auto request_kv = [&](const CUtensorMap* map, uint32_t dst, int full) {
-          const uint32_t fb = bar(full);
-          requested |= 1u << full;
+        auto request_kv = [&](const CUtensorMap* map, uint32_t dst, uint32_t fb) {
           mbar_expect_tx(fb, (uint32_t)kTileBytes);
           tma_tile4(dst, map, 0, t0 * kNMax, g, b, fb);
           if (C::kHalves == 2) tma_tile4(dst + (uint32_t)kHalfBytes, map, 64, t0 * kNMax, g, b, fb);
         };
         if (q_boxes) request_q(0);
-        if (early & 1) request_kv(&tma.k, smem_base + kOffK, K_FULL);
+        if (early & 1) request_kv(&tma.k, smem_base + kOffK, bar(K_FULL));
         if (q_boxes && n_sub == 2) request_q(1);
-        if (early & 2) request_kv(&tma.v, smem_base + kOffV, V_FULL);
+        if (early & 2) request_kv(&tma.v, smem_base + kOffV, bar(V_FULL));
       }
     }
   }
@@ -716,12 +712,17 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   // MMA tiles of four chunks; only the last one is narrower, or with kWalk the last one of every shard (see TileSeq)
   auto tile_chunks = [&](int i) { return min(4, (n_keys - kNMax * i + kChunk - 1) / kChunk); };
 
-  // Once a wait has given up, later calls on the plan write nothing.  Warp 11 looks the word up during the set-up and every role
-  // asks here before it goes to work; by then its first data are still on their way.  (Looked up by all before the set-up the
-  // word costs 1000 cycles, joined to the barrier above 500: 500 tokens, 32 / 8 heads, 15.4 -> 15.9 us.)
+  // Once a wait has given up, later calls on the plan write nothing.  Warp 11 looks the word up during the set-up; the others ask
+  // when their first data are there, and what they have requested lands before the CTA ends.  (Looked up by all before the
+  // set-up the word costs 1000 cycles, joined to the barrier above 900, asked for at once after it up to 1000 with 8 heads a
+  // tile: 1000 tokens, 64 / 8 heads, 26.0 -> 26.6 us.)
   auto goes_on = [&]() {
     wait_bar(wc, bar(CHECKED), 0u, 11);
     return wc.load(1) == 0;
+  };
+  auto landed = [&](uint32_t full) {  // a box that was requested, whatever the word says
+    for (int i = 0; i < 1 << 14 && !mbar_try_wait(full, 0u); ++i) {
+    }
   };
 
   if (warp < 8) {
@@ -768,7 +769,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> tensor-core reads
       mbar_arrive(bar(Q_FULL + s));
     }
-    if (s < n_sub && goes_on()) {
+    auto first_logits = [&]() {  // are issued only if the CTA goes on
+      if (n_tiles > 0) wait_bar(wc, s_full(s, 0), 0u, 1);
+      return goes_on();
+    };
+    if (s < n_sub && first_logits()) {
       const int m = tid & 127;  // MMA row = TMEM lane
       const int sub_row0 = row0 + s * R;
       const int sub_nrows = min(R, nrows - s * R);
@@ -1319,7 +1324,15 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       const uint32_t q_lo0 = desc_lo(smem_base + kOffQ, 16);
       const uint32_t k_lo0 = desc_lo(smem_base + kOffK, 16);
       const uint32_t v_lo0 = desc_lo(smem_base + kOffV, kHalfBytes);  // the two 64-column halves of d
-      if (n_tiles > 0 && goes_on()) {
+      auto first_data = [&]() {
+        wait_bar(wc, bar(K_FULL), 0u, 7);
+        wait_bar(wc, bar(Q_FULL), 0u, 6);
+        if (goes_on()) return true;
+        if (q_boxes)
+          for (int s = 0; s < n_sub; ++s) landed(bar(Q_FULL + s));
+        return false;
+      };
+      if (n_tiles > 0 && first_data()) {
         auto s_col = [&](int s, int i) {  // logit buffer of sub-tile s, tile i
           return tmem + (uint32_t)((kRing ? (2 * i + s) % 3 : s) * 128);
         };
@@ -1453,12 +1466,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           if (gave_up) wc.store(1, 1);
           mbar_arrive(bar(CHECKED));
         }
-      } else if (!goes_on()) {
-        // what was requested during the set-up lands before the CTA ends
-        for (uint32_t left = requested; left; left &= left - 1)
-          for (int i = 0; i < 1 << 20 && !mbar_try_wait(bar(__ffs(left) - 1), 0u); ++i) {
-          }
-        __syncwarp();
       } else if (n_tiles > 0) {
         const bool is_k = lw == 0;
         const CUtensorMap* map = is_k ? &tma.k : &tma.v;
@@ -1474,6 +1481,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         // (a no-op otherwise).  Nothing else in this kernel reads what the gather grid writes.
         grid_wait();
         for (int i = 0; i < n_tiles; ++i) {
+          if (i == 1 && !goes_on()) break;
           const int nch = kWalk ? min(4, cur.nc - cur.c) : tile_chunks(i);
           const int st = i % n_stages;
           note(8 * i + 1);
@@ -1503,6 +1511,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           __syncwarp();
           note(8 * i + 2);
         }
+        if (!goes_on()) landed(bar(full0));
       }
     }
     if (!kWalk && split > 1) {
