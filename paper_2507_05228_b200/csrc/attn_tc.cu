@@ -64,10 +64,11 @@ constexpr int kM = 128;                  // MMA rows per sub-tile
 constexpr int kNMax = 128;               // keys per KV tile (upper bound)
 constexpr int kHalfBytes = kM * 128;     // one 64-column half of a 128-row tile: 128 rows of 128 bytes
 constexpr uint32_t kTmemCols = 512;
-// How far a row may rise above its reference maximum before it is rescaled: by its logits (log2 units), or by the sum of a
-// tile's weights.  (bf16 and fp32 keep their relative precision at any scale; the sums of 2^20 tiles and the products with
-// values below 2^40 stay in range.)
-constexpr float kRescaleThreshold = 60.f;
+// How far a row may rise above its reference maximum before it is rescaled: by its logits (log2 units), or, where the maximum of
+// a tile comes after its weights (kLateMax), by the sum of the tile's weights.  (bf16 and fp32 keep their relative precision at
+// any scale; the sums of 2^20 tiles and the products with values below 2^40 stay in range.)  With weights of 8 bits and the
+// maximum at hand the bound is low: a row that a new key dominates is rescaled, so that the key's weight is 1 and exact.
+constexpr float kRescaleBf16 = 8.f, kRescaleTwoParts = 60.f;
 constexpr float kRescaleSum = 1.1529215e18f;  // 2^60
 // setmaxnreg only redistributes the registers the CTA was launched with (168 per thread x 384 threads = 64512), and
 // all four warps of an allocation group execute the same instruction: 8 warps x 32 x 216 + 4 warps x 32 x 72 = 64512.
@@ -793,9 +794,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       const uint32_t o_addr = kRing ? lane_base + C::kOCol + (uint32_t)(s * kD) : s_addr + C::kOCol;
       const float c = p.scale * 1.4426950408889634f;  // logits are kept in log2 units: x = s * scale * log2(e)
       const uint64_t c2 = pack2(c, c);
-      float m_run = -INFINITY;   // reference max the accumulators are scaled by (may lag by < 2^8)
+      float m_run = -INFINITY;   // reference max the accumulators are scaled by (may lag, see kRescaleBf16)
       float m_true = -INFINITY;  // exact running max
-      float l_run = 0.f;
+      float l_run = 0.f;         // sum of the weights; with !kLateMax and bf16 weights as the tensor core sees the largest
+      float l_fix = 0.f;         // kLateMax: what that adds to it, see top_error
       // This row's prefix lengths in the current and the next three active shards (a tile spans at most four), fetched
       // as the stream moves on so that the loads are off the critical path.
       auto row_vis = [&](int j) { return (kWalk && j < n_act && row_ok) ? __ldg(vis_row + tab->kk[j]) : 0; };
@@ -998,7 +1000,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           smax = row_max();
           m_true = fmaxf(m_true, smax * c);
           float m_new = m_run;
-          if (m_run == -INFINITY || m_true > m_run + kRescaleThreshold) m_new = m_true;
+          if (m_run == -INFINITY || m_true > m_run + (kRing ? kRescaleTwoParts : kRescaleBf16)) m_new = m_true;
           alpha = (m_run == -INFINITY) ? 0.f : ex2(m_run - m_new);
           changed = m_new != m_run;
           m_run = m_new;
@@ -1097,6 +1099,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
             neg_m2 = pack2(neg_m, neg_m);
             l_run *= alpha;
+            l_fix *= alpha;
             rescale();
             tmem_wait_st();  // the first weights, too: the second ones go to the same place
             psum2 = pack2(0.f, 0.f);
@@ -1115,7 +1118,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             smax = row_max();
             m_true = fmaxf(m_true, smax * c);
           }
-          l_run += (psum0 + psum1) + top_error();
+          l_run += psum0 + psum1;
+          l_fix += top_error();
         }
         note(8 * i + 2);
       }
@@ -1155,7 +1159,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         for (int to = 0; to < split; ++to)
           if (to != me)
             st_cluster(stats + (uint32_t)((slot_of(me, to) * 2 * kM + row) * 16), to, __float_as_uint(m_run),
-                       __float_as_uint(l_run), 0u, 0u);
+                       __float_as_uint(l_run), __float_as_uint(l_fix), 0u);
         cluster_barrier();
         const uint8_t* got_stats = smem + kOffQ + (split - 1) * 2 * kM * pitch + row * 16;
         float f_of[7], m_all = m_run, l_all;  // the others' maxima, then their factors
@@ -1167,12 +1171,16 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         const float m_use = m_all == -INFINITY ? 0.f : m_all;
         const float f_me = ex2(m_run - m_use);
         l_all = l_run * f_me;
+        float fix_all = l_fix * f_me;
 #pragma unroll
         for (int i = 0; i < 7; ++i) {
           f_of[i] = ex2(f_of[i] - m_use);
-          if (i < split - 1) l_all += f_of[i] * *reinterpret_cast<const float*>(got_stats + i * 2 * kM * 16 + 4);
+          if (i < split - 1) {
+            l_all += f_of[i] * *reinterpret_cast<const float*>(got_stats + i * 2 * kM * 16 + 4);
+            fix_all += f_of[i] * *reinterpret_cast<const float*>(got_stats + i * 2 * kM * 16 + 8);
+          }
         }
-        const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+        const float inv = l_all > 0.f ? 1.f / (l_all + fix_all) : 0.f;
         __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.o_out) + (int64_t)b * p.os.batch + (int64_t)slot * p.os.token +
                              (int64_t)head * p.os.head + me * cols;
         for (int c0 = 0; c0 < cols; c0 += 8) {
@@ -1232,7 +1240,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         wait_bar(wc, bar(O_FULL), 0u, 3, n_tiles);
         tc_fence_after();
         if (l_run > 0.f) {
-          o_scale = 1.f / l_run;
+          o_scale = 1.f / (l_run + l_fix);
           l_out = l_run * ex2(m_run - m_true);  // sum relative to the exact max
           m_out = m_true * 0.6931471805599453f;   // natural-log units
         }

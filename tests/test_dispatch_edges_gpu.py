@@ -319,6 +319,27 @@ def test_logits_of_minus_infinity_before_finite_ones(gu, n_q, n_kv, hidden):
     plan.destroy()
 
 
+@pytest.mark.parametrize("n_q,n_kv", [(700, 700), (100, 4000)])  # the second shares keys in clusters
+def test_row_sums_where_few_keys_dominate(gu, n_q, n_kv):
+    """One key in a hundred is eight times as long, so a row's weight sits on a few keys of any tile.  The fused call sums the
+    weights in fp32: 2^-22 of each, and logits of up to 40 in fp32, 4e-6 on average with room.  The partials sum the largest
+    weight of a tile as its bf16 rounding, which is exact where the key became the reference: on average below a fifth of
+    bf16's half step of 2^-9."""
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload("peaked", 1, n_q, n_kv, 8, 2, 128, "bf16", "random", "random", 4, 8, seed=n_q, symmetric=False,
+                         q_pos_offset=n_kv - n_q, outlier_frac=0.01)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    _, lse = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+    _, lse_ref = oracle.attention_unsharded(w.q, w.k, w.v, w.scale, q_pos_offset=w.q_pos_offset)
+    assert np.abs(lse.double().cpu().numpy() - lse_ref).mean() < 4e-6
+    _, _, l = cb.cascade_attn_partials(plan, q, k, v, w.scale)
+    _, _, e = oracle.attn_pass(w.q, w.k, w.v, w.scale, gu.oracle_plan(w))
+    there = e > 0
+    assert (np.abs(l.double().cpu().numpy() - e)[there] / e[there]).mean() < 2.0 ** -9 / 5
+    plan.destroy()
+
+
 @pytest.mark.parametrize("n_maps", [1, 2])
 def test_fused_route_over_resident_rows(gu, n_maps):
     """Rows with positions of their own: a query sees those at positions up to its own, and what lies behind may be NaN."""
