@@ -88,19 +88,19 @@ constexpr int kMaxStages = 4;
 //            (sub-tile s, tile i: buffer (2 i + s) mod 3), so the next logits of a sub-tile are computed while it is still
 //            in the softmax of the current tile.  P is kept to twice the precision there: a bf16 part and the bf16
 //            rest, which together fill the 128 columns of the buffer they overwrite.
-// kWalk (partials) at D = 64 has a staging area of its own for finished rows.
-template <int D, bool kWalk>
+// kBoxes (partials, see launch_attn_tc_partials) has a staging area of its own for finished rows, which at D = 128 takes the place
+// of the second K and V stages.
+template <int D, bool kBoxes>
 struct Cfg {
   static constexpr int kHalves = D / 64;
   static constexpr int kTileBytes = kHalves * kHalfBytes;  // [halves][128 rows][128 bytes]
-  static constexpr int kKStages = D == 64 ? 4 : 2;  // (D = 128: a third stage bought nothing)
-  static constexpr int kVStages = D == 64 ? 3 : 2;
+  static constexpr int kKStages = D == 64 ? 4 : (kBoxes ? 1 : 2);  // (D = 128: a third stage bought nothing)
+  static constexpr int kVStages = D == 64 ? 3 : (kBoxes ? 1 : 2);
   static constexpr bool kRing = D == 64;                   // three logit buffers, P in two parts
   static constexpr uint32_t kOCol = kRing ? 384u : 256u;   // first accumulator column
   // Output rows.  The last ones of a CTA are staged where Q and K were, padded by 16 bytes; with kBoxes all of them in an area
-  // of their own, per warp [32 rows][128 bytes], swizzled like the operand tiles.
-  static constexpr bool kBoxes = kWalk && D == 64;
-  static constexpr int kStageWarpBytes = 32 * 128, kRowBytes = D * 2, kStageRowBytes = kRowBytes + 16;
+  // of their own, per warp [halves][32 rows][128 bytes], swizzled like the operand tiles.
+  static constexpr int kStageWarpBytes = kHalves * 32 * 128, kRowBytes = D * 2, kStageRowBytes = kRowBytes + 16;
   static constexpr int kStageBytes = kBoxes ? 8 * kStageWarpBytes : 2 * kM * kStageRowBytes;
   // shared memory map (offsets from a 1024-byte aligned base)
   static constexpr int kOffQ = 0;
@@ -446,7 +446,7 @@ struct TmaArgs {
   // kWalk: where finished rows go, o_part as [batch * KV shards][n_q slots][heads][head_dim]; a box is the rows of one warp:
   // 32 / Gp slots x Gp heads
   CUtensorMap o;
-  int o_valid;  // 0 (always so at head_dim 128): the threads store their rows themselves
+  int o_valid;  // 0: the threads store their rows themselves
   // Fused route without a rotary step: the query rows as [batch][tokens][heads][head_dim]; a box is one sub-tile, 128 / Gp
   // tokens x Gp heads, 64 columns
   int q_valid;  // 0: the threads load them
@@ -459,11 +459,11 @@ struct TmaArgs {
 // one after another): the shards are walked as in the fused mode, but a tile never mixes two shards, and at a shard
 // boundary the softmax threads write that shard's (u, m, l) out and start over.  The query tile, the TMEM allocation,
 // the barriers and the K/V pipelines are set up once per query tile instead of once per (query tile, KV shard).
-template <int D, bool kRope, bool kWalk>
+template <int D, bool kRope, bool kWalk, bool kBoxes>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_constant__ AttnParams p, int lg,
                                                               int tile_major, int split, int early, int after_gather,
                                                               const __grid_constant__ TmaArgs tma) {
-  using C = Cfg<D, kWalk>;
+  using C = Cfg<D, kBoxes>;
   constexpr int kD = D, kTileBytes = C::kTileBytes, kKStages = C::kKStages, kVStages = C::kVStages;
   constexpr int kOffQ = C::kOffQ, kOffK = C::kOffK, kOffV = C::kOffV, kOffMisc = C::kOffMisc;
   constexpr bool kRing = C::kRing;
@@ -806,19 +806,16 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       if (kWalk) cur.start(tab, n_act);
       int kk_open = -1;  // kWalk: the shard whose partial is being accumulated
       int n_flushed = 0;  // kWalk: partials written so far
-      // kWalk: writes this warp's finished rows from TMEM, scaled.  kBoxes: through shared memory to the copy engine, as a box
-      // (4099 tokens in 16 shards, 32 / 8 heads of 64 columns: 389 -> 361 us); a box that would reach past the rows of the shard
-      // is left to the threads.  Otherwise every thread stores its own row, 32 bytes at a time.  (At D = 128 the staging area
-      // would have to take the place of the second K and V stages.  That gained 2 % at 4099 tokens in 16 shards of 8-token
-      // clusters and lost up to 25 % where shards are short or a KV head has few query heads, so that many boxes do not fit
-      // the rows of a shard: 500 tokens in 32 random shards, 8 / 8 heads, 146 us and 195 with boxes.  Staging half a row, with
-      // the second K stage back, still lost up to 16 %.)
+      // kWalk: writes this warp's finished rows from TMEM, scaled.  kBoxes: through shared memory to the copy engine, a box per 64
+      // columns; a box that would reach past the rows of the shard is left to the threads.  (Stores from the threads, 32 bytes
+      // into each of 32 rows per instruction, keep a CTA's memory pipe busy for 3200 cycles, one copy per row takes 2200
+      // cycles to issue.)  Otherwise every thread stores its own row.
       const int warp_row0 = sub_row0 + (((warp & 3) * 32) >> lg);
-      const bool boxed = C::kBoxes && tma.o_valid && warp_row0 + (32 >> lg) <= sub_row0 + sub_nrows;
+      const bool boxed = kBoxes && tma.o_valid && warp_row0 + (32 >> lg) <= sub_row0 + sub_nrows;
       const bool rows32 = (reinterpret_cast<uint64_t>(p.o_part) & 31) == 0;  // rows are multiples of 128 bytes
       auto store_rows = [&](float scale, bool have, int z, __nv_bfloat16* dst) {
         uint8_t* stage = smem + C::kOffStage + warp * C::kStageWarpBytes;
-        if constexpr (C::kBoxes) {
+        if constexpr (kBoxes) {
           if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the previous rows have left
           __syncwarp();
         }
@@ -844,7 +841,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           if (boxed) {
 #pragma unroll
             for (int j = 0; j < 64; j += 8)
-              *reinterpret_cast<uint4*>(stage + lane * 128 + (((j >> 3) ^ (lane & 7)) << 4)) = packed(j);
+              *reinterpret_cast<uint4*>(stage + half * 4096 + lane * 128 + (((j >> 3) ^ (lane & 7)) << 4)) = packed(j);
           } else if (row_ok) {
 #pragma unroll
             for (int j = 0; j < 64; j += 16) {
@@ -865,7 +862,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // this thread's writes -> the copy engine's reads
           __syncwarp();
           if (lane == 0) {
-            tma_store4(&tma.o, 0, h0, warp_row0, z, smem_u32(stage));
+#pragma unroll
+            for (int half = 0; half < C::kHalves; ++half)
+              tma_store4(&tma.o, half * 64, h0, warp_row0, z, smem_u32(stage + half * 4096));
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           }
         }
@@ -1253,7 +1252,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           p.l_part[stat] = l_out;
         }
       }
-      if constexpr (C::kBoxes) {
+      if constexpr (kBoxes) {
         store_rows(o_scale, n_tiles > 0, b * P + max(kk_open, 0), dst);
         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the rows have left shared memory
       } else {
@@ -1632,15 +1631,17 @@ bool encode_queries(CUtensorMap* map, const AttnParams& p, int lg) {
 struct TcLaunch {
   int lg, tile_major, split, early;
   bool after_gather;
+  bool boxes;  // partials at head_dim 128
 };
 
 cudaError_t launch_kernel(const AttnParams& p, bool walk, const TcLaunch& l, int64_t n_ctas, const tc::TmaArgs& tma,
                           cudaStream_t stream) {
-  auto kernel = p.d == 64 ? (walk ? tc::attn_tc_kernel<64, false, true> : tc::attn_tc_kernel<64, false, false>)
-                : p.rope  ? tc::attn_tc_kernel<128, true, false>
-                          : (walk ? tc::attn_tc_kernel<128, false, true> : tc::attn_tc_kernel<128, false, false>);
+  auto kernel = p.d == 64 ? (walk ? tc::attn_tc_kernel<64, false, true, true> : tc::attn_tc_kernel<64, false, false, false>)
+                : p.rope  ? tc::attn_tc_kernel<128, true, false, false>
+                : !walk   ? tc::attn_tc_kernel<128, false, false, false>
+                          : (l.boxes ? tc::attn_tc_kernel<128, false, true, true> : tc::attn_tc_kernel<128, false, true, false>);
   const int smem_bytes = p.d == 64 ? (walk ? tc::Cfg<64, true>::kSmemBytes : tc::Cfg<64, false>::kSmemBytes)
-                                   : (walk ? tc::Cfg<128, true>::kSmemBytes : tc::Cfg<128, false>::kSmemBytes);
+                                   : (l.boxes ? tc::Cfg<128, true>::kSmemBytes : tc::Cfg<128, false>::kSmemBytes);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
   if (n_ctas * l.split >= (int64_t)1 << 31) return cudaErrorInvalidConfiguration;
@@ -1685,12 +1686,18 @@ cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, c
   }
   const int lg = stacked_log2(p.G);
   const int64_t n_q = p.plan.n_q;
-  tma.o_valid = tc::Cfg<64, true>::kBoxes && p.d == 64 &&
-                encode_out(&tma.o, p.o_part, p.d, lg, p.H, n_q, (int64_t)p.batch * p.plan.n_kv_shards,
-                           {n_q * p.H * p.d, (int64_t)p.H * p.d, p.d});
-  const int64_t n_ctas = (int64_t)p.plan.n_qtiles[3 - lg] * (p.H >> lg) * p.batch;
+  // Boxes: at head_dim 64 always (4099 tokens in 16 shards, 32 / 8 heads: 389 -> 361 us with the post-pass).  At head_dim 128, where
+  // they cost the second K and V stages, with at least four heads a tile (a box is 32 rows of (slot, head), so it seldom
+  // reaches past a shard) and query tiles that are nine tenths full, so that two sub-tiles hide each other's loads: 32 / 8
+  // heads, 2000 tokens in 32 shards 289 -> 256 us, 4099 in 16 348 -> 336.  Elsewhere they lose up to a quarter: 16 / 8 heads,
+  // 2000 tokens in 32 shards 199 and 226, 8 / 8 heads 178 and 222; 32 / 8 heads, 500 tokens in 32 shards 160 and 200.
+  const int64_t slots = 256 >> lg, n_tiles = p.plan.n_qtiles[3 - lg];
+  const bool boxes = p.d == 64 || (lg >= 2 && 10 * n_q >= 9 * n_tiles * slots);
+  tma.o_valid = boxes && encode_out(&tma.o, p.o_part, p.d, lg, p.H, n_q, (int64_t)p.batch * p.plan.n_kv_shards,
+                                    {n_q * p.H * p.d, (int64_t)p.H * p.d, p.d});
+  const int64_t n_ctas = n_tiles * (p.H >> lg) * p.batch;
   // few CTAs per SM: balance matters more than L2 locality
-  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), 1, 0, true};
+  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), 1, 0, true, boxes && tma.o_valid};
   return launch_kernel(p, true, l, n_ctas, tma, stream);
 }
 
@@ -1703,7 +1710,7 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
   }
   const int lg = stacked_log2(p.G);
   tma.q_valid = !p.rope && encode_queries(&tma.q, p, lg);
-  const int64_t tilslots = 256 >> lg, n_qt = (p.plan.n_q + tilslots - 1) / tilslots;
+  const int64_t tile_slots = 256 >> lg, n_qt = (p.plan.n_q + tile_slots - 1) / tile_slots;
   const int64_t n_ctas = n_qt * (p.H >> lg) * p.batch;
   // Few query tiles (a chunk of a chunked prefill, a short prompt) leave SMs idle: a cluster then shares the keys of each
   // tile, as far as its CTAs fit at once with one per SM (clusters of 2, 4 and 8: 148, 132 and 120 CTAs) and have two
@@ -1718,7 +1725,7 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
       if (rule_ctas << i <= fit[i] && key_tiles >= (p.rope ? 3 : 2) << i) split = 1 << i;
   }
   const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), split,
-                      p.prefix_from_vis ? 0 : (k_gathered ? 0 : 1) | (v_gathered ? 0 : 2), k_gathered || v_gathered};
+                      p.prefix_from_vis ? 0 : (k_gathered ? 0 : 1) | (v_gathered ? 0 : 2), k_gathered || v_gathered, false};
   return launch_kernel(p, false, l, n_ctas, tma, stream);
 }
 
