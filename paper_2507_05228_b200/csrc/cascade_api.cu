@@ -816,8 +816,9 @@ static cascade_status_t run_tc(AttnParams p, const char* fn, const cascade_plan_
         after.k_sorted = ws;
       }
       after.v = ws + each;
+      after.after_attention = true;
     }
-    *launch_error = launch_gather_kv_rope(p, before, false, st);
+    *launch_error = launch_gather_kv_rope(p, before, st);
     k_gathered = true;
     v_gathered = !v_fits;
   } else if (!v_fits || !tc_rows_loadable(k, n_seen, p.Hkv, p.batch) || (p.prefix_from_vis && d.n_maps > 1)) {
@@ -830,7 +831,7 @@ static cascade_status_t run_tc(AttnParams p, const char* fn, const cascade_plan_
     *launch_error = cudaSuccess;
   }
   if (*launch_error == cudaSuccess) *launch_error = launch_attn_tc(p, k, v, n_seen, k_gathered, v_gathered, st);
-  if (*launch_error == cudaSuccess && after.v) *launch_error = launch_gather_kv_rope(p, after, true, st);
+  if (*launch_error == cudaSuccess && after.v) *launch_error = launch_gather_kv_rope(p, after, st);
   return CASCADE_OK;
 }
 

@@ -244,9 +244,9 @@ struct RopeCopies {
   void *k_sorted, *k_tokens;  // keys in shard-major order, in token order
   void* v;                    // values, shard-major or in token order
   bool v_token_order;
+  bool after_attention;  // made when the attention kernel in front is done, otherwise before it
 };
-// dependent: launched as a programmatic dependent of the kernel in front, which writes none of its inputs
-cudaError_t launch_gather_kv_rope(const AttnParams& p, const RopeCopies& c, bool dependent, cudaStream_t stream);
+cudaError_t launch_gather_kv_rope(const AttnParams& p, const RopeCopies& c, cudaStream_t stream);
 cudaError_t launch_rope_table(int32_t n_positions, int32_t head_dim, double base, float2* table, cudaStream_t stream);
 cudaError_t launch_rope_apply(cascade_dtype_t dtype, int32_t batch, int32_t n_rows, int32_t n_heads, int32_t head_dim,
                               const void* x, Strides xs, int32_t first_position, const float2* table, void* y, Strides ys,

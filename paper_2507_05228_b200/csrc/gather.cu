@@ -87,12 +87,14 @@ __device__ __forceinline__ void rotate8(uint4& lo, uint4& hi, const float2* __re
 // key rows on the way: a key row is turned by the angles of its own token index, so the rotation needs nothing but
 // the row and its row of the positional table.  A thread holds both halves of 8 rotation pairs (columns 8c.. and
 // 64 + 8c..), 8 threads per row; V rows are copied as they are.  Of the copies those that are asked for are made.
-// Launched as a dependent (of the attention kernel, which still reads what is overwritten here) it loads and turns its rows
-// under the end of that kernel and stores them when it has completed.
+// A programmatic dependent of what is in front of it.  Before the attention kernel it waits first, so that by the time that
+// kernel may be set up (see gather_kv_kernel) all that came before is complete.  After it (which still reads what is
+// overwritten here) it loads and turns its rows under the end of that kernel, and waits before it stores them.
 __global__ void __launch_bounds__(256) gather_kv_rope_kernel(const __grid_constant__ AttnParams p, const RopeCopies c) {
   constexpr int D = 128;
   constexpr int kPasses = kGatherRowsPerCta / 32;
-  grid_go();  // as in gather_kv_kernel
+  if (!c.after_attention) grid_wait();
+  grid_go();
   const PlanDev& pl = p.plan;
   const int g = blockIdx.y, b = blockIdx.z;
   const int map = pl.n_maps == 1 ? 0 : b;
@@ -136,7 +138,7 @@ __global__ void __launch_bounds__(256) gather_kv_rope_kernel(const __grid_consta
       if (slot0 + 32 * i + r0 < pl.n_kv)
         rotate8(klo[i], khi[i], p.rope + (int64_t)tok[i] * (D / 2) + chunk * 8);  // zeros stay zeros
   }
-  grid_wait();  // (returns at once unless launched as a dependent)
+  grid_wait();  // (returns at once the second time)
 #pragma unroll
   for (int i = 0; i < kPasses; ++i) {
     const int slot = slot0 + 32 * i + r0;
@@ -160,8 +162,8 @@ cudaError_t launch_gather_kv(const AttnParams& p, void* k_out, void* v_out, bool
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather_kv_rope(const AttnParams& p, const RopeCopies& c, bool dependent, cudaStream_t stream) {
-  return launch_dependent(gather_kv_rope_kernel, gather_grid(p), 256, 0, 1, dependent, stream, p, c);
+cudaError_t launch_gather_kv_rope(const AttnParams& p, const RopeCopies& c, cudaStream_t stream) {
+  return launch_dependent(gather_kv_rope_kernel, gather_grid(p), 256, 0, 1, true, stream, p, c);
 }
 
 // Positional table p of the rotary embedding (Section 5.1: p is set up before inference; the Pre-Pass algorithm takes its rows
