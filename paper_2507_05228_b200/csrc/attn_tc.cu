@@ -713,16 +713,17 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   // MMA tiles of four chunks; only the last one is narrower, or with kWalk the last one of every shard (see TileSeq)
   auto tile_chunks = [&](int i) { return min(4, (n_keys - kNMax * i + kChunk - 1) / kChunk); };
 
-  // Once a wait has given up, later calls on the plan write nothing.  Warp 11 looks the word up during the set-up; the others ask
-  // when their first data are there, and what they have requested lands before the CTA ends.  (Looked up by all before the
-  // set-up the word costs 1000 cycles, joined to the barrier above 900, asked for at once after it up to 1000 with 8 heads a
-  // tile: 1000 tokens, 64 / 8 heads, 26.0 -> 26.6 us.)
+  // Once a wait has given up, later calls on the plan write nothing.  Warp 11 looks the word up during the set-up; the issuing
+  // warp asks when the first logits are under way, the loaders when they have nothing left to do, and what is under way lands
+  // before the CTA ends.  From then on the softmax warps find the abort flag raised.  (The load takes as long as the first data:
+  // looked up by all before the set-up it costs 1000 cycles, joined to the barrier above 900, asked for before the first
+  // logits 400 to 1300: 33 tokens, 64 / 8 heads, 6.7 -> 7.6 us.)
   auto goes_on = [&]() {
     wait_bar(wc, bar(CHECKED), 0u, 11);
     return wc.load(1) == 0;
   };
-  auto landed = [&](uint32_t full) {  // a box that was requested, whatever the word says
-    for (int i = 0; i < 1 << 14 && !mbar_try_wait(full, 0u); ++i) {
+  auto landed = [&](uint32_t full, uint32_t parity) {  // what was requested, whatever the word says
+    for (int i = 0; i < 1 << 14 && !mbar_try_wait(full, parity); ++i) {
     }
   };
 
@@ -770,16 +771,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> tensor-core reads
       mbar_arrive(bar(Q_FULL + s));
     }
-    auto first_logits = [&]() {  // are issued only if the CTA goes on
-      if (n_tiles > 0) wait_bar(wc, s_full(s, 0), 0u, 1);
-      return goes_on();
-    };
-    if (s < n_sub && first_logits()) {
+    if (s < n_sub) {
       const int m = tid & 127;  // MMA row = TMEM lane
       const int sub_row0 = row0 + s * R;
       const int sub_nrows = min(R, nrows - s * R);
       const int slot_local = m >> lg;
-      const bool row_ok = slot_local < sub_nrows;
+      bool row_ok = slot_local < sub_nrows;
       const int slot = sub_row0 + (row_ok ? slot_local : 0);
       const int head = h0 + (m & (Gp - 1));
       const int32_t* vis_row = vis + (size_t)(kWalk ? slot : 0) * P;
@@ -878,6 +875,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           l_out = l_run * ex2(m_run - m_true);
           m_out = m_true * 0.6931471805599453f;
         }
+        if (wc.load(1)) return;  // nothing is written any more
         const int64_t stat = (((int64_t)b * P + kk) * pl.n_q + slot) * p.H + head;
         if (row_ok) {
           p.m_part[stat] = m_out;
@@ -1123,6 +1121,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         note(8 * i + 2);
       }
       note(8 * n_tiles + 3);
+      auto may_write = [&]() { return n_tiles > 0 ? wc.load(1) == 0 : goes_on(); };  // after the last product, see goes_on
       if (!kWalk && split > 1) {
         // ---- epilogue of a query tile whose keys were shared by the cluster: CTA r finishes columns r * cols .. of all
         // rows.  Every CTA sends it those columns of its accumulator and its row statistics (relative to its own m).
@@ -1133,6 +1132,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           wait_bar(wc, bar(O_FULL), 0u, 3, n_tiles);
           tc_fence_after();
         }
+        if (!may_write()) row_ok = false;
         cluster_barrier();  // every product of the cluster is done: its Q, K and V tiles may be overwritten
         const uint32_t from_me = smem_base + (uint32_t)kOffQ;
         auto slot_of = [&](int sender, int receiver) { return sender < receiver ? sender : sender - 1; };
@@ -1244,6 +1244,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           m_out = m_true * 0.6931471805599453f;   // natural-log units
         }
       }
+      const bool quiet = !may_write();
+      if (quiet) {
+        row_ok = false;
+        dst = nullptr;
+      }
       if (row_ok) {
         if (p.fused) {
           if (p.lse_out) p.lse_out[stat] = l_out > 0.f ? m_out + logf(l_out) : -INFINITY;
@@ -1253,7 +1258,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         }
       }
       if constexpr (kBoxes) {
-        store_rows(o_scale, n_tiles > 0, b * P + max(kk_open, 0), dst);
+        if (!quiet) store_rows(o_scale, n_tiles > 0, b * P + max(kk_open, 0), dst);
         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the rows have left shared memory
       } else {
         // Every product of the CTA has completed, so the Q / K tiles in shared memory are free: the thread stages its
@@ -1331,15 +1336,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       const uint32_t q_lo0 = desc_lo(smem_base + kOffQ, 16);
       const uint32_t k_lo0 = desc_lo(smem_base + kOffK, 16);
       const uint32_t v_lo0 = desc_lo(smem_base + kOffV, kHalfBytes);  // the two 64-column halves of d
-      auto first_data = [&]() {
-        wait_bar(wc, bar(K_FULL), 0u, 7);
-        wait_bar(wc, bar(Q_FULL), 0u, 6);
-        if (goes_on()) return true;
-        if (q_boxes)
-          for (int s = 0; s < n_sub; ++s) landed(bar(Q_FULL + s));
-        return false;
-      };
-      if (n_tiles > 0 && first_data()) {
+      if (n_tiles > 0) {
         auto s_col = [&](int s, int i) {  // logit buffer of sub-tile s, tile i
           return tmem + (uint32_t)((kRing ? (2 * i + s) % 3 : s) * 128);
         };
@@ -1389,6 +1386,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           issue_qk(s, 0, n_cur);
         }
         if (leader) mma_commit(bar(K_EMPTY));
+        int n_run = n_tiles;
         if constexpr (kRing) {
           // Order: QK_0(0) QK_1(0) QK_0(1), then per tile i: PV_0(i) QK_1(i+1) PV_1(i) QK_0(i+2).  QK_1(i+1) takes the
           // buffer PV_0(i) has read, QK_0(i+2) the one of PV_1(i); MMAs execute in issue order, so neither needs a
@@ -1406,8 +1404,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             issue_qk(0, 1, n_next);
             if (last_sub == 0 && leader) mma_commit(bar(K_EMPTY + 1 % kKStages));
           }
-          for (int i = 0; i < n_tiles; ++i) {
-            n_2 = i + 2 < n_tiles ? kChunk * seq.next(opens_2) : 0;
+          if (!goes_on()) n_run = 0;
+          for (int i = 0; i < n_run; ++i) {
+            n_2 = i + 2 < n_run ? kChunk * seq.next(opens_2) : 0;
             wait_bar(wc, bar(V_FULL + i % kVStages), (uint32_t)((i / kVStages) & 1), 4, i);
             for (int s = 0; s < n_sub; ++s) {
               note(8 * i + 2 + s);
@@ -1415,11 +1414,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
               tc_fence_after();
               issue_pv(s, i, n_cur, opens_cur);
               if (s == last_sub && leader) mma_commit(bar(V_EMPTY + i % kVStages));
-              if (s == 0 && n_sub == 2 && i + 1 < n_tiles) {
+              if (s == 0 && n_sub == 2 && i + 1 < n_run) {
                 issue_qk(1, i + 1, n_next);
                 if (leader) mma_commit(bar(K_EMPTY + (i + 1) % kKStages));
               }
-              if (s == last_sub && i + 2 < n_tiles) {
+              if (s == last_sub && i + 2 < n_run) {
                 wait_k(i + 2);
                 issue_qk(0, i + 2, n_2);
                 if (last_sub == 0 && leader) mma_commit(bar(K_EMPTY + (i + 2) % kKStages));
@@ -1430,9 +1429,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             n_next = n_2;
             opens_next = opens_2;
           }
-        } else
-        for (int i = 0; i < n_tiles; ++i) {
-          const bool has_next = i + 1 < n_tiles;
+        } else {
+        if (!goes_on()) n_run = 0;
+        for (int i = 0; i < n_run; ++i) {
+          const bool has_next = i + 1 < n_run;
           if (i > 0) {
             n_cur = n_next;
             opens_cur = opens_next;
@@ -1458,7 +1458,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             }
           }
         }
+        }
         if (leader) mma_commit(bar(O_FULL));
+        if (n_run == 0) {
+          if (q_boxes)
+            for (int s = 0; s < n_sub; ++s) landed(bar(Q_FULL + s), 0u);
+          landed(bar(O_FULL), 0u);
+        }
         note(7);
       }
       __syncwarp();
@@ -1487,14 +1493,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         // launched as its programmatic dependent it may have started early, so wait here for that grid to complete
         // (a no-op otherwise).  Nothing else in this kernel reads what the gather grid writes.
         grid_wait();
+        int n_issued = 0;
         for (int i = 0; i < n_tiles; ++i) {
-          if (i == 1 && !goes_on()) break;
           const int nch = kWalk ? min(4, cur.nc - cur.c) : tile_chunks(i);
           const int st = i % n_stages;
           note(8 * i + 1);
           // The first use of a stage waits for nothing, and must not: the products may have consumed a first tile that was
           // requested early before this warp gets here, and a wait for the phase before that would never end.
-          if (i >= n_stages) wait_bar(wc, bar(empty0 + st), (uint32_t)(((i / n_stages) & 1) ^ 1), is_k ? 9 : 10, i);
+          if (i >= n_stages && !wait_bar(wc, bar(empty0 + st), (uint32_t)(((i / n_stages) & 1) ^ 1), is_k ? 9 : 10, i)) break;
           const uint32_t dst = tiles_s + (uint32_t)(st * kTileBytes), fb = bar(full0 + st);
           if constexpr (kWalk) {
             if (leader) mbar_expect_tx(fb, (uint32_t)(nch * C::kHalves * kChunkBytes));
@@ -1516,9 +1522,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             if (C::kHalves == 2) tma_tile4(dst + (uint32_t)kHalfBytes, map, 64, key0 + kNMax * i, g, b, fb);
           }
           __syncwarp();
+          n_issued = i + 1;
           note(8 * i + 2);
         }
-        if (!goes_on()) landed(bar(full0));
+        if (!goes_on())
+          for (int i = max(0, n_issued - n_stages); i < n_issued; ++i) landed(bar(full0 + i % n_stages), (uint32_t)((i / n_stages) & 1));
       }
     }
     if (!kWalk && split > 1) {
@@ -1688,11 +1696,13 @@ cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, c
   const int64_t n_q = p.plan.n_q;
   // Boxes: at head_dim 64 always (4099 tokens in 16 shards, 32 / 8 heads: 389 -> 361 us with the post-pass).  At head_dim 128, where
   // they cost the second K and V stages, with at least four heads a tile (a box is 32 rows of (slot, head), so it seldom
-  // reaches past a shard) and query tiles that are nine tenths full, so that two sub-tiles hide each other's loads: 32 / 8
-  // heads, 2000 tokens in 32 shards 289 -> 256 us, 4099 in 16 348 -> 336.  Elsewhere they lose up to a quarter: 16 / 8 heads,
-  // 2000 tokens in 32 shards 199 and 226, 8 / 8 heads 178 and 222; 32 / 8 heads, 500 tokens in 32 shards 160 and 200.
-  const int64_t slots = 256 >> lg, n_tiles = p.plan.n_qtiles[3 - lg];
-  const bool boxes = p.d == 64 || (lg >= 2 && 10 * n_q >= 9 * n_tiles * slots);
+  // reaches past a shard), two sub-tiles in nearly every query tile, which hide each other's loads, and more than a chunk of
+  // keys in a shard: 32 / 8 heads, 2000 tokens in 32 shards 289 -> 256 us, 4099 in 16 348 -> 336, 16 / 4 heads, 3000 in 30 269
+  // -> 246.  Elsewhere they lose up to a quarter: 16 / 8 heads, 2000 tokens in 32 shards 199 and 226, 8 / 8 heads 178 and 222;
+  // 32 / 4 heads, 1000 tokens in 31 shards 171 and 202, in 10 shards 72 and 78.
+  const CutSize cut(p);
+  const int64_t n_tiles = p.plan.n_qtiles[3 - lg];
+  const bool boxes = p.d == 64 || (lg >= 2 && cut.keys >= 48 && cut.row_tiles(128 >> lg) >= 1.9 * cut.row_tiles(256 >> lg));
   tma.o_valid = boxes && encode_out(&tma.o, p.o_part, p.d, lg, p.H, n_q, (int64_t)p.batch * p.plan.n_kv_shards,
                                     {n_q * p.H * p.d, (int64_t)p.H * p.d, p.d});
   const int64_t n_ctas = n_tiles * (p.H >> lg) * p.batch;
@@ -1713,16 +1723,17 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
   const int64_t tile_slots = 256 >> lg, n_qt = (p.plan.n_q + tile_slots - 1) / tile_slots;
   const int64_t n_ctas = n_qt * (p.H >> lg) * p.batch;
   // Few query tiles (a chunk of a chunked prefill, a short prompt) leave SMs idle: a cluster then shares the keys of each
-  // tile, as far as its CTAs fit at once with one per SM (clusters of 2, 4 and 8: 148, 132 and 120 CTAs) and have two
-  // 128-key tiles each.  Three with a rotary step, where every CTA of a cluster turns the query rows for itself (32 / 8 heads,
-  // 500 tokens: 22.5 us in clusters of two, 18.5 without; 8 / 8 heads, 1000 tokens: 32.2 in clusters of four, 26.9 without;
-  // 1500 tokens 32.8 and 36.9).  The rule counts the heads of the whole problem, see AttnParams.
+  // tile, as far as its CTAs fit at once with one per SM (clusters of 2, 4 and 8: 148, 132 and 120 CTAs) and have three
+  // 128-key tiles each.  (With two each the exchange and, with a rotary step, query rows turned in every CTA cost more than
+  // they save: 500 tokens, 32 / 8 heads, 15.4 -> 14.1 us, with the rotary step 22.5 -> 18.5; 8 / 8 heads, 1000 tokens, 22.2 ->
+  // 19.4 and 32.2 -> 26.9.  12 tiles in clusters of four 32.8, alone 36.9.  The rule is the same with and without a rotary
+  // step, so that both sum in the same order.)  It counts the heads of the whole problem, see AttnParams.
   const int64_t rule_ctas = n_qt * ((int64_t)p.rule_kv_heads * p.G >> lg) * p.batch, key_tiles = (n_seen + 127) / 128;
   int split = 1;
   if (p.fused) {
     const int64_t fit[4] = {148, 148, 132, 120};
     for (int i = 1; i < 4; ++i)
-      if (rule_ctas << i <= fit[i] && key_tiles >= (p.rope ? 3 : 2) << i) split = 1 << i;
+      if (rule_ctas << i <= fit[i] && key_tiles >= 3 << i) split = 1 << i;
   }
   const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), split,
                       p.prefix_from_vis ? 0 : (k_gathered ? 0 : 1) | (v_gathered ? 0 : 2), k_gathered || v_gathered, false};
