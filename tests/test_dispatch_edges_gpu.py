@@ -442,3 +442,32 @@ def test_calls_on_a_plan_whose_status_word_is_set_write_nothing(gu, n_q, n_kv):
     o_ref, _ = oracle.attention_unsharded(w.q, w.k, w.v, w.scale, q_pos_offset=w.q_pos_offset)
     gu.check_output(o, None, o_ref, None, w.tol, "after the word was cleared")
     plan.destroy()
+
+
+@pytest.mark.parametrize("P", [1, 4])
+def test_captured_rotary_call(gu, P):
+    """Captured, the rotary call copies keys and values in token order; what lies behind the last query may be NaN, and the
+    workspace holds the same as after a plain call."""
+    from paper_2507_05228_b200 import binding as cb
+    n_q, n_kv, off = 64, 400, 200
+    w = wl.make_workload("captured_rope", 2, n_q, n_kv, 8, 2, 128, "bf16", "random", "random", 2, P, seed=P, symmetric=False,
+                         q_pos_offset=off)
+    q, k, v = gu.to_device(w)
+    k[:, off + n_q:], v[:, off + n_q:] = float("nan"), float("nan")
+    plan = gu.make_plan(w)
+    table = cb.cascade_rope_table(n_kv, 128, 10000.0)
+    size = cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED, cb.BF16, 2, 8, 2, 128)
+    ws = [torch.zeros(size, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    o = torch.zeros_like(q)
+    o_ref, _ = cb.cascade_attn_sharded_rope(plan, q, k, v, w.scale, table, workspace=ws[0])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        cb.cascade_attn_sharded_rope(plan, q, k, v, w.scale, table, out=o, want_lse=False, workspace=ws[1])
+    for _ in range(2):
+        o.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert (o.float() - o_ref.float()).abs().max() <= w.tol and torch.isfinite(o.float()).all()
+        assert torch.equal(*ws)
+    del graph
+    plan.destroy()
