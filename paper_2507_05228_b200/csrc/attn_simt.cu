@@ -475,7 +475,7 @@ double tiles_time(const AttnParams& p) {
 }
 
 cudaError_t launch_attn_simt(const AttnParams& p, cascade_dtype_t dtype, cudaStream_t stream) {
-  if (rows_time(p) < tiles_time(p)) return launch_attn_rows(p, dtype, stream);
+  if (0.97 * rows_time(p) < tiles_time(p)) return launch_attn_rows(p, dtype, stream);  // (a tie goes to the simpler kernel)
   if (dtype == CASCADE_BF16) {
     if (p.d == 128) return launch_one<__nv_bfloat16, 128>(p, stream);
     return launch_one<__nv_bfloat16, 64>(p, stream);

@@ -468,6 +468,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   constexpr int kOffQ = C::kOffQ, kOffK = C::kOffK, kOffV = C::kOffV, kOffMisc = C::kOffMisc;
   constexpr bool kRing = C::kRing;
   static_assert(!kRope || D == 128, "the rotary step is fused for head_dim 128 only");
+  constexpr bool kLateMax = !kWalk && !kRing;  // see below
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -776,7 +777,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       const int sub_row0 = row0 + s * R;
       const int sub_nrows = min(R, nrows - s * R);
       const int slot_local = m >> lg;
-      bool row_ok = slot_local < sub_nrows;
+      const bool row_ok = slot_local < sub_nrows;
       const int slot = sub_row0 + (row_ok ? slot_local : 0);
       const int head = h0 + (m & (Gp - 1));
       const int32_t* vis_row = vis + (size_t)(kWalk ? slot : 0) * P;
@@ -982,7 +983,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         // exponentials, and is taken while the products are under way (it was 320 of the 2200 cycles between the logits and
         // the weights; 2048 tokens 47 -> 44 us, 4 x 8192 with rotary step 2.22 -> 2.06 ms).  Not with kWalk, where most tiles
         // open a shard (434 -> 471 us on 4099 tokens in 16 shards), nor with kRing, whose next logits are there already.
-        constexpr bool kLateMax = !kWalk && !kRing;
         float smax = 0.f, alpha = 1.f;
         bool changed = false;
         if constexpr (kLateMax) {
@@ -1121,7 +1121,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         note(8 * i + 2);
       }
       note(8 * n_tiles + 3);
-      auto may_write = [&]() { return n_tiles > 0 ? wc.load(1) == 0 : goes_on(); };  // after the last product, see goes_on
+      auto may_write = [&]() {  // asked after the last product; see goes_on
+        return (n_tiles > 0 ? wc.load(1) : *reinterpret_cast<volatile const int32_t*>(wc.status)) == 0;
+      };
       if (!kWalk && split > 1) {
         // ---- epilogue of a query tile whose keys were shared by the cluster: CTA r finishes columns r * cols .. of all
         // rows.  Every CTA sends it those columns of its accumulator and its row statistics (relative to its own m).
@@ -1132,7 +1134,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           wait_bar(wc, bar(O_FULL), 0u, 3, n_tiles);
           tc_fence_after();
         }
-        if (!may_write()) row_ok = false;
+        const bool out_ok = may_write() && row_ok;
         cluster_barrier();  // every product of the cluster is done: its Q, K and V tiles may be overwritten
         const uint32_t from_me = smem_base + (uint32_t)kOffQ;
         auto slot_of = [&](int sender, int receiver) { return sender < receiver ? sender : sender - 1; };
@@ -1176,7 +1178,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           f_of[i] = ex2(f_of[i] - m_use);
           if (i < split - 1) {
             l_all += f_of[i] * *reinterpret_cast<const float*>(got_stats + i * 2 * kM * 16 + 4);
-            fix_all += f_of[i] * *reinterpret_cast<const float*>(got_stats + i * 2 * kM * 16 + 8);
+            if constexpr (kLateMax) fix_all += f_of[i] * *reinterpret_cast<const float*>(got_stats + i * 2 * kM * 16 + 8);
           }
         }
         const float inv = l_all > 0.f ? 1.f / (l_all + fix_all) : 0.f;
@@ -1202,7 +1204,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
               acc[6] = fmaf(d.z, f_of[i], acc[6]); acc[7] = fmaf(d.w, f_of[i], acc[7]);
             }
           }
-          if (row_ok) {
+          if (out_ok) {
             uint4 val;
             val.x = pack_bf16x2(acc[0] * inv, acc[1] * inv);
             val.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
@@ -1211,7 +1213,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             *reinterpret_cast<uint4*>(dst + c0) = val;
           }
         }
-        if (row_ok && me == 0 && p.lse_out)
+        if (out_ok && me == 0 && p.lse_out)
           p.lse_out[((int64_t)b * pl.n_q + slot) * p.H + head] =
               l_all > 0.f ? (m_use + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
       } else {
@@ -1245,11 +1247,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         }
       }
       const bool quiet = !may_write();
-      if (quiet) {
-        row_ok = false;
-        dst = nullptr;
-      }
-      if (row_ok) {
+      if (quiet) dst = nullptr;
+      if (dst) {
         if (p.fused) {
           if (p.lse_out) p.lse_out[stat] = l_out > 0.f ? m_out + logf(l_out) : -INFINITY;
         } else {
@@ -1301,7 +1300,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       }
       if constexpr (kWalk) {
         // the shards of which no row of the CTA sees anything were never walked: their partials are empty
-        if (row_ok) {
+        if (row_ok && may_write()) {
           int a = 0;
           for (int k = 0; k < P; ++k) {
             if (a < n_act && tab->kk[a] == k) {
@@ -1724,7 +1723,7 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
   const int64_t n_ctas = n_qt * (p.H >> lg) * p.batch;
   // Few query tiles (a chunk of a chunked prefill, a short prompt) leave SMs idle: a cluster then shares the keys of each
   // tile, as far as its CTAs fit at once with one per SM (clusters of 2, 4 and 8: 148, 132 and 120 CTAs) and have three
-  // 128-key tiles each.  (With two each the exchange and, with a rotary step, query rows turned in every CTA cost more than
+  // 128-key tiles each, or two at head_dim 64 (500 tokens, 12 heads, in clusters of two 12.0 us, alone 12.9).  (With two each the exchange and, with a rotary step, query rows turned in every CTA cost more than
   // they save: 500 tokens, 32 / 8 heads, 15.4 -> 14.1 us, with the rotary step 22.5 -> 18.5; 8 / 8 heads, 1000 tokens, 22.2 ->
   // 19.4 and 32.2 -> 26.9.  12 tiles in clusters of four 32.8, alone 36.9.  The rule is the same with and without a rotary
   // step, so that both sum in the same order.)  It counts the heads of the whole problem, see AttnParams.
@@ -1733,7 +1732,7 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
   if (p.fused) {
     const int64_t fit[4] = {148, 148, 132, 120};
     for (int i = 1; i < 4; ++i)
-      if (rule_ctas << i <= fit[i] && key_tiles >= 3 << i) split = 1 << i;
+      if (rule_ctas << i <= fit[i] && key_tiles >= (p.d == 64 ? 2 : 3) << i) split = 1 << i;
   }
   const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), split,
                       p.prefix_from_vis ? 0 : (k_gathered ? 0 : 1) | (v_gathered ? 0 : 2), k_gathered || v_gathered, false};
