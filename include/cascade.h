@@ -159,7 +159,7 @@ cascade_status_t cascade_plan_dense_mask(const cascade_plan_t* plan, int32_t map
 /* Reads the plan's device status word (SYNCHRONISES the device): 0 = no kernel that used this plan hit a
  * bounded-wait limit; otherwise a code identifying the wait.  Returns TIMEOUT if non-zero.
  * The word is sticky: once a wait inside the tensor-core kernel has given up (2 s without progress), every later
- * attention call on this plan returns CASCADE_OK from the host but its blocks exit at once and write nothing.  A
+ * tensor-core attention call on this plan returns CASCADE_OK from the host but its blocks write nothing.  A
  * non-zero status therefore invalidates the outputs of every call made on the plan since the last check that read 0;
  * destroy the plan and build a new one.  A caller that cannot afford stale outputs polls this after the calls whose
  * results it is about to use. */
@@ -239,8 +239,10 @@ cascade_status_t cascade_merge_peers(cascade_dtype_t dtype, int32_t batch, int32
  * Section 5.2.3 the result equals cascade_merge(cascade_attn_partials(...)).  Output in token order:
  *   o_out [batch][n_q][n_heads][head_dim] with strides; lse_out optional fp32 [batch][n_q][n_heads].
  * For n_q == 1 (decode, Appendix F "Caching") the KV shards are processed as independent partials that meet on chip, in
- * one launch (`workspace` is checked but not used).  The tensor-core route (bf16) reads K and V where
- * they are and uses `workspace` only for tensors whose strides its loads cannot take.  Size: cascade_workspace_bytes(CASCADE_CALL_SHARDED).
+ * one launch (`workspace` is checked but not used).  The tensor-core route (bf16) reads K and V where they are and uses
+ * `workspace` only for tensors whose strides its loads cannot take and for calls that are being captured into a graph; a
+ * graph follows cascade_plan_advance when it is replayed.  Size: cascade_workspace_bytes(CASCADE_CALL_SHARDED), the size of
+ * cascade_attn_partials' workspace on the tensor-core route; heads of 64 columns take the fp32 ALU kernel without it.
  */
 cascade_status_t cascade_attn_sharded(const cascade_plan_t* plan, cascade_dtype_t dtype, int32_t batch,
                                       int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, float scale,
@@ -275,7 +277,8 @@ cascade_status_t cascade_rope_table(int32_t n_positions, int32_t head_dim, doubl
  *   rope_table   DEVICE table written by cascade_rope_table for head_dim 128, 16-byte aligned, read-only
  *   n_positions  its row count; must cover max(q_pos_offset + n_q, n_kv).  A negative q_pos_offset is taken with the causal
  *                mask only (a row before position 0 sees nothing and yields zeros); INVALID_ARG without
- * All other arguments, the workspace and the outputs are those of cascade_attn_sharded.
+ * All other arguments, the workspace (used here: copies of the rotated keys and of the values) and the outputs are those of
+ * cascade_attn_sharded.  A graph that holds the call keeps the positions of its query rows.
  * Supported on the tensor-core route only (bf16, head_dim 128, n_q > 1, at most 256 KV shards); other shapes return
  * CASCADE_ERR_UNSUPPORTED and the caller rotates q and k beforehand.
  */

@@ -11,9 +11,10 @@
 // max / sum / output of the streaming softmax, and one output row is written at the end.  Only the last tile or two need the
 // causal mask.  Where there are few query tiles, a cluster of 2, 4 or 8 CTAs shares the keys of one and adds up through
 // distributed shared memory.
-// Measured, 32 query / 8 KV heads (before: shard by shard from gathered copies, query tiles inside one shard): 2048 tokens, 8
-// random shards 67 -> 47 us; 512 queries against 7168 cached tokens 127 -> 80 us; 32768 tokens, 64 / 8 heads, 32 random
-// shards 16.7 -> 16.0 ms; 2 x 3001 tokens, 16 / 4 heads of 64 columns 124 -> 85 us.
+// Measured, 32 query / 8 KV heads: 2048 tokens, 8 random shards 42.7 us; 512 queries against 7168 cached tokens 71 us; 32768
+// tokens, 64 / 8 heads, 32 random shards 15.5 ms; 2 x 3001 tokens, 16 / 4 heads of 64 columns 79 us.  (This order of work alone,
+// against shard by shard from gathered copies with query tiles inside one shard: 67 -> 47 us, 127 -> 80 us, 16.7 -> 16.0 ms and
+// 124 -> 85 us; the rest is what stands beside the code below.)
 //
 // Partials (kWalk, the Attention-Pass algorithm for every pair of the query tile).  The rows are consecutive slots of one
 // query shard and the KV shards are walked one after another: each shard's visible prefix (as seen by the CTA's last row,
@@ -26,8 +27,8 @@
 //         tcgen05.ld, applies the mask (the row sees a prefix of the keys), writes the weights P as bf16 back into the TMEM
 //         columns of S, keeps the running max / sum while the products run, rescales the output accumulator in TMEM in
 //         the rare case that a weight is far above the reference maximum, and runs the epilogue: the scaled output
-//         row goes through shared memory (the Q / K tiles are free by then) to the copy engine, one 256-byte bulk
-//         copy per row.
+//         row goes through shared memory (the Q / K tiles are free by then), from where the warp stores whole rows.
+//         kWalk writes rows out at every shard boundary, see store_rows.
 //   8     MMA issuer: S_s = Q_s K^T (operands in shared memory) and O_s += P_s V (P from TMEM), issued as
 //         PV_0(i), QK_0(i+1), PV_1(i), QK_1(i+1) so that the tensor pipe works on one sub-tile while the other is in
 //         its softmax.  QK_s(i+1) overwrites the columns PV_s(i) reads P from; MMAs execute in issue order, which
@@ -42,7 +43,7 @@
 //         sub-tiles come once per CTA, as boxes requested during the set-up; where their tokens are not consecutive (kWalk),
 //         where they are turned on the way (rotary step), or where their strides do not fit a tensor map, the softmax threads
 //         gather them themselves (plain 16-byte loads).
-//   11    works out the CTA's keys (kWalk: the table of the shards it sees anything of), then idles; it also keeps the
+//   11    works out the CTA's keys (kWalk: the table of the shards it sees anything of) and looks at the status word, then idles; it also keeps the
 //         register-reallocation groups of four warps whole.
 // The grid is launched as a programmatic dependent (partials: only after a gather).  After a gather everything up to the
 // loaders' first TMA load may run while the copies are still being written; otherwise the set-up of the block scheduler
@@ -981,7 +982,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         // The reference the weights are scaled by is the maximum of the first tile, and stays that unless a later tile rises
         // far above it.  kLateMax: that shows in the weights, so the maximum of this tile is not needed before its
         // exponentials, and is taken while the products are under way (it was 320 of the 2200 cycles between the logits and
-        // the weights; 2048 tokens 47 -> 44 us, 4 x 8192 with rotary step 2.22 -> 2.06 ms).  Not with kWalk, where most tiles
+        // the weights; when it was introduced, 2048 tokens 47 -> 44 us, 4 x 8192 with rotary step 2.22 -> 2.06 ms).  Not with kWalk, where most tiles
         // open a shard (434 -> 471 us on 4099 tokens in 16 shards), nor with kRing, whose next logits are there already.
         float smax = 0.f, alpha = 1.f;
         bool changed = false;
@@ -1028,19 +1029,19 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           if constexpr (kRing) CASCADE_TMEM_ST16(s_addr + 64u + (uint32_t)(16 * ch), pr);
         };
         auto exp_tile = [&]() {
-        if (nch == 4) {
-          // The full tile is one straight-line block, so that the scheduler can run the MUFU instructions of one chunk
-          // (8 issue cycles each) under the FMA / convert / store work of its neighbours; with a branch per chunk the
-          // two parts ran back to back (1600 cycles per tile instead of the ~1130 the MUFU unit needs).
-          exp_chunk(0);
-          exp_chunk(1);
-          exp_chunk(2);
-          exp_chunk(3);
-        } else {
+          if (nch == 4) {
+            // The full tile is one straight-line block, so that the scheduler can run the MUFU instructions of one chunk
+            // (8 issue cycles each) under the FMA / convert / store work of its neighbours; with a branch per chunk the
+            // two parts ran back to back (1600 cycles per tile instead of the ~1130 the MUFU unit needs).
+            exp_chunk(0);
+            exp_chunk(1);
+            exp_chunk(2);
+            exp_chunk(3);
+          } else {
 #pragma unroll
-          for (int ch = 0; ch < 3; ++ch)
-            if (ch < nch) exp_chunk(ch);  // warp-uniform
-        }
+            for (int ch = 0; ch < 3; ++ch)
+              if (ch < nch) exp_chunk(ch);  // warp-uniform
+          }
         };
         exp_tile();
         float psum0, psum1;

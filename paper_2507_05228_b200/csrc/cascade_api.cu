@@ -255,7 +255,6 @@ static cascade_status_t plan_host(int32_t n_maps, int32_t n_q, int32_t n_kv, con
     pl->kv_inv.assign((size_t)n_maps * n_kv, 0);
     pl->kv_slot_shard.assign((size_t)n_maps * n_kv, 0);
     if (kv_pos) pl->kv_pos.assign(kv_pos, kv_pos + (size_t)n_maps * n_kv);
-    int max_len = 0;
     // counting sort of token ids by shard id: ascending ids inside every shard
     auto sort_by_shard = [](const int32_t* shard_of, int n, int S, int32_t* off, int32_t* idx, int32_t* inv) {
       std::vector<int32_t> cursor(S + 1, 0);
@@ -277,11 +276,9 @@ static cascade_status_t plan_host(int32_t n_maps, int32_t n_q, int32_t n_kv, con
       sort_by_shard(kv_shard_of + (size_t)mp * n_kv, n_kv, P, ko, ki, pl->kv_inv.data() + (size_t)mp * n_kv);
       int32_t* slot_shard = pl->kv_slot_shard.data() + (size_t)mp * n_kv;
       for (int k = 0; k < P; ++k) {
-        max_len = std::max(max_len, (int)(ko[k + 1] - ko[k]));
         std::fill(slot_shard + ko[k], slot_shard + ko[k + 1], k);
       }
     }
-    pl->dev.max_kv_shard_len = max_len;
     pl->host_vis_stale = true;
     if (!vis_on_device || vis_from_host(*pl)) refresh_host_vis(*pl, true);
     // tile lists, padded to the same length for every map

@@ -34,7 +34,6 @@ struct PlanDev {
   int32_t n_qtiles[kNumTileSizes];  // per map (padded to the maximum over maps)
   int32_t* status;      // device status word, 0 = fine
   int32_t n_maps, n_q, n_kv, n_q_shards, n_kv_shards, q_pos_offset, causal;
-  int32_t max_kv_shard_len;
 };
 
 struct Strides {
@@ -261,10 +260,10 @@ cudaError_t launch_plan_set(const PlanDev& d, const int32_t* vis, int n_vis, con
 int64_t visible_keys(const cascade_plan& pl, int map, int64_t pos);
 // the fused decode of a checked call: cascade_attn_sharded, cascade_attn_decode_static
 cudaError_t run_decode_fused(const cascade_plan& plan, const AttnParams& p, cudaStream_t stream);
-// vis and pair_class of a device plan recomputed for a new q_pos_offset (plans without kv_pos)
 // Fills a new plan's lists, inverses and (visible) vis and pair_class from the uploaded row lists, 16 or 32 bits an id.
 cudaError_t launch_plan_fill(const PlanDev& d, const void* q_src, const void* kv_src, bool short_ids, bool visible,
                              cudaStream_t stream);
+// vis and pair_class of a device plan recomputed for a new q_pos_offset (plans without kv_pos)
 cudaError_t launch_plan_advance(const PlanDev& d, int32_t q_pos_offset, cudaStream_t stream);
 cudaError_t launch_merge(const MergeParams& p, cascade_dtype_t dtype, cudaStream_t stream);
 cudaError_t launch_merge_peers(const MergePeersParams& p, cascade_dtype_t dtype, cudaStream_t stream);

@@ -301,8 +301,8 @@ __global__ void __launch_bounds__(128, 4) decode_kernel(const __grid_constant__ 
 // With `step` the kernel is the whole decode step of a cache with rotary positions (the tail of the Pre-Pass algorithm,
 // then "Caching"): query rows are turned while they are loaded, and the new token's key row is turned and written, with its
 // value row, to the caches before anyone reads them.
-// Measured (32 query / 8 KV heads): 64 sequences of 16384 tokens in 16 shards 620 us = 6.93 TB/s (partials and merge as two
-// kernels 742 + 28), one sequence 23 us (44); the whole step of one sequence at 2500 of 4096 rows 10.5 us (38, four launches
+// Measured (32 query / 8 KV heads): 64 sequences of 16384 tokens in 16 shards 662 us on inputs new to the caches = 6.49 TB/s
+// (repeated on the same ones, of which L2 keeps a part, 608; partials and merge as two kernels 825), one sequence 23 us (44); the whole step of one sequence at 2500 of 4096 rows 10.5 us (38, four launches
 // and two copies).
 
 __device__ __forceinline__ uint32_t rotate_pair2(uint32_t x, uint32_t partner, const float4& cs, float sign) {

@@ -4,7 +4,8 @@
 // the visible prefix of a shard is a contiguous run of rows, which the attention kernel fetches with large TMA tile
 // loads; an index-mapped gather straight into shared memory could not feed the tensor cores (one 512-byte request
 // per ~36 cycles per SM with TMA row gathers, less with cp.async).  Bandwidth-bound: every K/V byte is read once
-// and written once, 16 bytes per thread.
+// and written once, 16 bytes per thread.  The same pass makes copies in token order for the fused route, where it cannot read
+// the caller's tensors as they are (strides that a tensor map cannot hold, a call that is being captured).
 // Positions of a shard's list that no query row of the plan sees (keys later than the last query position: the unwritten
 // tail of a preallocated cache) are written as zeros instead of copied.  The attention kernel loads whole 16-key
 // chunks and multiplies the rows past a prefix by zero weights, so what it loads there must be finite, whatever the
