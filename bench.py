@@ -34,18 +34,11 @@ HEADLINE_TEXT = ("c4_long_70b: batch 1 per GPU, 32768 tokens, 64 q / 8 kv heads,
 L2_FLUSH_BYTES = 256 << 20
 MIN_STEPS = 20  # timed launches behind every record
 
-# dram__bytes_read.sum + dram__bytes_write.sum per launch of each record's dominant kernel, from one ncu capture per
-# kernel and workload ((bytes of the captured case, launches of the captured size that make one full-size launch); None =
-# no capture of the kernel as it stands).  The prefill kernel's traffic grows with batch * KV heads (each (sequence, KV
-# head) streams its own K/V and writes its own output rows), the decode and merge kernels' with the batch.
+# dram__bytes_read.sum + dram__bytes_write.sum per launch of a record's dominant kernel, from one ncu capture of the kernel as it
+# stands ((bytes of the captured case, launches of the captured size that make one full-size launch)).  A kernel that has been
+# rewritten since its capture has no entry, and its record no traffic: the attention and decode kernels at present.
 NCU_TRAFFIC = {
-    "c2_prefill_8b/attn_tc_kernel": (25478656, 1),
-    "c3_batched/attn_tc_kernel": (136032256, 4),        # captured on one of the four sequences
-    "c4_long_70b/attn_tc_kernel": (1212214016, 1),
-    "c3_batched/attn_tc_kernel/partials": (1257771264, 4),
-    "c4_long_70b/attn_tc_kernel/partials": (4671739904, 4),  # captured with a quarter of the heads
-    "c5_decode/decode_kernel": (545430528, 8),          # captured with batch 8 of 64
-    "c3_batched/merge_kernel": (1135894528, 4),
+    "c3_batched/merge_kernel": (1135894528, 4),  # captured on one of the four sequences; the traffic grows with the batch
 }
 
 
