@@ -1724,10 +1724,11 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
   const int64_t n_ctas = n_qt * (p.H >> lg) * p.batch;
   // Few query tiles (a chunk of a chunked prefill, a short prompt) leave SMs idle: a cluster then shares the keys of each
   // tile, as far as its CTAs fit at once with one per SM (clusters of 2, 4 and 8: 148, 132 and 120 CTAs) and have three
-  // 128-key tiles each, or two at head_dim 64 (500 tokens, 12 heads, in clusters of two 12.0 us, alone 12.9).  (With two each the exchange and, with a rotary step, query rows turned in every CTA cost more than
-  // they save: 500 tokens, 32 / 8 heads, 15.4 -> 14.1 us, with the rotary step 22.5 -> 18.5; 8 / 8 heads, 1000 tokens, 22.2 ->
-  // 19.4 and 32.2 -> 26.9.  12 tiles in clusters of four 32.8, alone 36.9.  The rule is the same with and without a rotary
-  // step, so that both sum in the same order.)  It counts the heads of the whole problem, see AttnParams.
+  // 128-key tiles each, or two at head_dim 64 (500 tokens, 12 heads, in clusters of two 12.0 us, alone 12.9).  With two each
+  // at head_dim 128 the exchange and, with a rotary step, query rows turned in every CTA cost more than they save: 500
+  // tokens, 32 / 8 heads, 15.4 -> 14.1 us without, with the rotary step 22.5 -> 18.5; 8 / 8 heads, 1000 tokens, 22.2 -> 19.4
+  // and 32.2 -> 26.9.  12 tiles in clusters of four take 32.8, alone 36.9.  The rule is the same with and without a rotary
+  // step, so that both sum in the same order.  It counts the heads of the whole problem, see AttnParams.
   const int64_t rule_ctas = n_qt * ((int64_t)p.rule_kv_heads * p.G >> lg) * p.batch, key_tiles = (n_seen + 127) / 128;
   int split = 1;
   if (p.fused) {

@@ -905,7 +905,7 @@ cascade_status_t cascade_workspace_bytes(const cascade_plan_t* plan, int32_t whi
       set_error("cascade_workspace_bytes: the decode step needs a plan with one query row, bf16, head_dim 128");
       return CASCADE_ERR_UNSUPPORTED;
     }
-    // the partials of the decode kernel, then the rotated query rows
+    // what the interface asks for: partials and rotated query rows; the one-launch step keeps both on the chip
     *out_bytes = align_up(decode_ws_bytes(plan, dtype, batch, n_heads, head_dim), 256) +
                  align_up((size_t)batch * n_heads * head_dim * elt_size(dtype), 256);
   } else {
