@@ -174,15 +174,17 @@ cascade_status_t cascade_plan_device_status(const cascade_plan_t* plan, int32_t*
  *   m_part, l_part  fp32 [batch][n_kv_shards][n_q shard-major][n_heads], contiguous
  * (Together these are the paper's stage-B payload: n_kv_shards * (head_dim + 2) * n_heads * n_q values
  * per sequence, Appendix D.)  batch must equal n_maps when the plan has per-sequence maps.
- * head_dim in {64,128}; bf16 runs on the tensor cores (tcgen05), fp32 (and more than 256 KV shards, and head_dim 64
- * without a sufficient workspace) on the fp32 ALU kernel; n_q == 1 with bf16 runs the KV-streaming decode kernel.
+ * head_dim in {64,128}; bf16 runs on the tensor cores (tcgen05), and so does fp32 at head_dim 64, its operands split into
+ * three bf16 parts each, where that is the faster way; fp32 at head_dim 128, more than 256 KV shards, and head_dim 64
+ * without a sufficient workspace run on the fp32 ALU kernels; n_q == 1 with bf16 runs the KV-streaming decode kernel.
  * scale must be positive and finite (INVALID_ARG otherwise: the kernels take row maxima before scaling).
  * Only the k/v rows that some query row of the plan sees have to hold finite values: positions later than the last
  * query position (the unwritten tail of a preallocated cache) may hold anything, NaN bit patterns included; no route
  * lets them reach a result.  batch and n_heads may not exceed 65535 (and batch * n_kv_shards on the ALU route).
  * workspace: as reported by cascade_workspace_bytes(CASCADE_CALL_PARTIALS) (may be 0 -> NULL allowed).  The
  * tensor-core route first copies K and V into shard-major order there (the stage-A hand-over of each KV shard to
- * its AttnNodes, Appendix D): 2 * batch * n_kv_heads * n_kv * head_dim * 2 bytes, overwritten by every call.
+ * its AttnNodes, Appendix D): 2 * batch * n_kv_heads * n_kv * head_dim * 2 bytes, overwritten by every call.  fp32 at head_dim
+ * 64 keeps the split keys and values there, three times as much and a byte per 64 rows.
  */
 cascade_status_t cascade_attn_partials(const cascade_plan_t* plan, cascade_dtype_t dtype, int32_t batch,
                                        int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, float scale,
@@ -242,7 +244,8 @@ cascade_status_t cascade_merge_peers(cascade_dtype_t dtype, int32_t batch, int32
  * one launch (`workspace` is checked but not used).  The tensor-core route (bf16) reads K and V where they are and uses
  * `workspace` only for tensors whose strides its loads cannot take and for calls that are being captured into a graph; a
  * graph follows cascade_plan_advance when it is replayed.  Size: cascade_workspace_bytes(CASCADE_CALL_SHARDED), the size of
- * cascade_attn_partials' workspace on the tensor-core route; heads of 64 columns take the fp32 ALU kernel without it.
+ * cascade_attn_partials' workspace on the tensor-core route; heads of 64 columns take the fp32 ALU kernel without it.  fp32 at
+ * head_dim 64 as cascade_attn_partials.
  */
 cascade_status_t cascade_attn_sharded(const cascade_plan_t* plan, cascade_dtype_t dtype, int32_t batch,
                                       int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, float scale,

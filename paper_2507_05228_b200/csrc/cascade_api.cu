@@ -742,6 +742,24 @@ static bool tc_ws_given(const cascade_plan_t* plan, int batch, int Hkv, int d, c
   return workspace && bytes >= tc_ws_bytes(plan, batch, Hkv, d) && ((uintptr_t)workspace & 255) == 0;
 }
 
+// fp32 with heads of 64 columns on the tensor cores: whether the kernel takes the problem; whether the scratch for the split keys
+// and values is there and the kernel is the faster one.  The estimates of the ALU kernels leave out what a launch and a first
+// load take, hence the constants: at the 300 sizes of split_time the choice cost 1.9 % on average over the better kernel, and one
+// size got slower by more than 5 % (264 tokens in 5 of 32 shards).  16 x 512 tokens, 16 heads, 8 shards, no mask: partials 668 ->
+// 232 us, fused 540 -> 151; 1024 causal tokens, 8 sequences, fused 924 -> 161.
+static bool split_takes(const cascade_plan_t* plan, cascade_dtype_t dtype, int d) {
+  return dtype == CASCADE_F32 && d == 64 && plan->dev.n_q > 1 && plan->dev.n_kv_shards <= 256;
+}
+static bool use_split(const AttnParams& p, const cascade_plan_t* plan, cascade_dtype_t dtype, const void* workspace, size_t bytes) {
+  return split_takes(plan, dtype, p.d) && workspace && ((uintptr_t)workspace & 255) == 0 &&
+         bytes >= split_ws_bytes(plan->dev, p.batch, p.Hkv) && split_time(p) < 1.1 * std::min(tiles_time(p), rows_time(p)) + 4;
+}
+// Scratch of the routes with copies of K and V: bf16 on the tensor cores, or fp32 on the tensor cores.
+static size_t copies_ws_bytes(const cascade_plan_t* plan, cascade_dtype_t dtype, int batch, int Hkv, int d) {
+  if (use_tc(plan, dtype, d)) return tc_ws_bytes(plan, batch, Hkv, d);
+  return split_takes(plan, dtype, d) ? split_ws_bytes(plan->dev, batch, Hkv) : 0;
+}
+
 // Partials over short shards of heads of 64 columns, in bf16: whether the ALU kernels beat the tensor cores.
 static bool alu_partials_faster(const AttnParams& p) {
   return p.plan.n_kv_shards > 1 && (int64_t)p.batch * p.plan.n_kv_shards <= 65535 && rows_time(p) < tc_partials_time(p);
@@ -863,7 +881,7 @@ static HostCallLayout host_call_layout(const cascade_plan_t* plan, cascade_dtype
   // gs KV heads and their query heads per inner call
   const bool decode = use_decode(plan, dtype, G * gs, gs, d);
   L.inner_bytes = decode ? decode_ws_bytes(plan, dtype, batch, G * gs, d)
-                         : (use_tc(plan, dtype, d) ? tc_ws_bytes(plan, batch, gs, d) : 0);
+                         : copies_ws_bytes(plan, dtype, batch, gs, d);
   L.total = L.inner + align_up(L.inner_bytes, 256);
   return L;
 }
@@ -893,7 +911,7 @@ cascade_status_t cascade_workspace_bytes(const cascade_plan_t* plan, int32_t whi
     return CASCADE_ERR_INVALID_ARG;
   }
   const bool decode = use_decode(plan, dtype, n_heads, n_kv_heads, head_dim);
-  const size_t tc_bytes = !decode && use_tc(plan, dtype, head_dim) ? tc_ws_bytes(plan, batch, n_kv_heads, head_dim) : 0;
+  const size_t tc_bytes = decode ? 0 : copies_ws_bytes(plan, dtype, batch, n_kv_heads, head_dim);
   if (which_call == CASCADE_CALL_PARTIALS) {
     *out_bytes = tc_bytes;
   } else if (which_call == CASCADE_CALL_SHARDED) {
@@ -952,7 +970,7 @@ cascade_status_t cascade_attn_partials(const cascade_plan_t* plan, cascade_dtype
       set_error("cascade_attn_partials: batch * n_kv_shards exceeds 65535 on the route without tensor cores");
       return CASCADE_ERR_UNSUPPORTED;
     }
-    e = launch_attn_simt(p, dtype, st);
+    e = use_split(p, plan, dtype, workspace, workspace_bytes) ? launch_attn_split(p, workspace, st) : launch_attn_simt(p, dtype, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "cascade_attn_partials: launch");
   return CASCADE_OK;
@@ -1145,7 +1163,7 @@ static cascade_status_t attn_sharded_impl(const char* fn, const cascade_plan_t* 
     cascade_status_t ws = run_tc(p, fn, plan, workspace, workspace_bytes, st, &e);
     if (ws != CASCADE_OK) return ws;
   } else {
-    e = launch_attn_simt(p, dtype, st);
+    e = use_split(p, plan, dtype, workspace, workspace_bytes) ? launch_attn_split(p, workspace, st) : launch_attn_simt(p, dtype, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "attention (fused route): launch");
   return CASCADE_OK;
@@ -1328,9 +1346,11 @@ cascade_status_t cascade_attn_sharded_host(const cascade_plan_t* plan, cascade_d
     return CASCADE_ERR_UNSUPPORTED;
   }
   const HostCallLayout L = host_call_layout(plan, dtype, batch, n_heads, n_kv_heads, head_dim);
-  // heads of 64 columns do without the part for the head groups (on the ALU kernel), so a workspace without it is taken
+  // heads of 64 columns do without the part for the head groups (on the ALU kernel), so a workspace without it is taken; in fp32
+  // only one of exactly that size, which is all that this call used to ask for
   const bool inner = L.inner_bytes && (head_dim == 128 || workspace_bytes >= L.total);
-  const size_t need = head_dim == 128 ? L.total : L.inner;
+  const bool staging_only = head_dim == 64 && (dtype == CASCADE_BF16 || workspace_bytes < L.inner + 256);
+  const size_t need = staging_only ? L.inner : L.total;
   if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) {
     set_error("%s: workspace of %zu bytes (256-byte aligned) required, got %zu", fn, need, workspace_bytes);
     return CASCADE_ERR_WORKSPACE;

@@ -218,12 +218,16 @@ struct CutSize {
 };
 double rows_time(const AttnParams& p);         // attn_rows.cu
 double tiles_time(const AttnParams& p);        // attn_simt.cu
+double split_time(const AttnParams& p);        // attn_split.cu
 double tc_partials_time(const AttnParams& p);  // attn_tc.cu, partials of several shards at head_dim 64
 
 // Launchers; each returns a cudaError_t from the launch.
 cudaError_t launch_attn_rows(const AttnParams& p, cascade_dtype_t dtype, cudaStream_t stream);
 // the faster of attn_simt.cu and attn_rows.cu
 cudaError_t launch_attn_simt(const AttnParams& p, cascade_dtype_t dtype, cudaStream_t stream);
+// fp32, head_dim 64, at most 256 KV shards, on the tensor cores, and the scratch that it takes
+cudaError_t launch_attn_split(const AttnParams& p, void* workspace, cudaStream_t stream);
+size_t split_ws_bytes(const PlanDev& d, int batch, int Hkv);
 // K or V rows [batch][kv_heads][rows][d] for the tensor-core kernel (strides in elements)
 struct TcRows {
   const void* base;

@@ -1,0 +1,172 @@
+"""fp32 heads of 64 columns on the tensor cores (operands split into three bf16 parts): edges of its tiles, what it makes of
+values out of range, and its error next to that of the ALU kernels.  Two kernels per call tell that the route was taken."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2507_05228_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gu():
+    import gpu_util
+    return gpu_util
+
+
+def _fused(cb, plan, q, k, v, scale, workspace=True):
+    """The fused call with the workspace it asks for, or without any (then it runs on the ALUs); and how many kernels it ran."""
+    o, lse = torch.empty_like(q), torch.empty(q.shape[:3], dtype=torch.float32, device="cuda")
+    B, _, H, d = q.shape
+    need = cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED, cb.F32, B, H, k.shape[2], d)
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda") if workspace else None
+    S, n0 = cb._strides, cb.lib().cascade_launch_count()
+    assert 0 == cb.lib().cascade_attn_sharded(plan.handle, cb.F32, B, H, k.shape[2], d, scale, q.data_ptr(), S(q), k.data_ptr(), S(k),
+                                              v.data_ptr(), S(v), o.data_ptr(), S(o), lse.data_ptr(), ws.data_ptr() if workspace else None,
+                                              need if workspace else 0, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    return o, lse, cb.lib().cascade_launch_count() - n0
+
+
+@pytest.mark.parametrize("n_q,n_kv,H,Hkv,J,P,causal,off", [
+    (127, 127, 16, 16, 2, 2, False, 0),      # one sub-tile with a row missing
+    (129, 193, 16, 16, 3, 1, True, 64),      # a second sub-tile of one row, one key past three tiles
+    (257, 257, 16, 16, 4, 4, True, 0),       # a second query tile of one row; the first sub-tile skips tiles of the second
+    (300, 300, 16, 4, 5, 3, True, 0),        # four heads a tile
+    (40, 640, 16, 2, 1, 2, False, 0),        # eight heads a tile
+    (333, 333, 12, 4, 2, 5, True, 0),        # three heads per KV head: no stacking
+    (200, 500, 16, 16, 3, 4, True, -60),     # the first rows see nothing
+    (300, 300, 16, 16, 60, 2, True, 0),      # rows of many query shards in a tile
+])
+def test_split_route_at_its_edges(gu, n_q, n_kv, H, Hkv, J, P, causal, off):
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload(f"split_{n_q}_{n_kv}", 8, n_q, n_kv, H, Hkv, 64, "f32", "random", "random", J, P, seed=n_q + P, causal=causal,
+                         q_pos_offset=off, symmetric=J == P and n_q == n_kv)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    assert _fused(cb, plan, q, k, v, w.scale)[2] == 2
+    plan.destroy()
+    gu.full_parity(w)
+
+
+def test_split_route_where_shards_are_empty(gu):
+    """Shards without keys, and shards that a query tile sees nothing of."""
+    from paper_2507_05228_b200 import binding as cb
+    rng = np.random.default_rng(5)
+    n, B, H, P = 400, 8, 16, 6
+    w = wl.make_workload("split_empty", B, n, n, H, H, 64, "f32", "random", "random", 2, 2, seed=3)
+    w.kv_shard_of = np.where(np.arange(n) < 200, rng.integers(0, 2, n), 4).astype(np.int32)
+    w.n_kv_shards = P
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    assert _fused(cb, plan, q, k, v, w.scale)[2] == 2
+    plan.destroy()
+    gu.full_parity(w)
+
+
+@pytest.mark.parametrize("n,causal", [(512, False), (1000, True)])
+def test_split_route_is_as_exact_as_the_alu_kernels(gu, n, causal):
+    """Outputs closer to fp64 than those of the ALU kernels.  The logarithm of the row sum is 6 to 7 in size and rounded to fp32,
+    2.1e-8 of it on average, which both carry: 3e-8 in all, with room for the next digit."""
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload(f"split_err_{n}", 4, n, n, 12, 12, 64, "f32", "random", "random", 4, 4, seed=n, causal=causal)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    o_ref, lse_ref = oracle.attention_unsharded(w.q, w.k, w.v, w.scale, causal=causal)
+    err = {}
+    for ws in (True, False):
+        o, lse, n_kernels = _fused(cb, plan, q, k, v, w.scale, ws)
+        assert n_kernels == (2 if ws else 1)
+        err[ws] = [np.linalg.norm(a.double().cpu().numpy() - r) / np.linalg.norm(r) for a, r in ((o, o_ref), (lse, lse_ref))]
+    print(err)
+    assert err[True][0] <= err[False][0] and err[True][1] <= 3.2e-8, err
+    plan.destroy()
+
+
+def test_split_route_with_values_out_of_range(gu):
+    """Infinite, NaN and very large rows: rows that see none of them are untouched, the others as in fp64 (overflow aside)."""
+    from paper_2507_05228_b200 import binding as cb
+    B, n, H = 8, 300, 16
+    w = wl.make_workload("split_big", B, n, n, H, H, 64, "f32", "random", "random", 3, 3, seed=9)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    q[:, :, 1].abs_()
+    k[:, 70, 1] = -(2.0 ** 126)          # logits below every other one: no weight
+    k[:, 130, 2, 5] = 2.0 ** 80          # logits of either sign and 2^80
+    v[:, 200, 3, 7] = float("inf")
+    v[:, 210, 4, 9] = float("nan")
+    v[:, 220, 5] = 3.4e38
+    q[:, 33, 6, 2] = 2.0 ** 70
+    o, lse, n_kernels = _fused(cb, plan, q, k, v, w.scale)
+    assert n_kernels == 2 and plan.device_status() == 0
+    s = torch.einsum("bqhd,bkhd->bhqk", q.double(), k.double()) * float(np.float32(w.scale))
+    s = s.masked_fill(~torch.ones(n, n, dtype=torch.bool, device="cuda").tril(), -torch.inf)
+    a = torch.softmax(s, -1)
+    o_ref = torch.einsum("bhqk,bkhd->bqhd", a, v.double().nan_to_num(nan=0.0, posinf=0.0))
+    assert torch.isinf(o[:, 200:, 3, 7]).all() and torch.isnan(o[:, 210:, 4, 9]).all()
+    o[:, 200:, 3, 7] = 0
+    o[:, 210:, 4, 9] = 0
+    o_ref[:, 200:, 3, 7] = 0
+    o_ref[:, 210:, 4, 9] = 0
+    assert ((o.double() - o_ref).abs() <= w.tol * o_ref.abs().clamp_min(1.0)).all()
+    assert torch.allclose(lse.double(), torch.logsumexp(s, -1).transpose(1, 2), rtol=1e-5, atol=w.tol)
+    plan.destroy()
+
+
+def test_captured_split_calls_follow_the_plan(gu):
+    from paper_2507_05228_b200 import binding as cb
+    B, n_q, n_kv, H, P = 8, 128, 700, 16, 3
+    w = wl.make_workload("split_graph", B, n_kv, n_kv, H, H, 64, "f32", "random", "random", 1, 1, seed=4)
+    q, k, v = gu.to_device(w)
+    rng = np.random.default_rng(P)
+    kv_of, q_of = rng.integers(0, P, n_kv).astype(np.int32), rng.integers(0, 2, n_q).astype(np.int32)
+    plan = cb.cascade_shard_plan(q_of, kv_of, 2, P, 100, True)
+    qc, kc, vc = q[:, :n_q].clone(), k.clone(), v.clone()
+    ws = torch.empty(cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED, cb.F32, B, H, H, 64), dtype=torch.uint8, device="cuda")
+    o = torch.zeros_like(qc)
+    parts = [t.clone() for t in cb.cascade_attn_partials(plan, qc, k, v, w.scale, workspace=ws)]
+    n0 = cb.lib().cascade_launch_count()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        cb.cascade_attn_sharded(plan, qc, kc, vc, w.scale, out=o, want_lse=False, workspace=ws)
+        cb.cascade_attn_partials(plan, qc, kc, vc, w.scale, out=parts, workspace=ws)
+    assert cb.lib().cascade_launch_count() - n0 == 4
+    for off in (100, 572, 20):
+        seen = off + n_q
+        qc.copy_(q[:, off:seen])
+        kc.fill_(float("nan")), vc.fill_(float("nan"))
+        kc[:, :seen], vc[:, :seen] = k[:, :seen], v[:, :seen]
+        plan.advance(off)
+        graph.replay()
+        torch.cuda.synchronize()
+        o_ref, _ = oracle.attention_unsharded(w.q[:, off:seen], w.k, w.v, w.scale, q_pos_offset=off)
+        gu.check_output(o, None, o_ref, None, w.tol, f"replayed at {off}")
+        op = oracle.shard_plan(q_of, kv_of, 2, P, q_pos_offset=off, causal=True)
+        u, m, e = oracle.attn_pass(w.q[:, off:seen], w.k, w.v, w.scale, op)
+        gu.check_partials(tuple(t.double().cpu().numpy() for t in parts), (u, m, e), w.tol, f"partials at {off}")
+    del graph
+    plan.destroy()
+
+
+def test_split_calls_on_a_plan_whose_status_word_is_set_write_nothing(gu):
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload("split_gave_up", 8, 300, 300, 16, 16, 64, "f32", "random", "random", 2, 3, seed=2, symmetric=False)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    word = torch.as_tensor(gu._DevicePointer(plan.dev_ptr("q_off") - 256, 1, "<i4"), device="cuda")
+    o_ref, _ = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+    word.fill_(5)
+    o = torch.full_like(q, 7.0)
+    parts = cb.cascade_attn_partials(plan, q, k, v, w.scale)
+    for t in parts:
+        t.fill_(7.0)
+    cb.cascade_attn_sharded(plan, q, k, v, w.scale, out=o, want_lse=False)
+    cb.cascade_attn_partials(plan, q, k, v, w.scale, out=parts)
+    torch.cuda.synchronize()
+    assert (o == 7).all() and all((t == 7).all() for t in parts)
+    word.fill_(0)
+    cb.cascade_attn_sharded(plan, q, k, v, w.scale, out=o, want_lse=False)
+    assert torch.equal(o, o_ref) and plan.device_status() == 0
+    plan.destroy()
