@@ -124,12 +124,13 @@ enum Bar {
   V_EMPTY = V_FULL + kMaxStages,    // [kVStages]
   S_FULL = V_EMPTY + kMaxStages,    // [2]; kRing: [2][2], see s_full
   P_FULL = S_FULL + 4,              // [2]; kRing: [2][2], see p_full
-  O_FULL = P_FULL + 4,              // [1]
-  CHECKED = O_FULL + 1,             // [1] the plan's status word has been looked at
+  O_FULL = P_FULL + 4,              // [2] the last product of a sub-tile is in
+  CHECKED = O_FULL + 2,             // [1] the plan's status word has been looked at
   O_RDY = CHECKED + 1               // [2]  kWalk: the accumulator of a sub-tile holds a finished shard;
                                     //      kRing: the product of a sub-tile's latest tile is in its accumulator
 };
-static_assert(O_RDY + 2 <= Cfg<128, false>::kNumBars, "barrier table too small");
+constexpr int kBars = O_RDY + 2;
+static_assert(kBars <= Cfg<128, false>::kNumBars && kBars <= 32, "barrier table too small");
 
 // TMA box loads, 64 elements wide: rows land as 128 bytes each.  32 rows of the 3-D tensor [matrix z][row y][column x]
 // (shard-major copies), or 128 rows of the 4-D tensor [sequence w][head z][row y][column x].
@@ -241,7 +242,7 @@ struct TmaArgs {
 // the barriers and the K/V pipelines are set up once per query tile instead of once per (query tile, KV shard).
 template <int D, bool kRope, bool kWalk, bool kBoxes>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_constant__ AttnParams p, int lg,
-                                                              int tile_major, int split, int early, int after_gather,
+                                                              int tile_major, int lg_split, int early, int after_gather,
                                                               const __grid_constant__ TmaArgs tma) {
   using C = Cfg<D, kBoxes>;
   constexpr int kD = D, kTileBytes = C::kTileBytes, kKStages = C::kKStages, kVStages = C::kVStages;
@@ -269,27 +270,24 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   const int Gp = 1 << lg, R = kM >> lg;
   const PlanDev& pl = p.plan;
   const int P = pl.n_kv_shards;
-  // CTA index -> (query tile, batch, head group).  The tiles are listed by decreasing work.  With few CTAs per SM the
+  // Block index -> (query tile, sequence, head group).  The tiles are listed by decreasing work.  With few CTAs per SM the
   // query tile is the slowest index, so that the heaviest CTAs of all heads and sequences start first and the light ones
   // fill the tail.  For a large problem the head group is slowest instead: the CTAs running at any time then read the
-  // K/V of few KV heads, which keeps that stream in L2.
-  const int n_hg = p.H >> lg;
+  // K/V of few KV heads, which keeps that stream in L2.  (The grid has an axis for each, and what is a power of two is
+  // shifted: the divisions of a flat index took 900 of the 5300 cycles before a CTA's first logits.)
+  const int split = 1 << lg_split;
   const int ts = 3 - lg;  // kWalk: tile list of 2 R = 256 >> lg slots
-  const int n_qt = kWalk ? pl.n_qtiles[ts] : (pl.n_q + 2 * R - 1) / (2 * R);
-  const int cta = kWalk ? blockIdx.x : blockIdx.x / split;
-  const int part_of_keys = kWalk ? 0 : blockIdx.x % split;  // rank in the cluster that shares a query tile's keys
-  int tile_idx, hg, b;
+  const int n_qt = kWalk ? pl.n_qtiles[ts] : (pl.n_q + 2 * R - 1) >> (8 - lg);
+  int tile_idx, hg, b, part_of_keys = 0;  // part_of_keys: rank in the cluster that shares a query tile's keys
   if (tile_major) {
-    const int per_tile = n_hg * p.batch;
-    const int rem = cta % per_tile;
-    tile_idx = cta / per_tile;
-    hg = rem % n_hg;
-    b = rem / n_hg;
+    hg = (int)blockIdx.x >> lg_split;
+    part_of_keys = (int)blockIdx.x & (split - 1);
+    b = blockIdx.y;
+    tile_idx = blockIdx.z;
   } else {
-    const int rem = cta / n_qt;
-    tile_idx = cta % n_qt;
-    hg = rem % n_hg;
-    b = rem / n_hg;
+    tile_idx = blockIdx.x;
+    hg = blockIdx.y;
+    b = blockIdx.z;
   }
   // A gather right before this grid runs after all that came before it, and writes only what the loaders read: they wait
   // for it.
@@ -297,7 +295,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   if (!after_gather) grid_wait();
   const int map = pl.n_maps == 1 ? 0 : b;
   const int h0 = hg * Gp;  // first of the Gp stacked heads
-  const int g = h0 / p.G;  // their KV head
+  const int per_kv = p.G >> lg;  // head groups per KV head
+  const int g = per_kv == 1 ? hg : hg / per_kv;
   int row0, nrows;         // kWalk: slots of the shard-major order; otherwise tokens
   if constexpr (kWalk) {
     const int4 qt = pl.qtiles[ts][(size_t)map * pl.n_qtiles[ts] + tile_idx];
@@ -408,7 +407,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       // the keys the last row sees, in tiles of 128 from the first on; this CTA takes its part of the tiles
       const int seen = lane < 3 ? seen_by(lane == 0 ? row0 + nrows - 1 : row0 + (lane == 2 ? (n_sub - 1) * R : 0)) : 0;
       const int tiles = (__shfl_sync(0xffffffffu, seen, 0) + kNMax - 1) / kNMax;
-      const int t0 = tiles * part_of_keys / split, t1 = tiles * (part_of_keys + 1) / split;
+      const int t0 = tiles * part_of_keys >> lg_split, t1 = tiles * (part_of_keys + 1) >> lg_split;
       if (lane == 0) {
         tab->need[0] = max(0, min(seen, t1 * kNMax) - t0 * kNMax);  // keys of this CTA's part
         tab->slot0[0] = t0 * kNMax;
@@ -426,54 +425,44 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     if (lane == 0) wc.note(warp, v);
   };
 
-  if (tid == 9 * 32) {
-    mbar_init(bar(Q_FULL), q_boxes ? 1 : 128);  // 128: every thread of the sub-tile's softmax group brings a share of the rows
-    mbar_init(bar(Q_FULL + 1), q_boxes ? 1 : 128);
-    for (int s = 0; s < kKStages; ++s) {
-      mbar_init(bar(K_FULL + s), 1);  // TMA: one arrival that announces the byte count, then the bytes
-      mbar_init(bar(K_EMPTY + s), 1);
+  // Warp 9 sets the barriers up, a lane each, and has the first data on their way.  (A barrier that nobody else waits for it at, past
+  // the requests, costs the softmax threads registers: partials of 4099 tokens in 16 shards 392 -> 418 us.)
+  if (warp == 9) {
+    if (lane < kBars) {  // one arrival, except by the threads of a sub-tile; TMA: one that announces the byte count, then the bytes
+      const bool by_rows = lane < Q_FULL + 2 ? !q_boxes : lane >= P_FULL && lane < P_FULL + 4;
+      mbar_init(bar(lane), by_rows ? 128u : 1u);
     }
-    for (int s = 0; s < kVStages; ++s) {
-      mbar_init(bar(V_FULL + s), 1);
-      mbar_init(bar(V_EMPTY + s), 1);
-    }
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(bar(S_FULL + s), 1);
-      mbar_init(bar(S_FULL + 2 + s), 1);
-      mbar_init(bar(P_FULL + s), 128);
-      mbar_init(bar(P_FULL + 2 + s), 128);
-    }
-    mbar_init(bar(O_FULL), 1);
-    mbar_init(bar(CHECKED), 1);
-    mbar_init(bar(O_RDY), 1);
-    mbar_init(bar(O_RDY + 1), 1);
-    wc.store(1, 0);
-    for (int w = 0; w < kThreads / 32; ++w) wc.store(2 + w, 0);
+    if (lane < kThreads / 32) wc.store(2 + lane, 0);
+    if (lane == 0) wc.store(1, 0);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    __syncwarp();
     if constexpr (!kWalk) {
-      // The query rows and the first tiles of K and V (early, bit 0: K, bit 1: V; not what a gather in front of this grid
-      // writes) are requested here, under the rest of the set-up.  (Query rows loaded by the softmax threads cost a CTA 2700
-      // cycles before its first product: 2048 tokens 40.3 -> 38.5 us, 2 x 3001 tokens of head_dim 64 78.2 -> 76.7.)
-      const int tiles = (seen_by(row0 + nrows - 1) + kNMax - 1) / kNMax;
-      const int t0 = tiles * part_of_keys / split;
-      if (tiles * (part_of_keys + 1) / split > t0) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        auto request_q = [&](int s) {
-          mbar_expect_tx(bar(Q_FULL + s), (uint32_t)kTileBytes);
-          for (int half = 0; half < C::kHalves; ++half)
-            tma_tile4(smem_base + (uint32_t)(kOffQ + s * kTileBytes + half * kHalfBytes), &tma.q, 64 * half, h0, row0 + s * R, b,
-                      bar(Q_FULL + s));
-        };
-        auto request_kv = [&](const CUtensorMap* map, uint32_t dst, uint32_t fb) {
-          mbar_expect_tx(fb, (uint32_t)kTileBytes);
-          tma_tile4(dst, map, 0, t0 * kNMax, g, b, fb);
-          if (C::kHalves == 2) tma_tile4(dst + (uint32_t)kHalfBytes, map, 64, t0 * kNMax, g, b, fb);
-        };
-        if (q_boxes) request_q(0);
-        if (early & 1) request_kv(&tma.k, smem_base + kOffK, bar(K_FULL));
-        if (q_boxes && n_sub == 2) request_q(1);
-        if (early & 2) request_kv(&tma.v, smem_base + kOffV, bar(V_FULL));
+      if (lane == 0) {
+        // The query rows and the first tiles of K and V (early, bit 0: K, bit 1: V; not what a gather in front of this grid
+        // writes) are requested here, under the rest of the set-up.  (Query rows loaded by the softmax threads cost a CTA 2700
+        // cycles before its first product: 2048 tokens 40.3 -> 38.5 us, 2 x 3001 tokens of head_dim 64 78.2 -> 76.7.)
+        const int tiles = (seen_by(row0 + nrows - 1) + kNMax - 1) / kNMax;
+        const int t0 = tiles * part_of_keys >> lg_split;
+        if (tiles * (part_of_keys + 1) >> lg_split > t0) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          auto request_q = [&](int s) {
+            mbar_expect_tx(bar(Q_FULL + s), (uint32_t)kTileBytes);
+            for (int half = 0; half < C::kHalves; ++half)
+              tma_tile4(smem_base + (uint32_t)(kOffQ + s * kTileBytes + half * kHalfBytes), &tma.q, 64 * half, h0, row0 + s * R, b,
+                        bar(Q_FULL + s));
+          };
+          auto request_kv = [&](const CUtensorMap* map, uint32_t dst, uint32_t fb) {
+            mbar_expect_tx(fb, (uint32_t)kTileBytes);
+            tma_tile4(dst, map, 0, t0 * kNMax, g, b, fb);
+            if (C::kHalves == 2) tma_tile4(dst + (uint32_t)kHalfBytes, map, 64, t0 * kNMax, g, b, fb);
+          };
+          if (q_boxes) request_q(0);
+          if (early & 1) request_kv(&tma.k, smem_base + kOffK, bar(K_FULL));
+          if (q_boxes && n_sub == 2) request_q(1);
+          if (early & 2) request_kv(&tma.v, smem_base + kOffV, bar(V_FULL));
+        }
       }
+      __syncwarp();
     }
   }
   if (warp == 8) {
@@ -911,7 +900,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         const int pitch = cols * 4 + 16;  // bytes between received rows: spreads a warp's 16-byte stores over the banks
         const int row = s * kM + m;
         if (n_tiles > 0) {
-          wait_bar(wc, bar(O_FULL), 0u, 3, n_tiles);
+          wait_bar(wc, bar(O_FULL + s), 0u, 3, n_tiles);
           tc_fence_after();
         }
         const bool out_ok = may_write() && row_ok;
@@ -1018,7 +1007,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       }
       float o_scale = 0.f, m_out = -INFINITY, l_out = 0.f;
       if (n_tiles > 0) {
-        wait_bar(wc, bar(O_FULL), 0u, 3, n_tiles);
+        wait_bar(wc, bar(O_FULL + s), 0u, 3, n_tiles);
         tc_fence_after();
         if (l_run > 0.f) {
           o_scale = 1.f / (l_run + l_fix);
@@ -1192,6 +1181,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
               wait_bar(wc, p_full(s, i), s_parity(i), 5, i);
               tc_fence_after();
               issue_pv(s, i, n_cur, opens_cur);
+              if (i == n_run - 1 && leader) mma_commit(bar(O_FULL + s));
               if (s == last_sub && leader) mma_commit(bar(V_EMPTY + i % kVStages));
               if (s == 0 && n_sub == 2 && i + 1 < n_run) {
                 issue_qk(1, i + 1, n_next);
@@ -1224,6 +1214,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             wait_bar(wc, p_full(s, i), s_parity(i), 5, i);
             tc_fence_after();
             issue_pv(s, i, n_cur, opens_cur);
+            if (!has_next && leader) mma_commit(bar(O_FULL + s));
             if (kWalk && has_next && opens_next && leader) mma_commit(bar(O_RDY + s));
             if (s == n_sub - 1 && leader) mma_commit(bar(V_EMPTY + i % kVStages));
             if (has_next) {
@@ -1238,8 +1229,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           }
         }
         }
-        if (leader) mma_commit(bar(O_FULL));
         if (n_run == 0) {
+          if (leader) mma_commit(bar(O_FULL));
           if (q_boxes)
             for (int s = 0; s < n_sub; ++s) landed(bar(Q_FULL + s), 0u);
           landed(bar(O_FULL), 0u);
@@ -1399,12 +1390,12 @@ bool encode_queries(CUtensorMap* map, const AttnParams& p, int lg) {
 }
 
 struct TcLaunch {
-  int lg, tile_major, split, early;
+  int lg, tile_major, lg_split, early;
   bool after_gather;
   bool boxes;  // partials at head_dim 128
 };
 
-cudaError_t launch_kernel(const AttnParams& p, bool walk, const TcLaunch& l, int64_t n_ctas, const tc::TmaArgs& tma,
+cudaError_t launch_kernel(const AttnParams& p, bool walk, const TcLaunch& l, int64_t n_tiles, const tc::TmaArgs& tma,
                           cudaStream_t stream) {
   auto kernel = p.d == 64 ? (walk ? tc::attn_tc_kernel<64, false, true, true> : tc::attn_tc_kernel<64, false, false, false>)
                 : p.rope  ? tc::attn_tc_kernel<128, true, false, false>
@@ -1414,10 +1405,12 @@ cudaError_t launch_kernel(const AttnParams& p, bool walk, const TcLaunch& l, int
                                    : (l.boxes ? tc::Cfg<128, true>::kSmemBytes : tc::Cfg<128, false>::kSmemBytes);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
-  if (n_ctas * l.split >= (int64_t)1 << 31) return cudaErrorInvalidConfiguration;
+  // (few CTAs if tile_major; a head group has a head, so n_hg and the batch fit the short axes as the entry points check)
+  const unsigned n_hg = (unsigned)(p.H >> l.lg), batch = (unsigned)p.batch, tiles = (unsigned)n_tiles;
+  const dim3 grid = l.tile_major ? dim3(n_hg << l.lg_split, batch, tiles) : dim3(tiles, n_hg, batch);
   TimedLaunch timed(stream);
-  return launch_dependent(kernel, dim3((unsigned)(n_ctas * l.split)), tc::kThreads, smem_bytes, l.split,
-                          !walk || l.after_gather, stream, p, l.lg, l.tile_major, l.split, l.early, (int)l.after_gather, tma);
+  return launch_dependent(kernel, grid, tc::kThreads, smem_bytes, 1u << l.lg_split, !walk || l.after_gather, stream, p, l.lg,
+                          l.tile_major, l.lg_split, l.early, (int)l.after_gather, tma);
 }
 
 // stack as many of the G heads of a KV head into one MMA tile as divide G (at most 8)
@@ -1469,8 +1462,8 @@ cudaError_t launch_attn_tc_partials(const AttnParams& p, const void* k_sorted, c
                                     {n_q * p.H * p.d, (int64_t)p.H * p.d, p.d});
   const int64_t n_ctas = n_tiles * (p.H >> lg) * p.batch;
   // few CTAs per SM: balance matters more than L2 locality
-  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), 1, 0, true, boxes && tma.o_valid};
-  return launch_kernel(p, true, l, n_ctas, tma, stream);
+  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), 0, 0, true, boxes && tma.o_valid};
+  return launch_kernel(p, true, l, n_tiles, tma, stream);
 }
 
 cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v, int64_t n_seen, bool k_gathered, bool v_gathered,
@@ -1492,15 +1485,15 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TcRows& k, const TcRows& v
   // and 32.2 -> 26.9.  12 tiles in clusters of four take 32.8, alone 36.9.  The rule is the same with and without a rotary
   // step, so that both sum in the same order.  It counts the heads of the whole problem, see AttnParams.
   const int64_t rule_ctas = n_qt * ((int64_t)p.rule_kv_heads * p.G >> lg) * p.batch, key_tiles = (n_seen + 127) / 128;
-  int split = 1;
+  int lg_split = 0;
   if (p.fused) {
     const int64_t fit[4] = {148, 148, 132, 120};
     for (int i = 1; i < 4; ++i)
-      if (rule_ctas << i <= fit[i] && key_tiles >= (p.d == 64 ? 2 : 3) << i) split = 1 << i;
+      if (rule_ctas << i <= fit[i] && key_tiles >= (p.d == 64 ? 2 : 3) << i) lg_split = i;
   }
-  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), split,
+  const TcLaunch l = {lg, n_ctas <= 8 * (int64_t)sm_count(), lg_split,
                       p.prefix_from_vis ? 0 : (k_gathered ? 0 : 1) | (v_gathered ? 0 : 2), k_gathered || v_gathered, false};
-  return launch_kernel(p, false, l, n_ctas, tma, stream);
+  return launch_kernel(p, false, l, n_qt, tma, stream);
 }
 
 }  // namespace cascade
