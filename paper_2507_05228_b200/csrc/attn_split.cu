@@ -425,7 +425,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
       TileSeq seq(longest(s), n_parts);
       while (seq.next()) {
         if (i > 0) fold(prev_k, prev_t0, prev_n, i - 1, alpha);
-        note(8 * i + 1);
         const int n = seq.n;
         const int seen = seen_of(seq.k, seq.t0, n);  // (ahead of the wait, which hides the load)
         wait_bar(wc, bar(S_FULL + s), (uint32_t)(i & 1), 1, i);
@@ -502,7 +501,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
         const uint64_t alpha2 = pack2(alpha, alpha);
         l_run[0] = ffma2(l_run[0], alpha2, fadd2(sum[0], sum[1]));
         l_run[1] = ffma2(l_run[1], alpha2, fadd2(sum[2], sum[3]));
-        note(8 * i + 2);
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(bar(P_FULL + s));
@@ -569,39 +567,41 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
           mma_commit(bar(O_FULL + s));
         };
         uint32_t done0 = 0;  // tiles of sub-tile 0 that are finished (the other one sees them all)
-        wait_bar(wc, bar(K_FULL), 0u, 7);
+        // When a wait has given up, no stage is given back that may not be full (the loader would have a second load counted on its
+        // barrier while the first is under way), and the loop ends.
+        bool fed = wait_bar(wc, bar(K_FULL), 0u, 7);
         int info = tile_info[0];
         wait_bar(wc, bar(Q_FULL), 0u, 6);
         if (n_sub == 2) wait_bar(wc, bar(Q_FULL + 1), 0u, 6);
         tc_fence_after();
         if (info & 256) issue_qk(0, 0);
         if (n_sub == 2) issue_qk(1, 0);
-        mma_commit(bar(K_EMPTY));
-        for (int i = 0; i < n_tiles && !wc.load(1); ++i) {
+        if (fed) mma_commit(bar(K_EMPTY));
+        for (int i = 0; i < n_tiles && fed && !wc.load(1); ++i) {
           const bool more = i + 1 < n_tiles;
           int next = 0;
-          wait_bar(wc, bar(V_FULL + (i & 1)), (uint32_t)((i >> 1) & 1), 4, i);
+          fed = wait_bar(wc, bar(V_FULL + (i & 1)), (uint32_t)((i >> 1) & 1), 4, i);
           if (info & 256) {
             wait_bar(wc, bar(P_FULL), done0 & 1, 5, i);
             tc_fence_after();
             issue_pv(0, i, info & 255);
             ++done0;
           }
-          if (n_sub == 1) mma_commit(bar(V_EMPTY + (i & 1)));
+          if (n_sub == 1 && fed) mma_commit(bar(V_EMPTY + (i & 1)));
           if (more) {
-            wait_bar(wc, bar(K_FULL + ((i + 1) & 1)), (uint32_t)(((i + 1) >> 1) & 1), 7, i);
+            fed = wait_bar(wc, bar(K_FULL + ((i + 1) & 1)), (uint32_t)(((i + 1) >> 1) & 1), 7, i) && fed;
             next = tile_info[(i + 1) & 1];
             if (next & 256) issue_qk(0, i + 1);
-            if (n_sub == 1) mma_commit(bar(K_EMPTY + ((i + 1) & 1)));
+            if (n_sub == 1 && fed) mma_commit(bar(K_EMPTY + ((i + 1) & 1)));
           }
           if (n_sub == 2) {
             wait_bar(wc, bar(P_FULL + 1), (uint32_t)(i & 1), 5, i);
             tc_fence_after();
             issue_pv(1, i, info & 255);
-            mma_commit(bar(V_EMPTY + (i & 1)));
+            if (fed) mma_commit(bar(V_EMPTY + (i & 1)));
             if (more) {
               issue_qk(1, i + 1);
-              mma_commit(bar(K_EMPTY + ((i + 1) & 1)));
+              if (fed) mma_commit(bar(K_EMPTY + ((i + 1) & 1)));
             }
           }
           info = next;

@@ -421,6 +421,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   if constexpr (kWalk) wc.words = reinterpret_cast<volatile int*>(smem + kOffMisc);
   else wc.misc = smem_base + (uint32_t)kOffMisc;
   wc.status = pl.status;
+
   auto note = [&](int v) {
     if (lane == 0) wc.note(warp, v);
   };
@@ -685,7 +686,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             }
           }
         }
-        note(8 * i + 1);
         if constexpr (kWalk) {
           // The issuing warp commits O_RDY right after the last product of a shard, before it issues the logits of
           // this tile, so the previous shard's partial is written out while those logits are computed.  The first
@@ -887,9 +887,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           l_run += psum0 + psum1;
           l_fix += top_error();
         }
-        note(8 * i + 2);
       }
-      note(8 * n_tiles + 3);
       auto may_write = [&]() {  // asked after the last product; see goes_on
         return (n_tiles > 0 ? wc.load(1) : *reinterpret_cast<volatile const int32_t*>(wc.status)) == 0;
       };
@@ -1147,21 +1145,23 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         TileSeq<kWalk> seq(tab, n_act, n_keys);
         bool opens_cur = true, opens_next = false;
         int n_cur = kChunk * seq.next(opens_cur), n_next = 0;
-        wait_bar(wc, bar(K_FULL), 0u, 7);
+        // A wait that gives up ends the role: nothing more is issued, and no stage given back that may not be full (the loader
+        // would have a second load counted on its barrier while the first is under way).
+        bool fed = wait_bar(wc, bar(K_FULL), 0u, 7);
         for (int s = 0; s < n_sub; ++s) {
-          wait_bar(wc, bar(Q_FULL + s), 0u, 6);
+          fed = fed && wait_bar(wc, bar(Q_FULL + s), 0u, 6);
           tc_fence_after();
-          issue_qk(s, 0, n_cur);
+          if (fed) issue_qk(s, 0, n_cur);
         }
-        if (leader) mma_commit(bar(K_EMPTY));
-        int n_run = n_tiles;
+        if (fed && leader) mma_commit(bar(K_EMPTY));
+        int n_run = fed ? n_tiles : 0;
         if constexpr (kRing) {
           // Order: QK_0(0) QK_1(0) QK_0(1), then per tile i: PV_0(i) QK_1(i+1) PV_1(i) QK_0(i+2).  QK_1(i+1) takes the
           // buffer PV_0(i) has read, QK_0(i+2) the one of PV_1(i); MMAs execute in issue order, so neither needs a
           // barrier.  K(j) is released after QK_1(j), the later of its two readers.
           const int last_sub = n_sub - 1;
           auto wait_k = [&](int i) {
-            wait_bar(wc, bar(K_FULL + i % kKStages), (uint32_t)((i / kKStages) & 1), 7, i);
+            fed = fed && wait_bar(wc, bar(K_FULL + i % kKStages), (uint32_t)((i / kKStages) & 1), 7, i);
             tc_fence_after();
           };
           bool opens_2 = false;
@@ -1169,16 +1169,16 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           if (n_tiles > 1) {
             n_next = kChunk * seq.next(opens_next);
             wait_k(1);
-            issue_qk(0, 1, n_next);
-            if (last_sub == 0 && leader) mma_commit(bar(K_EMPTY + 1 % kKStages));
+            if (fed) issue_qk(0, 1, n_next);
+            if (fed && last_sub == 0 && leader) mma_commit(bar(K_EMPTY + 1 % kKStages));
           }
-          if (!goes_on()) n_run = 0;
+          if (!fed || !goes_on()) n_run = 0;
           for (int i = 0; i < n_run; ++i) {
             n_2 = i + 2 < n_run ? kChunk * seq.next(opens_2) : 0;
-            wait_bar(wc, bar(V_FULL + i % kVStages), (uint32_t)((i / kVStages) & 1), 4, i);
-            for (int s = 0; s < n_sub; ++s) {
-              note(8 * i + 2 + s);
-              wait_bar(wc, p_full(s, i), s_parity(i), 5, i);
+            fed = wait_bar(wc, bar(V_FULL + i % kVStages), (uint32_t)((i / kVStages) & 1), 4, i);
+            for (int s = 0; s < n_sub && fed; ++s) {
+              fed = wait_bar(wc, p_full(s, i), s_parity(i), 5, i);
+              if (!fed) break;
               tc_fence_after();
               issue_pv(s, i, n_cur, opens_cur);
               if (i == n_run - 1 && leader) mma_commit(bar(O_FULL + s));
@@ -1189,29 +1189,30 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
               }
               if (s == last_sub && i + 2 < n_run) {
                 wait_k(i + 2);
+                if (!fed) break;
                 issue_qk(0, i + 2, n_2);
                 if (last_sub == 0 && leader) mma_commit(bar(K_EMPTY + (i + 2) % kKStages));
               }
             }
+            if (!fed) break;
             n_cur = n_next;
             opens_cur = opens_next;
             n_next = n_2;
             opens_next = opens_2;
           }
         } else {
-        if (!goes_on()) n_run = 0;
-        for (int i = 0; i < n_run; ++i) {
+        if (!fed || !goes_on()) n_run = 0;
+        for (int i = 0; i < n_run && fed; ++i) {
           const bool has_next = i + 1 < n_run;
           if (i > 0) {
             n_cur = n_next;
             opens_cur = opens_next;
           }
           n_next = has_next ? kChunk * seq.next(opens_next) : 0;
-          note(8 * i + 1);
-          wait_bar(wc, bar(V_FULL + i % kVStages), (uint32_t)((i / kVStages) & 1), 4, i);
-          for (int s = 0; s < n_sub; ++s) {
-            note(8 * i + 2 + s);
-            wait_bar(wc, p_full(s, i), s_parity(i), 5, i);
+          fed = wait_bar(wc, bar(V_FULL + i % kVStages), (uint32_t)((i / kVStages) & 1), 4, i);
+          for (int s = 0; s < n_sub && fed; ++s) {
+            fed = wait_bar(wc, p_full(s, i), s_parity(i), 5, i);
+            if (!fed) break;
             tc_fence_after();
             issue_pv(s, i, n_cur, opens_cur);
             if (!has_next && leader) mma_commit(bar(O_FULL + s));
@@ -1219,8 +1220,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             if (s == n_sub - 1 && leader) mma_commit(bar(V_EMPTY + i % kVStages));
             if (has_next) {
               if (s == 0) {
-                note(8 * i + 4);
-                wait_bar(wc, bar(K_FULL + (i + 1) % kKStages), (uint32_t)(((i + 1) / kKStages) & 1), 7, i);
+                fed = wait_bar(wc, bar(K_FULL + (i + 1) % kKStages), (uint32_t)(((i + 1) / kKStages) & 1), 7, i);
+                if (!fed) break;
                 tc_fence_after();
               }
               issue_qk(s, i + 1, n_next);
@@ -1229,13 +1230,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           }
         }
         }
-        if (n_run == 0) {
+        if (n_run == 0 || !fed) {
           if (leader) mma_commit(bar(O_FULL));
           if (q_boxes)
             for (int s = 0; s < n_sub; ++s) landed(bar(Q_FULL + s), 0u);
           landed(bar(O_FULL), 0u);
         }
-        note(7);
       }
       __syncwarp();
     } else {
