@@ -99,11 +99,16 @@ __device__ __forceinline__ void decode_init(DecodeState& st) {
 // block instead of two and the arithmetic (a block took 3200 cycles one after another).  Without it nothing is spilled,
 // which is the better trade where 16 warps per SM cover the latencies anyway (partials of 64 sequences of 16384 tokens: 630
 // us without, 820 with; all shards in one kernel: 711 without, 620 with).
-template <bool kAhead, typename Get>
+// gate() is called before the first rows are requested, ready() before the query is used; by a warp without blocks, too.
+template <bool kAhead, typename Get, typename Gate, typename Ready>
 __device__ __forceinline__ void decode_walk(DecodeState& st, const DecodeQuery& q, const PlanDev& pl, const int32_t* kv_idx,
                                             int count, Get get, const __nv_bfloat16* kp, int64_t k_token,
-                                            const __nv_bfloat16* vp, int64_t v_token, int lane, float cs) {
-  if (count <= 0) return;
+                                            const __nv_bfloat16* vp, int64_t v_token, int lane, float cs, Gate gate, Ready ready) {
+  if (count <= 0) {
+    gate();
+    ready();
+    return;
+  }
   const int x = lane >> 2, j = lane & 3;
   uint32_t ka[16], kb[16], vr[4][8];
   auto token = [&](int2 e) {  // lane l: token of key l (clamped to the last key; masked below)
@@ -128,9 +133,11 @@ __device__ __forceinline__ void decode_walk(DecodeState& st, const DecodeQuery& 
   if constexpr (kAhead) {
     e = get(0);
     tok = token(e);
+    gate();
     load_k(tok);
     load_v(tok);
     if (count > 1) tok = token(get(1));
+    ready();
   }
 #pragma unroll 1
   for (int t = 0; t < count; ++t) {
@@ -277,7 +284,7 @@ __global__ void __launch_bounds__(128, 4) decode_kernel(const __grid_constant__ 
   decode_init(st);
   decode_walk<false>(st, s_q, pl, kv_idx, (n_vis - warp * 16 + NW * 16 - 1) / (NW * 16),
                      [&](int t) { const int k0 = (t * NW + warp) * 16; return make_int2(k0, n_vis - k0); }, kb, p.ks.token,
-                     vb, p.vs.token, lane, cs);
+                     vb, p.vs.token, lane, cs, []() {}, []() {});
   decode_publish<G, NW>(sh, st, warp, lane);
   __syncthreads();
   // thread = output column
@@ -302,8 +309,8 @@ __global__ void __launch_bounds__(128, 4) decode_kernel(const __grid_constant__ 
 // then "Caching"): query rows are turned while they are loaded, and the new token's key row is turned and written, with its
 // value row, to the caches before anyone reads them.
 // Measured (32 query / 8 KV heads): 64 sequences of 16384 tokens in 16 shards 662 us on inputs new to the caches = 6.49 TB/s
-// (repeated on the same ones, of which L2 keeps a part, 608; partials and merge as two kernels 825), one sequence 23 us (44); the whole step of one sequence at 2500 of 4096 rows 10.5 us (38, four launches
-// and two copies).
+// (repeated on the same ones, of which L2 keeps a part, 608; partials and merge as two kernels 825), one sequence 22 us (30 with
+// eight warps a CTA); the whole step of one sequence at 2500 of 4096 rows 7.7 us (9.4 with eight warps and the table behind a barrier).
 
 __device__ __forceinline__ uint32_t rotate_pair2(uint32_t x, uint32_t partner, const float4& cs, float sign) {
   // two neighbouring columns of one half: y = x cos + sign * partner * sin  (sign -1: lower half, +1: upper half)
@@ -315,11 +322,12 @@ __device__ __forceinline__ uint32_t rotate_pair2(uint32_t x, uint32_t partner, c
 constexpr int kMaxCluster = 16;
 constexpr int kFusedShards = 256;  // KV shards whose table fits in the kernel's shared memory at a time
 
-template <int G, int NW>
+template <int G, int NW, bool kOneList>
 __global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __grid_constant__ AttnParams p,
                                                                        const __grid_constant__ DecodeStep step) {
   constexpr int D = 128;
-  __shared__ DecodeShared<G, NW> sh;
+  extern __shared__ __align__(16) uint8_t smem_decode[];
+  DecodeShared<G, NW>& sh = *reinterpret_cast<DecodeShared<G, NW>*>(smem_decode);
   __shared__ DecodeQuery s_q;
   // what the CTAs of the cluster send for this CTA's part of the outputs: [sender][output], and n, w of every head
   __shared__ float s_o[G * D + kMaxCluster], s_n[kMaxCluster][G], s_w[kMaxCluster][G];
@@ -385,15 +393,13 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __
       s_most = most;
     }
   };
-  if (warp == 0) fill_table(0);
-  if (warp == 1) {
+  if (warp == 0 && !kOneList) fill_table(0);
+  if (warp == NW - 1) {
     uint32_t qf[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) qf[c] = 0u;
-    if (x < G) {
-      const int tok_q = (int)CASCADE_CHECKED((int64_t)pl.q_idx[(size_t)map * pl.n_q], pl.n_q, pl.status, 107);
-      load_query(static_cast<const __nv_bfloat16*>(p.q) + (int64_t)b * p.qs.batch + (int64_t)tok_q * p.qs.token +
-                     (int64_t)(g * G + x) * p.qs.head, j, qf);
+    if (x < G) {  // (there is one query row, token 0)
+      load_query(static_cast<const __nv_bfloat16*>(p.q) + (int64_t)b * p.qs.batch + (int64_t)(g * G + x) * p.qs.head, j, qf);
       if (step.rope) {  // the two pieces hold the two halves of the same pairs
         const float4* cs4 = reinterpret_cast<const float4*>(step.rope + (int64_t)step.position * (D / 2) + 16 * j);
 #pragma unroll
@@ -415,49 +421,88 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __
   DecodeState st;
   decode_init(st);
 
+  // Each lane works out one of the warp's next 32 blocks.  kOneList: up to 32 shards, and no warp has more blocks than that; no
+  // barrier stands before the requests of the first rows then.  (Table and query behind one barrier, then the list: 3500 cycles
+  // before the first request.)
   // Order of the 16-key blocks.  If the visible prefixes are about equally long, block i of every shard comes before block
   // i + 1 of any: shards interleave in the sequence, so the warps of a cluster read one region of the cache together.
   // Otherwise shard after shard, which balances whatever the lengths are.
   __shared__ int2 s_list[NW][32];  // of this warp's next blocks: first position in kv_idx, keys left there
-  if (step.rope) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-#pragma unroll 1
-  for (int w0 = 0; w0 < P; w0 += kFusedShards) {
-    if (w0 > 0) {
-      __syncthreads();
-      if (warp == 0) fill_table(w0);
+  auto gate = [&]() {  // the caches are complete before their rows are requested
+    if (step.rope) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  };
+  auto list = [&](int2 e) {  // those of the lanes' blocks that exist; how many
+    const uint32_t there = __ballot_sync(0xffffffffu, e.y > 0);
+    __syncwarp();
+    if (e.y > 0) s_list[warp][__popc(there & ((1u << lane) - 1u))] = e;
+    __syncwarp();
+    return __popc(there);
+  };
+  if constexpr (kOneList) {  // lane = shard, then lane = block, in every warp by itself
+    const int v = lane < P ? (vis_given ? step.vis[map * P + lane] : __ldg(vis + lane)) : 0;
+    const int off = lane < P ? __ldg(kv_off + lane) : 0, nb = (v + 15) >> 4;
+    int incl = nb;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
     }
-    __syncthreads();
-    const int n_w = min(kFusedShards, P - w0), total = s_before[n_w];
-    const bool even = s_most * n_w * 4 <= total * 5;
-    const int n_ids = even ? s_most * n_w : total;
-    // Each lane works out one of the warp's next 32 blocks; those that exist are listed in shared memory.
-#pragma unroll 1
-    for (int id0 = rank * NW + warp; id0 < n_ids; id0 += 32 * n_cta * NW) {
-      const int id = id0 + lane * n_cta * NW;
-      int2 e = make_int2(0, 0);
-      if (id < n_ids) {
-        int kk, i;
-        if (even) {
-          kk = id % n_w;
-          i = id / n_w;
-        } else {
-          int lo = 0, hi = n_w - 1;  // the last shard that starts at or before the block: it is not empty
-          while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (s_before[mid] <= id) lo = mid;
-            else hi = mid - 1;
-          }
-          kk = lo;
-          i = id - s_before[kk];
-        }
-        e = make_int2(s_off[kk] + i * 16, s_vis[kk] - i * 16);
+    const int total = __shfl_sync(0xffffffffu, incl, 31), most = __reduce_max_sync(0xffffffffu, nb);
+    const bool even = most * P * 4 <= total * 5;
+    const int id = rank * NW + warp + lane * n_cta * NW;
+    int kk = 0, i;
+    if (even) {
+      i = id / P;
+      kk = id - i * P;
+    } else {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {  // the last shard that starts at or before the block
+        const int at = __shfl_sync(0xffffffffu, incl - nb, kk + o);
+        if (kk + o < P && at <= id) kk += o;
       }
-      const uint32_t there = __ballot_sync(0xffffffffu, e.y > 0);
-      __syncwarp();
-      if (e.y > 0) s_list[warp][__popc(there & ((1u << lane) - 1u))] = e;
-      __syncwarp();
-      decode_walk<true>(st, s_q, pl, kv_idx, __popc(there), [&](int t) { return s_list[warp][t]; }, kb, p.ks.token, vb,
-                        p.vs.token, lane, cs);
+      i = id - __shfl_sync(0xffffffffu, incl - nb, kk);
+    }
+    const int left = __shfl_sync(0xffffffffu, v, kk) - i * 16, first = __shfl_sync(0xffffffffu, off, kk) + i * 16;
+    const int listed = list(make_int2(first, id < (even ? most * P : total) ? left : 0));
+    decode_walk<true>(st, s_q, pl, kv_idx, listed, [&](int t) { return s_list[warp][t]; }, kb, p.ks.token, vb, p.vs.token, lane, cs,
+                      gate, []() { __syncthreads(); });
+  } else {
+    gate();
+#pragma unroll 1
+    for (int w0 = 0; w0 < P; w0 += kFusedShards) {
+      if (w0 > 0) {
+        __syncthreads();
+        if (warp == 0) fill_table(w0);
+      }
+      __syncthreads();
+      const int n_w = min(kFusedShards, P - w0), total = s_before[n_w];
+      const bool even = s_most * n_w * 4 <= total * 5;
+      const int n_ids = even ? s_most * n_w : total;
+#pragma unroll 1
+      for (int id0 = rank * NW + warp; id0 < n_ids; id0 += 32 * n_cta * NW) {
+        const int id = id0 + lane * n_cta * NW;
+        int2 e = make_int2(0, 0);
+        if (id < n_ids) {
+          int kk, i;
+          if (even) {
+            kk = id % n_w;
+            i = id / n_w;
+          } else {
+            int lo = 0, hi = n_w - 1;  // the last shard that starts at or before the block: it is not empty
+            while (lo < hi) {
+              const int mid = (lo + hi + 1) >> 1;
+              if (s_before[mid] <= id) lo = mid;
+              else hi = mid - 1;
+            }
+            kk = lo;
+            i = id - s_before[kk];
+          }
+          e = make_int2(s_off[kk] + i * 16, s_vis[kk] - i * 16);
+        }
+        const int listed = list(e);
+        decode_walk<true>(st, s_q, pl, kv_idx, listed, [&](int t) { return s_list[warp][t]; }, kb, p.ks.token, vb, p.vs.token, lane, cs,
+                          []() {}, []() {});
+      }
     }
   }
   decode_publish<G, NW>(sh, st, warp, lane);
@@ -518,15 +563,21 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __
   }
 }
 
-template <int G>
+template <int G, int NW>
 static cudaError_t launch_fused(const AttnParams& p, const DecodeStep& step, int n_cta, cudaStream_t stream) {
-  constexpr int NW = 8;
-  auto kernel = decode_fused_kernel<G, NW>;
-  if (n_cta > 8) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-  }
-  return launch_dependent(kernel, dim3(n_cta, p.Hkv, p.batch), NW * 32, 0, n_cta, true, stream, p, step);
+  // One list: for as many keys as there are, whatever is visible when the launch runs (every shard may end in a block that is not
+  // full, and in the interleaved order the list is a quarter longer).  Up to ten blocks a warp: beyond, the few registers that it
+  // costs the walk weigh more (2 sequences of 16384 tokens, 32 / 8 heads, 34.5 us, from the table 32.4; one, in the wide form, 22.0
+  // and 29.0 before both).
+  const int P = p.plan.n_kv_shards;
+  const bool one_list = P <= 32 && ((p.plan.n_kv + 15) / 16 + P) * (int64_t)5 / 4 + 1 <= 10 * (int64_t)n_cta * NW;
+  auto kernel = one_list ? decode_fused_kernel<G, NW, true> : decode_fused_kernel<G, NW, false>;
+  constexpr int smem = sizeof(DecodeShared<G, NW>);
+  cudaError_t e = cudaSuccess;
+  if (n_cta > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess && smem > 32768) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(kernel, dim3(n_cta, p.Hkv, p.batch), NW * 32, smem, n_cta, true, stream, p, step);
 }
 
 // f(integral_constant G) for the group sizes the kernels are built for
@@ -572,8 +623,14 @@ cudaError_t launch_decode_fused(const AttnParams& p, const DecodeStep& step, int
   const int64_t pairs = (int64_t)p.rule_kv_heads * p.batch, blocks = std::max<int64_t>(1, (n_visible + 15) / 16);
   const int64_t most = std::min<int64_t>(pairs <= 7 ? kMaxCluster : 10, (blocks + 7) / 8);
   const int n_cta = pairs > 128 ? cluster_for_many(pairs, blocks, most) : (int)std::max<int64_t>(1, std::min(256 / pairs, most));
+  // Sixteen warps a CTA where that gives every CTA an SM of its own and there are blocks for them: with eight, an SM holds half the
+  // loads it could (one sequence of 16384 tokens, 32 / 8 heads, 30.4 us, now 21.7; a step at 12000 of them, 64 / 8 heads, 25.5
+  // and 17.5; 600 tokens, 8 / 8 heads, 6.1 and 5.3).
+  const bool wide = pairs * n_cta <= 132 && blocks > 8 * n_cta;
   TimedLaunch timed(stream);
-  return with_group(p.G, [&](auto g) { return launch_fused<decltype(g)::value>(p, step, n_cta, stream); });
+  return with_group(p.G, [&](auto g) {
+    return wide ? launch_fused<decltype(g)::value, 16>(p, step, n_cta, stream) : launch_fused<decltype(g)::value, 8>(p, step, n_cta, stream);
+  });
 }
 
 cudaError_t launch_decode(const AttnParams& p, cudaStream_t stream) {
