@@ -9,15 +9,18 @@
 //          no duplicating moves (8 loads per 32 packed FMAs).
 // Every one of these loads is a single conflict-free wavefront.  K of the next tile is fetched with cp.async while the
 // current weights are formed and multiplied with V, and V while the next logits are.
-// The key stream is cut into chunks of 16 keys of one shard, so the shard mask is one limit per (row, chunk); tiles that the
-// CTA's first row sees completely skip it.
+// The key stream is cut into chunks of 16 keys, of one shard (partials) or of the sequence (kTokens, the fused route), so the mask is
+// one limit per (row, chunk); tiles that the CTA's first row sees completely skip it.
+// Fused, of all shards a query sees a prefix in token order, so rows and keys are taken as they lie: nothing is looked up in the
+// plan before they are requested, and a shard of a few keys does not end in a chunk of its own.  (Shard by shard, one sequence of
+// 128 tokens had its key rows requested after 7000 of 14000 cycles.)
 //
 // RW = 4: the four warps own different rows and share the K/V tiles.  RW = 1: all four warps own the same rows and take the
 // tiles (32 keys) of the stream in turn; their (m, l, o) are combined at the end.  Small problems and short shards use the
 // latter: four times as many CTAs, four times shorter chains, less padding.
 // Measured (fp32): 16 sequences of 512 tokens, 16 heads of 64, 8 shards, bidirectional, fused 540 us = 32 TFLOP/s (partials
-// and merge 708 us, before 1662 us with one row at a time per warp); one sequence of 128 tokens, 12 heads, 2 shards: 11 us
-// (before 35).  What bounds it now is shared-memory bandwidth: 448 16-byte loads (4 cycles each) against 2048 packed FMAs
+// and merge 708 us, before 1662 us with one row at a time per warp); one sequence of 128 tokens, 12 heads, 2 shards: 8.4 us
+// (in token order; shard by shard 10.5, a row at a time 35).  What bounds it now is shared-memory bandwidth: 448 16-byte loads (4 cycles each) against 2048 packed FMAs
 // per warp and 16 x 64 tile.
 #include "cascade_internal.cuh"
 
@@ -97,14 +100,14 @@ struct SimtCfg {
 
 constexpr int64_t kEnough = 2 * 148;  // CTAs that fill the chip, two per SM
 
-// A tile of the key stream: per chunk of 16 keys its shard, its first key in the shard's list and its keys.
+// A tile of the key stream: per chunk of 16 keys its first key in the stream and in the plan's list, and the keys from there on.
 template <int NC>
 struct SimtTile {
-  int kk[NC], t0[NC], n[NC], at[NC];
+  int t0[NC], n[NC], at[NC];
   bool any, masked;
 };
 
-template <typename T, int D, int RW>
+template <typename T, int D, int RW, bool kTokens>
 __global__ void __launch_bounds__(128, SimtCfg<D, RW>::kCtas)
 attn_simt_kernel(const __grid_constant__ AttnParams p, int parts_per_cta) {
   using C = SimtCfg<D, RW>;
@@ -124,18 +127,24 @@ attn_simt_kernel(const __grid_constant__ AttnParams p, int parts_per_cta) {
 
   const PlanDev& pl = p.plan;
   const int P = pl.n_kv_shards;
-  const int n_pg = p.fused ? 1 : (P + parts_per_cta - 1) / parts_per_cta;
-  const int b = blockIdx.z / n_pg;
-  const int pg = blockIdx.z % n_pg;
+  const int n_pg = kTokens ? 1 : (P + parts_per_cta - 1) / parts_per_cta;
+  const int b = kTokens ? blockIdx.z : blockIdx.z / n_pg;
+  const int pg = kTokens ? 0 : blockIdx.z % n_pg;
   const int map = pl.n_maps == 1 ? 0 : b;
   const int h = blockIdx.y;
-  const int g = h / p.G;
+  const int g = p.G == 1 ? h : h / p.G;
   // the plan's tiles of 64 slots, or of 32 slots in two pieces
   constexpr int kList = RW == 4 ? 1 : 0, kPieces = (32 << kList) / C::R;
-  const int4 qt = pl.qtiles[kList][(size_t)map * pl.n_qtiles[kList] + blockIdx.x / kPieces];
-  const int row0 = qt.x + (blockIdx.x % kPieces) * C::R;
-  const int nrows = min(C::R, qt.y - (int)(blockIdx.x % kPieces) * C::R);
-  if (nrows <= 0) return;
+  int row0, nrows;  // slots of a query shard, or tokens, the last ones (which see most) first
+  if constexpr (kTokens) {
+    row0 = (int)(gridDim.x - 1 - blockIdx.x) * C::R;
+    nrows = min(C::R, pl.n_q - row0);
+  } else {
+    const int4 qt = pl.qtiles[kList][(size_t)map * pl.n_qtiles[kList] + blockIdx.x / kPieces];
+    row0 = qt.x + (blockIdx.x % kPieces) * C::R;
+    nrows = min(C::R, qt.y - (int)(blockIdx.x % kPieces) * C::R);
+    if (nrows <= 0) return;
+  }
   const int32_t* q_idx = pl.q_idx + (size_t)map * pl.n_q;
   const int32_t* kv_idx = pl.kv_idx + (size_t)map * pl.n_kv;
   const int32_t* kv_off = pl.kv_off + (size_t)map * (P + 1);
@@ -143,14 +152,26 @@ attn_simt_kernel(const __grid_constant__ AttnParams p, int parts_per_cta) {
   // rows ascend: the first has the shortest prefix of every shard, the last the longest
   const int32_t* vis_first = vis + (size_t)row0 * P;
   const int32_t* vis_last = vis + (size_t)(row0 + nrows - 1) * P;
+  auto token_of = [&](int r) {
+    if constexpr (kTokens) return (int64_t)(row0 + r);
+    else return (int64_t)CASCADE_CHECKED((int64_t)__ldg(q_idx + row0 + r), pl.n_q, pl.status, 104);
+  };
+  auto seen_by = [&](int r) {  // kTokens: keys of the sequence that the row sees
+    if (!pl.causal) return pl.n_kv;
+    if (!p.prefix_from_vis) return (int)max((int64_t)0, min((int64_t)pl.n_kv, (int64_t)pl.q_pos_offset + row0 + r + 1));
+    const int32_t* of = vis + (size_t)__ldg(pl.q_inv + (size_t)map * pl.n_q + row0 + r) * P;
+    int n = 0;
+    for (int k = 0; k < P; ++k) n += __ldg(of + k);
+    return n;
+  };
+  const int seen_first = kTokens ? seen_by(0) : 0, seen_last = kTokens ? seen_by(nrows - 1) : 0;
   const T* qb = static_cast<const T*>(p.q) + (int64_t)b * p.qs.batch + (int64_t)h * p.qs.head;
   const T* kb = static_cast<const T*>(p.k) + (int64_t)b * p.ks.batch + (int64_t)g * p.ks.head;
   const T* vb = static_cast<const T*>(p.v) + (int64_t)b * p.vs.batch + (int64_t)g * p.vs.head;
 
   for (int i = tid; i < C::R * (D / 4); i += 128) {
     const int r = i / (D / 4), c4 = (i % (D / 4)) * 4;
-    const int64_t tok =
-        r < nrows ? CASCADE_CHECKED((int64_t)__ldg(q_idx + row0 + r), pl.n_q, pl.status, 104) : (int64_t)0;
+    const int64_t tok = r < nrows ? token_of(r) : (int64_t)0;
     stage4(sQ + r * C::QP + c4, qb + tok * p.qs.token + c4, r < nrows);
   }
   stage_commit();
@@ -168,19 +189,28 @@ attn_simt_kernel(const __grid_constant__ AttnParams p, int parts_per_cta) {
       for (int i = 0; i < 16 / kRowsAtOnce; ++i) {
         const int x = i * kRowsAtOnce + lr;
         const bool there = x < t.n[j];
-        const int64_t tok =
-            there ? CASCADE_CHECKED((int64_t)__ldg(kv_idx + t.at[j] + x), pl.n_kv, pl.status, 105) : (int64_t)0;
+        int64_t tok = 0;
+        if constexpr (kTokens) {
+          if (there) tok = t.at[j] + x;
+        } else if (there) {
+          tok = CASCADE_CHECKED((int64_t)__ldg(kv_idx + t.at[j] + x), pl.n_kv, pl.status, 105);
+        }
         stage4(dst + (j * 16 + x) * pitch + lc, base + tok * token_stride + lc, there);
       }
     stage_commit();
   };
   const int my_row = wrow + rg;  // this thread's rows: my_row + 4 r
+  int seen[kTokens ? TR : 1];
+  if constexpr (kTokens) {
+#pragma unroll
+    for (int r = 0; r < TR; ++r) seen[r] = seen_by(min(my_row + 4 * r, nrows - 1));
+  }
   const float cs = p.scale * 1.4426950408889634f;  // raw logits -> log2 units
 
   float m_run[TR], l_run[TR];  // raw logits; l is this thread's share (its key columns)
   uint64_t acc[TR][2 * DJ];
 
-  const int k_first = p.fused ? 0 : pg * parts_per_cta, k_last = p.fused ? 1 : min(P, (pg + 1) * parts_per_cta);
+  const int k_first = kTokens ? 0 : pg * parts_per_cta, k_last = kTokens ? 1 : min(P, (pg + 1) * parts_per_cta);
   for (int part = k_first; part < k_last; ++part) {
 #pragma unroll
     for (int r = 0; r < TR; ++r) {
@@ -189,33 +219,23 @@ attn_simt_kernel(const __grid_constant__ AttnParams p, int parts_per_cta) {
 #pragma unroll
       for (int j = 0; j < 2 * DJ; ++j) acc[r][j] = 0;
     }
-    // cursor over the chunks: of all shards one after another (fused), or of shard `part`
-    const int kk_end = p.fused ? P : part + 1;
-    int kk = p.fused ? 0 : part, c = group * NC, need = vis_last[kk];
-    auto settle = [&]() {  // to the next existing chunk
-      while (kk < kk_end && c * 16 >= need) {
-        c -= (need + 15) >> 4;
-        if (++kk < kk_end) need = __ldg(vis_last + kk);
-      }
-    };
+    // cursor over the chunks of shard `part`, or of the sequence
+    int c = group * NC;
+    const int need = kTokens ? seen_last : __ldg(vis_last + part);
+    const int first = kTokens ? seen_first : __ldg(vis_first + part), at0 = kTokens ? 0 : __ldg(kv_off + part);
     auto next_tile = [&](SimtTile<NC>& t) {
       t.masked = false;
-      t.any = kk < kk_end;
+      t.any = c * 16 < need;
 #pragma unroll
       for (int j = 0; j < NC; ++j) {
-        const bool there = kk < kk_end;
-        t.kk[j] = there ? kk : 0;
         t.t0[j] = c * 16;
-        t.n[j] = there ? need - c * 16 : 0;
-        t.at[j] = there ? __ldg(kv_off + kk) + c * 16 : 0;
-        t.masked = t.masked || !there || __ldg(vis_first + kk) < c * 16 + 16;
+        t.n[j] = need - c * 16;
+        t.at[j] = at0 + c * 16;
+        t.masked = t.masked || first < c * 16 + 16;
         ++c;
-        settle();
       }
       c += (C::KW - 1) * NC;  // the other groups' tiles
-      settle();
     };
-    settle();
     SimtTile<NC> cur, nxt;
     next_tile(cur);
     group_sync();  // the tiles of the previous part are consumed
@@ -268,12 +288,11 @@ attn_simt_kernel(const __grid_constant__ AttnParams p, int parts_per_cta) {
       if (cur.masked) {
 #pragma unroll
         for (int r = 0; r < TR; ++r) {
-          const int32_t* vis_row = vis + (size_t)(row0 + min(my_row + 4 * r, nrows - 1)) * P;
+          const int sees = kTokens ? seen[kTokens ? r : 0] : __ldg(vis + (size_t)(row0 + min(my_row + 4 * r, nrows - 1)) * P + part);
 #pragma unroll
           for (int j = 0; j < KJ; ++j) {
             const int ch = j >> 1;
-            const int limit = cur.n[ch] > 0 ? __ldg(vis_row + cur.kk[ch]) - cur.t0[ch] : 0;
-            if (cg + 8 * (j & 1) >= limit) s[r][j] = -INFINITY;
+            if (cg + 8 * (j & 1) >= sees - cur.t0[ch]) s[r][j] = -INFINITY;
           }
         }
       }
@@ -349,9 +368,9 @@ attn_simt_kernel(const __grid_constant__ AttnParams p, int parts_per_cta) {
       o.y *= inv;
       o.z *= inv;
       o.w *= inv;
-      if (p.fused) {
-        const int tok = (int)CASCADE_CHECKED((int64_t)__ldg(q_idx + row0 + row), pl.n_q, pl.status, 104);
-        store4(static_cast<T*>(p.o_out) + (int64_t)b * p.os.batch + (int64_t)tok * p.os.token + (int64_t)h * p.os.head + col,
+      if constexpr (kTokens) {
+        const int64_t tok = row0 + row;
+        store4(static_cast<T*>(p.o_out) + (int64_t)b * p.os.batch + tok * p.os.token + (int64_t)h * p.os.head + col,
                o);
         if (stats && p.lse_out)
           p.lse_out[((int64_t)b * pl.n_q + tok) * p.H + h] = l > 0.f ? m_raw * p.scale + logf(l) : -INFINITY;
@@ -414,24 +433,29 @@ attn_simt_kernel(const __grid_constant__ AttnParams p, int parts_per_cta) {
 template <typename T, int D, int RW>
 cudaError_t launch_rows(const AttnParams& p, int parts_per_cta, cudaStream_t stream) {
   using C = SimtCfg<D, RW>;
+  auto kernel = p.fused ? attn_simt_kernel<T, D, RW, true> : attn_simt_kernel<T, D, RW, false>;
   // per function and per device; cheap enough to repeat on every launch
-  cudaError_t e = cudaFuncSetAttribute(attn_simt_kernel<T, D, RW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)C::kBytes);
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kBytes);
   if (e != cudaSuccess) return e;
   constexpr int kList = RW == 4 ? 1 : 0, kPieces = (32 << kList) / C::R;
   const int n_pg = p.fused ? 1 : (p.plan.n_kv_shards + parts_per_cta - 1) / parts_per_cta;
-  const dim3 grid(p.plan.n_qtiles[kList] * kPieces, p.H, p.batch * n_pg);
-  attn_simt_kernel<T, D, RW><<<grid, 128, C::kBytes, stream>>>(p, parts_per_cta);
+  const dim3 grid(p.fused ? (p.plan.n_q + C::R - 1) / C::R : p.plan.n_qtiles[kList] * kPieces, p.H, p.batch * n_pg);
+  kernel<<<grid, 128, C::kBytes, stream>>>(p, parts_per_cta);
   count_launch();
   return cudaGetLastError();
+}
+
+// Tiles of `height` rows (16 or 64): of tokens (fused), or of the plan's list.
+int64_t simt_tiles(const AttnParams& p, int height) {
+  return p.fused ? (p.plan.n_q + height - 1) / height : height == 64 ? p.plan.n_qtiles[1] : p.plan.n_qtiles[0];
 }
 
 // Whether four row warps share a CTA: when that fills the chip (two CTAs per SM) and does not pad the rows by more than what the
 // narrow form's four times larger K/V traffic costs.  It decides how sums are split, so it goes by the heads of the whole
 // problem (see AttnParams).
 bool use_wide(const AttnParams& p) {
-  const int64_t tiles = p.plan.n_qtiles[1], heads = (int64_t)p.rule_kv_heads * p.G * p.batch;
-  const int64_t narrow_rows = (int64_t)p.plan.n_q + (int64_t)p.plan.n_q_shards * 8;  // padded by half a piece a shard
+  const int64_t tiles = simt_tiles(p, 64), heads = (int64_t)p.rule_kv_heads * p.G * p.batch;
+  const int64_t narrow_rows = (int64_t)p.plan.n_q + (int64_t)(p.fused ? 1 : p.plan.n_q_shards) * 8;  // padded by half a piece a shard
   return tiles * heads * (p.fused ? 1 : p.plan.n_kv_shards) >= kEnough && tiles * 64 * 4 <= narrow_rows * 6;
 }
 
@@ -447,7 +471,7 @@ int64_t narrow_pieces(const AttnParams& p) {
 template <typename T, int D>
 cudaError_t launch_one(const AttnParams& p, cudaStream_t stream) {
   const int64_t heads = (int64_t)p.H * p.batch;
-  if (use_wide(p)) return launch_rows<T, D, 4>(p, parts_per_cta(p, p.plan.n_qtiles[1] * heads), stream);
+  if (use_wide(p)) return launch_rows<T, D, 4>(p, parts_per_cta(p, simt_tiles(p, 64) * heads), stream);
   return launch_rows<T, D, 1>(p, parts_per_cta(p, narrow_pieces(p) * heads), stream);
 }
 
@@ -459,14 +483,15 @@ double tiles_time(const AttnParams& p) {
   const CutSize c(p);
   const bool d64 = p.d == 64;
   if (use_wide(p)) {
-    const double list = p.plan.n_qtiles[1];
-    const double seen = c.seen_by_last(list), chunks = c.pieces(seen, 16) * c.shards;  // of 16 keys, fused route
+    const double list = simt_tiles(p, 64);
+    const double seen = p.fused ? c.seen_at((list + 1) / (2 * list)) : c.seen_by_last(list), chunks = std::ceil(seen * c.n_kv / 16);
     const double cta = d64 ? 2 + 6.2 * (p.fused ? chunks / 4 : c.pieces(seen, 64))
                            : 2 + 5 * (p.fused ? chunks / 2 : c.pieces(seen, 32));
     return list * c.heads * cta * (p.fused ? 1 : c.shards) / kEstimateSms;
   }
-  const double pieces = c.row_tiles(16), seen = c.seen_by_last(pieces);
-  const double tiles = p.fused ? c.pieces(seen, 16) * c.shards / 2 : c.pieces(seen, 32);
+  const double pieces = p.fused ? simt_tiles(p, 16) : c.row_tiles(16);
+  const double seen = p.fused ? c.seen_at((pieces + 1) / (2 * pieces)) : c.seen_by_last(pieces);
+  const double tiles = p.fused ? std::ceil(seen * c.n_kv / 32) : c.pieces(seen, 32);
   const double cta = d64 ? 2.4 + 0.45 * std::min(tiles, 4.0) + 0.71 * std::max(0.0, tiles - 4)
                          : 1 + (p.fused ? 10 : 7.2) * std::max(1.0, tiles / 4);
   const double parts = parts_per_cta(p, std::max<int64_t>(1, (int64_t)(narrow_pieces(p) * c.heads)));

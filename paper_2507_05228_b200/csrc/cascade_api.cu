@@ -744,15 +744,15 @@ static bool tc_ws_given(const cascade_plan_t* plan, int batch, int Hkv, int d, c
 
 // fp32 with heads of 64 columns on the tensor cores: whether the kernel takes the problem; whether the scratch for the split keys
 // and values is there and the kernel is the faster one.  The estimates of the ALU kernels leave out what a launch and a first
-// load take, hence the constants: at the 300 sizes of split_time the choice cost 1.9 % on average over the better kernel, and one
-// size got slower by more than 5 % (264 tokens in 5 of 32 shards).  16 x 512 tokens, 16 heads, 8 shards, no mask: partials 668 ->
+// load take, hence the constants: at the 300 sizes of split_time the choice cost 1.9 % on average over the better kernel (partials),
+// at 160 more 0.2 % (fused).  16 x 512 tokens, 16 heads, 8 shards, no mask: partials 668 ->
 // 232 us, fused 540 -> 151; 1024 causal tokens, 8 sequences, fused 924 -> 161.
 static bool split_takes(const cascade_plan_t* plan, cascade_dtype_t dtype, int d) {
   return dtype == CASCADE_F32 && d == 64 && plan->dev.n_q > 1 && plan->dev.n_kv_shards <= 256;
 }
 static bool use_split(const AttnParams& p, const cascade_plan_t* plan, cascade_dtype_t dtype, const void* workspace, size_t bytes) {
   return split_takes(plan, dtype, p.d) && workspace && ((uintptr_t)workspace & 255) == 0 &&
-         bytes >= split_ws_bytes(plan->dev, p.batch, p.Hkv) && split_time(p) < 1.1 * std::min(tiles_time(p), rows_time(p)) + 4;
+         bytes >= split_ws_bytes(plan->dev, p.batch, p.Hkv) && split_time(p) < (p.fused ? 1.3 : 1.1) * std::min(tiles_time(p), rows_time(p)) + (p.fused ? 5 : 4);
 }
 // Scratch of the routes with copies of K and V: bf16 on the tensor cores, or fp32 on the tensor cores.
 static size_t copies_ws_bytes(const cascade_plan_t* plan, cascade_dtype_t dtype, int batch, int Hkv, int d) {
@@ -1163,6 +1163,7 @@ static cascade_status_t attn_sharded_impl(const char* fn, const cascade_plan_t* 
     cascade_status_t ws = run_tc(p, fn, plan, workspace, workspace_bytes, st, &e);
     if (ws != CASCADE_OK) return ws;
   } else {
+    p.prefix_from_vis = is_capturing(st) || !plan->kv_pos.empty();  // see run_tc
     e = use_split(p, plan, dtype, workspace, workspace_bytes) ? launch_attn_split(p, workspace, st) : launch_attn_simt(p, dtype, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "attention (fused route): launch");
