@@ -22,56 +22,87 @@ __device__ __forceinline__ int32_t visible_prefix(const PlanDev& d, const T* q_i
   if (pos < 0) return 0;
   if (pos >= d.n_kv) return len;
   const T* list = kv_idx + (size_t)mp * d.n_kv + begin;
-  int lo = 0, hi = len;  // first entry greater than pos
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if ((int32_t)list[mid] <= (int32_t)pos) lo = mid + 1;
-    else hi = mid;
+  // First entry greater than pos.  Each step reads seven entries at once and keeps an eighth of the range: what bounds
+  // these kernels is the chain of dependent reads, 4 of them for 512 keys where halving makes 10.
+  int lo = 0, n = len;
+  while (n > 0) {
+    const int step = n / 8 + 1;
+    int below = 0;
+#pragma unroll
+    for (int i = 1; i < 8; ++i) {
+      const int at = i * step - 1;
+      below += at < n && (int32_t)list[lo + at] <= (int32_t)pos;
+    }
+    lo += below * step;
+    n = min(n - below * step, step - 1);
   }
   return lo;
 }
 
-// Entry t of vis[map][r][k], or after those EMPTY / PARTIAL / FULL per (query shard, KV shard) from the prefix lengths of the
-// shard's first and last row (rows ascend in position, so the first row has the shortest prefix and the last the longest;
-// both are searched for again here, so that one launch does everything: the launch is what costs).
+// The threads that visible_entry takes, a whole number of warps: one for a group of kWarpRows query slots (over all maps) and
+// kWarpShards KV shards, then two threads for each pair of a query shard and a KV shard.
+constexpr int kWarpShards = 4, kWarpRows = 32 / kWarpShards;
+struct VisThreads {
+  int64_t vis, all;
+};
+__host__ __device__ __forceinline__ VisThreads vis_threads(const PlanDev& d) {
+  const int64_t vis = ((int64_t)d.n_maps * d.n_q + kWarpRows - 1) / kWarpRows *
+                      ((d.n_kv_shards + kWarpShards - 1) / kWarpShards) * 32;
+  return {vis, vis + ((int64_t)d.n_maps * d.n_q_shards * d.n_kv_shards * 2 + 31) / 32 * 32};
+}
+
+// Thread t's entry of vis[map][r][k] or, after those, its half of EMPTY / PARTIAL / FULL per (query shard, KV shard), from the
+// prefix lengths of the shard's first and last row (rows ascend in position, so the first row has the shortest prefix and the
+// last the longest; both are searched for again here, a thread each, so that one launch does everything: the launch is what
+// costs).  Called by whole warps.  The lanes of a warp search few shards for neighbouring rows, so most of their reads are of
+// the same lines, and write 16 bytes of a row.
+// Measured back to back, 16 shards: 512 rows at 8192 keys 4.9 -> 3.3 us (halving, a thread per entry, shards first -> this), 1024
+// at 16384 5.3 -> 3.7, 4096 at 4096 4.9 -> 5.0; 16384 rows at 32768 keys, 32 shards, 20.5 -> 11.6.  Sixteenths: 3.6, 4.1, 7.9
+// and 16.0 with one shard a warp; eighths with one shard a warp 3.2, 3.6, 5.2 and 12.0, with eight 3.3, 3.7, 6.2 and 13.0.
 template <typename T>
 __device__ __forceinline__ void visible_entry(const PlanDev& d, const T* q_idx, const T* kv_idx, int32_t q_pos_offset, int64_t t,
                                               int64_t n_vis, int32_t* __restrict__ vis, uint8_t* __restrict__ pair_class) {
   const int J = d.n_q_shards, P = d.n_kv_shards;
-  const int64_t e = t < n_vis ? t : t - n_vis;
-  const int k = (int)(e % P);
-  const int64_t row = e / P;
   if (t < n_vis) {
-    vis[t] = visible_prefix(d, q_idx, kv_idx, q_pos_offset, (int)(row / d.n_q), (int)(row % d.n_q), k);
+    // 32-bit divisions: those of 64 bits take as long as a read
+    const uint32_t warp = (uint32_t)(t / 32), across = (P + kWarpShards - 1) / kWarpShards;
+    const int k = (int)(warp % across) * kWarpShards + (int)(t % kWarpShards);
+    const int64_t row = (int64_t)(warp / across) * kWarpRows + t % 32 / kWarpShards;
+    if (k < P && row < (int64_t)d.n_maps * d.n_q) {
+      const int mp = d.n_maps == 1 ? 0 : (int)(row / d.n_q);
+      vis[row * P + k] = visible_prefix(d, q_idx, kv_idx, q_pos_offset, mp, (int)(row - (int64_t)mp * d.n_q), k);
+    }
     return;
   }
-  const int mp = (int)(row / J), j = (int)(row % J);
-  const int32_t* qo = d.q_off + (size_t)mp * (J + 1);
-  const int32_t* ko = d.kv_off + (size_t)mp * (P + 1);
-  const int len = ko[k + 1] - ko[k];
-  uint8_t cls = CASCADE_PAIR_EMPTY;
-  if (qo[j + 1] > qo[j] && len > 0) {
-    const int lo = visible_prefix(d, q_idx, kv_idx, q_pos_offset, mp, qo[j], k);
-    const int hi = visible_prefix(d, q_idx, kv_idx, q_pos_offset, mp, qo[j + 1] - 1, k);
-    cls = hi == 0 ? CASCADE_PAIR_EMPTY : (lo == len ? CASCADE_PAIR_FULL : CASCADE_PAIR_PARTIAL);
+  const uint32_t e = (uint32_t)((t - n_vis) / 2);
+  const bool last = t & 1, valid = e < (int64_t)d.n_maps * J * P;
+  int seen = 0, len = 0;
+  if (valid) {
+    const int k = (int)(e % P), at = (int)(e / P), mp = at / J, j = at % J;
+    const int32_t* qo = d.q_off + (size_t)mp * (J + 1);
+    const int32_t* ko = d.kv_off + (size_t)mp * (P + 1);
+    const int first = qo[j], end = qo[j + 1];
+    if (end > first) len = ko[k + 1] - ko[k];
+    if (len > 0) seen = visible_prefix(d, q_idx, kv_idx, q_pos_offset, mp, last ? end - 1 : first, k);
   }
-  pair_class[e] = cls;
+  const int other = __shfl_xor_sync(0xffffffffu, seen, 1);  // (even lanes write: the last row's)
+  if (valid && !last)
+    pair_class[e] = other == 0 ? CASCADE_PAIR_EMPTY : (seen == len ? CASCADE_PAIR_FULL : CASCADE_PAIR_PARTIAL);
 }
 
-// One thread per entry.
+// One thread per entry, two per pair.  128 a block measured faster than 256 (3.6 against 4.2 us at 512 rows, 16 shards).
 __global__ void plan_advance_kernel(PlanDev d, int32_t q_pos_offset, int32_t* __restrict__ vis,
                                     uint8_t* __restrict__ pair_class) {
   grid_go();
   grid_wait();
-  const int64_t n_vis = (int64_t)d.n_maps * d.n_q * d.n_kv_shards;
-  const int64_t n = n_vis + (int64_t)d.n_maps * d.n_q_shards * d.n_kv_shards;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-    visible_entry(d, d.q_idx, d.kv_idx, q_pos_offset, t, n_vis, vis, pair_class);
+  const VisThreads n = vis_threads(d);
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n.all; t += (int64_t)gridDim.x * blockDim.x)
+    visible_entry(d, d.q_idx, d.kv_idx, q_pos_offset, t, n.vis, vis, pair_class);
 }
 
 // The arrays of a new plan that follow from its row lists kv_src and q_src (ids of T, as they were uploaded): the lists
 // themselves, their inverses, the shard of every K/V slot and, unless the host has them (n_visible = 0), vis and pair_class.
-// One thread per entry of each.
+// One thread per entry of each, those of visible_entry first.
 template <typename T>
 __global__ void plan_fill_kernel(PlanDev d, const T* __restrict__ q_src, const T* __restrict__ kv_src, int64_t n_vis,
                                  int64_t n_visible) {
@@ -130,8 +161,8 @@ cudaError_t launch_plan_set(const PlanDev& d, const int32_t* vis, int n_vis, con
 
 cudaError_t launch_plan_fill(const PlanDev& d, const void* q_src, const void* kv_src, bool short_ids, bool visible,
                              cudaStream_t stream) {
-  const int64_t n_vis = (int64_t)d.n_maps * d.n_q * d.n_kv_shards;
-  const int64_t n_visible = visible ? n_vis + (int64_t)d.n_maps * d.n_q_shards * d.n_kv_shards : 0;
+  const int64_t n_vis = vis_threads(d).vis;
+  const int64_t n_visible = visible ? vis_threads(d).all : 0;
   const int64_t n = n_visible + (int64_t)d.n_maps * ((int64_t)d.n_q + d.n_kv);
   const int threads = 256;
   const int blocks = (int)std::min<int64_t>((n + threads - 1) / threads, 8 * 1024);
@@ -146,8 +177,8 @@ cudaError_t launch_plan_fill(const PlanDev& d, const void* q_src, const void* kv
 }
 
 cudaError_t launch_plan_advance(const PlanDev& d, int32_t q_pos_offset, cudaStream_t stream) {
-  const int64_t n = (int64_t)d.n_maps * (d.n_q + d.n_q_shards) * d.n_kv_shards;
-  const int threads = 256;
+  const int64_t n = vis_threads(d).all;
+  const int threads = 128;  // spread over the SMs: 512 rows in 16 shards are 8704 threads
   const int blocks = (int)std::min<int64_t>((n + threads - 1) / threads, 8 * 1024);
   // a dependent too: the chain plan -> attention of a 512-token chunk at 8192 keys 70.3 -> 68.8 us back to back
   return launch_dependent(plan_advance_kernel, dim3(blocks), threads, 0, 1, true, stream, d, q_pos_offset,
