@@ -11,8 +11,8 @@
 // max / sum / output of the streaming softmax, and one output row is written at the end.  Only the last tile or two need the
 // causal mask.  Where there are few query tiles, a cluster of 2, 4 or 8 CTAs shares the keys of one and adds up through
 // distributed shared memory.
-// Measured, 32 query / 8 KV heads: 2048 tokens, 8 random shards 42.7 us; 512 queries against 7168 cached tokens 71 us; 32768
-// tokens, 64 / 8 heads, 32 random shards 15.5 ms; 2 x 3001 tokens, 16 / 4 heads of 64 columns 79 us.  (This order of work alone,
+// Measured, 32 query / 8 KV heads: 2048 tokens, 8 random shards 41.9 us; 512 queries against 7168 cached tokens 69 us; 32768
+// tokens, 64 / 8 heads, 32 random shards 15.6 ms; 2 x 3001 tokens, 16 / 4 heads of 64 columns 76 us.  (This order of work alone,
 // against shard by shard from gathered copies with query tiles inside one shard: 67 -> 47 us, 127 -> 80 us, 16.7 -> 16.0 ms and
 // 124 -> 85 us; the rest is what stands beside the code below.)
 //
