@@ -19,6 +19,7 @@
 // 64 registers hold the loads in flight.  Anything else kept through the loop ends up spilled, and a spilled value comes back
 // from L2, because the streaming loads evict it from L1: the query fragments therefore live in shared memory.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "cascade_internal.cuh"
@@ -94,13 +95,14 @@ __device__ __forceinline__ void decode_init(DecodeState& st) {
 
 // Walks `count` blocks of 16 keys; block t is the keys kv_idx[at .. at + n - 1] (n >= 1; 16 at most are taken) with
 // (at, n) = get(t).
-// kAhead: the key rows of block t + 1 are requested as soon as the logits of block t are formed, its value rows after the
-// product of block t, its tokens a block earlier still, all into registers that have just come free: one memory latency per
-// block instead of two and the arithmetic (a block took 3200 cycles one after another).  Without it nothing is spilled,
+// kAhead: the key rows of block t + kAhead are requested as soon as the logits of block t are formed, its value rows after the
+// product of block t, its tokens a block earlier still, all into registers that have just come free: with 1, one memory latency
+// per block instead of two and the arithmetic (a block took 3200 cycles one after another).  With 0 nothing is spilled,
 // which is the better trade where 16 warps per SM cover the latencies anyway (partials of 64 sequences of 16384 tokens: 630
-// us without, 820 with; all shards in one kernel: 711 without, 620 with).
+// us without, 820 with; all shards in one kernel: 711 without, 620 with).  With 2 a warp keeps twice the loads in flight, in
+// registers that it has where an SM holds eight warps and no more.  The sums are the same whatever kAhead is.
 // gate() is called before the first rows are requested, ready() before the query is used; by a warp without blocks, too.
-template <bool kAhead, typename Get, typename Gate, typename Ready>
+template <int kAhead, typename Get, typename Gate, typename Ready>
 __device__ __forceinline__ void decode_walk(DecodeState& st, const DecodeQuery& q, const PlanDev& pl, const int32_t* kv_idx,
                                             int count, Get get, const __nv_bfloat16* kp, int64_t k_token,
                                             const __nv_bfloat16* vp, int64_t v_token, int lane, float cs, Gate gate, Ready ready) {
@@ -109,55 +111,60 @@ __device__ __forceinline__ void decode_walk(DecodeState& st, const DecodeQuery& 
     ready();
     return;
   }
+  constexpr int kBuffers = kAhead > 1 ? kAhead : 1;  // of block t: t % kBuffers
   const int x = lane >> 2, j = lane & 3;
-  uint32_t ka[16], kb[16], vr[4][8];
+  uint32_t ka[kBuffers][16], kb[kBuffers][16], vr[kBuffers][4][8];
   auto token = [&](int2 e) {  // lane l: token of key l (clamped to the last key; masked below)
     return (int)CASCADE_CHECKED((int64_t)__ldg(kv_idx + e.x + min(lane & 15, e.y - 1)), pl.n_kv, pl.status, 106);
   };
-  auto load_k = [&](int tok) {  // rows x and x + 8
+  auto load_k = [&](int buf, int tok) {  // rows x and x + 8
     const __nv_bfloat16* r0 = kp + (int64_t)__shfl_sync(0xffffffffu, tok, x) * k_token;
     const __nv_bfloat16* r1 = kp + (int64_t)__shfl_sync(0xffffffffu, tok, x + 8) * k_token;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      load32(r0 + 64 * c, ka + 8 * c);
-      load32(r1 + 64 * c, kb + 8 * c);
+      load32(r0 + 64 * c, ka[buf] + 8 * c);
+      load32(r1 + 64 * c, kb[buf] + 8 * c);
     }
   };
-  auto load_v = [&](int tok) {  // rows 2j, 2j + 1, 2j + 8, 2j + 9
+  auto load_v = [&](int buf, int tok) {  // rows 2j, 2j + 1, 2j + 8, 2j + 9
 #pragma unroll
     for (int rr = 0; rr < 4; ++rr)
-      load32(vp + (int64_t)__shfl_sync(0xffffffffu, tok, 2 * j + (rr & 1) + (rr >> 1) * 8) * v_token, vr[rr]);
+      load32(vp + (int64_t)__shfl_sync(0xffffffffu, tok, 2 * j + (rr & 1) + (rr >> 1) * 8) * v_token, vr[buf][rr]);
   };
   int2 e;
   int tok;
-  if constexpr (kAhead) {
+  if constexpr (kAhead > 0) {
     e = get(0);
     tok = token(e);
+    const int tok1 = kAhead > 1 && count > 1 ? token(get(1)) : 0;
     gate();
-    load_k(tok);
-    load_v(tok);
-    if (count > 1) tok = token(get(1));
+    load_k(0, tok);
+    load_v(0, tok);
+    if (kAhead > 1 && count > 1) {
+      load_k(kBuffers - 1, tok1);
+      load_v(kBuffers - 1, tok1);
+    }
+    if (count > kAhead) tok = token(get(kAhead));
     ready();
   }
-#pragma unroll 1
-  for (int t = 0; t < count; ++t) {
-    if constexpr (!kAhead) {
+  auto block = [&](int t, int buf) {
+    if constexpr (kAhead == 0) {
       e = get(t);
       tok = token(e);
-      load_k(tok);
-      load_v(tok);
+      load_k(buf, tok);
+      load_v(buf, tok);
     }
-    const int n_keys = e.y;
-    const bool more = kAhead && t + 1 < count;
+    const int n_keys = kAhead > 1 ? get(t).y : e.y;
+    const bool more = kAhead > 0 && t + kAhead < count;
     float sc[4] = {0.f, 0.f, 0.f, 0.f};  // (key x, head 2j), (x, 2j + 1), (x + 8, 2j), (x + 8, 2j + 1)
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const uint2 b = q.frag[i][lane];
-      mma_16816(sc, ka[2 * i], kb[2 * i], ka[2 * i + 1], kb[2 * i + 1], b.x, b.y);
+      mma_16816(sc, ka[buf][2 * i], kb[buf][2 * i], ka[buf][2 * i + 1], kb[buf][2 * i + 1], b.x, b.y);
     }
     if (more) {
-      e = get(t + 1);
-      load_k(tok);
+      if (kAhead == 1) e = get(t + 1);
+      load_k(buf, tok);
     }
     float alpha[2], p0[2], p1[2];
 #pragma unroll
@@ -183,12 +190,18 @@ __device__ __forceinline__ void decode_walk(DecodeState& st, const DecodeQuery& 
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-      mma_16816(st.o[i], __byte_perm(vr[0][i], vr[1][i], 0x5410), __byte_perm(vr[0][i], vr[1][i], 0x7632),
-                __byte_perm(vr[2][i], vr[3][i], 0x5410), __byte_perm(vr[2][i], vr[3][i], 0x7632), pa, pb);
+      mma_16816(st.o[i], __byte_perm(vr[buf][0][i], vr[buf][1][i], 0x5410), __byte_perm(vr[buf][0][i], vr[buf][1][i], 0x7632),
+                __byte_perm(vr[buf][2][i], vr[buf][3][i], 0x5410), __byte_perm(vr[buf][2][i], vr[buf][3][i], 0x7632), pa, pb);
     if (more) {
-      load_v(tok);
-      if (t + 2 < count) tok = token(get(t + 2));
+      load_v(buf, tok);
+      if (t + kAhead + 1 < count) tok = token(get(t + kAhead + 1));
     }
+  };
+#pragma unroll 1
+  for (int t = 0; t < count; t += kBuffers) {
+    block(t, 0);
+    if constexpr (kBuffers == 2)
+      if (t + 1 < count) block(t + 1, 1);
   }
 }
 
@@ -282,7 +295,7 @@ __global__ void __launch_bounds__(128, 4) decode_kernel(const __grid_constant__ 
 
   DecodeState st;
   decode_init(st);
-  decode_walk<false>(st, s_q, pl, kv_idx, (n_vis - warp * 16 + NW * 16 - 1) / (NW * 16),
+  decode_walk<0>(st, s_q, pl, kv_idx, (n_vis - warp * 16 + NW * 16 - 1) / (NW * 16),
                      [&](int t) { const int k0 = (t * NW + warp) * 16; return make_int2(k0, n_vis - k0); }, kb, p.ks.token,
                      vb, p.vs.token, lane, cs, []() {}, []() {});
   decode_publish<G, NW>(sh, st, warp, lane);
@@ -309,8 +322,9 @@ __global__ void __launch_bounds__(128, 4) decode_kernel(const __grid_constant__ 
 // then "Caching"): query rows are turned while they are loaded, and the new token's key row is turned and written, with its
 // value row, to the caches before anyone reads them.
 // Measured (32 query / 8 KV heads): 64 sequences of 16384 tokens in 16 shards 662 us on inputs new to the caches = 6.49 TB/s
-// (repeated on the same ones, of which L2 keeps a part, 608; partials and merge as two kernels 825), one sequence 22 us (30 with
-// eight warps a CTA); the whole step of one sequence at 2500 of 4096 rows 7.7 us (9.4 with eight warps and the table behind a barrier).
+// (repeated on the same ones, of which L2 keeps a part, 608; partials and merge as two kernels 825), one sequence 25 us (23
+// repeated); the whole step of one sequence at 2500 of 4096 rows 7.6 us (7.1 repeated; with the table behind a barrier and one block
+// ahead 10.4 and 9.6).
 
 __device__ __forceinline__ uint32_t rotate_pair2(uint32_t x, uint32_t partner, const float4& cs, float sign) {
   // two neighbouring columns of one half: y = x cos + sign * partner * sin  (sign -1: lower half, +1: upper half)
@@ -322,12 +336,12 @@ __device__ __forceinline__ uint32_t rotate_pair2(uint32_t x, uint32_t partner, c
 constexpr int kMaxCluster = 16;
 constexpr int kFusedShards = 256;  // KV shards whose table fits in the kernel's shared memory at a time
 
-template <int G, int NW, bool kOneList>
-__global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __grid_constant__ AttnParams p,
-                                                                       const __grid_constant__ DecodeStep step) {
-  constexpr int D = 128;
-  extern __shared__ __align__(16) uint8_t smem_decode[];
-  DecodeShared<G, NW>& sh = *reinterpret_cast<DecodeShared<G, NW>*>(smem_decode);
+// kAhead: blocks that a warp requests ahead, see decode_walk; with 2 a CTA has an SM to itself.
+template <int G, int kAhead, bool kOneList>
+__global__ void __launch_bounds__(256, 3 - kAhead) decode_fused_kernel(const __grid_constant__ AttnParams p,
+                                                                      const __grid_constant__ DecodeStep step) {
+  constexpr int D = 128, NW = 8;
+  __shared__ DecodeShared<G, NW> sh;
   __shared__ DecodeQuery s_q;
   // what the CTAs of the cluster send for this CTA's part of the outputs: [sender][output], and n, w of every head
   __shared__ float s_o[G * D + kMaxCluster], s_n[kMaxCluster][G], s_w[kMaxCluster][G];
@@ -464,7 +478,7 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __
     }
     const int left = __shfl_sync(0xffffffffu, v, kk) - i * 16, first = __shfl_sync(0xffffffffu, off, kk) + i * 16;
     const int listed = list(make_int2(first, id < (even ? most * P : total) ? left : 0));
-    decode_walk<true>(st, s_q, pl, kv_idx, listed, [&](int t) { return s_list[warp][t]; }, kb, p.ks.token, vb, p.vs.token, lane, cs,
+    decode_walk<kAhead>(st, s_q, pl, kv_idx, listed, [&](int t) { return s_list[warp][t]; }, kb, p.ks.token, vb, p.vs.token, lane, cs,
                       gate, []() { __syncthreads(); });
   } else {
     gate();
@@ -500,7 +514,7 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __
           e = make_int2(s_off[kk] + i * 16, s_vis[kk] - i * 16);
         }
         const int listed = list(e);
-        decode_walk<true>(st, s_q, pl, kv_idx, listed, [&](int t) { return s_list[warp][t]; }, kb, p.ks.token, vb, p.vs.token, lane, cs,
+        decode_walk<kAhead>(st, s_q, pl, kv_idx, listed, [&](int t) { return s_list[warp][t]; }, kb, p.ks.token, vb, p.vs.token, lane, cs,
                           []() {}, []() {});
       }
     }
@@ -563,21 +577,47 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) decode_fused_kernel(const __
   }
 }
 
-template <int G, int NW>
+template <int G, int kAhead>
 static cudaError_t launch_fused(const AttnParams& p, const DecodeStep& step, int n_cta, cudaStream_t stream) {
   // One list: for as many keys as there are, whatever is visible when the launch runs (every shard may end in a block that is not
   // full, and in the interleaved order the list is a quarter longer).  Up to ten blocks a warp: beyond, the few registers that it
-  // costs the walk weigh more (2 sequences of 16384 tokens, 32 / 8 heads, 34.5 us, from the table 32.4; one, in the wide form, 22.0
-  // and 29.0 before both).
+  // costs the walk weigh more (2 sequences of 16384 tokens, 32 / 8 heads, 34.5 us, from the table 32.4).
   const int P = p.plan.n_kv_shards;
-  const bool one_list = P <= 32 && ((p.plan.n_kv + 15) / 16 + P) * (int64_t)5 / 4 + 1 <= 10 * (int64_t)n_cta * NW;
-  auto kernel = one_list ? decode_fused_kernel<G, NW, true> : decode_fused_kernel<G, NW, false>;
-  constexpr int smem = sizeof(DecodeShared<G, NW>);
-  cudaError_t e = cudaSuccess;
-  if (n_cta > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess && smem > 32768) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  return launch_dependent(kernel, dim3(n_cta, p.Hkv, p.batch), NW * 32, smem, n_cta, true, stream, p, step);
+  const bool one_list = P <= 32 && ((p.plan.n_kv + 15) / 16 + P) * (int64_t)5 / 4 + 1 <= 10 * (int64_t)n_cta * 8;
+  auto kernel = one_list ? decode_fused_kernel<G, kAhead, true> : decode_fused_kernel<G, kAhead, false>;
+  if (n_cta > 8) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_dependent(kernel, dim3(n_cta, p.Hkv, p.batch), 256, 0, n_cta, true, stream, p, step);
+}
+
+// How many clusters of n_cta CTAs that have an SM each the device holds at a time.
+static int clusters_alone(int n_cta) {
+  static std::atomic<int16_t> known[64][kMaxCluster + 1];  // number + 1; 0: not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  std::atomic<int16_t>& entry = known[dev][n_cta];
+  if (const int n = entry.load(std::memory_order_relaxed)) return n - 1;
+  auto kernel = decode_fused_kernel<8, 2, true>;  // (all forms with two blocks ahead take a whole SM)
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_cta);
+  cfg.blockDim = dim3(256);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = n_cta;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  cudaError_t e = n_cta > 8 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  entry.store((int16_t)(std::min(n, 1000) + 1), std::memory_order_relaxed);
+  return n;
 }
 
 // f(integral_constant G) for the group sizes the kernels are built for
@@ -623,13 +663,16 @@ cudaError_t launch_decode_fused(const AttnParams& p, const DecodeStep& step, int
   const int64_t pairs = (int64_t)p.rule_kv_heads * p.batch, blocks = std::max<int64_t>(1, (n_visible + 15) / 16);
   const int64_t most = std::min<int64_t>(pairs <= 7 ? kMaxCluster : 10, (blocks + 7) / 8);
   const int n_cta = pairs > 128 ? cluster_for_many(pairs, blocks, most) : (int)std::max<int64_t>(1, std::min(256 / pairs, most));
-  // Sixteen warps a CTA where that gives every CTA an SM of its own and there are blocks for them: with eight, an SM holds half the
-  // loads it could (one sequence of 16384 tokens, 32 / 8 heads, 30.4 us, now 21.7; a step at 12000 of them, 64 / 8 heads, 25.5
-  // and 17.5; 600 tokens, 8 / 8 heads, 6.1 and 5.3).
-  const bool wide = pairs * n_cta <= 132 && blocks > 8 * n_cta;
+  // Two blocks ahead where every CTA gets an SM of its own all the same and its warps have a second block: with one, an SM holds
+  // half the loads it could (one block ahead -> two, us, on caches new to L2: a step at 2500 rows, 32 / 8 heads, 9.9 -> 7.6; decode on
+  // 1400 keys, 8 / 8 heads, 8.2 -> 6.7, on 16384, 32 / 8 heads, 30.7 -> 25.0, on 32768 54 -> 42).  Where the clusters do not all fit
+  // that way, a second round costs more: 3 sequences of 8000 keys, 4 KV heads, 21 us, and 28 when CTAs that take a whole SM were
+  // launched for them.  Sixteen warps a CTA, with a block ahead each, kept as many loads in flight (16384 keys 22 us, 2500 rows 8.2),
+  // but a warp rounds its weights to bf16 against a maximum of its own, so another number of warps changes the result.
+  const bool two_ahead = blocks > 8 * n_cta && (int64_t)p.Hkv * p.batch <= clusters_alone(n_cta);
   TimedLaunch timed(stream);
   return with_group(p.G, [&](auto g) {
-    return wide ? launch_fused<decltype(g)::value, 16>(p, step, n_cta, stream) : launch_fused<decltype(g)::value, 8>(p, step, n_cta, stream);
+    return two_ahead ? launch_fused<decltype(g)::value, 2>(p, step, n_cta, stream) : launch_fused<decltype(g)::value, 1>(p, step, n_cta, stream);
   });
 }
 

@@ -1,5 +1,5 @@
-"""Fused decode where a warp lists its blocks by itself (up to 32 shards, up to ten blocks a warp) and where a CTA has sixteen
-warps (few KV heads and sequences): edges of both, against the oracle."""
+"""Fused decode where a warp lists its blocks by itself (up to 32 shards, up to ten blocks a warp) and where it requests two blocks
+ahead (few KV heads and sequences): edges of both, against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -17,11 +17,13 @@ def gu():
 
 
 @pytest.mark.parametrize("B,n_kv,H,Hkv,P,kv_map,pos", [
-    (1, 2049, 64, 8, 8, "random", 2048),      # sixteen warps, eight heads: partials of more than 48 KiB; one key past a block
+    (1, 2049, 64, 8, 8, "random", 2048),      # two blocks ahead, eight heads; one key past a block
     (1, 4097, 32, 8, 32, "contiguous", 4000), # 32 shards, the last ones empty: shard after shard, found by search
     (1, 4097, 32, 8, 33, "contiguous", 4000), # one shard more: the table
-    (1, 1281, 8, 8, 5, "random", 1280),       # sixteen warps a CTA, nearly every warp with one block
-    (1, 20000, 16, 8, 16, "random", 19000),   # sixteen warps, more than ten blocks each
+    (1, 1281, 8, 8, 5, "random", 1280),       # two blocks ahead, nearly every warp with one block
+    (1, 20000, 16, 8, 16, "random", 19000),   # more than ten blocks a warp: two ahead, from the table
+    (1, 45000, 16, 8, 5, "random", 44990),    # more than 32 blocks a warp: the list is made a second time
+    (3, 3000, 8, 4, 8, "random", 2999),       # 12 KV heads and sequences: their clusters do not all get an SM for each CTA
     (2, 12000, 32, 8, 8, "random", 11999),    # ten CTAs of eight warps a pair, from the table
     (1, 17, 4, 1, 2, "contiguous", 16),       # two blocks, one of them a single key
     (3, 200, 2, 2, 32, "random", 3),          # four keys in all, most shards empty
@@ -29,6 +31,25 @@ def gu():
 def test_decode_lists_and_widths(gu, B, n_kv, H, Hkv, P, kv_map, pos):
     gu.full_parity(wl.make_workload(f"lists_{B}_{n_kv}_{P}", B, 1, n_kv, H, Hkv, 128, "bf16", "round_robin", kv_map, 1, P, seed=n_kv + P,
                                     q_pos_offset=pos))
+
+
+@pytest.mark.parametrize("n_kv,H,Hkv,P,pos", [
+    (1500, 8, 8, 8, 1400),      # one block a warp, some with two
+    (4096, 32, 8, 8, 2500),     # two and three
+    (8192, 16, 2, 40, 8000),    # 33 shards and more: the table
+    (24000, 16, 8, 16, 23000),  # 18, from the table
+])
+def test_a_sequence_has_the_same_bits_alone_and_beside_another(gu, n_kv, H, Hkv, P, pos):
+    """As many CTAs a sequence in both calls; alone, a warp requests two blocks ahead.  What it adds up, and in which order, stays."""
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload(f"alone_{n_kv}", 2, 1, n_kv, H, Hkv, 128, "bf16", "round_robin", "random", 1, P, seed=n_kv, q_pos_offset=pos)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    o, lse = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+    for b in range(2):
+        o1, lse1 = cb.cascade_attn_sharded(plan, q[b:b + 1], k[b:b + 1], v[b:b + 1], w.scale)
+        assert torch.equal(o1[0], o[b]) and torch.equal(lse1[0], lse[b])
+    plan.destroy()
 
 
 def test_captured_decode_follows_the_plan(gu):
