@@ -184,7 +184,8 @@ cascade_status_t cascade_plan_device_status(const cascade_plan_t* plan, int32_t*
  * workspace: as reported by cascade_workspace_bytes(CASCADE_CALL_PARTIALS) (may be 0 -> NULL allowed).  The
  * tensor-core route first copies K and V into shard-major order there (the stage-A hand-over of each KV shard to
  * its AttnNodes, Appendix D): 2 * batch * n_kv_heads * n_kv * head_dim * 2 bytes, overwritten by every call.  fp32 at head_dim
- * 64 keeps the split keys and values there, three times as much and a byte per 64 rows.
+ * 64 keeps the split keys and values there, three times as much and a byte per 64 rows; none is asked for where the ALU kernels
+ * are the faster way, and without it they are taken.
  */
 cascade_status_t cascade_attn_partials(const cascade_plan_t* plan, cascade_dtype_t dtype, int32_t batch,
                                        int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, float scale,

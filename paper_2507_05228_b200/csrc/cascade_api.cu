@@ -750,14 +750,29 @@ static bool tc_ws_given(const cascade_plan_t* plan, int batch, int Hkv, int d, c
 static bool split_takes(const cascade_plan_t* plan, cascade_dtype_t dtype, int d) {
   return dtype == CASCADE_F32 && d == 64 && plan->dev.n_q > 1 && plan->dev.n_kv_shards <= 256;
 }
+static bool split_faster(const AttnParams& p) {
+  return split_time(p) < (p.fused ? 1.3 : 1.1) * std::min(tiles_time(p), rows_time(p)) + (p.fused ? 5 : 4);
+}
 static bool use_split(const AttnParams& p, const cascade_plan_t* plan, cascade_dtype_t dtype, const void* workspace, size_t bytes) {
   return split_takes(plan, dtype, p.d) && workspace && ((uintptr_t)workspace & 255) == 0 &&
-         bytes >= split_ws_bytes(plan->dev, p.batch, p.Hkv) && split_time(p) < (p.fused ? 1.3 : 1.1) * std::min(tiles_time(p), rows_time(p)) + (p.fused ? 5 : 4);
+         bytes >= split_ws_bytes(plan->dev, p.batch, p.Hkv) && split_faster(p);
 }
-// Scratch of the routes with copies of K and V: bf16 on the tensor cores, or fp32 on the tensor cores.
-static size_t copies_ws_bytes(const cascade_plan_t* plan, cascade_dtype_t dtype, int batch, int Hkv, int d) {
+// Scratch of the routes with copies of K and V: bf16 on the tensor cores, or fp32 on the tensor cores where that is the faster way
+// from where the plan's query block is, or from the end of the keys, to which it may be moved.  rule_kv_heads: see AttnParams.
+static size_t copies_ws_bytes(const cascade_plan_t* plan, cascade_dtype_t dtype, int batch, int H, int Hkv, int d, bool fused,
+                              int rule_kv_heads) {
   if (use_tc(plan, dtype, d)) return tc_ws_bytes(plan, batch, Hkv, d);
-  return split_takes(plan, dtype, d) ? split_ws_bytes(plan->dev, batch, Hkv) : 0;
+  if (!split_takes(plan, dtype, d)) return 0;
+  const cascade_strides_t none = {0, 0, 0};
+  AttnParams p = make_params(plan, batch, H, Hkv, d, 1.f, nullptr, none, nullptr, none, nullptr, none);
+  p.fused = fused;
+  p.rule_kv_heads = rule_kv_heads;
+  bool wanted = split_faster(p);
+  if (const int last = plan->dev.n_kv - plan->dev.n_q; !wanted && plan->dev.causal && plan->dev.q_pos_offset < last) {
+    p.plan.q_pos_offset = last;
+    wanted = split_faster(p);
+  }
+  return wanted ? split_ws_bytes(plan->dev, batch, Hkv) : 0;
 }
 
 // Partials over short shards of heads of 64 columns, in bf16: whether the ALU kernels beat the tensor cores.
@@ -881,7 +896,7 @@ static HostCallLayout host_call_layout(const cascade_plan_t* plan, cascade_dtype
   // gs KV heads and their query heads per inner call
   const bool decode = use_decode(plan, dtype, G * gs, gs, d);
   L.inner_bytes = decode ? decode_ws_bytes(plan, dtype, batch, G * gs, d)
-                         : copies_ws_bytes(plan, dtype, batch, gs, d);
+                         : copies_ws_bytes(plan, dtype, batch, G * gs, gs, d, true, Hkv);
   L.total = L.inner + align_up(L.inner_bytes, 256);
   return L;
 }
@@ -911,11 +926,13 @@ cascade_status_t cascade_workspace_bytes(const cascade_plan_t* plan, int32_t whi
     return CASCADE_ERR_INVALID_ARG;
   }
   const bool decode = use_decode(plan, dtype, n_heads, n_kv_heads, head_dim);
-  const size_t tc_bytes = decode ? 0 : copies_ws_bytes(plan, dtype, batch, n_kv_heads, head_dim);
+  auto copies = [&](bool fused) {
+    return decode ? 0 : copies_ws_bytes(plan, dtype, batch, n_heads, n_kv_heads, head_dim, fused, n_kv_heads);
+  };
   if (which_call == CASCADE_CALL_PARTIALS) {
-    *out_bytes = tc_bytes;
+    *out_bytes = copies(false);
   } else if (which_call == CASCADE_CALL_SHARDED) {
-    *out_bytes = decode ? decode_ws_bytes(plan, dtype, batch, n_heads, head_dim) : tc_bytes;
+    *out_bytes = decode ? decode_ws_bytes(plan, dtype, batch, n_heads, head_dim) : copies(true);
   } else if (which_call == CASCADE_CALL_SHARDED_HOST) {
     *out_bytes = host_call_layout(plan, dtype, batch, n_heads, n_kv_heads, head_dim).total;
   } else if (which_call == CASCADE_CALL_DECODE_STEP_ROPE) {

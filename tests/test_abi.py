@@ -100,6 +100,28 @@ def test_workspace_of_the_tensor_core_route_is_two_copies(binding):
     plan.destroy()
 
 
+def test_workspace_of_split_fp32_operands_is_asked_for_where_they_are_used(binding):
+    """fp32, heads of 64: three bf16 copies of K and of V and their flags, or nothing where the ALU kernels are taken."""
+    def need(n_q, n_kv, B, H, off, causal, call):
+        plan = binding.cascade_shard_plan_host(np.arange(n_q, dtype=np.int32) % 4, np.arange(n_kv, dtype=np.int32) % 4, 4, 4, off, causal)
+        n = binding.cascade_workspace_bytes(plan, call, binding.F32, B, H, H, 64)
+        plan.destroy()
+        return n
+
+    def copies(n_kv, mats):
+        return 2 * (-(-3 * mats * n_kv * 128 // 256) * 256) + -(-2 * mats * -(-n_kv // 64) // 256) * 256
+
+    sharded, partials, host = binding.CALL_SHARDED, binding.CALL_PARTIALS, binding.CALL_SHARDED_HOST
+    for call in (sharded, partials):
+        assert need(512, 512, 16, 16, 0, False, call) == copies(512, 256)
+        assert need(33, 33, 1, 8, 0, False, call) == 0
+        # a block of queries that is moved along a cache: the same wherever it stands, as scratch is taken once
+        assert need(256, 8192, 4, 16, 0, True, call) == need(256, 8192, 4, 16, 7936, True, call) == copies(8192, 64)
+    staging = lambda n, B, H: 4 * (B * n * H * 64 * 4)  # (multiples of 256)
+    assert need(256, 256, 1, 8, 0, True, host) == staging(256, 1, 8)
+    assert need(512, 512, 16, 16, 0, False, host) == staging(512, 16, 16) + copies(512, 16 * 4)  # four heads at a time
+
+
 def test_tensors_without_storage_raise(binding):
     """torch.func.vmap hands out tensors that throw when asked for their data pointer.  In a child process: an exception that
     leaves the interpreter lock released takes the interpreter down with it."""
