@@ -353,7 +353,9 @@ cascade_status_t cascade_kl_gaps(int32_t n_tokens, const uint8_t* r_held, const 
  *   q_host, o_host  HOST, dense [batch][n_q][n_heads][head_dim]; k_host, v_host  HOST, dense
  *                   [batch][n_kv][n_kv_heads][head_dim].  Pinned memory is needed for the copies to be asynchronous.
  *   workspace       DEVICE, 256-byte aligned, cascade_workspace_bytes(CASCADE_CALL_SHARDED_HOST) bytes: staging for
- *                   q, k, v, o and the scratch of one head group.  Overwritten by every call.
+ *                   q, k, v, o and the scratch of one head group.  Overwritten by every call.  Heads of 64 columns take any
+ *                   size from the staging alone on (each of the four rounded up to 256 bytes), and the ALU kernels without
+ *                   the rest.
  * All work is ordered after what `stream` holds at the time of the call, and `stream` waits for the last output
  * copy: synchronising `stream` makes o_host valid.  The first call on a device creates two internal copy streams and
  * their events (no device memory); all calls on a device share them, so calls from several host threads for the same

@@ -1364,11 +1364,9 @@ cascade_status_t cascade_attn_sharded_host(const cascade_plan_t* plan, cascade_d
     return CASCADE_ERR_UNSUPPORTED;
   }
   const HostCallLayout L = host_call_layout(plan, dtype, batch, n_heads, n_kv_heads, head_dim);
-  // heads of 64 columns do without the part for the head groups (on the ALU kernel), so a workspace without it is taken; in fp32
-  // only one of exactly that size, which is all that this call used to ask for
+  // heads of 64 columns do without the part for the head groups (on the ALU kernel), so a workspace without all of it is taken
   const bool inner = L.inner_bytes && (head_dim == 128 || workspace_bytes >= L.total);
-  const bool staging_only = head_dim == 64 && (dtype == CASCADE_BF16 || workspace_bytes < L.inner + 256);
-  const size_t need = staging_only ? L.inner : L.total;
+  const size_t need = head_dim == 64 ? L.inner : L.total;
   if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) {
     set_error("%s: workspace of %zu bytes (256-byte aligned) required, got %zu", fn, need, workspace_bytes);
     return CASCADE_ERR_WORKSPACE;

@@ -108,6 +108,31 @@ def test_head_dim_64_with_too_small_a_workspace(gu):
     plan.destroy()
 
 
+def test_fp32_host_call_with_any_workspace_that_holds_the_staging(gu):
+    """fp32, heads of 64: from the staging alone up to a byte less than all, the head groups take the ALU kernel."""
+    from paper_2507_05228_b200 import binding as cb
+    B, n, H = 8, 300, 16
+    w = wl.make_workload("d64_f32_host_ws", B, n, n, H, H, 64, "f32", "random", "random", 3, 3, seed=10)
+    plan = gu.make_plan(w)
+    o_ref, _ = oracle.attention_unsharded(w.q, w.k, w.v, w.scale)
+    hq, hk, hv = (torch.from_numpy(a).pin_memory() for a in (w.q, w.k, w.v))
+    ho = torch.empty_like(hq).pin_memory()
+    staging = 4 * ((hq.numel() * 4 + 255) // 256 * 256)
+    total = cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED_HOST, cb.F32, B, H, H, 64)
+    assert total > staging + 512  # the head groups would use the rest
+    raw = torch.full((total + 256,), 0x5A, dtype=torch.uint8, device="cuda")
+    for size in (staging, staging + 256, staging + 257, total - 1):
+        ho.zero_()
+        cb.cascade_attn_sharded_host(plan, hq, hk, hv, w.scale, ho, raw[:size])
+        torch.cuda.synchronize()
+        gu.check_output(ho.double().numpy(), None, o_ref, None, w.tol, f"host call with {size - staging} bytes of scratch")
+        assert (raw[staging:] == 0x5A).all()
+    with pytest.raises(cb.CascadeError) as ei:
+        cb.cascade_attn_sharded_host(plan, hq, hk, hv, w.scale, ho, raw[:staging - 1])
+    assert ei.value.status == 4
+    plan.destroy()
+
+
 @pytest.mark.parametrize("n_q,n_kv,H,Hkv,d,B,shards,dtype,causal", [
     (1, 1, 2, 2, 64, 1, 1, "f32", True),          # one key
     (1, 300, 6, 2, 64, 2, 3, "bf16", True),       # one query row on the ALU route: key groups share the row
