@@ -27,8 +27,9 @@
 // What bounds it: the chain of a sub-tile, weights -> output -> (logits) -> weights, about 5500 cycles a tile, in which the tensor
 // cores are busy for 3500; with partials the stores (60 of 234 us at 16 x 512 tokens in 8 shards).
 //
-// Values of 2^63 and beyond, infinities and NaN, whose parts could turn a result into NaN that fp32 arithmetic keeps: from a tile
-// that holds any on, a CTA works its tiles out in plain fp32 by the softmax threads, slowly.
+// Values of 2^63 and beyond, infinities and NaN, whose parts could turn a result into NaN that fp32 arithmetic keeps: a tile with such
+// keys or values, and every tile of a CTA with such queries, is worked out in plain fp32 by the softmax threads, slowly: fused,
+// 16 x 512 tokens, 16 heads, 148 us; with one such key, or value, in every head 1.1 ms, or 1.6; with all of them 7.4, or 12.
 #include "tcgen05.cuh"
 
 namespace cascade {
@@ -52,12 +53,15 @@ constexpr int kOffMax = kOffV + 2 * kKvTile;        // float [2][sub-tile][half]
 constexpr int kOffTab = kOffMax + 3 * 4 * kM * 4;   // int32 [2][2][kMaxShards]: longest and shortest prefix of a sub-tile's rows
 constexpr int kOffBar = kOffTab + 4 * kMaxShards * 4;
 constexpr int kOffMisc = kOffBar + 32 * 8;          // TMEM address, abort flag, progress words, see WaitCtx
-constexpr int kOffBad = kOffMisc + 8 + 4 * kWarps;  // [0]: a query row, or a key row of a tile so far, is out of range, [1]: a value row
-constexpr int kOffInfo = kOffBad + 8;               // int32 [3]: see tile_info
-constexpr int kSmemBytes = kOffInfo + 12 + 1024;
+constexpr int kOffFar = kOffMisc + 8 + 4 * kWarps;  // int32: kFarQ, kFarK, kFarV, whether any such row of the CTA is out of range
+constexpr int kOffInfo = kOffFar + 4;               // int32 [3]: see tile_info
+constexpr int kFarWords = 128;                      // keys, values: a bit for every 64 << far_shift rows, whether one is out of range
+constexpr int kOffFarRows = kOffInfo + 12;          // uint32 [2][kFarWords]
+constexpr int kSmemBytes = kOffFarRows + 2 * kFarWords * 4 + 1024;
 static_assert(kSmemBytes <= 232448, "exceeds the 227 KiB a CTA may use");
 
 // two of each: by sub-tile, or by stage
+enum { kFarQ = 1, kFarK = 2, kFarV = 4 };
 enum Bar { Q_FULL = 0, S_FULL = 2, P_FULL = 6, O_FULL = 8, K_FULL = 10, K_EMPTY = 12, V_FULL = 14, V_EMPTY = 16, DONE = 18 };
 
 __device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
@@ -227,7 +231,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
     }
   }
 
-  auto bad = [&](int i) -> volatile int& { return reinterpret_cast<volatile int*>(smem + kOffBad)[i]; };  // see kOffBad
+  int* const any_far = reinterpret_cast<int*>(smem + kOffFar);
+  auto far_kinds = [&]() { return *const_cast<volatile int*>(any_far); };
+  auto far_rows = [&](int is_v) { return reinterpret_cast<volatile uint32_t*>(smem + kOffFarRows) + is_v * kFarWords; };
+  const int blocks = (pl.n_kv + 63) / 64, far_shift = max(0, 32 - __clz((blocks - 1) / (32 * kFarWords)));
   // [0], [1]: tile of either stage: keys, + 256 if sub-tile 0 sees any of them (sub-tile 1 sees all that there are); [2]: tiles
   volatile int* const tile_info = reinterpret_cast<volatile int*>(smem + kOffInfo);
   WaitCtx<false, kWarps> wc;
@@ -252,7 +259,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
       asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(gave_up) : "l"(pl.status) : "memory");
       wc.store(1, gave_up != 0);
       for (int w = 0; w < kWarps; ++w) wc.store(2 + w, 0);
-      bad(0) = bad(1) = 0;
+      *any_far = 0;
     }
     __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_base + (uint32_t)kOffMisc),
@@ -307,7 +314,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
         const int r = ((tid & 255) >> 3) + 32 * j;
         store_split8(smem + kOffQ + s * kQTile + r * 128 + (((tid & 7) ^ (r & 7)) << 4), kQPart, qu[j], qv[j], big);
       }
-      if (is_big(big)) bad(0) = 1;
+      if (is_big(big)) atomicOr(any_far, kFarQ);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> tensor-core reads
       mbar_arrive(bar(Q_FULL + s));
 
@@ -367,6 +374,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
         }
       };
       auto seen_of = [&](int k, int t0, int n) { return min(n, (kParts ? __ldg(my_vis + k) : seen_all) - t0); };
+      // whether a key (is_v: value) row that the products of tile (k, t0) read is out of range
+      auto far_tile = [&](int is_v, int k, int t0, int n) {
+        const int row = (kParts ? __ldg(kv_off + k) : 0) + t0, last = min(row + (n + 15) / 16 * 16, pl.n_kv) - 1;
+        const int b0 = row / 64 >> far_shift, b1 = last / 64 >> far_shift;
+        return (((far_rows(is_v)[b0 / 32] >> (b0 & 31)) | (far_rows(is_v)[b1 / 32] >> (b1 & 31))) & 1u) != 0;
+      };
       auto slow_dot = [&](int k, int t0, int x) {  // the logit of key x of tile (k, t0) in plain fp32
         const float4 *q4 = reinterpret_cast<const float4*>(q_row(s, m)), *k4 = reinterpret_cast<const float4*>(kb + kv_row(k, t0, x) * p.ks.token);
         float dot = 0.f;
@@ -385,28 +398,34 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
         wait_bar(wc, bar(O_FULL + s), (uint32_t)(i & 1), 3, i);
         tc_fence_after();
         const bool opens = t0 == 0, closes = t0 + kN >= longest(s)[k];
-        if (__any_sync(0xffffffffu, bad(1))) {
-          const int seen = seen_of(k, t0, n);
-#pragma unroll 1
-          for (int c = kCols * half; c < kCols * half + kCols; c += 4) {  // (the weights themselves are gone by now)
-            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-            for (int x = 0; x < seen; ++x) {
-              const float w = ex2((slow_dot(k, t0, x) - (m_run == -INFINITY ? 0.f : m_run)) * cs);
-              const float4 v = __ldg(reinterpret_cast<const float4*>(vb + kv_row(k, t0, x) * p.vs.token + c));
-              o = make_float4(fmaf(w, v.x, o.x), fmaf(w, v.y, o.y), fmaf(w, v.z, o.z), fmaf(w, v.w, o.w));
-            }
-            __syncwarp();
-            tmem_st1(o_addr + (uint32_t)c, __float_as_uint(o.x));
-            tmem_st1(o_addr + (uint32_t)c + 1, __float_as_uint(o.y));
-            tmem_st1(o_addr + (uint32_t)c + 2, __float_as_uint(o.z));
-            tmem_st1(o_addr + (uint32_t)c + 3, __float_as_uint(o.w));
-          }
-          tmem_wait_st();
-        }
         uint32_t o[kCols];
-        CASCADE_TMEM_LD32(o_addr + (uint32_t)(kCols * half), o, 0);
-        tmem_wait_ld();
+        auto products = [&]() {
+          CASCADE_TMEM_LD32(o_addr + (uint32_t)(kCols * half), o, 0);
+          tmem_wait_ld();
+        };
+        if (kParts) products();  // (in front 228.4 -> 221.2 us at 16 x 512 tokens, 8 shards; fused 147.7, in front 151.2)
+        if (__any_sync(0xffffffffu, (far_kinds() & kFarV) && far_tile(1, k, t0, n))) {
+          const int seen = seen_of(k, t0, n);
+          const float m_use = m_run == -INFINITY ? 0.f : m_run;
+#pragma unroll
+          for (int c = 0; c < kCols; ++c) o[c] = 0u;
+#pragma unroll 1
+          for (int x = 0; x < seen; ++x) {  // (the weights themselves are gone by now)
+            const float w = ex2((slow_dot(k, t0, x) - m_use) * cs);
+            const float4* v4 = reinterpret_cast<const float4*>(vb + kv_row(k, t0, x) * p.vs.token + kCols * half);
+#pragma unroll
+            for (int c = 0; c < kCols; c += 4) {
+              const float4 v = __ldg(v4 + c / 4);
+              o[c] = __float_as_uint(fmaf(w, v.x, __uint_as_float(o[c])));
+              o[c + 1] = __float_as_uint(fmaf(w, v.y, __uint_as_float(o[c + 1])));
+              o[c + 2] = __float_as_uint(fmaf(w, v.z, __uint_as_float(o[c + 2])));
+              o[c + 3] = __float_as_uint(fmaf(w, v.w, __uint_as_float(o[c + 3])));
+            }
+          }
+          __syncwarp();
+        } else if (!kParts) {
+          products();
+        }
 #pragma unroll
         for (int j = 0; j < kCols; ++j) acc[j] = opens ? __uint_as_float(o[j]) : fmaf(acc[j], alpha, __uint_as_float(o[j]));
         if (closes) {
@@ -429,7 +448,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
         const int seen = seen_of(seq.k, seq.t0, n);  // (ahead of the wait, which hides the load)
         wait_bar(wc, bar(S_FULL + s), (uint32_t)(i & 1), 1, i);
         tc_fence_after();
-        if (__any_sync(0xffffffffu, bad(0))) {
+        const int far = far_kinds();
+        if (__any_sync(0xffffffffu, (far & (kFarQ | kFarK)) && ((far & kFarQ) || far_tile(0, seq.k, seq.t0, n)))) {
 #pragma unroll 1
           for (int x = kCols * half; x < min(n, kCols * half + kCols); ++x) {
             const float dot = slow_dot(seq.k, seq.t0, x);
@@ -616,6 +636,21 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
       const int full = is_v ? V_FULL : K_FULL, empty = is_v ? V_EMPTY : K_EMPTY;
       const uint32_t to = smem_base + (uint32_t)(is_v ? kOffV : kOffK);
       grid_wait();  // the copies are written by the grid in front
+      // The rows out of range, for the softmax threads: all of them before the first tile, so that which tiles are worked out in plain
+      // fp32 depends on the rows alone and not on how far ahead this warp is.
+      auto note_far = [&]() {
+        volatile uint32_t* bits = far_rows(is_v);
+        for (int w = lane; w < kFarWords; w += 32) bits[w] = 0u;
+        __syncwarp();
+        const volatile uint8_t* flags = (is_v ? sp.v_far : sp.k_far) + ((int64_t)b * p.Hkv + g) * blocks;
+#pragma unroll 4
+        for (int x = lane; x < blocks; x += 32)
+          if (flags[x]) {
+            atomicOr(const_cast<uint32_t*>(bits) + (x >> far_shift) / 32, 1u << ((x >> far_shift) & 31));
+            atomicOr(any_far, is_v ? kFarV : kFarK);
+          }
+        __syncwarp();
+      };
       TileSeq seq(longest(n_sub - 1), n_parts);  // the later sub-tile sees all that the earlier one does
       int i = 0;
       for (; seq.next(); ++i) {
@@ -626,12 +661,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
           mbar_expect_tx(bar(full + (i & 1)), kKvTile);
           const int row = (kParts ? __ldg(kv_off + seq.k) : 0) + seq.t0;  // first row of the tile in the split copies
           tma_box4(to + (uint32_t)((i & 1) * kKvTile), is_v ? &sp.v : &sp.k, 0, row, b * p.Hkv + g, 0, bar(full + (i & 1)));
-          // whether a row of the box is out of range (looked up while the box is on its way)
-          const int blocks = (pl.n_kv + 63) / 64;
-          const volatile uint8_t* flags = (is_v ? sp.v_far : sp.k_far) + ((int64_t)b * p.Hkv + g) * blocks;
-          if (flags[row / 64] | flags[min(row / 64 + 1, blocks - 1)]) bad(is_v) = 1;
-          mbar_arrive(bar(full + (i & 1)));
         }
+        if (i == 0) note_far();  // (while the box is on its way)
+        if (leader) mbar_arrive(bar(full + (i & 1)));
         __syncwarp();
       }
       if (wc.load(1))

@@ -115,6 +115,35 @@ def test_split_route_with_values_out_of_range(gu):
     plan.destroy()
 
 
+@pytest.mark.parametrize("far", ["key", "value"])
+def test_values_out_of_range_touch_their_own_tiles_only(gu, far):
+    """Partials of the shards without such a row, and fused rows before the tile that holds it, keep their bits."""
+    from paper_2507_05228_b200 import binding as cb
+    B, n, H, P = 8, 400, 16, 4
+    w = wl.make_workload("split_far", B, n, n, H, H, 64, "f32", "random", "random", 2, P, seed=21, symmetric=False)
+    w.kv_shard_of = (np.arange(n) // 8 % P).astype(np.int32)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    ws = torch.empty(cb.cascade_workspace_bytes(plan, cb.CALL_PARTIALS, cb.F32, B, H, H, 64), dtype=torch.uint8, device="cuda")
+    n0 = cb.lib().cascade_launch_count()
+    clean = [t.clone() for t in cb.cascade_attn_partials(plan, q, k, v, w.scale, workspace=ws)]
+    assert cb.lib().cascade_launch_count() - n0 == 2
+    o = _fused(cb, plan, q, k, v, w.scale)[0]
+    if far == "key":  # in the tile of tokens 192 to 255 both; no other shard has rows in the same block of 64 slots
+        k[:, 192, :, 3] = 2.0 ** 70
+    else:
+        v[:, 200, :, 3] = 2.0 ** 70
+    k0 = 0 if far == "key" else 1
+    parts = [t.clone() for t in cb.cascade_attn_partials(plan, q, k, v, w.scale, workspace=ws)]
+    o_far = _fused(cb, plan, q, k, v, w.scale)[0]
+    assert not torch.equal(parts[0][:, k0], clean[0][:, k0])
+    for a, b in zip(parts, clean):
+        for kk in set(range(P)) - {k0}:
+            assert torch.equal(a[:, kk], b[:, kk]), kk
+    assert torch.equal(o_far[:, :192], o[:, :192]) and not torch.equal(o_far[:, 192:], o[:, 192:])
+    plan.destroy()
+
+
 def test_captured_split_calls_follow_the_plan(gu):
     from paper_2507_05228_b200 import binding as cb
     B, n_q, n_kv, H, P = 8, 128, 700, 16, 3
