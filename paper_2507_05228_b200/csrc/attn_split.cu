@@ -1,7 +1,7 @@
 // fp32 attention-pass on the tensor cores (the Attention-Pass algorithm, and the fused route), head_dim 64.
 //
 // Every fp32 operand is taken apart into three bf16 numbers, x = x0 + x1 + x2 (each the rounded rest of what came before; 24 bits
-// in all, so nothing is left out), and a product x y becomes six bf16 products, those of order up to 2^-16:
+// in all, so from 2^-110 on, where the last bit is bf16's smallest number, nothing is left out), and a product x y becomes six bf16 products, those of order up to 2^-16:
 //   x0 y2 + x2 y0 + x1 y1 + x0 y1 + x1 y0 + x0 y0;  what is left out (x1 y2, x2 y1, x2 y2) is below 2^-24 |x y|.
 // The tensor core cuts its fp32 sums off at every step.  So the small products come first, the large ones of a logit are shared by two
 // accumulators (two steps at full size each), and those and the outputs of different key tiles are added up in registers.
@@ -27,8 +27,11 @@
 // What bounds it: the chain of a sub-tile, weights -> output -> (logits) -> weights, about 5500 cycles a tile, in which the tensor
 // cores are busy for 3500; with partials the stores (60 of 234 us at 16 x 512 tokens in 8 shards).
 //
-// Values of 2^63 and beyond, infinities and NaN, whose parts could turn a result into NaN that fp32 arithmetic keeps: a tile with such
-// keys or values, and every tile of a CTA with such queries, is worked out in plain fp32 by the softmax threads, slowly: fused,
+// Out of range are values of 2^63 and beyond, infinities and NaN, whose parts could turn a result into NaN that fp32 arithmetic keeps;
+// queries and keys all of whose columns are below 2^-100, and columns of values that are in 64 rows, unless they are zero: of those the
+// parts lose bits (relative error of the output with all values of size 2^-110 1.2e-7 as ever, 2^-115 1.1e-6, 2^-120 3.5e-5).  Beside a
+// larger one, what is lost of a value is below 2^-34 of it.  A tile with such keys or values, and every tile of a CTA with such
+// queries, is worked out in plain fp32 by the softmax threads, slowly: fused,
 // 16 x 512 tokens, 16 heads, 148 us; with one such key, or value, in every head 1.1 ms, or 1.6; with all of them 7.4, or 12.
 #include "tcgen05.cuh"
 
@@ -97,6 +100,21 @@ __device__ __forceinline__ bool is_big(uint64_t big) {
   return !(a + b == 0.f);
 }
 
+// bits i of `some` and `most`: whether x[i] is not zero, and whether it is 2^-100 or more
+__device__ __forceinline__ void note_size(const float4& u, const float4& v, uint32_t& some, uint32_t& most) {
+  const float x[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    some |= x[i] != 0.f ? 1u << i : 0u;
+    most |= fabsf(x[i]) >= 7.888609e-31f ? 1u << i : 0u;
+  }
+}
+// Whether the row of eight threads that this thread is in has no such value of 2^-100 or more, and is not zero.  By whole warps.
+__device__ __forceinline__ bool is_small_row(uint32_t some, uint32_t most, int lane) {
+  const uint32_t any = __ballot_sync(0xffffffffu, some != 0), big = __ballot_sync(0xffffffffu, most != 0), row = 0xffu << (lane & 24);
+  return (any & row) != 0 && (big & row) == 0;
+}
+
 __device__ __forceinline__ void tma_box4(uint32_t dst, const CUtensorMap* map, int x, int y, int z, int w, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
@@ -140,15 +158,33 @@ __global__ void __launch_bounds__(256) split_kv_kernel(const __grid_constant__ A
   }
   const int64_t mat = (int64_t)b * p.Hkv + g, part_bytes = (int64_t)p.batch * p.Hkv * pl.n_kv * 128;
   uint64_t far[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  bool small_k = false;
+  uint32_t some_v = 0, most_v = 0;  // a bit for each column of this thread
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int r = r0 + 32 * j;
+    uint32_t some = 0, most = 0;
+    note_size(x[j][0], x[j][1], some, most);
+    note_size(x[j][2], x[j][3], some_v, most_v);
+    small_k |= is_small_row(some, most, lane);
     if (r >= pl.n_kv) continue;
     const int64_t at = (mat * pl.n_kv + r) * 128 + c8 * 16;
     store_split8(k_out + at, part_bytes, x[j][0], x[j][1], far[0]);
     store_split8(v_out + at, part_bytes, x[j][2], x[j][3], far[1]);
   }
-  const int any_k = __syncthreads_or(is_big(far[0])), any_v = __syncthreads_or(is_big(far[1]));
+  __shared__ uint32_t s_size[8][4];  // of the warp's rows: columns 0 to 31 and 32 to 63 that are not zero, and that reach 2^-100
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const uint32_t bits = __reduce_or_sync(0xffffffffu, (c8 >> 2) == (w & 1) ? (w < 2 ? some_v : most_v) << 8 * (c8 & 3) : 0u);
+    if (lane == 0) s_size[warp][w] = bits;
+  }
+  const int any_k = __syncthreads_or(is_big(far[0]) || small_k);
+  uint32_t size[4] = {0, 0, 0, 0};
+  if (warp == 0)
+    for (int w = 0; w < 8; ++w)
+      for (int i = 0; i < 4; ++i) size[i] |= s_size[w][i];
+  const int any_v = __syncthreads_or(is_big(far[1]) || (size[0] & ~size[2]) || (size[1] & ~size[3]));
   if (threadIdx.x == 0) {
     k_far[mat * gridDim.x + blockIdx.x] = any_k != 0;
     v_far[mat * gridDim.x + blockIdx.x] = any_v != 0;
@@ -309,12 +345,16 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
     const int s = warp >> 3, half = (warp >> 2) & 1, m = tid & 127;  // sub-tile, keys and columns 32 * half .., MMA row
     if (s < n_sub) {
       uint64_t big = pack2(0.f, 0.f);
+      bool small = false;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int r = ((tid & 255) >> 3) + 32 * j;
+        uint32_t some = 0, most = 0;
+        note_size(qu[j], qv[j], some, most);
+        small |= is_small_row(some, most, lane);
         store_split8(smem + kOffQ + s * kQTile + r * 128 + (((tid & 7) ^ (r & 7)) << 4), kQPart, qu[j], qv[j], big);
       }
-      if (is_big(big)) atomicOr(any_far, kFarQ);
+      if (is_big(big) || small) atomicOr(any_far, kFarQ);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> tensor-core reads
       mbar_arrive(bar(Q_FULL + s));
 
@@ -382,16 +422,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_split_kernel(const __grid_co
       };
       auto slow_dot = [&](int k, int t0, int x) {  // the logit of key x of tile (k, t0) in plain fp32
         const float4 *q4 = reinterpret_cast<const float4*>(q_row(s, m)), *k4 = reinterpret_cast<const float4*>(kb + kv_row(k, t0, x) * p.ks.token);
-        float dot = 0.f;
+        float4 dot = make_float4(0.f, 0.f, 0.f, 0.f);  // in four sums, whose roundings average out
 #pragma unroll 1
         for (int c = 0; c < kD / 4; ++c) {
           const float4 a = __ldg(q4 + c), d = __ldg(k4 + c);
-          dot = fmaf(a.x, d.x, dot);
-          dot = fmaf(a.y, d.y, dot);
-          dot = fmaf(a.z, d.z, dot);
-          dot = fmaf(a.w, d.w, dot);
+          dot = make_float4(fmaf(a.x, d.x, dot.x), fmaf(a.y, d.y, dot.y), fmaf(a.z, d.z, dot.z), fmaf(a.w, d.w, dot.w));
         }
-        return dot;
+        return (dot.x + dot.y) + (dot.z + dot.w);
       };
       // The output of tile (k, t0): added to what the shard's earlier tiles gave, scaled by alpha, and written if it is the shard's last.
       auto fold = [&](int k, int t0, int n, int i, float alpha) {

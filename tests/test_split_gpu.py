@@ -144,6 +144,36 @@ def test_values_out_of_range_touch_their_own_tiles_only(gu, far):
     plan.destroy()
 
 
+@pytest.mark.parametrize("what,size", [("q", -118), ("k", -118), ("v", -118), ("v", -101), ("k", -112), ("one column of v", -120)])
+def test_small_values_keep_their_bits(gu, what, size):
+    """Below 2^-110 three bf16 parts do not hold an fp32 number.  Rows of queries and keys and columns of values that small go another
+    way, in plain fp32.  Bound: a sum of n terms in a chain is off by 2^-24 / sqrt(3) * sqrt(n / 2) of itself in the mean, half an ulp of
+    rounding at each of its parts: 1.9e-7 for the 64 products of a tile, 1e-7 for logits near 1 in chains of 16, in the weights and in
+    the row sums; 2.4e-7 together, and the worst of 64 columns a tenth more."""
+    from paper_2507_05228_b200 import binding as cb
+    w = wl.make_workload("split_small", 8, 300, 300, 16, 16, 64, "f32", "random", "random", 3, 3, seed=17)
+    q, k, v = gu.to_device(w)
+    scale = w.scale
+    if what == "one column of v":
+        v[..., 5] *= 2.0 ** size
+    else:
+        {"q": q, "k": k, "v": v}[what].mul_(2.0 ** size)
+        if what != "v":
+            scale = w.scale * 2.0 ** -size
+    s = torch.einsum("bqhd,bkhd->bhqk", q.double(), k.double()) * float(np.float32(scale))
+    s = s.masked_fill(~torch.ones(300, 300, dtype=torch.bool, device="cuda").tril(), -torch.inf)
+    ref = torch.einsum("bhqk,bkhd->bqhd", torch.softmax(s, -1), v.double())
+    plan = gu.make_plan(w)
+    err = {}
+    for ws in (True, False):
+        o, _, n_kernels = _fused(cb, plan, q, k, v, scale, ws)
+        assert n_kernels == (2 if ws else 1)
+        off = (o.double() - ref).square().sum((0, 1, 2)).sqrt() / ref.square().sum((0, 1, 2)).sqrt()  # of every column
+        err[ws] = off.max().item()
+    assert err[True] <= 2.7e-7 and err[False] <= 2.7e-7, err
+    plan.destroy()
+
+
 def test_captured_split_calls_follow_the_plan(gu):
     from paper_2507_05228_b200 import binding as cb
     B, n_q, n_kv, H, P = 8, 128, 700, 16, 3
