@@ -75,7 +75,8 @@ struct WaitCtx<true, kWarps> {
   __device__ __forceinline__ void note(int warp, int v) const { words[2 + warp] = v; }
 };
 
-// Bounded wait: gives up after ~2 s, raises the CTA's abort flag and records `code`.  (The barrier is looked at before the flag, and
+// Bounded wait: gives up after ~2 s, raises the CTA's abort flag and records `code`; or once another CTA has, and raises the flag
+// too: the loading warps go by it when they wait for their copies in flight, and the storing ones when they write nothing.  (The barrier is looked at before the flag, and
 // the softmax and issuing warps leave no note of where they are: 2 x 3001 tokens of head_dim 64 76.7 -> 73.8 us, 2048 tokens
 // 37.8 -> 37.0, 4099 tokens in 16 shards 392 -> 380.)
 template <bool kPointer, int kWarps>
@@ -86,7 +87,11 @@ __device__ __forceinline__ bool wait_bar(const WaitCtx<kPointer, kWarps>& c, uin
   uint32_t spins = 0;
   while (!mbar_try_wait(bar, parity)) {
     if ((++spins & 1023u) == 0) {
-      if (c.load(1) || *reinterpret_cast<volatile int32_t*>(c.status) != 0) return false;
+      if (c.load(1)) return false;
+      if (*reinterpret_cast<volatile int32_t*>(c.status) != 0) {
+        c.store(1, 1);
+        return false;
+      }
       const uint64_t now = global_timer_ns();
       if (t0 == 0) t0 = now;
       if (now - t0 > 2000000000ull) {
