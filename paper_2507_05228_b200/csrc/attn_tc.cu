@@ -1231,10 +1231,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         }
         }
         if (n_run == 0 || !fed) {
-          if (leader) mma_commit(bar(O_FULL));
+          // Everything issued so far, at the barrier of the later sub-tile: that of the first may have had its one arrival already,
+          // when the wait for the other's last weights ran out, and would then say nothing of the products issued since.
+          const uint32_t done = bar(O_FULL + n_sub - 1);
+          if (leader) mma_commit(done);
           if (q_boxes)
             for (int s = 0; s < n_sub; ++s) landed(bar(Q_FULL + s), 0u);
-          landed(bar(O_FULL), 0u);
+          landed(done, 0u);
         }
       }
       __syncwarp();
