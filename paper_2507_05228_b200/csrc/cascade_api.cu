@@ -610,16 +610,17 @@ cascade_status_t cascade_plan_device_status(const cascade_plan_t* plan, int32_t*
     set_error("cascade_plan_device_status: null pointer or host-only plan");
     return CASCADE_ERR_INVALID_ARG;
   }
-  int32_t words[20] = {0};
+  int32_t words[kStatusWords] = {0};  // see WaitCtx
   cudaError_t e = cudaDeviceSynchronize();
   if (e == cudaSuccess) e = cudaMemcpy(words, plan->dev.status, sizeof(words), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "cascade_plan_device_status");
   *out_code = words[0];
   if (*out_code != 0) {
-    set_error("device status word = %d: a bounded wait inside a kernel gave up (block %d,%d,%d tile %d; warp progress "
-              "%d %d %d %d | %d %d %d %d | %d | %d %d %d)",
-              words[0], words[1], words[2], words[3], words[4], words[8], words[9], words[10], words[11], words[12],
-              words[13], words[14], words[15], words[16], words[17], words[18], words[19]);
+    char progress[12 * kMaxWaitWarps + 1];
+    int n = 0;
+    for (int w = 0; w < kMaxWaitWarps; ++w) n += snprintf(progress + n, sizeof(progress) - n, " %d", words[8 + w]);
+    set_error("device status word = %d: a bounded wait inside a kernel gave up (block %d,%d,%d tile %d; warp progress%s)", words[0],
+              words[1], words[2], words[3], words[4], progress);
     return CASCADE_ERR_TIMEOUT;
   }
   return CASCADE_OK;

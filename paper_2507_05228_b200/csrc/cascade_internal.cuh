@@ -16,6 +16,9 @@ namespace cascade {
 
 constexpr int kNumTileSizes = 4;  // query-tile heights 32, 64, 128, 256
 
+// The report of a wait that gave up, see WaitCtx: code, block, tile, and from word 8 on a progress word for each warp of the CTA.
+constexpr int kMaxWaitWarps = 20, kStatusWords = 8 + kMaxWaitWarps;
+
 // Device-side view of a plan.  All arrays have a leading n_maps dimension.
 struct PlanDev {
   const int32_t* q_off;
@@ -32,7 +35,7 @@ struct PlanDev {
   // One list per tile height: qtiles[i] holds tiles of up to (32 << i) slots.
   const int4* qtiles[kNumTileSizes];
   int32_t n_qtiles[kNumTileSizes];  // per map (padded to the maximum over maps)
-  int32_t* status;      // device status word, 0 = fine
+  int32_t* status;      // device status word, 0 = fine; kStatusWords of them
   int32_t n_maps, n_q, n_kv, n_q_shards, n_kv_shards, q_pos_offset, causal;
 };
 

@@ -53,7 +53,8 @@ __device__ __forceinline__ bool elect_one() {  // true in exactly one lane of a 
 template <bool kPointer, int kWarps>
 struct WaitCtx {
   uint32_t misc;
-  int32_t* status;  // global: [0] code, [1..3] block index, [4] tile of the waiter, [8..19] progress words
+  int32_t* status;  // global: [0] code, [1..3] block index, [4] tile of the waiter, [8..] progress words
+  static_assert(kWarps <= kMaxWaitWarps, "the status words end");
   __device__ __forceinline__ int load(int w) const {
     int v;
     asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(v) : "r"(misc + 4 * w) : "memory");
