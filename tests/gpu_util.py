@@ -84,8 +84,11 @@ def _check_routes_agree(o_f, o_m, w):
     assert excess <= 0, f"{w.name}: fused vs merge(partials): {diff.max().item():.3e}, {excess:.3e} over the bound"
 
 
-def full_parity(w, check_lse=True):
-    """Every element of partials, merge and the fused call against the oracle.  Returns the error triple."""
+def full_parity(w, check_lse=True, scratch=True):
+    """Every element of partials, merge and the fused call against the oracle.  Returns the error triple.  scratch=False: with a
+    workspace too small for copies of K and V, which heads of 64 columns take the ALU kernels with, one a call."""
+    ws = None if scratch else torch.empty(16, dtype=torch.uint8, device="cuda")
+    launches = cb.lib().cascade_launch_count
     q, k, v = to_device(w)
     plan = make_plan(w)
     oplan = oracle_plan(w)
@@ -94,14 +97,18 @@ def full_parity(w, check_lse=True):
     u, m, e = oracle.attn_pass(w.q, w.k, w.v, w.scale, oplan)
     o_ref, lse_ref = oracle.attention_unsharded(w.q, w.k, w.v, w.scale, causal=w.causal,
                                                 q_pos_offset=w.q_pos_offset)
-    o_part, m_part, l_part = cb.cascade_attn_partials(plan, q, k, v, w.scale)
+    n0 = launches()
+    o_part, m_part, l_part = cb.cascade_attn_partials(plan, q, k, v, w.scale, workspace=ws)
+    assert scratch or launches() - n0 == 1
     torch.cuda.synchronize()
     errs = check_partials((o_part.double().cpu().numpy(), m_part.double().cpu().numpy(),
                            l_part.double().cpu().numpy()), (u, m, e), w.tol, w.name + " partials")
     o_m, lse_m = cb.cascade_merge(o_part, m_part, l_part, plan.dev_ptr("q_idx"))
     e_merge = check_output(o_m, lse_m if check_lse else None, o_ref, lse_ref, w.tol, w.name + " merge",
                            stored_partials=True)
-    o_f, lse_f = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+    n0 = launches()
+    o_f, lse_f = cb.cascade_attn_sharded(plan, q, k, v, w.scale, workspace=ws)
+    assert scratch or launches() - n0 == 1
     e_fused = check_output(o_f, lse_f if check_lse else None, o_ref, lse_ref, w.tol, w.name + " fused")
     # both routes are within their bound of the exact result, hence within the sum of the bounds of each other
     _check_routes_agree(o_f, o_m, w)

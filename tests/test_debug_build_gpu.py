@@ -26,6 +26,21 @@ cases = [wl.config("c2_prefill_8b", n_q=512, n_kv=512, H=8, Hkv=2), wl.config("c
          wl.make_workload("dbg_chunk", 1, 96, 400, 8, 2, 128, "bf16", "random", "random", 3, 7, seed=96)]
 for w in cases:
     gu.full_parity(w)   # plan arrays, partials, merge, fused; asserts the status word is 0
+w = wl.make_workload("dbg_split", 8, 300, 300, 16, 8, 64, "f32", "random", "random", 3, 5, seed=97, symmetric=False)
+n0 = cb.lib().cascade_launch_count()
+gu.full_parity(w)       # fp32 on the tensor cores: two kernels for the partials and two for the fused call, and the merge
+assert cb.lib().cascade_launch_count() - n0 >= 5
+# a key and a value out of range: rows that see neither are untouched, those of plain fp32 arithmetic go through the indexes again
+q, k, v = gu.to_device(w)
+plan = gu.make_plan(w)
+o, _ = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+o = o.clone()
+k[:, 250, :, 3] = 2.0 ** 70
+v[:, 251, :, 3] = 2.0 ** 70
+o_far, _ = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+parts = cb.cascade_attn_partials(plan, q, k, v, w.scale)
+assert torch.equal(o_far[:, :192], o[:, :192]) and plan.device_status() == 0
+cases.append(w)
 print("debug build: %%d cases clean" %% len(cases))
 """
 

@@ -137,13 +137,25 @@ def test_fp32_host_call_with_any_workspace_that_holds_the_staging(gu):
     (1, 1, 2, 2, 64, 1, 1, "f32", True),          # one key
     (1, 300, 6, 2, 64, 2, 3, "bf16", True),       # one query row on the ALU route: key groups share the row
     (17, 33, 3, 1, 128, 1, 2, "f32", False),      # one row and one key more than a piece / a tile
-    (640, 640, 8, 8, 64, 8, 4, "f32", True),      # wide form: 64-row tiles, masked and unmasked 64-key tiles
+    (640, 640, 8, 8, 64, 8, 4, "f32", True),      # on the tensor cores; on the ALUs see the next test
     (512, 512, 4, 4, 128, 12, 4, "f32", False),   # wide form at head_dim 128
-    (300, 300, 8, 8, 64, 8, 60, "f32", True),     # five keys per shard: chunks of many shards in a tile
+    (300, 300, 8, 8, 64, 8, 60, "f32", True),     # the same, with five keys per shard
 ])
 def test_alu_kernel_forms(gu, n_q, n_kv, H, Hkv, d, B, shards, dtype, causal):
     gu.full_parity(wl.make_workload(f"alu_{n_q}_{d}", B, n_q, n_kv, H, Hkv, d, dtype, "random", "random",
                                     1 if n_q == 1 else shards, shards, seed=n_q + d, causal=causal))
+
+
+@pytest.mark.parametrize("n,H,Hkv,B,J,P,causal", [
+    (640, 8, 8, 8, 4, 4, True),     # wide form: 64-row tiles, masked and unmasked 64-key tiles
+    (512, 8, 8, 8, 4, 4, False),    # the same without a mask
+    (300, 8, 8, 8, 60, 60, True),   # partials a row at a time over five keys per shard; the fused call in the wide form
+    (64, 4, 2, 8, 64, 4, True),     # partials of one row per query shard: one row of a tile of 32
+])
+def test_alu_kernels_without_scratch(gu, n, H, Hkv, B, J, P, causal):
+    """fp32, heads of 64: problems that the tensor cores take when a caller brings the scratch, without it."""
+    w = wl.make_workload(f"alu_no_ws_{n}", B, n, n, H, Hkv, 64, "f32", "random", "random", J, P, seed=n + 1, causal=causal, symmetric=False)
+    gu.full_parity(w, scratch=False)
 
 
 @pytest.mark.parametrize("n_q,n_kv,P,causal", [(128, 128, 2, True), (129, 200, 2, True), (300, 900, 7, False), (40, 64, 64, True)])
@@ -170,7 +182,8 @@ def test_new_plans_have_the_same_arrays_on_the_device(gu, n_q, n_kv, P, causal):
 
 @pytest.mark.parametrize("n_q,n_kv,H,Hkv,d,B,J,P,dtype,causal", [
     (64, 64, 16, 16, 64, 1, 32, 32, "f32", True),     # partials of two rows and two keys each
-    (64, 64, 4, 2, 64, 8, 64, 4, "f32", True),        # fused route, one row per shard: one row of a tile of 32
+    (64, 64, 4, 2, 64, 8, 64, 4, "f32", True),        # one row per query shard: partials on the tensor cores, without scratch see above
+    (64, 64, 2, 2, 128, 1, 64, 1, "f32", True),       # fused route, a row at a time
     (333, 333, 8, 8, 64, 1, 32, 12, "f32", False),    # tiles of 10 rows, the last tile of a shard short of keys
     (130, 130, 12, 12, 64, 1, 40, 40, "bf16", True),  # heads of 64 in bf16: partials on the ALUs, the fused call on the tensor cores
     (128, 128, 8, 2, 128, 2, 128, 2, "f32", True),    # head_dim 128
@@ -178,7 +191,7 @@ def test_new_plans_have_the_same_arrays_on_the_device(gu, n_q, n_kv, P, causal):
     (300, 300, 4, 2, 128, 1, 290, 280, "bf16", True), # more shards than the tensor cores take, some of them empty
 ])
 def test_row_kernel_forms(gu, n_q, n_kv, H, Hkv, d, B, J, P, dtype, causal):
-    """Problems cut so fine that a query row at a time is the faster way."""
+    """Problems cut so fine that a query row at a time is the faster way for the partials.  (The fused call of most takes tiles of tokens.)"""
     gu.full_parity(wl.make_workload(f"rows_{n_q}_{d}", B, n_q, n_kv, H, Hkv, d, dtype, "random", "random", J, P, seed=n_q + d,
                                     causal=causal, symmetric=False, q_pos_offset=n_kv - n_q))
 

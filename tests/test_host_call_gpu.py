@@ -61,18 +61,25 @@ def test_host_call_matches_oracle_and_device_call(cb, gu, case):
     plan.destroy()
 
 
-def test_head_groups_take_the_form_of_the_whole_problem(cb, gu):
-    """512 fp32 tokens, 8 sequences, 8 heads: enough tiles for four row warps a block as a whole, not per head group.  The
-    host call computes the groups one by one and still gives the same bits as the device call."""
+@pytest.mark.parametrize("scratch", [True, False])
+def test_head_groups_take_the_form_of_the_whole_problem(cb, gu, scratch):
+    """512 fp32 tokens, 8 sequences, 8 heads: on the tensor cores; without the scratch on the ALUs, where as a whole, not per
+    head group, there are enough tiles for four row warps a block.  The host call computes the groups (of four heads) one by one and
+    still gives the same bits as the device call."""
     w = wl.make_workload("host_wide", 8, 512, 512, 8, 8, 64, "f32", "random", "random", 4, 4, seed=33)
     plan = gu.make_plan(w)
     hq, hk, hv = _host(w, w.q), _host(w, w.k), _host(w, w.v)
     ho = torch.empty_like(hq).pin_memory()
-    ws = torch.empty(cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED_HOST, cb.F32, w.B, w.H, w.Hkv, w.d), dtype=torch.uint8,
-                     device="cuda")
+    need = cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED_HOST, cb.F32, w.B, w.H, w.Hkv, w.d)
+    ws = torch.empty(need if scratch else 4 * hq.numel() * 4, dtype=torch.uint8, device="cuda")
+    n0 = cb.lib().cascade_launch_count()
     cb.cascade_attn_sharded_host(plan, hq, hk, hv, w.scale, ho, ws)
     torch.cuda.current_stream().synchronize()
+    assert cb.lib().cascade_launch_count() - n0 == (4 if scratch else 2)
     q, k, v = gu.to_device(w)
-    o_dev, _ = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+    o_dev, _ = cb.cascade_attn_sharded(plan, q, k, v, w.scale,
+                                       workspace=None if scratch else torch.empty(16, dtype=torch.uint8, device="cuda"))
     assert torch.equal(o_dev.cpu(), ho)
+    o_ref, _ = oracle.attention_unsharded(w.q, w.k, w.v, w.scale)
+    gu.check_output(ho.double().numpy(), None, o_ref, None, w.tol, "host call")
     plan.destroy()

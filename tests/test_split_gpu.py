@@ -229,3 +229,134 @@ def test_split_calls_on_a_plan_whose_status_word_is_set_write_nothing(gu):
     cb.cascade_attn_sharded(plan, q, k, v, w.scale, out=o, want_lse=False)
     assert torch.equal(o, o_ref) and plan.device_status() == 0
     plan.destroy()
+
+
+def _partials(cb, plan, q, k, v, scale):
+    """The partials with the workspace that they ask for; and how many kernels ran."""
+    n0 = cb.lib().cascade_launch_count()
+    parts = cb.cascade_attn_partials(plan, q, k, v, scale)
+    torch.cuda.synchronize()
+    return parts, cb.lib().cascade_launch_count() - n0
+
+
+@pytest.mark.parametrize("n_kv", [16, 64, 512])
+@pytest.mark.parametrize("signs", ["values", "queries and keys", "all"])
+def test_split_route_on_values_of_one_sign(gu, n_kv, signs):
+    """The tensor core cuts its sums off, which adds up where all products have one sign and one tile holds the keys.  Outputs, maxima
+    and sums are closer to fp64 than those of the ALU kernels all the same.  The logarithm of the row sum is 5 to 9 in size and
+    rounded to fp32, 2^-24 of it at most; the cut-off logits add as much at most."""
+    from paper_2507_05228_b200 import binding as cb
+    B, n_q, H, P = 16, 128, 16, 2
+    w = wl.make_workload(f"split_sign_{n_kv}", B, n_q, n_kv, H, H, 64, "f32", "random", "random", 2, P, seed=n_kv, causal=False, symmetric=False)
+    if signs != "values":
+        w.q, w.k = np.abs(w.q), np.abs(w.k)
+    if signs != "queries and keys":
+        w.v = np.abs(w.v)
+    q, k, v = gu.to_device(w)
+    plan = gu.make_plan(w)
+    o_ref, lse_ref = oracle.attention_unsharded(w.q, w.k, w.v, w.scale, causal=False)
+    refs = (o_ref, lse_ref) + oracle.attn_pass(w.q, w.k, w.v, w.scale, gu.oracle_plan(w))
+    err = {}
+    for ws in (True, False):
+        o, lse, n_kernels = _fused(cb, plan, q, k, v, w.scale, ws)
+        assert n_kernels == (2 if ws else 1)
+        n0 = cb.lib().cascade_launch_count()
+        parts = cb.cascade_attn_partials(plan, q, k, v, w.scale, workspace=None if ws else torch.empty(16, dtype=torch.uint8, device="cuda"))
+        torch.cuda.synchronize()
+        assert cb.lib().cascade_launch_count() - n0 == (2 if ws else 1)
+        err[ws] = [np.linalg.norm(a.double().cpu().numpy() - r) / np.linalg.norm(r) for a, r in zip((o, lse) + tuple(parts), refs)]
+    print(err)
+    assert all(a <= b for i, (a, b) in enumerate(zip(err[True], err[False])) if i != 1) and err[True][1] <= 2.0 ** -23, err
+    plan.destroy()
+
+
+def test_split_route_with_a_map_per_sequence(gu):
+    from paper_2507_05228_b200 import binding as cb
+    B, n, H, P = 8, 260, 16, 3
+    w = wl.make_workload("split_maps", B, n, n, H, H, 64, "f32", "random", "random", 1, 1, seed=41)
+    rng = np.random.default_rng(42)
+    q_of, kv_of = rng.integers(0, 2, (B, n)).astype(np.int32), rng.integers(0, P, (B, n)).astype(np.int32)
+    q, k, v = gu.to_device(w)
+    plan = cb.cascade_shard_plan(q_of, kv_of, 2, P)
+    o, lse, n_kernels = _fused(cb, plan, q, k, v, w.scale)
+    parts, n_parts = _partials(cb, plan, q, k, v, w.scale)
+    assert n_kernels == 2 and n_parts == 2 and plan.device_status() == 0
+    o_ref, lse_ref = oracle.attention_unsharded(w.q, w.k, w.v, w.scale)
+    gu.check_output(o, lse, o_ref, lse_ref, w.tol, "a map per sequence")
+    for b in range(B):
+        ref = oracle.attn_pass(w.q[b:b + 1], w.k[b:b + 1], w.v[b:b + 1], w.scale, oracle.shard_plan(q_of[b], kv_of[b], 2, P))
+        gu.check_partials(tuple(t[b:b + 1].double().cpu().numpy() for t in parts), ref, w.tol, f"a map per sequence, b={b}")
+    plan.destroy()
+
+
+def test_split_route_over_resident_rows(gu):
+    """Rows with positions of their own, a set of them per sequence; those that no query sees hold NaN."""
+    from paper_2507_05228_b200 import binding as cb
+    B, n, n_q, n_kv, H, off = 8, 600, 130, 300, 16, 300
+    rng = np.random.default_rng(43)
+    w = wl.make_workload("split_resident", B, n, n, H, H, 64, "f32", "random", "random", 1, 1, seed=44)
+    q, k, v = gu.to_device(w)
+    pos = np.sort(np.stack([rng.choice(n, n_kv, replace=False) for _ in range(B)]), axis=1).astype(np.int32)
+    q_of, kv_of = rng.integers(0, 2, (B, n_q)).astype(np.int32), rng.integers(0, 4, (B, n_kv)).astype(np.int32)
+    plan = cb.cascade_shard_plan_resident(q_of, kv_of, pos, 2, 4, off)
+    at = torch.from_numpy(pos.astype(np.int64)).cuda()
+    kr, vr = (torch.stack([t[b, at[b]] for b in range(B)]) for t in (k, v))
+    for b in range(B):
+        kr[b, at[b] > off + n_q - 1] = float("nan")
+        vr[b, at[b] > off + n_q - 1] = float("nan")
+    qr = q[:, off:off + n_q]
+    o, lse, n_kernels = _fused(cb, plan, qr, kr, vr, w.scale)
+    parts, n_parts = _partials(cb, plan, qr, kr, vr, w.scale)
+    assert n_kernels == 2 and n_parts == 2 and plan.device_status() == 0
+    seen = at[:, None, :] <= torch.arange(off, off + n_q, device="cuda")[None, :, None]
+    s = torch.einsum("bqhd,bkhd->bhqk", qr.double(), kr.double().nan_to_num(0.0)) * float(np.float32(w.scale))
+    s = s.masked_fill(~seen[:, None], -torch.inf)
+    o_ref = torch.einsum("bhqk,bkhd->bqhd", torch.softmax(s, -1), vr.double().nan_to_num(0.0)).cpu().numpy()
+    lse_ref = torch.logsumexp(s, -1).transpose(1, 2).cpu().numpy()
+    gu.check_output(o, lse, o_ref, lse_ref, w.tol, "resident rows")
+    merged, _ = cb.cascade_merge(*parts, plan.dev_ptr("q_idx"), n_q)
+    gu.check_output(merged, None, o_ref, None, w.tol, "resident rows, merged")
+    plan.destroy()
+
+
+@pytest.mark.parametrize("form", ["columns of one tensor", "keys and values of one sequence for all"])
+def test_split_route_on_strided_and_expanded_rows(gu, form):
+    from paper_2507_05228_b200 import binding as cb
+    B, n, H, Hkv = 8, 200, 16, 8
+    w = wl.make_workload("split_strides", B, n, n, H, Hkv, 64, "f32", "random", "random", 3, 3, seed=45)
+    if form == "columns of one tensor":
+        rows = torch.full((B, n, H + 2 * Hkv + 1, 64), float("nan"), device="cuda")
+        q, k, v = rows[:, :, :H], rows[:, :, H:H + Hkv], rows[:, :, H + Hkv:H + 2 * Hkv]
+        for t, src in zip((q, k, v), gu.to_device(w)):
+            t.copy_(src)
+    else:
+        w.k, w.v = (np.broadcast_to(a[:1], a.shape).copy() for a in (w.k, w.v))
+        q, k, v = gu.to_device(w)
+        k, v = k[:1].expand(B, -1, -1, -1), v[:1].expand(B, -1, -1, -1)
+    plan = gu.make_plan(w)
+    need = cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED, cb.F32, B, H, Hkv, 64)
+    n0 = cb.lib().cascade_launch_count()
+    o, lse = cb.cascade_attn_sharded(plan, q, k, v, w.scale)
+    assert need > 0 and cb.lib().cascade_launch_count() - n0 == 2
+    parts, n_parts = _partials(cb, plan, q, k, v, w.scale)
+    assert n_parts == 2
+    gu.check_output(o, lse, *oracle.attention_unsharded(w.q, w.k, w.v, w.scale), w.tol, form)
+    gu.check_partials(tuple(t.double().cpu().numpy() for t in parts), oracle.attn_pass(w.q, w.k, w.v, w.scale, gu.oracle_plan(w)), w.tol, form)
+    plan.destroy()
+
+
+def test_split_route_from_host_buffers(gu):
+    """The head groups of the host call, two kernels each, against the oracle."""
+    from paper_2507_05228_b200 import binding as cb
+    B, n, H = 8, 300, 16
+    w = wl.make_workload("split_host", B, n, n, H, H, 64, "f32", "random", "random", 3, 3, seed=46)
+    plan = gu.make_plan(w)
+    hq, hk, hv = (torch.from_numpy(a).pin_memory() for a in (w.q, w.k, w.v))
+    ho = torch.empty_like(hq).pin_memory()
+    ws = torch.empty(cb.cascade_workspace_bytes(plan, cb.CALL_SHARDED_HOST, cb.F32, B, H, H, 64), dtype=torch.uint8, device="cuda")
+    n0 = cb.lib().cascade_launch_count()
+    cb.cascade_attn_sharded_host(plan, hq, hk, hv, w.scale, ho, ws)
+    torch.cuda.synchronize()
+    assert cb.lib().cascade_launch_count() - n0 == 2 * H // 4  # four heads at a time
+    gu.check_output(ho.double().numpy(), None, oracle.attention_unsharded(w.q, w.k, w.v, w.scale)[0], None, w.tol, "host buffers")
+    plan.destroy()
