@@ -578,12 +578,16 @@ __global__ void __launch_bounds__(256, 3 - kAhead) decode_fused_kernel(const __g
 }
 
 template <int G, int kAhead>
-static cudaError_t launch_fused(const AttnParams& p, const DecodeStep& step, int n_cta, cudaStream_t stream) {
+static cudaError_t launch_fused(const AttnParams& p, const DecodeStep& step, int64_t blocks, int n_cta, cudaStream_t stream) {
   // One list: for as many keys as there are, whatever is visible when the launch runs (every shard may end in a block that is not
   // full, and in the interleaved order the list is a quarter longer).  Up to ten blocks a warp: beyond, the few registers that it
-  // costs the walk weigh more (2 sequences of 16384 tokens, 32 / 8 heads, 34.5 us, from the table 32.4).
+  // costs the walk weigh more (2 sequences of 16384 tokens, 32 / 8 heads, 34.5 us, from the table 32.4).  With four and eight
+  // heads and one block ahead they do from the second block on (table -> list, us, 32 / 8 heads: 2 sequences of 1200 keys 9.6 ->
+  // 9.2, of 3000 12.5 -> 12.8, of 6500 18.3 -> 19.0; 4 of 700 9.8 -> 9.4, of 1200 11.2 -> 11.7, of 6500 22.7 -> 24.3); with one and
+  // two heads the walk from the table spills more (4 sequences of 3000 keys, 16 / 8 heads, 16.3 -> 14.6).
   const int P = p.plan.n_kv_shards;
-  const bool one_list = P <= 32 && ((p.plan.n_kv + 15) / 16 + P) * (int64_t)5 / 4 + 1 <= 10 * (int64_t)n_cta * 8;
+  const bool one_list = P <= 32 && ((p.plan.n_kv + 15) / 16 + P) * (int64_t)5 / 4 + 1 <= 10 * (int64_t)n_cta * 8 &&
+                        (kAhead == 2 || G <= 2 || blocks <= 8 * n_cta);
   auto kernel = one_list ? decode_fused_kernel<G, kAhead, true> : decode_fused_kernel<G, kAhead, false>;
   if (n_cta > 8) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -672,7 +676,8 @@ cudaError_t launch_decode_fused(const AttnParams& p, const DecodeStep& step, int
   const bool two_ahead = blocks > 8 * n_cta && (int64_t)p.Hkv * p.batch <= clusters_alone(n_cta);
   TimedLaunch timed(stream);
   return with_group(p.G, [&](auto g) {
-    return two_ahead ? launch_fused<decltype(g)::value, 2>(p, step, n_cta, stream) : launch_fused<decltype(g)::value, 1>(p, step, n_cta, stream);
+    return two_ahead ? launch_fused<decltype(g)::value, 2>(p, step, blocks, n_cta, stream)
+                     : launch_fused<decltype(g)::value, 1>(p, step, blocks, n_cta, stream);
   });
 }
 

@@ -25,6 +25,8 @@ def gu():
     (1, 45000, 16, 8, 5, "random", 44990),    # more than 32 blocks a warp: the list is made a second time
     (3, 3000, 8, 4, 8, "random", 2999),       # 12 KV heads and sequences: their clusters do not all get an SM for each CTA
     (2, 12000, 32, 8, 8, "random", 11999),    # ten CTAs of eight warps a pair, from the table
+    (2, 1280, 32, 8, 8, "random", 1279),      # four heads, one block ahead: a block a warp, listed
+    (2, 1281, 64, 8, 8, "random", 1280),      # eight heads: a block more, from the table
     (1, 17, 4, 1, 2, "contiguous", 16),       # two blocks, one of them a single key
     (3, 200, 2, 2, 32, "random", 3),          # four keys in all, most shards empty
 ])
