@@ -1027,8 +1027,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         if (!quiet) store_rows(o_scale, n_tiles > 0, b * P + max(kk_open, 0), dst);
         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the rows have left shared memory
       } else {
-        // Every product of the CTA has completed, so the Q / K tiles in shared memory are free: the thread stages its
-        // output row there (rows 16 bytes further apart than they are long, which spreads a warp's accesses over all banks)
+        // The products Q K^T of the CTA have completed, those of the other sub-tile among them: its last one is issued before this
+        // sub-tile's last product with V, and a commit waits for all that was issued before it.  So the Q and K tiles in shared
+        // memory are free (V may still be read, and is not touched): the thread stages its output row there (rows 16 bytes further apart than they are long, which spreads a warp's accesses over all banks)
         // and the warp stores whole rows, 512 bytes per instruction.  (A bulk copy per row took 2200 cycles to issue; boxes as
         // with kWalk are issued once here, and the first use of a tensor map costs more: 2048 tokens 43.6 -> 45.0 us.)
         uint8_t* stage = smem + C::kOffStage + (s * kM + m) * C::kStageRowBytes;
