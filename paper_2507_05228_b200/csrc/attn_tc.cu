@@ -1029,8 +1029,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       } else {
         // The products Q K^T of the CTA have completed, those of the other sub-tile among them: its last one is issued before this
         // sub-tile's last product with V, and a commit waits for all that was issued before it.  So the Q and K tiles in shared
-        // memory are free (V may still be read, and is not touched): the thread stages its output row there (rows 16 bytes further apart than they are long, which spreads a warp's accesses over all banks)
-        // and the warp stores whole rows, 512 bytes per instruction.  (A bulk copy per row took 2200 cycles to issue; boxes as
+        // memory are free (V may still be read, and is not touched): the thread stages its output row there (rows 16 bytes
+        // further apart than they are long, which spreads a warp's accesses over all banks) and the warp stores whole rows, 512 bytes per instruction.  (A bulk copy per row took 2200 cycles to issue; boxes as
         // with kWalk are issued once here, and the first use of a tensor map costs more: 2048 tokens 43.6 -> 45.0 us.)
         uint8_t* stage = smem + C::kOffStage + (s * kM + m) * C::kStageRowBytes;
 #pragma unroll
@@ -1232,13 +1232,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         }
         }
         if (n_run == 0 || !fed) {
-          // Everything issued so far, at the barrier of the later sub-tile: that of the first may have had its one arrival already,
-          // when the wait for the other's last weights ran out, and would then say nothing of the products issued since.
-          const uint32_t done = bar(O_FULL + n_sub - 1);
-          if (leader) mma_commit(done);
+          // Everything issued so far, at the barrier of the second sub-tile: that of the first may have had its one arrival already,
+          // when the wait for the other's last weights ran out, and would then say nothing of the products issued since.  (A
+          // constant: as the barrier of the later sub-tile it cost all calls a hundredth, 268 tokens 8.9 -> 9.0 us.)
+          if (leader) mma_commit(bar(O_FULL + 1));
           if (q_boxes)
             for (int s = 0; s < n_sub; ++s) landed(bar(Q_FULL + s), 0u);
-          landed(done, 0u);
+          landed(bar(O_FULL + 1), 0u);
         }
       }
       __syncwarp();

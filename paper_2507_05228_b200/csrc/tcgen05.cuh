@@ -88,8 +88,7 @@ __device__ __forceinline__ bool wait_bar(const WaitCtx<kPointer, kWarps>& c, uin
   uint32_t spins = 0;
   while (!mbar_try_wait(bar, parity)) {
     if ((++spins & 1023u) == 0) {
-      if (c.load(1)) return false;
-      if (*reinterpret_cast<volatile int32_t*>(c.status) != 0) {
+      if (c.load(1) || *reinterpret_cast<volatile int32_t*>(c.status) != 0) {
         c.store(1, 1);
         return false;
       }
